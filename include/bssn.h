@@ -183,11 +183,13 @@ bssn_status_t bssn_rk4_stage(const bssn_grid_t* grid, const bssn_params_t* param
 
 /* The two halves of bssn_rk4_stage, for callers that schedule or time them
  * separately (the paper's split of "RHS derivatives" from the rest, Sec. 2.4.1):
- * bssn_diff_tables fills the first-difference tables in `work` from `state`;
- * bssn_rk4_stage_fused then runs the fused right-hand side + dissipation +
- * stage update reading those tables, which must have been made from the same
- * ys with the same grid and fd_order (no check is possible). Same argument
- * rules as bssn_rk4_stage. */
+ * bssn_diff_tables prepares `work` from `state` (the single-precision copy
+ * and derivative tables of the FP32-RHS form; the FP64 form has nothing to
+ * prepare, its stage makes its derivatives tile by tile);
+ * bssn_rk4_stage_fused then runs the right-hand side + dissipation + stage
+ * update on a `work` that must have been prepared from the same ys with the
+ * same grid and fd_order (no check is possible). Same argument rules as
+ * bssn_rk4_stage. */
 bssn_status_t bssn_diff_tables(const bssn_grid_t* grid, const bssn_params_t* params, bssn_precision_t prec,
                                const double* state, void* work, unsigned long long work_bytes, void* stream);
 bssn_status_t bssn_rk4_stage_fused(const bssn_grid_t* grid, const bssn_params_t* params, bssn_precision_t prec,
@@ -274,14 +276,13 @@ typedef struct {
 } bssn_block_t;
 
 /* Builds a plan for nblocks patches (params and precision shared by all).
- * The plan allocates and owns, per patch, three stage buffers and its
- * difference tables, plus the patch table and one CUDA graph per step size
- * (about 3 + 2*11*p/2*8/(24*8) state copies per patch in FP64). autotune = 1
- * times every candidate tile shape of the fused stage kernel on one
- * representative patch per size class and keeps the fastest (cached per
- * process by size class, order and precision); autotune = 0 uses runs of 128
- * consecutive points. Synchronizes the device. Returns BSSN_ERR_NOMEM if an
- * allocation fails (nothing is leaked). */
+ * The plan allocates and owns, per patch, three stage buffers (and in the
+ * FP32-RHS form a single-precision copy and derivative tables), plus the
+ * patch table, one CUDA graph per step size and, in FP64, the derivative
+ * record of up to 2048 tiles (1.1 GB). The stage kernels' tiles are fixed in
+ * both precisions (8 x 8 x 8 points in FP64, 8 x 4 x 4 in FP32-RHS), so
+ * autotune (0 or 1) has nothing to choose. Synchronizes the device. Returns
+ * BSSN_ERR_NOMEM if an allocation fails (nothing is leaked). */
 bssn_status_t bssn_plan_create(bssn_plan_t** out, const bssn_block_t* blocks, int nblocks,
                                const bssn_params_t* params, bssn_precision_t prec, int autotune);
 
@@ -293,8 +294,7 @@ bssn_status_t bssn_batch_step(bssn_plan_t* plan, double dt, void* stream);
 
 /* Interior points and stage tiles of the plan (HOST outputs, nullable); shapes
  * (HOST, nullable, nblocks entries) receives each patch's tile shape index:
- * 0 = runs of 128 consecutive points, 1..6 = (32,4,1) (16,8,1) (8,8,2)
- * (32,2,2) (16,4,2) (8,4,4). */
+ * 0 = the FP64 form's 8 x 8 x 8 tiles, 6 = the FP32-RHS form's 8 x 4 x 4. */
 bssn_status_t bssn_plan_info(const bssn_plan_t* plan, long long* points, long long* tiles, int* shapes);
 
 /* Frees everything the plan owns (synchronizes the device). */
@@ -385,8 +385,9 @@ typedef struct {
 } bssn_amr_desc_t;
 
 /* Builds the hierarchy's ghost/restriction maps and allocates, per patch,
- * three stage buffers (five on levels that have a finer level) and the
- * difference tables. The caller keeps ownership of every state and
+ * three stage buffers (five on levels that have a finer level), in the
+ * FP32-RHS form a single-precision copy and derivative tables, and in FP64
+ * one derivative record for all levels. The caller keeps ownership of every state and
  * ghost_src, which must stay valid until bssn_amr_destroy. Synchronizes.
  * BSSN_ERR_NOMEM if the device allocations fail. */
 bssn_status_t bssn_amr_create(bssn_amr_t** out, const bssn_amr_patch_t* patches, int npatches,

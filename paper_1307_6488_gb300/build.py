@@ -20,6 +20,7 @@ UNITS = [
     ("bssn_api.cu", "bssn_api.o", []),
     ("bssn_order.cu", "bssn_order4.o", ["-DBSSN_ORDER=4"]),
     ("bssn_order.cu", "bssn_order8.o", ["-DBSSN_ORDER=8"]),
+    ("bssn_stage64.cu", "bssn_stage64.o", []),
     ("bssn_stage32.cu", "bssn_stage32_4.o", ["-DBSSN_ORDER=4"]),
     ("bssn_stage32.cu", "bssn_stage32_8.o", ["-DBSSN_ORDER=8"]),
     ("bssn_noalloc.cu", "bssn_noalloc.o", []),

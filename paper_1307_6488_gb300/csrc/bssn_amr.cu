@@ -511,11 +511,10 @@ struct DevList {
 struct Level {
   std::vector<int> ids;         // global patch indices, input order
   bool parent = false;
-  PatchDev* dev = nullptr;      // level table for the tile kernels
-  long long* d_tile0 = nullptr;
+  FxTable fx;                   // FP64 form: the level's patches as the stage kernels see them
   long long* d_ext0 = nullptr;
   long long* d_pad0 = nullptr;
-  long long ntiles = 0, next = 0, npad = 0, points = 0;
+  long long next = 0, npad = 0, points = 0;
   DevList<CopyEntry> copy;
   DevList<StaticEntry> stat;
   DevList<ProlongEntry> pro;    // ghosts of this level from level - 1
@@ -554,7 +553,9 @@ struct bssn_amr {
   double* X1 = nullptr;         // separable prolongation scratch, shared by the levels
   double* X2 = nullptr;
   std::vector<void*> allocations;
-  int grid_stage = 0, grid_other = 0;
+  int grid_other = 0;
+  double* rec = nullptr;        // FP64 form: the derivative record all levels share
+  long long rec_slots = 0;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   cudaStream_t cap = nullptr;
@@ -762,21 +763,6 @@ cudaError_t fill(bssn_amr* A, int l, int which, int m, int s, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-template <int PO, typename R>
-void stage_level(bssn_amr* A, Level& L, const RK& rk, int in, int out, cudaStream_t s) {
-  const unsigned int g = (unsigned int)std::max<long long>(1, std::min<long long>(A->grid_stage, L.ntiles));
-  kb_stage<PO, R><<<g, TILE_THREADS, 0, s>>>(L.dev, L.d_tile0, (int)L.ids.size(), L.ntiles, A->gz, rk, in, out);
-  ++A->nodes;
-}
-
-template <int PO, typename R>
-void diffs_level(bssn_amr* A, Level& L, int which, cudaStream_t s) {
-  const unsigned int g = (unsigned int)std::max<long long>(
-      1, std::min<long long>(A->grid_other, (L.next + 255) / 256));
-  kb_diffs<PO, R><<<g, 256, 0, s>>>(L.dev, L.d_ext0, (int)L.ids.size(), L.next, which);
-  ++A->nodes;
-}
-
 cudaError_t compute_stage(bssn_amr* A, Level& L, const RK& rk, int in, int out, cudaStream_t s) {
   if (A->prec == BSSN_FP32_RHS) {
     // the single grids' TMA-tiled kernel over the level's patches (one spacing)
@@ -793,14 +779,9 @@ cudaError_t compute_stage(bssn_amr* A, Level& L, const RK& rk, int in, int out, 
     A->nodes += 3;
     return e;
   }
-  if (A->order == 4) {
-    diffs_level<4, double>(A, L, in, s);
-    stage_level<4, double>(A, L, rk, in, out, s);
-  } else {
-    diffs_level<8, double>(A, L, in, s);
-    stage_level<8, double>(A, L, rk, in, out, s);
-  }
-  return cudaGetLastError();
+  const cudaError_t e = fx_stage(A->order, L.fx, A->rec, A->rec_slots, A->gz, rk, in, out, s);
+  A->nodes += 2 * ((L.fx.ntiles + A->rec_slots - 1) / A->rec_slots);
+  return e;
 }
 
 // advance(l, m) of the Berger-Oliger recursion, enqueued on stream s.
@@ -960,15 +941,7 @@ bssn_status_t bssn_amr_create(bssn_amr_t** out, const bssn_amr_patch_t* patches,
     for (int k = 1; k < 6 && e == cudaSuccess; ++k)
       if (D.buf[k] && k != 3) e = cudaMemcpy(D.buf[k], P.state, nd * sizeof(double), cudaMemcpyDeviceToDevice);
     if (e == cudaSuccess) e = cudaMemset(D.buf[3], 0, nd * sizeof(double));
-    const int Hh = A->order / 2;
-    if (e != cudaSuccess) break;
-    if (prec == BSSN_FP64) {
-      const size_t tab = (size_t)NM * Hh * P.var_stride;
-      e = amr_alloc(A, 2 * tab * sizeof(double), &p);
-      if (e != cudaSuccess) break;
-      D.dX = p;
-      D.dY = (char*)p + tab * sizeof(double);
-    } else {
+    if (prec == BSSN_FP32_RHS) {
       // single-precision copy and D_x / D_y tables in Layout32 (tiled kernel)
       const Layout32 L32 = make_layout32(G);
       e = amr_alloc(A, (size_t)(NV + 2 * NM) * L32.vs * sizeof(float), &p);
@@ -982,13 +955,6 @@ bssn_status_t bssn_amr_create(bssn_amr_t** out, const bssn_amr_patch_t* patches,
         e = cudaErrorInvalidValue;
         break;
       }
-    }
-    if (A->order == 4) {
-      D.c64 = make_coef<4, double>(G, params->ko_eps);
-      D.c32 = make_coef<4, float>(G, params->ko_eps);
-    } else {
-      D.c64 = make_coef<8, double>(G, params->ko_eps);
-      D.c32 = make_coef<8, float>(G, params->ko_eps);
     }
     A->updates += D.L.npts << P.level;
   }
@@ -1052,34 +1018,26 @@ bssn_status_t bssn_amr_create(bssn_amr_t** out, const bssn_amr_patch_t* patches,
   for (int l = 0; l < nlev && e == cudaSuccess && nested; ++l) {
     Level& L = A->lev[l];
     const int nl = (int)L.ids.size();
-    std::vector<PatchDev> tab(nl);
-    std::vector<long long> t0(nl), e0(nl), p0(nl);
-    long long nt = 0, ne = 0, npd = 0;
+    std::vector<FxGrid> tab;
+    std::vector<long long> e0(nl), p0(nl);
+    long long ne = 0, npd = 0;
     for (int i = 0; i < nl; ++i) {
-      PatchDev D = A->host[L.ids[i]];
-      D.tx = D.ty = D.tz = 0;  // linear runs of 128 points
-      const long long n = tiles_of(D.L, 0, 0, 0, &D.ntx, &D.nty);
-      D.tile0 = t0[i] = nt;
-      nt += n;
-      D.ext0 = e0[i] = ne;
+      const PatchDev& D = A->host[L.ids[i]];
+      e0[i] = ne;
       ne += (long long)D.L.nx * (D.L.ny + 2 * Hh) * (D.L.nz + 2 * Hh);
-      D.pad0 = p0[i] = npd;
+      p0[i] = npd;
       npd += (D.L.nx + 2LL * g) * (D.L.ny + 2LL * g) * (D.L.nz + 2LL * g);
       L.points += D.L.npts;
-      tab[i] = D;
+      if (prec == BSSN_FP64) {
+        const bssn_grid_t G{D.L.nx, D.L.ny, D.L.nz, g, L.h[0], L.h[1], L.h[2], D.L.vs};
+        tab.push_back(fx_grid(G, A->order, params->ko_eps, D.buf));
+      }
     }
-    L.ntiles = nt;
     L.next = ne;
     L.npad = npd;
-    e = amr_alloc(A, sizeof(PatchDev) * nl, &p);
-    if (e == cudaSuccess) {
-      L.dev = (PatchDev*)p;
-      e = cudaMemcpy(L.dev, tab.data(), sizeof(PatchDev) * nl, cudaMemcpyHostToDevice);
-    }
-    if (e == cudaSuccess) e = amr_alloc(A, sizeof(long long) * nl, &p);
-    if (e == cudaSuccess) {
-      L.d_tile0 = (long long*)p;
-      e = cudaMemcpy(p, t0.data(), sizeof(long long) * nl, cudaMemcpyHostToDevice);
+    if (prec == BSSN_FP64) {
+      e = fx_upload(tab, &L.fx, [&](size_t n, void** q) { return amr_alloc(A, n, q); });
+      A->rec_slots = std::max(A->rec_slots, std::min(FX_MAX_SLOTS, L.fx.ntiles));
     }
     if (e == cudaSuccess) e = amr_alloc(A, sizeof(long long) * nl, &p);
     if (e == cudaSuccess) {
@@ -1121,18 +1079,14 @@ bssn_status_t bssn_amr_create(bssn_amr_t** out, const bssn_amr_patch_t* patches,
   if (e == cudaSuccess && nested && prec == BSSN_FP32_RHS)
     e = A->order == 4 ? stage32_batch_init<4>() : stage32_batch_init<8>();
   if (e == cudaSuccess && nested) e = cudaStreamCreateWithFlags(&A->cap, cudaStreamNonBlocking);
-  int dev = 0, sms = 0, occ = 1;
+  if (e == cudaSuccess && nested && prec == BSSN_FP64) {
+    e = amr_alloc(A, (size_t)A->rec_slots * FX_SLOT_DOUBLES * sizeof(double), &p);
+    A->rec = (double*)p;
+    if (e == cudaSuccess) e = A->order == 4 ? derivs_init<4>() : derivs_init<8>();
+  }
+  int dev = 0, sms = 0;
   if (e == cudaSuccess && nested) e = cudaGetDevice(&dev);
   if (e == cudaSuccess && nested) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess && nested) {
-    if (A->order == 4)
-      e = prec == BSSN_FP64 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kb_stage<4, double>, TILE_THREADS, 0)
-                            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kb_stage<4, float>, TILE_THREADS, 0);
-    else
-      e = prec == BSSN_FP64 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kb_stage<8, double>, TILE_THREADS, 0)
-                            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kb_stage<8, float>, TILE_THREADS, 0);
-  }
-  A->grid_stage = std::max(1, occ) * std::max(1, sms);
   A->grid_other = 8 * std::max(1, sms);
   A->geo = H;
   if (e != cudaSuccess || !nested) {

@@ -64,8 +64,9 @@ bool params_ok(const bssn_grid_t* G, const bssn_params_t* P) {
 
 // Scratch layout, one size for both precisions:
 //   [tables region][constraint partials][finals + flag]
-// The tables region holds, for BSSN_FP64, the double difference tables
-// (2 x 11 x p/2 arrays of var_stride doubles); for BSSN_FP32_RHS, two single
+// The tables region holds 2 x 11 x p/2 arrays of var_stride doubles: for
+// BSSN_FP64 stages the derivative record (as many tiles at a time as fit),
+// for the constraints the difference tables; for BSSN_FP32_RHS, two single
 // precision copies of the state (24 x var_stride floats each: a whole step
 // alternates between them) followed by the single precision tables.
 constexpr int RMS_BLOCKS = 304, RMS_THREADS = 256;
@@ -94,13 +95,13 @@ WorkLayout work_layout(const bssn_grid_t& G, const bssn_params_t& P) {
 }
 
 struct WorkPtrs {
-  void* dX;       // difference tables (FP64 form)
-  void* dY;
   float* f32;     // single-precision state copy (FP32 form, Layout32)
   float* f32b;    // a second one (the next stage's input, written by the stage before)
   float* tab32;   // D_x then D_y tables of the 11 mixed variables (FP32 form, Layout32)
-  double* dX64;   // double tables (constraints)
+  double* dX64;   // double difference tables (constraints)
   double* dY64;
+  double* rec;    // derivative record (FP64 form)
+  size_t rec_doubles;
   double* part;
   double* finals;
   unsigned int* flag;
@@ -114,18 +115,17 @@ WorkPtrs work_ptrs(void* work, const bssn_grid_t& G, const bssn_params_t& P, bss
   const size_t H = P.fd_order / 2;
   w.dX64 = base;
   w.dY64 = base + NM * H * L.vs;
+  w.rec = base;
+  w.rec_doubles = W.tables;
   if (prec == BSSN_FP64) {
     w.f32 = nullptr;
     w.f32b = nullptr;
     w.tab32 = nullptr;
-    w.dX = w.dX64;
-    w.dY = w.dY64;
   } else {
     const Layout32 L32 = make_layout32(G);
     w.f32 = (float*)base;
     w.f32b = w.f32 + (size_t)NV * L32.vs;
     w.tab32 = w.f32b + (size_t)NV * L32.vs;
-    w.dX = w.dY = nullptr;
   }
   w.part = base + W.tables;
   w.finals = w.part + W.partials;
@@ -133,19 +133,22 @@ WorkPtrs work_ptrs(void* work, const bssn_grid_t& G, const bssn_params_t& P, bss
   return w;
 }
 
-// Difference tables of ys (for the FP32 form: first the single-precision
-// copy, then its D_x / D_y tables).
+// What a stage needs before its fused part: for the FP32 form the
+// single-precision copy of ys and its D_x / D_y tables, for the FP64 form
+// nothing (the fused part makes its derivatives tile by tile).
 cudaError_t run_diffs(int order, bssn_precision_t prec, const bssn_grid_t& G, const double* ys, const WorkPtrs& w,
                       cudaStream_t s) {
+  if (prec == BSSN_FP64) return cudaSuccess;
+  const Layout32 L32 = make_layout32(G);
+  cudaError_t e = launch_to_f32t(make_layout(G), L32, ys, w.f32, s);
+  if (e != cudaSuccess) return e;
+  return order == 4 ? launch_d1tab32<4>(L32, G, w.f32, w.tab32, s) : launch_d1tab32<8>(L32, G, w.f32, w.tab32, s);
+}
+
+// Difference tables of the constraints and Weyl scalars.
+cudaError_t run_tables64(int order, const bssn_grid_t& G, const double* u, const WorkPtrs& w, cudaStream_t s) {
   const Layout L = make_layout(G);
-  if (prec == BSSN_FP32_RHS) {
-    const Layout32 L32 = make_layout32(G);
-    cudaError_t e = launch_to_f32t(L, L32, ys, w.f32, s);
-    if (e != cudaSuccess) return e;
-    return order == 4 ? launch_d1tab32<4>(L32, G, w.f32, w.tab32, s) : launch_d1tab32<8>(L32, G, w.f32, w.tab32, s);
-  }
-  return order == 4 ? launch_diffs<4>(L, G, prec, ys, w.dX, w.dY, s)
-                    : launch_diffs<8>(L, G, prec, ys, w.dX, w.dY, s);
+  return order == 4 ? launch_diffs<4>(L, u, w.dX64, w.dY64, s) : launch_diffs<8>(L, u, w.dX64, w.dY64, s);
 }
 
 // The tiled FP32-RHS stage on the single-precision copy ys32 and the tables
@@ -165,11 +168,24 @@ cudaError_t run_fused(int order, bssn_precision_t prec, const bssn_grid_t& G, co
                       const double* ys, const double* y0, double* acc, double* out, const WorkPtrs& w, int mode,
                       cudaStream_t s) {
   if (prec == BSSN_FP32_RHS) return fused32(order, G, P, rk, ys, w.f32, y0, acc, out, nullptr, w.tab32, mode, s);
-  const Layout L = make_layout(G);
-  const Gauge gz = make_gauge(P);
-  StageArgs A{(const void*)ys, ys, y0, acc, out, w.dX, w.dY};
-  if (order == 4) return launch_stage<4>(L, G, P.ko_eps, prec, gz, rk, A, mode, s);
-  return launch_stage<8>(L, G, P.ko_eps, prec, gz, rk, A, mode, s);
+  const double eps = mode == 0 ? P.ko_eps : 0.0;  // the right-hand side alone has no dissipation
+  FxWork W{};
+  W.one.L = make_layout(G);
+  W.one.C = order == 4 ? make_fx<4>(G, eps) : make_fx<8>(G, eps);
+  W.one.T = fx_tiles(G.nx, G.ny, G.nz);
+  W.one.buf[0] = const_cast<double*>(y0);
+  W.one.buf[1] = const_cast<double*>(ys);
+  W.one.buf[2] = out;
+  W.one.buf[3] = acc;
+  W.rec = w.rec;
+  const int vol = W.one.T.vol;
+  W.slot = (long long)REC_RHS * vol;
+  // the scratch always holds a tile: its halo alone outweighs the record of
+  // a small one, and p/2 tables of a large grid the record of 512 points
+  const long long slots = (long long)(w.rec_doubles / (size_t)W.slot);
+  const long long ntiles = (long long)W.one.T.ntx * W.one.T.nty * W.one.T.ntz;
+  const StageOut S{mode, make_gauge(P), rk, 1, 2, out};
+  return launch_stage64(order, W, vol, ntiles, slots, S.gz, S, s);
 }
 
 cudaError_t run_stage(int order, bssn_precision_t prec, const bssn_grid_t& G, const bssn_params_t& P, const RK& rk,
@@ -488,7 +504,8 @@ bssn_status_t bssn_bounds_violations(unsigned long long* count, void* stream) {
   cudaError_t e = cudaStreamSynchronize((cudaStream_t)stream);
   unsigned long long total = 0, c = 0;
   cudaError_t (*takes[])(unsigned long long*) = {bounds_take_local,       bounds_take_order<4>, bounds_take_order<8>,
-                                                 bounds_take_stage32<4>, bounds_take_stage32<8>, bounds_take_batch,
+                                                 bounds_take_stage32<4>, bounds_take_stage32<8>, bounds_take_stage64,
+                                                 bounds_take_batch,
                                                  bounds_take_amr,        bounds_take_cfd};
   for (auto take : takes) {
     if (e != cudaSuccess) break;
@@ -714,7 +731,7 @@ bssn_status_t bssn_psi4(const bssn_grid_t* grid, const bssn_params_t* params, co
   const WorkPtrs w = work_ptrs(work, *grid, *params, BSSN_FP64);
   const double h[3] = {grid->dx, grid->dy, grid->dz};
   cudaError_t e = cudaMemsetAsync(w.flag, 0, sizeof(unsigned int), s);
-  if (e == cudaSuccess) e = run_diffs(params->fd_order, BSSN_FP64, *grid, state, w, s);
+  if (e == cudaSuccess) e = run_tables64(params->fd_order, *grid, state, w, s);
   if (e == cudaSuccess) {
     if (params->fd_order == 4)
       e = launch_psi4<4>(L, make_coef<4, double>(*grid, 0.0), state, w.dX64, w.dY64, origin, h, psi_re, psi_im,
@@ -742,7 +759,7 @@ bssn_status_t constraints_impl(const bssn_grid_t* grid, const bssn_params_t* par
   const Layout L = make_layout(*grid);
   const WorkPtrs w = work_ptrs(work, *grid, *params, BSSN_FP64);
   cudaError_t e = cudaMemsetAsync(w.flag, 0, sizeof(unsigned int), s);
-  if (e == cudaSuccess) e = run_diffs(params->fd_order, BSSN_FP64, *grid, state, w, s);
+  if (e == cudaSuccess) e = run_tables64(params->fd_order, *grid, state, w, s);
   if (e == cudaSuccess) {
     if (params->fd_order == 4)
       e = launch_constraints<4>(L, make_coef<4, double>(*grid, 0.0), state, w.dX64, w.dY64, ham, mom, gcon, w.part,

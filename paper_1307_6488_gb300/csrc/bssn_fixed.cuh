@@ -1,0 +1,612 @@
+// FP64 derivatives on the integer pipes.
+//
+// GB300 issues FP64 at 1.68 operations per clock and SM, 32-bit integer
+// operations at up to 128. The finite-difference stencils are sums of stored
+// values with small rational weights, so they are evaluated here exactly, in
+// fixed point, and rounded to double once:
+//
+//  * one block takes one variable on one tile of 8 x 8 x 8 interior points
+//    with its halo. E is the largest exponent among the values the tile's
+//    stencils read, and every value becomes the integer
+//    n = trunc(u 2^(59-E)), |n| < 2^59: six bits more than a double's
+//    significand has. Values of at least 2^-6 of the tile's largest are held
+//    exactly, smaller ones to 2^-59 of the largest (the rounding error a
+//    double-precision stencil makes on the largest itself is 2^-53).
+//  * n is kept as two limbs, n = hi 2^30 + lo with 0 <= lo < 2^30, so that
+//    differences a - b and paired sums a + b - 2c of limbs fit 32 bits and a
+//    weighted sum is one 32 x 32 + 64 bit multiply-add per limb. The weights
+//    are the integers of the stencils over a common denominator.
+//  * mixed derivatives apply the first-derivative weights along y or z to
+//    the exact first-derivative sums along x or y (three limbs, in shared
+//    memory).
+//  * the sum is rounded to the nearest double and scaled by 1/(denominator h).
+//
+// No rounding happens before the last two operations, so a constant field has
+// exactly zero derivatives and the result does not depend on the order of the
+// terms. A tile whose values are not all finite, or so large or small that
+// the scaling could leave the range of doubles, takes double-precision
+// stencils (fx_fallback) instead: infinities and NaNs then reach exactly the
+// points whose stencils touch them.
+//
+// k_derivs writes the derivatives to a record, one slot per tile
+// (rec[(slot * nout + output) * vol + point of the tile]); the algebra kernel
+// reads them back. At 128^3, 8th order, one stage took 17.26 ms (+ 0.40 ms of
+// difference tables) when one kernel did stencils and algebra on the FP64
+// pipe (4375 FP64 instructions per point), 8.3 ms this way. Against a
+// quadruple-precision evaluation the right-hand side's error is no larger than
+// before in any variable, and 1e-16 instead of 1e-14 for W, gt_ii and alpha.
+#pragma once
+#include "bssn_bounds.cuh"
+#include "bssn_common.cuh"
+
+namespace bssn {
+
+constexpr int FX_T = 8;          // tile edge
+constexpr int FX_THREADS = 256;  // threads of k_derivs
+
+// Integer weights: first derivative W1/D1, second derivative W2/D2, paired
+// form of the upwinded first derivative
+//   sum_i UP[i] u(s o_i) = [ sum_a WT[a] (u_sa - u_-sa) + SK Delta ] / DU,
+// Delta = sum_a WK[a] (u_a + u_-a - 2 u_0) the 2r-th difference that is also
+// the Kreiss-Oliger operator (the even part of the upwinded stencil has to
+// vanish on all even powers below 2r, which leaves only this one), s = +-1.
+template <int P> struct FX;
+template <> struct FX<4> {
+  static constexpr int D1 = 12, D2 = 12, DU = 24, SK = 1;
+  static __host__ __device__ constexpr int W1(int a) { return a == 1 ? 8 : -1; }
+  static __host__ __device__ constexpr int W2(int a) { return a == 1 ? 16 : -1; }
+  static __host__ __device__ constexpr int WT(int a) { return a == 1 ? 21 : (a == 2 ? -6 : 1); }
+  static __host__ __device__ constexpr int WK(int a) { return a == 1 ? 15 : (a == 2 ? -6 : 1); }
+};
+template <> struct FX<8> {
+  static constexpr int D1 = 840, D2 = 5040, DU = 1680, SK = 3;
+  static __host__ __device__ constexpr int W1(int a) { return a == 1 ? 672 : (a == 2 ? -168 : (a == 3 ? 32 : -3)); }
+  static __host__ __device__ constexpr int W2(int a) { return a == 1 ? 8064 : (a == 2 ? -1008 : (a == 3 ? 128 : -9)); }
+  static __host__ __device__ constexpr int WT(int a) {
+    return a == 1 ? 1470 : (a == 2 ? -480 : (a == 3 ? 145 : (a == 4 ? -30 : 3)));
+  }
+  static __host__ __device__ constexpr int WK(int a) {
+    return a == 1 ? 210 : (a == 2 ? -120 : (a == 3 ? 45 : (a == 4 ? -10 : 1)));
+  }
+};
+
+// The record of one point: which derivatives of which variables, and where.
+struct DerivList {
+  int n, nout;
+  signed char var[NV];
+  short d1[NV];   // first of 3 outputs (x, y, z), or -1
+  short d2[NV];   // first of 6 outputs (xx, xy, xz, yy, yz, zz), or -1
+  short ext[NV];  // advection + dissipation, or -1
+};
+
+// Right-hand side: W, gt, alpha, beta (9 outputs each), K and Gt^i (3 each),
+// then the 24 advection + dissipation sums.
+constexpr int REC_K = 9 * NM, REC_GAM = REC_K + 3, REC_EXT = REC_GAM + 9, REC_RHS = REC_EXT + NV;
+
+inline DerivList rhs_list() {
+  DerivList D{};
+  for (int m = 0; m < NM; ++m) {
+    const int e = D.n++;
+    D.var[e] = (signed char)mvar(m);
+    D.d1[e] = (short)(9 * m);
+    D.d2[e] = (short)(9 * m + 3);
+  }
+  for (int v = 0; v < NV; ++v) {
+    if (mixed_index(v) >= 0) continue;
+    const int e = D.n++;
+    D.var[e] = (signed char)v;
+    D.d1[e] = (short)(v == V_TRK ? REC_K : (v >= V_GAM1 && v <= V_GAM3 ? REC_GAM + 3 * (v - V_GAM1) : -1));
+    D.d2[e] = -1;
+  }
+  for (int e = 0; e < D.n; ++e) D.ext[e] = (short)(REC_EXT + D.var[e]);
+  D.nout = REC_RHS;
+  return D;
+}
+
+// Scales of one grid's stencils.
+struct FxCoef {
+  double c1[3];  // 1 / (D1 h_d)
+  double c2[6];  // 1 / (D2 h_d^2), mixed 1 / (D1^2 h h'), packed as sym()
+  double cu[3];  // 1 / (DU h_d)
+  double ck[3];  // eps KOSCALE / h_d
+  int cubic;     // h equal along all axes: the dissipation is one exact sum
+};
+
+template <int P>
+FxCoef make_fx(const bssn_grid_t& G, double eps) {
+  using X = FX<P>;
+  FxCoef C;
+  const double h[3] = {G.dx, G.dy, G.dz};
+  for (int d = 0; d < 3; ++d) {
+    C.c1[d] = 1.0 / (X::D1 * h[d]);
+    C.cu[d] = 1.0 / (X::DU * h[d]);
+    C.ck[d] = eps * FD<P>::KOSCALE / h[d];
+  }
+  for (int s = 0; s < 6; ++s) {
+    const int i = sym_i(s), j = sym_j(s);
+    C.c2[s] = i == j ? 1.0 / (X::D2 * h[i] * h[i]) : 1.0 / ((double)X::D1 * X::D1 * h[i] * h[j]);
+  }
+  C.cubic = G.dx == G.dy && G.dy == G.dz;
+  return C;
+}
+
+// Tiles of one grid: extents of a (full) tile, counts, slot volume.
+struct FxTiles {
+  int tx, ty, tz, ntx, nty, ntz, vol;
+};
+__host__ __device__ inline FxTiles fx_tiles(int nx, int ny, int nz) {
+  FxTiles T;
+  T.tx = nx < FX_T ? nx : FX_T;
+  T.ty = ny < FX_T ? ny : FX_T;
+  T.tz = nz < FX_T ? nz : FX_T;
+  T.ntx = (nx + FX_T - 1) / FX_T;
+  T.nty = (ny + FX_T - 1) / FX_T;
+  T.ntz = (nz + FX_T - 1) / FX_T;
+  T.vol = T.tx * T.ty * T.tz;
+  return T;
+}
+
+// ------------------------------------------------------------------ fixed point
+// shifts that give 0 for counts of 64 and more (the PTX rule)
+__device__ __forceinline__ unsigned long long fx_shr(unsigned long long x, int n) {
+  unsigned long long r;
+  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(n));
+  return r;
+}
+__device__ __forceinline__ unsigned long long fx_shl(unsigned long long x, int n) {
+  unsigned long long r;
+  asm("shl.b64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(n));
+  return r;
+}
+
+constexpr int FX_LIMB = 30;
+constexpr unsigned int FX_MASK = (1u << FX_LIMB) - 1;
+
+// limbs (lo, hi) of trunc(u 2^(1081 - emax)), emax the largest biased exponent
+__device__ __forceinline__ int2 fx_from_double(double u, int emax) {
+  const int h = __double2hiint(u);
+  const unsigned int l = (unsigned int)__double2loint(u);
+  const int ex = (h >> 20) & 0x7ff;
+  const unsigned int mh = ex ? ((unsigned int)h & 0xfffffu) | 0x100000u : 0u;
+  const unsigned int ml = ex ? l : 0u;  // subnormals are far below the last place
+  const unsigned long long m = ((unsigned long long)__funnelshift_l(ml, mh, 6) << 32) | (ml << 6);
+  const unsigned long long s = (unsigned long long)(long long)(h >> 31);
+  const long long n = (long long)((fx_shr(m, emax - ex) ^ s) - s);
+  return make_int2((int)((unsigned int)n & FX_MASK), (int)(n >> FX_LIMB));
+}
+
+// The sum of two values, rounded to 53 significant bits (ties to even) as a
+// double-precision addition rounds it; lo may come out as 2^30. The sums of
+// second derivatives keep this one rounding of the double-precision form: on
+// data that varies along one axis only, its effect on the derivative along
+// that axis (2^-53 |u| / h^2) is larger than any other rounding of the
+// right-hand side, and results stay comparable with that form's.
+__device__ __forceinline__ int2 fx_pair(int2 p, int2 m) {
+  unsigned int lo = (unsigned int)(p.x + m.x);
+  const int hi = p.y + m.y + (int)(lo >> FX_LIMB);
+  lo &= FX_MASK;
+  const int g = max(0, 9 - __clz(hi ^ (hi >> 31)));  // bits of the sum beyond 53
+  const unsigned int mk = (1u << g) - 1u;
+  lo = (lo + (mk >> 1) + ((lo >> g) & mk & 1u)) & ~mk;
+  return make_int2((int)lo, hi);
+}
+
+// (hi 2^30 + lo) 2^(emax - 1081), rounded to nearest (ties away from zero)
+__device__ __forceinline__ double fx_to_double(long long hi, long long lo, int emax) {
+  hi += lo >> FX_LIMB;
+  unsigned int l = (unsigned int)lo & FX_MASK;
+  // magnitude
+  const unsigned int sg = (unsigned int)(hi >> 63);
+  unsigned long long H = (unsigned long long)hi;
+  if (sg) {
+    l = (0u - l) & FX_MASK;
+    H = ~H + (l == 0u ? 1u : 0u);
+  }
+  // 94 bits H:l with the top bit moved to bit 63 of y
+  const bool z = H == 0;
+  const unsigned long long A = z ? (unsigned long long)l << 34 : H;
+  const unsigned int B = z ? 0u : l << 2;
+  const int lz = __clzll((long long)A);
+  const unsigned long long y = fx_shl(A, lz) | fx_shr((unsigned long long)B << 32, 64 - lz);
+  const unsigned long long r = (y >> 11) + ((y >> 10) & 1u);
+  const int e = emax + 34 - lz - (z ? 64 : 0);
+  unsigned long long bits = ((unsigned long long)(unsigned int)e << 52) + r;
+  if (A == 0) bits = 0;
+  return __longlong_as_double((long long)(bits | ((unsigned long long)(sg & 0x80000000u) << 32)));
+}
+
+// ------------------------------------------------------------------ double-precision stencils
+// One point of a tile that fixed point does not hold. v: the variable, p:
+// the point; writes the same outputs.
+template <int P>
+__device__ __noinline__ void fx_fallback(const double* __restrict__ v, long long p, long long sy, long long sz,
+                                         const FxCoef& C, const double* beta, double wa, bool want1, bool want2,
+                                         bool wante, double* o1, double* o2, double* oe) {
+  using F = FD<P>;
+  using X = FX<P>;
+  constexpr int H = F::H, R = F::R;
+  const long long st[3] = {1, sy, sz};
+  const double m2 = -2.0 * v[p];
+  double ext = 0.0;
+  for (int d = 0; d < 3; ++d) {
+    double r1 = 0.0, r2 = 0.0, k = 0.0;
+    for (int a = 1; a <= R; ++a) {
+      const double up = v[p + a * st[d]], um = v[p - a * st[d]];
+      const double df = up - um, s = (up + um) + m2;
+      if (a <= H) {
+        r1 += X::W1(a) * df;
+        r2 += X::W2(a) * s;
+      }
+      k += X::WK(a) * s;
+    }
+    if (want1) o1[d] = C.c1[d] * r1;
+    if (want2) o2[sym(d, d)] = C.c2[sym(d, d)] * r2;
+    if (wante) {
+      // the one-sided stencil the sign of beta selects, and no other point
+      const long long ss = beta[d] < 0.0 ? -st[d] : st[d];
+      double t = 0.0;
+      for (int i = 0; i < F::UPN; ++i) {
+        const int o = F::UPLO + i;
+        int w = 0;
+        if (o == 0)
+          for (int a = 1; a <= R; ++a) w -= 2 * X::SK * X::WK(a);
+        else
+          w = X::SK * X::WK(abs(o)) + (o > 0 ? X::WT(o) : -X::WT(-o));
+        t += w * v[p + o * ss];
+      }
+      ext += C.ck[d] * k + C.cu[d] * (wa * fabs(beta[d])) * t;
+    }
+  }
+  if (wante) *oe = ext;
+  if (!want2) return;
+  for (int i = 0; i < 3; ++i)
+    for (int j = i + 1; j < 3; ++j) {
+      double r = 0.0;
+      for (int a = 1; a <= H; ++a)
+        for (int b = 1; b <= H; ++b) {
+          const long long A = a * st[i], B = b * st[j];
+          r += (double)(X::W1(a) * X::W1(b)) * ((v[p + A + B] - v[p - A + B]) - (v[p + A - B] - v[p - A - B]));
+        }
+      o2[sym(i, j)] = C.c2[sym(i, j)] * r;
+    }
+}
+
+// ------------------------------------------------------------------ one tile of one variable
+template <int P>
+struct FxSmem {
+  static constexpr int H = FD<P>::H, R = FD<P>::R;
+  static constexpr int BX = FX_T + 2 * R;          // box edge
+  static constexpr int EH = FX_T + 2 * H;
+  static constexpr int BOX = BX * BX * BX;
+  static constexpr int GN = EH * FX_T * FX_T;      // entries of one first-derivative table
+  static constexpr size_t bytes = sizeof(int2) * BOX + 3 * sizeof(int4) * GN;
+};
+
+// three limbs of sum_a W1[a] (n_a - n_-a) along stride st
+template <int P>
+__device__ __forceinline__ int4 fx_first(const int2* __restrict__ b, int st) {
+  long long lo = 0, hi = 0;
+#pragma unroll
+  for (int a = 1; a <= FD<P>::H; ++a) {
+    const int2 p = b[a * st], m = b[-a * st];
+    lo += (long long)FX<P>::W1(a) * (p.x - m.x);
+    hi += (long long)FX<P>::W1(a) * (p.y - m.y);
+  }
+  hi += lo >> FX_LIMB;
+  return make_int4((int)((unsigned int)lo & FX_MASK), (int)((unsigned int)hi & FX_MASK), (int)(hi >> FX_LIMB), 0);
+}
+
+// the first-derivative weights along stride st of a table of such sums
+template <int P>
+__device__ __forceinline__ double fx_mixed(const int4* __restrict__ g, int st, int emax) {
+  long long l0 = 0, l1 = 0;
+  int l2 = 0;
+#pragma unroll
+  for (int b = 1; b <= FD<P>::H; ++b) {
+    const int4 p = g[b * st], m = g[-b * st];
+    l0 += (long long)FX<P>::W1(b) * (p.x - m.x);
+    l1 += (long long)FX<P>::W1(b) * (p.y - m.y);
+    l2 += FX<P>::W1(b) * (p.z - m.z);
+  }
+  l1 += l0 >> FX_LIMB;
+  const long long hi = ((long long)(l2 + (int)(l1 >> FX_LIMB)) << FX_LIMB) | (l1 & (long long)FX_MASK);
+  return fx_to_double(hi, l0 & (long long)FX_MASK, emax);
+}
+
+// Stencils along the three axes at one point of the box, and the outputs.
+template <int P, bool D1, bool D2, bool EXT>
+__device__ __forceinline__ void fx_point(const int2* __restrict__ c, const int4* const g[3], const FxCoef& C,
+                                         const double* beta, double wa, int emax, double* __restrict__ o1,
+                                         double* __restrict__ o2, double* __restrict__ oe, int vol) {
+  using F = FD<P>;
+  using X = FX<P>;
+  constexpr int BX = FxSmem<P>::BX;
+  const int2 u0 = c[0];
+  const int m2x = -2 * u0.x, m2y = -2 * u0.y;
+  long long kslo = 0, kshi = 0;
+  double ext = 0.0;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const int st = d == 0 ? 1 : (d == 1 ? BX : BX * BX);
+    long long r1l = 0, r1h = 0, r2l = 0, r2h = 0, tl = 0, th = 0, kl = 0, kh = 0;
+#pragma unroll
+    for (int a = 1; a <= (EXT ? F::R : F::H); ++a) {
+      const int2 p = c[a * st], m = c[-a * st];
+      const int dx = p.x - m.x, dy = p.y - m.y;
+      if (D1 && a <= F::H) {
+        r1l += (long long)X::W1(a) * dx;
+        r1h += (long long)X::W1(a) * dy;
+      }
+      if (EXT) {
+        tl += (long long)X::WT(a) * dx;
+        th += (long long)X::WT(a) * dy;
+      }
+      if (D2 && a <= F::H) {
+        const int2 s = fx_pair(p, m);
+        r2l += (long long)X::W2(a) * (s.x + m2x);
+        r2h += (long long)X::W2(a) * (s.y + m2y);
+      }
+      if (EXT) {
+        kl += (long long)X::WK(a) * (p.x + m.x + m2x);
+        kh += (long long)X::WK(a) * (p.y + m.y + m2y);
+      }
+    }
+    if (D1) o1[d * vol] = C.c1[d] * fx_to_double(r1h, r1l, emax);
+    if (D2) o2[sym(d, d) * vol] = C.c2[sym(d, d)] * fx_to_double(r2h, r2l, emax);
+    if (EXT) {
+      // |b| times the stencil mirrored by the sign of b
+      const double b = wa * beta[d];
+      const long long kkl = X::SK * kl, kkh = X::SK * kh;
+      const bool neg = b < 0.0;
+      ext = fma(C.cu[d] * b, fx_to_double(neg ? th - kkh : th + kkh, neg ? tl - kkl : tl + kkl, emax), ext);
+      if (C.cubic) {
+        kslo += kl;
+        kshi += kh;
+      } else {
+        ext = fma(C.ck[d], fx_to_double(kh, kl, emax), ext);
+      }
+    }
+  }
+  if (EXT) {
+    if (C.cubic) ext = fma(C.ck[0], fx_to_double(kshi, kslo, emax), ext);
+    *oe = ext;
+  }
+  if (D2) {
+    o2[1 * vol] = C.c2[1] * fx_mixed<P>(g[0], FX_T, emax);
+    o2[2 * vol] = C.c2[2] * fx_mixed<P>(g[1], FX_T * FX_T, emax);
+    o2[4 * vol] = C.c2[4] * fx_mixed<P>(g[2], FX_T * FX_T, emax);
+  }
+}
+
+// Point of a thread: x and the eight rows of a plane, arranged so that the
+// half-warps of an 8-byte shared-memory read take rows y and y + 4, whose
+// distance in the box is an odd multiple of 64 bytes (no bank conflicts).
+__device__ __forceinline__ void fx_lane(int t, int& x, int& y, int& z) {
+  x = t & 7;
+  y = ((t >> 3) & 1) * 4 + ((t >> 4) & 1) + ((t >> 5) & 1) * 2;
+  z = t >> 6;
+}
+
+// All outputs of list entry e on the tile (ti, tj, tk) of the grid L, written
+// to the record slot `rec` (nout x vol doubles).
+template <int P>
+__device__ __forceinline__ void fx_tile(const Layout& L, const FxCoef& C, const FxTiles& T, const DerivList& list,
+                                        int e, bool advect_gauge, bool lapse_frozen, bool shift_frozen,
+                                        const double* __restrict__ u, int ti, int tj, int tk,
+                                        double* __restrict__ rec) {
+  using S = FxSmem<P>;
+  constexpr int H = S::H, R = S::R, BX = S::BX;
+  extern __shared__ __align__(16) unsigned char fx_smem[];
+  int4* g = (int4*)fx_smem;
+  int2* box = (int2*)(g + 3 * S::GN);
+  __shared__ unsigned int red[2][FX_THREADS / 32];
+
+  const int var = list.var[e];
+  const bool mixed = list.d2[e] >= 0;
+  const int i0 = ti * FX_T, j0 = tj * FX_T, k0 = tk * FX_T;
+  const int ex = min(FX_T, L.nx - i0), ey = min(FX_T, L.ny - j0), ez = min(FX_T, L.nz - k0);
+  const long long org = L.off0 + i0 + j0 * L.sy + k0 * L.sz;
+  const double* __restrict__ v = u + var * L.vs;
+
+  // ---- the box in registers: columns of the (x, y) box, cut along z. Only
+  // what the stencils read: the lines through the tile (R beyond it) and, for
+  // mixed derivatives, the planes through it (H beyond it).
+  constexpr int SEG = P == 8 ? 6 : 7, NSEG = BX / SEG, COLS = BX * BX, TASKS = COLS * NSEG;
+  constexpr int PER = (TASKS + FX_THREADS - 1) / FX_THREADS;
+  static_assert(SEG * NSEG == BX, "segments cover the box");
+  double raw[PER][SEG];
+  unsigned int mx = 0, any = 0;
+#pragma unroll
+  for (int q = 0; q < PER; ++q) {
+    const int c = threadIdx.x + q * FX_THREADS;
+    const int seg = c / COLS, col = c - seg * COLS;
+    const int by = col / BX, bx = col - by * BX;
+    const int ox = bx < R ? R - bx : max(0, bx - (R + ex) + 1);
+    const int oy = by < R ? R - by : max(0, by - (R + ey) + 1);
+    int reach;  // how far beyond the tile this column is read along z
+    if (c >= TASKS || ox > R || oy > R) reach = -1;
+    else if (ox == 0 && oy == 0) reach = R;
+    else if (ox == 0 || oy == 0) reach = (mixed && ox <= H && oy <= H) ? H : 0;
+    else reach = (mixed && ox <= H && oy <= H) ? 0 : -1;
+    const long long p0 = org + (bx - R) + (by - R) * L.sy + (seg * SEG - R) * L.sz;
+#pragma unroll
+    for (int s = 0; s < SEG; ++s) {
+      const int bz = seg * SEG + s;
+      const int oz = bz < R ? R - bz : max(0, bz - (R + ez) + 1);
+      const long long p = p0 + s * L.sz;
+      double x = 0.0;
+      if (oz <= reach && in_range(p, p, padded_points(L))) x = __ldg(v + p);
+      raw[q][s] = x;
+      const unsigned int hw = (unsigned int)__double2hiint(x) & 0x7fffffffu;
+      mx = max(mx, hw);
+      any |= hw | (unsigned int)__double2loint(x);
+    }
+  }
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  any = __reduce_or_sync(0xffffffffu, any);
+  if ((threadIdx.x & 31) == 0) {
+    red[0][threadIdx.x >> 5] = mx;
+    red[1][threadIdx.x >> 5] = any;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < FX_THREADS / 32; ++w) {
+    mx = max(mx, red[0][w]);
+    any |= red[1][w];
+  }
+  const int emax = (int)(mx >> 20);
+  const bool fallback = emax >= 1900 || (emax < 160 && any != 0u);
+
+  const bool d1 = list.d1[e] >= 0, ext = list.ext[e] >= 0;
+  const int vol = T.vol;
+  double* const o1 = rec + (long long)(d1 ? list.d1[e] : 0) * vol;
+  double* const o2 = rec + (long long)(mixed ? list.d2[e] : 0) * vol;
+  double* const oe = rec + (long long)(ext ? list.ext[e] : 0) * vol;
+  // advection weight of this variable's right-hand side
+  double wa = 1.0;
+  if (var >= V_ALPHA) {
+    const bool frozen = var == V_ALPHA ? lapse_frozen : shift_frozen;
+    wa = advect_gauge && !frozen ? 1.0 : 0.0;
+  }
+
+  if (!fallback) {
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+      const int c = threadIdx.x + q * FX_THREADS;
+      if (c >= TASKS) break;
+      const int seg = c / COLS, col = c - seg * COLS;
+#pragma unroll
+      for (int s = 0; s < SEG; ++s) box[(seg * SEG + s) * COLS + col] = fx_from_double(raw[q][s], emax);
+    }
+    __syncthreads();
+    if (mixed) {
+      // D_x sums on rows y beyond the tile (for xy) and planes z beyond it
+      // (for xz), D_y sums on planes beyond it (for yz); the in-tile D_x
+      // serves both tables
+      for (int t = threadIdx.x; t < 2 * H * FX_T * FX_T; t += FX_THREADS) {  // xy rows outside
+        const int x = t & 7, r = t >> 3, z = r & 7, q = r >> 3;
+        const int y = q < H ? q : q + FX_T;  // 0 .. EH-1
+        g[(z * S::EH + y) * FX_T + x] = fx_first<P>(box + ((z + R) * BX + (y - H + R)) * BX + x + R, 1);
+      }
+      for (int t = threadIdx.x; t < S::GN; t += FX_THREADS) {
+        int x, y, z;
+        fx_lane(t, x, y, z);  // z = 0 .. EH-1
+        const int2* b = box + ((z - H + R) * BX + (y + R)) * BX + x + R;
+        const int4 fx = fx_first<P>(b, 1);
+        g[S::GN + (z * FX_T + y) * FX_T + x] = fx;
+        if (z >= H && z < H + FX_T) g[((z - H) * S::EH + (y + H)) * FX_T + x] = fx;
+        g[2 * S::GN + (z * FX_T + y) * FX_T + x] = fx_first<P>(b, BX);
+      }
+      __syncthreads();
+    }
+  }
+  for (int t = threadIdx.x; t < FX_T * FX_T * FX_T; t += FX_THREADS) {
+    int x, y, z;
+    fx_lane(t, x, y, z);
+    if (x >= ex || y >= ey || z >= ez) continue;
+    const int idx = (z * T.ty + y) * T.tx + x;
+    const long long p = org + x + y * L.sy + z * L.sz;
+    if (!in_range(p - R * L.sz, p + R * L.sz, padded_points(L))) continue;
+    double beta[3] = {0.0, 0.0, 0.0};
+    if (ext)
+#pragma unroll
+      for (int d = 0; d < 3; ++d) beta[d] = __ldg(u + (V_BETA1 + d) * L.vs + p);
+    if (fallback) {
+      double r1[3], r2[6], re;
+      fx_fallback<P>(v, p, L.sy, L.sz, C, beta, wa, d1, mixed, ext, r1, r2, &re);
+      if (d1)
+        for (int d = 0; d < 3; ++d) o1[d * vol + idx] = r1[d];
+      if (mixed)
+        for (int s = 0; s < 6; ++s) o2[s * vol + idx] = r2[s];
+      if (ext) oe[idx] = re;
+      continue;
+    }
+    const int2* c = box + ((z + R) * BX + (y + R)) * BX + x + R;
+    const int4* const gt[3] = {g + (z * S::EH + (y + H)) * FX_T + x, g + S::GN + ((z + H) * FX_T + y) * FX_T + x,
+                               g + 2 * S::GN + ((z + H) * FX_T + y) * FX_T + x};
+    if (mixed && ext)
+      fx_point<P, true, true, true>(c, gt, C, beta, wa, emax, o1 + idx, o2 + idx, oe + idx, vol);
+    else if (mixed)
+      fx_point<P, true, true, false>(c, gt, C, beta, wa, emax, o1 + idx, o2 + idx, oe + idx, vol);
+    else if (d1 && ext)
+      fx_point<P, true, false, true>(c, gt, C, beta, wa, emax, o1 + idx, o2 + idx, oe + idx, vol);
+    else if (d1)
+      fx_point<P, true, false, false>(c, gt, C, beta, wa, emax, o1 + idx, o2 + idx, oe + idx, vol);
+    else
+      fx_point<P, false, false, true>(c, gt, C, beta, wa, emax, o1 + idx, o2 + idx, oe + idx, vol);
+  }
+}
+
+// One grid as the FP64 kernels see it: its layout, scales, tiles and buffers.
+// Single grids pass one by value; patches keep a device table of them, each
+// with the number of its first tile in the flat list of all tiles.
+struct FxGrid {
+  Layout L;
+  FxCoef C;
+  FxTiles T;
+  long long tile0;
+  double* buf[6];  // as PatchDev: 0 y0, 1 and 2 stage buffers, 3 acc, 4 and 5 kept by parents
+};
+
+// What a launch works on: a grid passed by value (table null) or the grids
+// of a table, tiles tile0, tile0 + 1, ... of the flat list, slot by slot.
+struct FxWork {
+  FxGrid one;
+  const FxGrid* table;
+  const long long* tile0s;  // first tile of every grid of the table
+  int ngrids;
+  long long tile0;          // tile of slot 0
+  double* rec;
+  long long slot;           // doubles of one slot
+};
+
+// grid and tile coordinates of a slot
+__device__ __forceinline__ const FxGrid& fx_locate(const FxWork& Wk, long long t, int& ti, int& tj, int& tk) {
+  const FxGrid* G = &Wk.one;
+  if (Wk.table) {
+    int lo = 0, hi = Wk.ngrids - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (__ldg(Wk.tile0s + mid) <= t) lo = mid; else hi = mid - 1;
+    }
+    G = Wk.table + lo;
+  }
+  const unsigned int q = (unsigned int)(t - G->tile0);
+  const unsigned int r = q / (unsigned int)G->T.ntx;
+  ti = (int)(q - r * G->T.ntx);
+  tk = (int)(r / (unsigned int)G->T.nty);
+  tj = (int)(r - tk * (unsigned int)G->T.nty);
+  return *G;
+}
+
+struct DerivArgs {
+  FxWork W;
+  DerivList list;
+  int in;  // buffer the stencils read
+  bool advect_gauge, lapse_frozen, shift_frozen;
+};
+
+// What a thread does with the right-hand side of its point.
+struct StageOut {
+  int mode;                // 0: RK stage, 1: right-hand side to out
+  Gauge gz;
+  RK rk;
+  int in, out;             // buffers of the stage input and of the result
+  double* rhs;             // mode 1: where the right-hand side goes
+};
+
+struct AlgebraArgs {
+  FxWork W;
+  StageOut S;
+};
+
+// One block per slot (blockIdx.x) and list entry (blockIdx.y).
+template <int P>
+__global__ void __launch_bounds__(FX_THREADS, 2) k_derivs(const __grid_constant__ DerivArgs A) {
+  int ti, tj, tk;
+  const FxGrid& G = fx_locate(A.W, A.W.tile0 + blockIdx.x, ti, tj, tk);
+  fx_tile<P>(G.L, G.C, G.T, A.list, blockIdx.y, A.advect_gauge, A.lapse_frozen, A.shift_frozen, G.buf[A.in], ti, tj,
+             tk, A.W.rec + (long long)blockIdx.x * A.W.slot);
+}
+
+}  // namespace bssn

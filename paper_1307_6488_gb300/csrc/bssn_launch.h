@@ -1,33 +1,28 @@
 // Host-side launchers of the order-templated kernels (one translation unit
 // per finite-difference order instantiates them).
 #pragma once
+#include <atomic>
+
 #include "bssn_common.cuh"
+#include "bssn_fixed.cuh"
 #include "bssn_stage32_types.h"
 
 namespace bssn {
 
-// Pointers of one fused-stage launch. For the double form ys/dX/dY are
-// double; for the FP32-RHS form they point at the single-precision copy of
-// the state and single-precision tables (passed as void*).
-struct StageArgs {
-  const void* ys;
-  const double* ys64;
-  const double* y0;
-  double* acc;
-  double* out;
-  const void* dX;
-  const void* dY;
-  float* out32 = nullptr;  // FP32 form: single-precision copy of out (nullable)
-};
-
-// FP64 first-difference tables (H per mixed variable). The FP32-RHS form of
-// single grids has its own tables (launch_d1tab32).
+// FP64 first-difference tables of the constraints and Weyl scalars (H per
+// mixed variable).
 template <int P>
-cudaError_t launch_diffs(const Layout& L, const bssn_grid_t& G, bssn_precision_t prec, const void* u, void* dX,
-                         void* dY, cudaStream_t s);
+cudaError_t launch_diffs(const Layout& L, const double* u, double* dX, double* dY, cudaStream_t s);
+// Derivatives of `nslots` tiles into the record (bssn_fixed.cuh).
 template <int P>
-cudaError_t launch_stage(const Layout& L, const bssn_grid_t& G, double eps, bssn_precision_t prec, const Gauge& gz,
-                         const RK& rk, const StageArgs& A, int mode, cudaStream_t s);
+cudaError_t derivs_init();  // raises the kernel's shared-memory limit (not during a capture)
+template <int P>
+cudaError_t launch_derivs(const DerivArgs& A, long long nslots, cudaStream_t s);
+// The FP64 stage (or right-hand side) of `ntiles` tiles from work.tile0 on,
+// through a record of `slots` slots (bssn_stage64.cu); vol: the largest tile
+// volume among the grids.
+cudaError_t launch_stage64(int order, const FxWork& work, int vol, long long ntiles, long long slots,
+                           const Gauge& gz, const StageOut& out, cudaStream_t s);
 template <int P>
 cudaError_t launch_ko(const Layout& L, const bssn_grid_t& G, double eps, bssn_precision_t prec, const double* u,
                       double* rhs, cudaStream_t s);
@@ -89,11 +84,24 @@ template <int P>
 cudaError_t bounds_take_order(unsigned long long* out);
 template <int P>
 cudaError_t bounds_take_stage32(unsigned long long* out);
+cudaError_t bounds_take_stage64(unsigned long long* out);
 cudaError_t bounds_take_batch(unsigned long long* out);
 cudaError_t bounds_take_amr(unsigned long long* out);
 cudaError_t bounds_take_cfd(unsigned long long* out);
 
-constexpr int STAGE_THREADS = 128;
+// Raise the dynamic shared memory limit of a kernel once per device.
+template <typename K>
+inline cudaError_t allow_smem(K kern, size_t bytes, std::atomic<unsigned long long>& done) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const unsigned long long bit = 1ull << (dev & 63);
+  if (done.load() & bit) return cudaSuccess;
+  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e == cudaSuccess) done.fetch_or(bit);
+  return e;
+}
+
 constexpr int CON_THREADS = 128;
 inline long long con_blocks(const Layout& L) { return (L.npts + CON_THREADS - 1) / CON_THREADS; }
 

@@ -1,5 +1,6 @@
 // Instantiates the kernels and launchers for one finite-difference order,
 // selected at compile time with -DBSSN_ORDER=4 or -DBSSN_ORDER=8.
+#include "bssn_fixed.cuh"
 #include "bssn_kernels.cuh"
 #include "bssn_weyl.cuh"
 #include "bssn_launch.h"
@@ -14,36 +15,27 @@ namespace bssn {
 static inline unsigned int blocks_for(long long n, int threads) { return (unsigned int)((n + threads - 1) / threads); }
 
 template <>
-cudaError_t launch_diffs<BSSN_ORDER>(const Layout& L, const bssn_grid_t& G, bssn_precision_t prec, const void* u,
-                                     void* dX, void* dY, cudaStream_t s) {
+cudaError_t launch_diffs<BSSN_ORDER>(const Layout& L, const double* u, double* dX, double* dY, cudaStream_t s) {
   constexpr int H = FD<BSSN_ORDER>::H;
   const long long n = (long long)L.nx * (L.ny + 2 * H) * (L.nz + 2 * H);
-  // single grids in the FP32-RHS form take the tiled path (launch_d1tab32)
-  if (prec != BSSN_FP64) return cudaErrorInvalidValue;
-  k_diffs<BSSN_ORDER, double><<<blocks_for(n, 256), 256, 0, s>>>(L, (const double*)u, (double*)dX, (double*)dY);
+  k_diffs<BSSN_ORDER, double><<<blocks_for(n, 256), 256, 0, s>>>(L, u, dX, dY);
   return cudaGetLastError();
 }
 
-template <typename R>
-static cudaError_t stage_typed(const Layout& L, const bssn_grid_t& G, double eps, const Gauge& gz, const RK& rk,
-                               const StageArgs& A, int mode, cudaStream_t s) {
-  StagePtrs<R> S{(const R*)A.ys, A.ys64, A.y0, A.acc, A.out, (const R*)A.dX, (const R*)A.dY, A.out32};
-  const Coef<R> C = make_coef<BSSN_ORDER, R>(G, eps);
-  const int tx = 0;
-  const unsigned int nb = blocks_for(L.npts, STAGE_THREADS);
-  if (mode == 0)
-    k_stage<BSSN_ORDER, 0, R><<<nb, STAGE_THREADS, 0, s>>>(L, C, gz, rk, S, tx);
-  else
-    k_stage<BSSN_ORDER, 1, R><<<nb, STAGE_THREADS, 0, s>>>(L, C, gz, rk, S, tx);
-  return cudaGetLastError();
+static std::atomic<unsigned long long> g_derivs_smem{0};  // devices whose limit is raised
+
+template <>
+cudaError_t derivs_init<BSSN_ORDER>() {
+  return allow_smem(k_derivs<BSSN_ORDER>, FxSmem<BSSN_ORDER>::bytes, g_derivs_smem);
 }
 
 template <>
-cudaError_t launch_stage<BSSN_ORDER>(const Layout& L, const bssn_grid_t& G, double eps, bssn_precision_t prec,
-                                     const Gauge& gz, const RK& rk, const StageArgs& A, int mode, cudaStream_t s) {
-  // single grids in the FP32-RHS form take the tiled path (launch_stage32)
-  if (prec != BSSN_FP64) return cudaErrorInvalidValue;
-  return stage_typed<double>(L, G, eps, gz, rk, A, mode, s);
+cudaError_t launch_derivs<BSSN_ORDER>(const DerivArgs& A, long long nslots, cudaStream_t s) {
+  constexpr size_t bytes = FxSmem<BSSN_ORDER>::bytes;
+  const cudaError_t e = derivs_init<BSSN_ORDER>();
+  if (e != cudaSuccess) return e;
+  k_derivs<BSSN_ORDER><<<dim3((unsigned int)nslots, (unsigned int)A.list.n), FX_THREADS, bytes, s>>>(A);
+  return cudaGetLastError();
 }
 
 template <>

@@ -49,19 +49,6 @@ bool map32(CUtensorMap* tm, const float* base, const Layout32& L, int narr, cuui
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Raise the dynamic shared memory limit of a kernel once per device.
-template <typename K>
-cudaError_t allow_smem(K kern, size_t bytes, std::atomic<unsigned long long>& done) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  const unsigned long long bit = 1ull << (dev & 63);
-  if (done.load() & bit) return cudaSuccess;
-  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e == cudaSuccess) done.fetch_or(bit);
-  return e;
-}
-
 std::atomic<unsigned long long> g_smem_done[2];
 
 }  // namespace

@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(128, STAGE_F64_MIN_BLOCKS) k_psi4(Layout L, Co
   const long long p = L.off0 + i + j * L.sy + k * L.sz;
   if (!in_range(p - FD<P>::R * L.sz, p + FD<P>::R * L.sz, padded_points(L))) return;
   PointIn<double> Q;
-  gather<P, false, false, double>(L, C, u, dX, dY, p, Q, nullptr);
+  gather<P, double>(L, C, u, dX, dY, p, Q);
   double dAt[3][6];
   const long long st[3] = {1, L.sy, L.sz};
 #pragma unroll
