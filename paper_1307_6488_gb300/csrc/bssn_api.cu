@@ -64,9 +64,9 @@ bool params_ok(const bssn_grid_t* G, const bssn_params_t* P) {
 
 // Scratch layout, one size for both precisions:
 //   [tables region][constraint partials][finals + flag]
-// The tables region holds 2 x 11 x p/2 arrays of var_stride doubles: for
-// BSSN_FP64 stages the derivative record (as many tiles at a time as fit),
-// for the constraints the difference tables; for BSSN_FP32_RHS, two single
+// The tables region is as large as 2 x 11 x p/2 arrays of var_stride doubles:
+// for BSSN_FP64 stages and the constraints it holds the derivative record (as
+// many tiles at a time as fit); for BSSN_FP32_RHS, two single
 // precision copies of the state (24 x var_stride floats each: a whole step
 // alternates between them) followed by the single precision tables.
 constexpr int RMS_BLOCKS = 304, RMS_THREADS = 256;
@@ -98,25 +98,21 @@ struct WorkPtrs {
   float* f32;     // single-precision state copy (FP32 form, Layout32)
   float* f32b;    // a second one (the next stage's input, written by the stage before)
   float* tab32;   // D_x then D_y tables of the 11 mixed variables (FP32 form, Layout32)
-  double* dX64;   // double difference tables (constraints)
-  double* dY64;
-  double* rec;    // derivative record (FP64 form)
+  double* rec;    // derivative record (FP64 form, constraints)
   size_t rec_doubles;
+  size_t part_doubles;
   double* part;
   double* finals;
   unsigned int* flag;
 };
 
 WorkPtrs work_ptrs(void* work, const bssn_grid_t& G, const bssn_params_t& P, bssn_precision_t prec) {
-  Layout L = make_layout(G);
   WorkLayout W = work_layout(G, P);
   double* base = (double*)work;
   WorkPtrs w;
-  const size_t H = P.fd_order / 2;
-  w.dX64 = base;
-  w.dY64 = base + NM * H * L.vs;
   w.rec = base;
   w.rec_doubles = W.tables;
+  w.part_doubles = W.partials;
   if (prec == BSSN_FP64) {
     w.f32 = nullptr;
     w.f32b = nullptr;
@@ -145,10 +141,15 @@ cudaError_t run_diffs(int order, bssn_precision_t prec, const bssn_grid_t& G, co
   return order == 4 ? launch_d1tab32<4>(L32, G, w.f32, w.tab32, s) : launch_d1tab32<8>(L32, G, w.f32, w.tab32, s);
 }
 
-// Difference tables of the constraints and Weyl scalars.
-cudaError_t run_tables64(int order, const bssn_grid_t& G, const double* u, const WorkPtrs& w, cudaStream_t s) {
-  const Layout L = make_layout(G);
-  return order == 4 ? launch_diffs<4>(L, u, w.dX64, w.dY64, s) : launch_diffs<8>(L, u, w.dX64, w.dY64, s);
+// The grid as the FP64 kernels see it, on the stencil input u, and the record.
+FxWork fx_work(int order, const bssn_grid_t& G, double eps, const double* u, const WorkPtrs& w) {
+  FxWork W{};
+  W.one.L = make_layout(G);
+  W.one.C = order == 4 ? make_fx<4>(G, eps) : make_fx<8>(G, eps);
+  W.one.T = fx_tiles(G.nx, G.ny, G.nz);
+  W.one.buf[1] = const_cast<double*>(u);
+  W.rec = w.rec;
+  return W;
 }
 
 // The tiled FP32-RHS stage on the single-precision copy ys32 and the tables
@@ -169,15 +170,10 @@ cudaError_t run_fused(int order, bssn_precision_t prec, const bssn_grid_t& G, co
                       cudaStream_t s) {
   if (prec == BSSN_FP32_RHS) return fused32(order, G, P, rk, ys, w.f32, y0, acc, out, nullptr, w.tab32, mode, s);
   const double eps = mode == 0 ? P.ko_eps : 0.0;  // the right-hand side alone has no dissipation
-  FxWork W{};
-  W.one.L = make_layout(G);
-  W.one.C = order == 4 ? make_fx<4>(G, eps) : make_fx<8>(G, eps);
-  W.one.T = fx_tiles(G.nx, G.ny, G.nz);
+  FxWork W = fx_work(order, G, eps, ys, w);
   W.one.buf[0] = const_cast<double*>(y0);
-  W.one.buf[1] = const_cast<double*>(ys);
   W.one.buf[2] = out;
   W.one.buf[3] = acc;
-  W.rec = w.rec;
   const int vol = W.one.T.vol;
   W.slot = (long long)REC_RHS * vol;
   // the scratch always holds a tile: its halo alone outweighs the record of
@@ -731,15 +727,9 @@ bssn_status_t bssn_psi4(const bssn_grid_t* grid, const bssn_params_t* params, co
   const WorkPtrs w = work_ptrs(work, *grid, *params, BSSN_FP64);
   const double h[3] = {grid->dx, grid->dy, grid->dz};
   cudaError_t e = cudaMemsetAsync(w.flag, 0, sizeof(unsigned int), s);
-  if (e == cudaSuccess) e = run_tables64(params->fd_order, *grid, state, w, s);
-  if (e == cudaSuccess) {
-    if (params->fd_order == 4)
-      e = launch_psi4<4>(L, make_coef<4, double>(*grid, 0.0), state, w.dX64, w.dY64, origin, h, psi_re, psi_im,
-                         inv_re, inv_im, E, B, w.flag, s);
-    else
-      e = launch_psi4<8>(L, make_coef<8, double>(*grid, 0.0), state, w.dX64, w.dY64, origin, h, psi_re, psi_im,
-                         inv_re, inv_im, E, B, w.flag, s);
-  }
+  if (e == cudaSuccess)
+    e = launch_psi4(params->fd_order, fx_work(params->fd_order, *grid, 0.0, state, w), w.rec_doubles, origin, h, psi_re,
+                    psi_im, inv_re, inv_im, E, B, w.flag, s);
   return latch(e);
 }
 
@@ -759,17 +749,12 @@ bssn_status_t constraints_impl(const bssn_grid_t* grid, const bssn_params_t* par
   const Layout L = make_layout(*grid);
   const WorkPtrs w = work_ptrs(work, *grid, *params, BSSN_FP64);
   cudaError_t e = cudaMemsetAsync(w.flag, 0, sizeof(unsigned int), s);
-  if (e == cudaSuccess) e = run_tables64(params->fd_order, *grid, state, w, s);
+  int nparts = 0;
+  if (e == cudaSuccess)
+    e = launch_constraints(params->fd_order, fx_work(params->fd_order, *grid, 0.0, state, w), w.rec_doubles, ham, mom,
+                           gcon, w.part, (long long)(w.part_doubles / 14), &nparts, w.flag, ham_only, s);
   if (e == cudaSuccess) {
-    if (params->fd_order == 4)
-      e = launch_constraints<4>(L, make_coef<4, double>(*grid, 0.0), state, w.dX64, w.dY64, ham, mom, gcon, w.part,
-                                w.flag, ham_only, s);
-    else
-      e = launch_constraints<8>(L, make_coef<8, double>(*grid, 0.0), state, w.dX64, w.dY64, ham, mom, gcon, w.part,
-                                w.flag, ham_only, s);
-  }
-  if (e == cudaSuccess) {
-    k_reduce_partials<<<1, 256, 0, s>>>(w.part, con_blocks(L), w.finals);
+    k_reduce_partials<<<1, 256, 0, s>>>(w.part, nparts, w.finals);
     e = cudaGetLastError();
   }
   double host[16];

@@ -83,6 +83,32 @@ struct DerivList {
 // then the 24 advection + dissipation sums.
 constexpr int REC_K = 9 * NM, REC_GAM = REC_K + 3, REC_EXT = REC_GAM + 9, REC_RHS = REC_EXT + NV;
 
+// Constraints and Weyl scalars: W and gt (9 each), Gt^i (3 each) - all the
+// Hamiltonian constraint needs - then K (3) and At (3 each).
+constexpr int REC_C_GAM = 9 * 7, REC_HAM = REC_C_GAM + 9, REC_C_K = REC_HAM, REC_C_AT = REC_C_K + 3,
+              REC_CON = REC_C_AT + 18;
+
+inline DerivList con_list(bool ham_only) {
+  DerivList D{};
+  for (int m = 0; m < 7; ++m) {
+    const int e = D.n++;
+    D.var[e] = (signed char)m;
+    D.d1[e] = (short)(9 * m);
+    D.d2[e] = (short)(9 * m + 3);
+  }
+  for (int v = V_TRK; v < V_ALPHA; ++v) {
+    const bool gam = v >= V_GAM1;
+    if (ham_only && !gam) continue;
+    const int e = D.n++;
+    D.var[e] = (signed char)v;
+    D.d1[e] = (short)(v == V_TRK ? REC_C_K : (gam ? REC_C_GAM + 3 * (v - V_GAM1) : REC_C_AT + 3 * (v - V_AT11)));
+    D.d2[e] = -1;
+  }
+  for (int e = 0; e < D.n; ++e) D.ext[e] = -1;
+  D.nout = ham_only ? REC_HAM : REC_CON;
+  return D;
+}
+
 inline DerivList rhs_list() {
   DerivList D{};
   for (int m = 0; m < NM; ++m) {

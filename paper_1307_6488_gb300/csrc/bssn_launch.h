@@ -9,10 +9,6 @@
 
 namespace bssn {
 
-// FP64 first-difference tables of the constraints and Weyl scalars (H per
-// mixed variable).
-template <int P>
-cudaError_t launch_diffs(const Layout& L, const double* u, double* dX, double* dY, cudaStream_t s);
 // Derivatives of `nslots` tiles into the record (bssn_fixed.cuh).
 template <int P>
 cudaError_t derivs_init();  // raises the kernel's shared-memory limit (not during a capture)
@@ -26,15 +22,16 @@ cudaError_t launch_stage64(int order, const FxWork& work, int vol, long long nti
 template <int P>
 cudaError_t launch_ko(const Layout& L, const bssn_grid_t& G, double eps, bssn_precision_t prec, const double* u,
                       double* rhs, cudaStream_t s);
-template <int P>
-cudaError_t launch_constraints(const Layout& L, const Coef<double>& C, const double* u, const double* dX,
-                               const double* dY, double* ham, double* mom, double* gcon, double* part,
-                               unsigned int* flag, bool ham_only, cudaStream_t s);
-
-template <int P>
-cudaError_t launch_psi4(const Layout& L, const Coef<double>& C, const double* u, const double* dX, const double* dY,
-                        const double origin[3], const double h[3], double* psi_re, double* psi_im, double* inv_re,
-                        double* inv_im, double* E, double* B, unsigned int* flag, cudaStream_t s);
+// The constraints at every point (or, ham_only, the Hamiltonian alone), with
+// sums and maxima per block in part (14 doubles each; *nparts of at most
+// max_parts are written), and the Weyl scalars. Single grids, through a record
+// of rec_doubles.
+cudaError_t launch_constraints(int order, FxWork work, size_t rec_doubles, double* ham, double* mom, double* gcon,
+                               double* part, long long max_parts, int* nparts, unsigned int* flag, bool ham_only,
+                               cudaStream_t s);
+cudaError_t launch_psi4(int order, FxWork work, size_t rec_doubles, const double origin[3], const double h[3],
+                        double* psi_re, double* psi_im, double* inv_re, double* inv_im, double* E, double* B,
+                        unsigned int* flag, cudaStream_t s);
 
 // Tiled FP32-RHS path of single grids (bssn_stage32.cu): the single-precision
 // copy and tables live in Layout32 (tables: 11 D_x arrays, then 11 D_y).

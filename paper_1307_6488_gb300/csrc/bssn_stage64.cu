@@ -1,15 +1,32 @@
-// The FP64 stage of single grids, patches and refined levels: derivatives on
-// the integer pipes (k_derivs, bssn_fixed.cuh), then the pointwise algebra
-// and the stage update on the FP64 pipe, tile by tile through a record that
-// holds as many tiles as the caller's scratch takes.
+// The FP64 stage of single grids, patches and refined levels, the constraints
+// and the Weyl scalars: derivatives on the integer pipes (k_derivs,
+// bssn_fixed.cuh), then the pointwise algebra on the FP64 pipe, tile by tile
+// through a record that holds as many tiles as the caller's scratch takes.
 #include <algorithm>
 
 #include "bssn_bounds.cuh"
 #include "bssn_fixed.cuh"
 #include "bssn_launch.h"
 #include "bssn_point.cuh"
+#include "bssn_weyl.cuh"
 
 namespace bssn {
+
+// Point idx of a tile; false outside the grid.
+struct TilePoint {
+  int i, j, k;
+  long long p;
+};
+__device__ __forceinline__ bool tile_point(const FxGrid& G, int ti, int tj, int tk, int idx, TilePoint& q) {
+  if (idx >= G.T.vol) return false;
+  const int yz = idx / G.T.tx;
+  q.i = ti * FX_T + idx - yz * G.T.tx;
+  q.j = tj * FX_T + yz % G.T.ty;
+  q.k = tk * FX_T + yz / G.T.ty;
+  if (q.i >= G.L.nx || q.j >= G.L.ny || q.k >= G.L.nz) return false;
+  q.p = G.L.off0 + q.i + q.j * G.L.sy + q.k * G.L.sz;
+  return in_range(q.p, q.p, padded_points(G.L));
+}
 
 // Threads of a block and resident blocks per SM. The kernel is bound by the
 // FP64 pipe (~1100 instructions per point at 1.68 per clock and SM), which a
@@ -30,15 +47,10 @@ __global__ void __launch_bounds__(ALG_THREADS, ALG_MIN_BLOCKS) k_algebra(const _
   const int idx = (int)(blockIdx.x - slot * blocks_per_slot) * ALG_THREADS + threadIdx.x;
   int ti, tj, tk;
   const FxGrid& G = fx_locate(A.W, A.W.tile0 + slot, ti, tj, tk);
-  const Layout& L = G.L;
+  TilePoint pt;
+  if (!tile_point(G, ti, tj, tk, idx, pt)) return;
+  const long long p = pt.p, vs = G.L.vs;
   const int vol = G.T.vol;
-  if (idx >= vol) return;
-  const int x = idx % G.T.tx, yz = idx / G.T.tx;
-  const int i = ti * FX_T + x, j = tj * FX_T + yz % G.T.ty, k = tk * FX_T + yz / G.T.ty;
-  if (i >= L.nx || j >= L.ny || k >= L.nz) return;
-  const long long p = L.off0 + i + j * L.sy + k * L.sz;
-  if (!in_range(p, p, padded_points(L))) return;
-  const long long vs = L.vs;
   const double* __restrict__ rec = A.W.rec + (long long)slot * A.W.slot + idx;
   const double* __restrict__ ys = G.buf[A.S.in] + p;
   PointIn<double> Q;
@@ -106,6 +118,199 @@ __global__ void __launch_bounds__(ALG_THREADS, ALG_MIN_BLOCKS) k_algebra(const _
     }
     out[o] = yn;
   }
+}
+
+// The set of the constraints and Weyl scalars at one point.
+template <bool HONLY>
+__device__ __forceinline__ void load_con(const double* __restrict__ rec, int vol, const double* __restrict__ u,
+                                         long long vs, PointIn<double>& Q, double dAt[3][6]) {
+  auto r = [&](int o) { return __ldg(rec + o * vol); };
+#pragma unroll
+  for (int v = 0; v < NV; ++v) Q.u[v] = __ldg(u + v * vs);
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    Q.dW[d] = r(d);
+    Q.dK[d] = HONLY ? 0.0 : r(REC_C_K + d);
+#pragma unroll
+    for (int s = 0; s < 6; ++s) {
+      Q.dg[d][s] = r(9 * (1 + s) + d);
+      dAt[d][s] = HONLY ? 0.0 : r(REC_C_AT + 3 * s + d);
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) Q.dGam[d][c] = r(REC_C_GAM + 3 * c + d);
+  }
+#pragma unroll
+  for (int s = 0; s < 6; ++s) {
+    Q.ddW[s] = r(3 + s);
+#pragma unroll
+    for (int c = 0; c < 6; ++c) Q.ddg[c][s] = r(9 * (1 + c) + 3 + s);
+  }
+}
+
+struct ConArgs {
+  FxWork W;
+  double *ham, *mom, *gcon, *part;
+  unsigned int* flag;
+};
+
+// Constraints of the points of `nblocks` blocks of CON_THREADS points
+// (blocks_per_slot to a slot), grid-stride. Per-block partial results, 7 sums
+// of squares and 7 maxima, are added to part[blockIdx.x * 14 + q] (written by
+// the first chunk), so that one small array serves any number of tiles in a
+// fixed order. With HONLY the Hamiltonian constraint alone (the momentum and
+// Gamma slots stay 0); its values are the same bits as in the full evaluation.
+// Bound by the FP64 pipe (128 registers and 4 blocks an SM, as the algebra).
+template <bool HONLY>
+__global__ void __launch_bounds__(CON_THREADS, 4) k_constraints(const __grid_constant__ ConArgs A, unsigned int nblocks,
+                                                               int blocks_per_slot, bool first) {
+  double sum[7], top[7];
+#pragma unroll
+  for (int q = 0; q < 7; ++q) sum[q] = top[q] = 0.0;
+  bool bad = false;
+  for (unsigned int b = blockIdx.x; b < nblocks; b += gridDim.x) {
+    const unsigned int slot = b / (unsigned int)blocks_per_slot;
+    const int idx = (int)(b - slot * blocks_per_slot) * CON_THREADS + threadIdx.x;
+    int ti, tj, tk;
+    const FxGrid& G = fx_locate(A.W, A.W.tile0 + slot, ti, tj, tk);
+    TilePoint pt;
+    if (!tile_point(G, ti, tj, tk, idx, pt)) continue;
+    const long long p = pt.p, vs = G.L.vs;
+    PointIn<double> Q;
+    double dAt[3][6], c[7];
+    load_con<HONLY>(A.W.rec + (long long)slot * A.W.slot + idx, G.T.vol, G.buf[1] + p, vs, Q, dAt);
+    constraints_point<double>(Q, dAt, 1.0 / Q.u[V_W], c);
+    if (HONLY)
+#pragma unroll
+      for (int q = 1; q < 7; ++q) c[q] = 0.0;
+    if (A.ham) A.ham[p] = c[0];
+    if (A.mom && !HONLY)
+#pragma unroll
+      for (int a = 0; a < 3; ++a) A.mom[a * vs + p] = c[1 + a];
+    if (A.gcon && !HONLY)
+#pragma unroll
+      for (int a = 0; a < 3; ++a) A.gcon[a * vs + p] = c[4 + a];
+#pragma unroll
+    for (int q = 0; q < 7; ++q) {
+      bad |= !isfinite(c[q]);
+      sum[q] += c[q] * c[q];
+      top[q] = fmax(top[q], fabs(c[q]));  // a NaN is left out here and reported by the flag
+    }
+    bad |= !(Q.u[V_W] > 0.0);  // the conformal factor must stay positive
+  }
+  if (bad) atomicOr(A.flag, 1u);
+  __shared__ double red[CON_THREADS / 32][14];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int q = 0; q < 7; ++q) {
+    double s = sum[q], m = top[q];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      s += __shfl_down_sync(0xffffffffu, s, o);
+      m = fmax(m, __shfl_down_sync(0xffffffffu, m, o));
+    }
+    if (lane == 0) {
+      red[warp][q] = s;
+      red[warp][7 + q] = m;
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < 14) {
+    const int q = threadIdx.x;
+    double* out = A.part + (long long)blockIdx.x * 14 + q;
+    double r = first ? 0.0 : *out;
+    for (int w = 0; w < CON_THREADS / 32; ++w) r = (q < 7) ? r + red[w][q] : fmax(r, red[w][q]);
+    *out = r;
+  }
+}
+
+struct WeylArgs {
+  FxWork W;
+  double o[3], h[3];
+  double *psi_re, *psi_im, *inv_re, *inv_im, *E, *B;
+  unsigned int* flag;
+};
+
+// Weyl scalars, one point per thread; outputs in the state's padded layout
+// (E and B as 6 arrays var_stride apart), each nullable. FP64-pipe bound.
+__global__ void __launch_bounds__(CON_THREADS, 4) k_psi4(const __grid_constant__ WeylArgs A, int blocks_per_slot) {
+  const unsigned int slot = blockIdx.x / (unsigned int)blocks_per_slot;
+  const int idx = (int)(blockIdx.x - slot * blocks_per_slot) * CON_THREADS + threadIdx.x;
+  int ti, tj, tk;
+  const FxGrid& G = fx_locate(A.W, A.W.tile0 + slot, ti, tj, tk);
+  TilePoint pt;
+  if (!tile_point(G, ti, tj, tk, idx, pt)) return;
+  const long long p = pt.p, vs = G.L.vs;
+  PointIn<double> Q;
+  double dAt[3][6];
+  load_con<false>(A.W.rec + (long long)slot * A.W.slot + idx, G.T.vol, G.buf[1] + p, vs, Q, dAt);
+  const double xyz[3] = {A.o[0] + pt.i * A.h[0], A.o[1] + pt.j * A.h[1], A.o[2] + pt.k * A.h[2]};
+  WeylOut O;
+  weyl_point(Q, dAt, xyz, O);
+  const bool bad = !isfinite(O.psi_re) || !isfinite(O.psi_im) || !isfinite(O.inv_re) || !isfinite(O.inv_im);
+  if (A.psi_re) A.psi_re[p] = O.psi_re;
+  if (A.psi_im) A.psi_im[p] = O.psi_im;
+  if (A.inv_re) A.inv_re[p] = O.inv_re;
+  if (A.inv_im) A.inv_im[p] = O.inv_im;
+#pragma unroll
+  for (int s = 0; s < 6; ++s) {
+    if (A.E) A.E[s * vs + p] = O.E[s];
+    if (A.B) A.B[s * vs + p] = O.B[s];
+  }
+  if (bad) atomicOr(A.flag, 1u);
+}
+
+// Runs derivatives and `use` (called with the slots of the chunk and whether
+// it is the first) over the grid's tiles, as many at a time as the record holds.
+template <typename F>
+static cudaError_t through_record(int order, const FxWork& work, const DerivList& list, size_t rec_doubles,
+                                  cudaStream_t s, F use) {
+  const FxTiles& T = work.one.T;
+  DerivArgs D{work, list, 1, false, false, false};
+  D.W.slot = (long long)list.nout * T.vol;
+  const long long ntiles = (long long)T.ntx * T.nty * T.ntz, slots = (long long)(rec_doubles / (size_t)D.W.slot);
+  if (slots < 1) return cudaErrorInvalidValue;
+  const long long chunks = (ntiles + slots - 1) / slots, per = (ntiles + chunks - 1) / chunks;
+  for (long long t = 0; t < ntiles; t += per) {
+    const long long n = std::min(per, ntiles - t);
+    D.W.tile0 = t;
+    cudaError_t e = order == 4 ? launch_derivs<4>(D, n, s) : launch_derivs<8>(D, n, s);
+    if (e != cudaSuccess) return e;
+    use(D.W, n, t == 0);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+cudaError_t launch_constraints(int order, FxWork work, size_t rec_doubles, double* ham, double* mom, double* gcon,
+                               double* part, long long max_parts, int* nparts, unsigned int* flag, bool ham_only,
+                               cudaStream_t s) {
+  ConArgs A{work, ham, mom, gcon, part, flag};
+  const int bps = (work.one.T.vol + CON_THREADS - 1) / CON_THREADS;
+  *nparts = 0;
+  return through_record(order, work, con_list(ham_only), rec_doubles, s, [&](const FxWork& W, long long n, bool first) {
+    A.W = W;
+    // as many blocks as are resident (4 on each of 152 SMs): each takes the
+    // points of several tiles, and the partial sums stay few
+    const unsigned int nb = (unsigned int)(n * bps);
+    if (first) *nparts = (int)std::min<long long>(std::min<long long>(nb, max_parts), 608);
+    const unsigned int g = (unsigned int)*nparts;  // the last chunk may be smaller: idle blocks add nothing
+    if (ham_only)
+      k_constraints<true><<<g, CON_THREADS, 0, s>>>(A, nb, bps, first);
+    else
+      k_constraints<false><<<g, CON_THREADS, 0, s>>>(A, nb, bps, first);
+  });
+}
+
+cudaError_t launch_psi4(int order, FxWork work, size_t rec_doubles, const double origin[3], const double h[3],
+                        double* psi_re, double* psi_im, double* inv_re, double* inv_im, double* E, double* B,
+                        unsigned int* flag, cudaStream_t s) {
+  WeylArgs A{work, {origin[0], origin[1], origin[2]}, {h[0], h[1], h[2]}, psi_re, psi_im, inv_re, inv_im, E, B, flag};
+  const int bps = (work.one.T.vol + CON_THREADS - 1) / CON_THREADS;
+  return through_record(order, work, con_list(false), rec_doubles, s, [&](const FxWork& W, long long n, bool) {
+    A.W = W;
+    k_psi4<<<(unsigned int)(n * bps), CON_THREADS, 0, s>>>(A, bps);
+  });
 }
 
 cudaError_t launch_stage64(int order, const FxWork& work, int vol, long long ntiles, long long slots,

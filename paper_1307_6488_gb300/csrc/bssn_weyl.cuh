@@ -11,7 +11,7 @@
 // (x, y, z), (xz, yz, -(x^2 + y^2)), (-y, x, 0) about the coordinate origin;
 // Psi_4 = 0 where x = y = 0.
 #pragma once
-#include "bssn_kernels.cuh"
+#include "bssn_point.cuh"
 
 namespace bssn {
 
@@ -140,46 +140,6 @@ __device__ __forceinline__ void weyl_point(const PointIn<double>& P, const doubl
   const double Btt = sdot3(O.B, et, et), Bpp = sdot3(O.B, ep, ep), Btp = sdot3(O.B, et, ep);
   O.psi_re = 0.5 * (Ett - Epp) - Btp;
   O.psi_im = -0.5 * (Btt - Bpp) - Etp;
-}
-
-// One thread per interior point; outputs in the state's padded layout
-// (E and B as 6 arrays var_stride apart), each nullable.
-template <int P>
-__global__ void __launch_bounds__(128, STAGE_F64_MIN_BLOCKS) k_psi4(Layout L, Coef<double> C, const double* __restrict__ u,
-                                              const double* __restrict__ dX, const double* __restrict__ dY,
-                                              double ox, double oy, double oz, double hx, double hy, double hz,
-                                              double* psi_re, double* psi_im, double* inv_re, double* inv_im,
-                                              double* Eo, double* Bo, unsigned int* flag) {
-  constexpr int H = FD<P>::H;
-  const long long lin = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (lin >= L.npts) return;
-  int i, j, k;
-  i = (int)(lin % L.nx);
-  brick_row<STAGE_BRICK_Y64, STAGE_BRICK_Z64>(lin / L.nx, L.ny, L.nz, j, k);  // rows in brick order, as k_stage
-  const long long p = L.off0 + i + j * L.sy + k * L.sz;
-  if (!in_range(p - FD<P>::R * L.sz, p + FD<P>::R * L.sz, padded_points(L))) return;
-  PointIn<double> Q;
-  gather<P, double>(L, C, u, dX, dY, p, Q);
-  double dAt[3][6];
-  const long long st[3] = {1, L.sy, L.sz};
-#pragma unroll
-  for (int d = 0; d < 3; ++d)
-#pragma unroll
-    for (int s = 0; s < 6; ++s) dAt[d][s] = d1_direct<H>(u + (V_AT11 + s) * L.vs, p, st[d], C.c1[d]);
-  const double xyz[3] = {ox + i * hx, oy + j * hy, oz + k * hz};
-  WeylOut O;
-  weyl_point(Q, dAt, xyz, O);
-  bool bad = !isfinite(O.psi_re) || !isfinite(O.psi_im) || !isfinite(O.inv_re) || !isfinite(O.inv_im);
-  if (psi_re) psi_re[p] = O.psi_re;
-  if (psi_im) psi_im[p] = O.psi_im;
-  if (inv_re) inv_re[p] = O.inv_re;
-  if (inv_im) inv_im[p] = O.inv_im;
-#pragma unroll
-  for (int s = 0; s < 6; ++s) {
-    if (Eo) Eo[s * L.vs + p] = O.E[s];
-    if (Bo) Bo[s * L.vs + p] = O.B[s];
-  }
-  if (bad) atomicOr(flag, 1u);
 }
 
 }  // namespace bssn
