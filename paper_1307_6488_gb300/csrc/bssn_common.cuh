@@ -212,14 +212,8 @@ inline RK make_rk3(int stage, double dt) {
   return r;
 }
 
-// Pointers of the difference tables inside the work buffer: dX holds the
-// x-differences u(i+a) - u(i-a), dY the y-differences, for the NM mixed
-// variables and a = 1..H, each table var_stride doubles.
-struct Diffs {
-  double* dX;
-  double* dY;
-};
-
+// Doubles of the tables region of the work buffer that the p/2-dependent part
+// of its size comes from: 2 x 11 x p/2 arrays.
 inline size_t diff_doubles(const Layout& L, int H) { return (size_t)2 * NM * H * (size_t)L.vs; }
 
 }  // namespace bssn

@@ -77,6 +77,18 @@ struct DerivList {
   short d1[NV];   // first of 3 outputs (x, y, z), or -1
   short d2[NV];   // first of 6 outputs (xx, xy, xz, yy, yz, zz), or -1
   short ext[NV];  // advection + dissipation, or -1
+  float f1[NV], f2[NV];  // factors (powers of two) of the first and second derivatives
+
+  void add(int v, int o1, int o2, int oe) {
+    const bool gt = v >= V_GT11 && v <= V_GT33, gam = v >= V_GAM1 && v <= V_GAM3;
+    var[n] = (signed char)v;
+    d1[n] = (short)o1;
+    d2[n] = (short)o2;
+    ext[n] = (short)oe;
+    f1[n] = gt || gam ? 0.5f : 1.0f;  // the algebra takes half of these (Point64)
+    f2[n] = gt ? -0.5f : 1.0f;
+    ++n;
+  }
 };
 
 // Right-hand side: W, gt, alpha, beta (9 outputs each), K and Gt^i (3 each),
@@ -90,41 +102,23 @@ constexpr int REC_C_GAM = 9 * 7, REC_HAM = REC_C_GAM + 9, REC_C_K = REC_HAM, REC
 
 inline DerivList con_list(bool ham_only) {
   DerivList D{};
-  for (int m = 0; m < 7; ++m) {
-    const int e = D.n++;
-    D.var[e] = (signed char)m;
-    D.d1[e] = (short)(9 * m);
-    D.d2[e] = (short)(9 * m + 3);
+  for (int m = 0; m < 7; ++m) D.add(m, 9 * m, 9 * m + 3, -1);
+  for (int i = 0; i < 3; ++i) D.add(V_GAM1 + i, REC_C_GAM + 3 * i, -1, -1);
+  if (!ham_only) {
+    D.add(V_TRK, REC_C_K, -1, -1);
+    for (int s = 0; s < 6; ++s) D.add(V_AT11 + s, REC_C_AT + 3 * s, -1, -1);
   }
-  for (int v = V_TRK; v < V_ALPHA; ++v) {
-    const bool gam = v >= V_GAM1;
-    if (ham_only && !gam) continue;
-    const int e = D.n++;
-    D.var[e] = (signed char)v;
-    D.d1[e] = (short)(v == V_TRK ? REC_C_K : (gam ? REC_C_GAM + 3 * (v - V_GAM1) : REC_C_AT + 3 * (v - V_AT11)));
-    D.d2[e] = -1;
-  }
-  for (int e = 0; e < D.n; ++e) D.ext[e] = -1;
   D.nout = ham_only ? REC_HAM : REC_CON;
   return D;
 }
 
 inline DerivList rhs_list() {
   DerivList D{};
-  for (int m = 0; m < NM; ++m) {
-    const int e = D.n++;
-    D.var[e] = (signed char)mvar(m);
-    D.d1[e] = (short)(9 * m);
-    D.d2[e] = (short)(9 * m + 3);
-  }
+  for (int m = 0; m < NM; ++m) D.add(mvar(m), 9 * m, 9 * m + 3, REC_EXT + mvar(m));
   for (int v = 0; v < NV; ++v) {
     if (mixed_index(v) >= 0) continue;
-    const int e = D.n++;
-    D.var[e] = (signed char)v;
-    D.d1[e] = (short)(v == V_TRK ? REC_K : (v >= V_GAM1 && v <= V_GAM3 ? REC_GAM + 3 * (v - V_GAM1) : -1));
-    D.d2[e] = -1;
+    D.add(v, v == V_TRK ? REC_K : (v >= V_GAM1 && v <= V_GAM3 ? REC_GAM + 3 * (v - V_GAM1) : -1), -1, REC_EXT + v);
   }
-  for (int e = 0; e < D.n; ++e) D.ext[e] = (short)(REC_EXT + D.var[e]);
   D.nout = REC_RHS;
   return D;
 }
@@ -342,8 +336,9 @@ __device__ __forceinline__ double fx_mixed(const int4* __restrict__ g, int st, i
 // Stencils along the three axes at one point of the box, and the outputs.
 template <int P, bool D1, bool D2, bool EXT>
 __device__ __forceinline__ void fx_point(const int2* __restrict__ c, const int4* const g[3], const FxCoef& C,
-                                         const double* beta, double wa, int emax, double* __restrict__ o1,
-                                         double* __restrict__ o2, double* __restrict__ oe, int vol) {
+                                         const double* beta, double wa, double f1, double f2, int emax,
+                                         double* __restrict__ o1, double* __restrict__ o2, double* __restrict__ oe,
+                                         int vol) {
   using F = FD<P>;
   using X = FX<P>;
   constexpr int BX = FxSmem<P>::BX;
@@ -377,8 +372,8 @@ __device__ __forceinline__ void fx_point(const int2* __restrict__ c, const int4*
         kh += (long long)X::WK(a) * (p.y + m.y + m2y);
       }
     }
-    if (D1) o1[d * vol] = C.c1[d] * fx_to_double(r1h, r1l, emax);
-    if (D2) o2[sym(d, d) * vol] = C.c2[sym(d, d)] * fx_to_double(r2h, r2l, emax);
+    if (D1) o1[d * vol] = (f1 * C.c1[d]) * fx_to_double(r1h, r1l, emax);
+    if (D2) o2[sym(d, d) * vol] = (f2 * C.c2[sym(d, d)]) * fx_to_double(r2h, r2l, emax);
     if (EXT) {
       // |b| times the stencil mirrored by the sign of b
       const double b = wa * beta[d];
@@ -398,9 +393,9 @@ __device__ __forceinline__ void fx_point(const int2* __restrict__ c, const int4*
     *oe = ext;
   }
   if (D2) {
-    o2[1 * vol] = C.c2[1] * fx_mixed<P>(g[0], FX_T, emax);
-    o2[2 * vol] = C.c2[2] * fx_mixed<P>(g[1], FX_T * FX_T, emax);
-    o2[4 * vol] = C.c2[4] * fx_mixed<P>(g[2], FX_T * FX_T, emax);
+    o2[1 * vol] = (f2 * C.c2[1]) * fx_mixed<P>(g[0], FX_T, emax);
+    o2[2 * vol] = (f2 * C.c2[2]) * fx_mixed<P>(g[1], FX_T * FX_T, emax);
+    o2[4 * vol] = (f2 * C.c2[4]) * fx_mixed<P>(g[2], FX_T * FX_T, emax);
   }
 }
 
@@ -485,6 +480,7 @@ __device__ __forceinline__ void fx_tile(const Layout& L, const FxCoef& C, const 
 
   const bool d1 = list.d1[e] >= 0, ext = list.ext[e] >= 0;
   const int vol = T.vol;
+  const double f1 = list.f1[e], f2 = list.f2[e];
   double* const o1 = rec + (long long)(d1 ? list.d1[e] : 0) * vol;
   double* const o2 = rec + (long long)(mixed ? list.d2[e] : 0) * vol;
   double* const oe = rec + (long long)(ext ? list.ext[e] : 0) * vol;
@@ -541,9 +537,9 @@ __device__ __forceinline__ void fx_tile(const Layout& L, const FxCoef& C, const 
       double r1[3], r2[6], re;
       fx_fallback<P>(v, p, L.sy, L.sz, C, beta, wa, d1, mixed, ext, r1, r2, &re);
       if (d1)
-        for (int d = 0; d < 3; ++d) o1[d * vol + idx] = r1[d];
+        for (int d = 0; d < 3; ++d) o1[d * vol + idx] = f1 * r1[d];
       if (mixed)
-        for (int s = 0; s < 6; ++s) o2[s * vol + idx] = r2[s];
+        for (int s = 0; s < 6; ++s) o2[s * vol + idx] = f2 * r2[s];
       if (ext) oe[idx] = re;
       continue;
     }
@@ -551,15 +547,15 @@ __device__ __forceinline__ void fx_tile(const Layout& L, const FxCoef& C, const 
     const int4* const gt[3] = {g + (z * S::EH + (y + H)) * FX_T + x, g + S::GN + ((z + H) * FX_T + y) * FX_T + x,
                                g + 2 * S::GN + ((z + H) * FX_T + y) * FX_T + x};
     if (mixed && ext)
-      fx_point<P, true, true, true>(c, gt, C, beta, wa, emax, o1 + idx, o2 + idx, oe + idx, vol);
+      fx_point<P, true, true, true>(c, gt, C, beta, wa, f1, f2, emax, o1 + idx, o2 + idx, oe + idx, vol);
     else if (mixed)
-      fx_point<P, true, true, false>(c, gt, C, beta, wa, emax, o1 + idx, o2 + idx, oe + idx, vol);
+      fx_point<P, true, true, false>(c, gt, C, beta, wa, f1, f2, emax, o1 + idx, o2 + idx, oe + idx, vol);
     else if (d1 && ext)
-      fx_point<P, true, false, true>(c, gt, C, beta, wa, emax, o1 + idx, o2 + idx, oe + idx, vol);
+      fx_point<P, true, false, true>(c, gt, C, beta, wa, f1, f2, emax, o1 + idx, o2 + idx, oe + idx, vol);
     else if (d1)
-      fx_point<P, true, false, false>(c, gt, C, beta, wa, emax, o1 + idx, o2 + idx, oe + idx, vol);
+      fx_point<P, true, false, false>(c, gt, C, beta, wa, f1, f2, emax, o1 + idx, o2 + idx, oe + idx, vol);
     else
-      fx_point<P, false, false, true>(c, gt, C, beta, wa, emax, o1 + idx, o2 + idx, oe + idx, vol);
+      fx_point<P, false, false, true>(c, gt, C, beta, wa, f1, f2, emax, o1 + idx, o2 + idx, oe + idx, vol);
   }
 }
 

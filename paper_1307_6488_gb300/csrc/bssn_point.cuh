@@ -1,4 +1,5 @@
-// Pointwise algebra of the BSSN right-hand side and constraints.
+// Pointwise algebra of the BSSN right-hand side, FP32-RHS form (the FP64
+// forms' is bssn_point64.cuh).
 //
 // The evolution system is the vacuum BSSN system in the conformal variable
 // W = (det gamma)^(-1/6) (the paper's Sec. 1.1 cites the BSSN formulation
@@ -27,24 +28,11 @@
 
 namespace bssn {
 
-template <typename R>
-struct PointIn {
-  R u[NV];
-  R dW[3], dK[3], da[3];
-  R dg[3][6];    // dg[d][s]   = d_d gt_s
-  R dGam[3][3];  // dGam[d][i] = d_d Gt^i
-  R db[3][3];    // db[d][i]   = d_d beta^i
-  R ddW[6], dda[6];
-  R ddb[3][6];   // ddb[i][s]  = d_s beta^i (s a packed pair of directions)
-  R ddg[6][6];   // ddg[s][t]  = d_t gt_s
-  R adv[NV];     // beta^k dhat_k u_v
-};
-
 // The FP32-RHS form's per-point set. The second derivatives of gt_ij and of
 // beta^i enter the right-hand side only through contractions with gt^ij, so
-// the gather forms those contractions as each derivative is produced and
-// keeps 12 values instead of 54; advection enters additively and is carried
-// by the caller together with the dissipation.
+// the stencil loop forms those contractions as each derivative is produced
+// and keeps 12 values instead of 54; advection enters additively and is
+// carried by the caller together with the dissipation.
 template <typename R>
 struct PointLean {
   R u[NV];
@@ -72,40 +60,16 @@ __device__ __forceinline__ void inverse_metric(const R* g, R gu[6]) {
   gu[3] = c3 * idet; gu[4] = c4 * idet; gu[5] = c5 * idet;
 }
 
-// -1/2 gt^lm d_l d_m gt_s, given hgu = -1/2 gt^lm with the off-diagonal
-// entries doubled
-template <typename R>
-__device__ __forceinline__ R metric_laplacian(const PointIn<R>& P, const R hgu[6], int s) {
-  R r = hgu[0] * P.ddg[s][0];
-#pragma unroll
-  for (int t = 1; t < 6; ++t) r += hgu[t] * P.ddg[s][t];
-  return r;
-}
 template <typename R>
 __device__ __forceinline__ R metric_laplacian(const PointLean<R>& P, const R*, int s) { return P.lapg[s]; }
 
-// gt^jk d_j d_k beta^i (gu2: gt^jk with the off-diagonal entries doubled)
-template <typename R>
-__device__ __forceinline__ R shift_laplacian(const PointIn<R>& P, const R gu2[6], int i) {
-  R t3 = gu2[0] * P.ddb[i][0];
-#pragma unroll
-  for (int s = 1; s < 6; ++s) t3 += gu2[s] * P.ddb[i][s];
-  return t3;
-}
 template <typename R>
 __device__ __forceinline__ R shift_laplacian(const PointLean<R>& P, const R*, int i) { return P.lapb[i]; }
 
-// d_j d_k beta^k
-template <typename R>
-__device__ __forceinline__ R grad_div_shift(const PointIn<R>& P, int j) {
-  return P.ddb[0][sym(j, 0)] + P.ddb[1][sym(j, 1)] + P.ddb[2][sym(j, 2)];
-}
 template <typename R>
 __device__ __forceinline__ R grad_div_shift(const PointLean<R>& P, int j) { return P.dddb[j]; }
 
-// advection of variable v, or 0 where the caller adds it
-template <typename R>
-__device__ __forceinline__ R advection(const PointIn<R>& P, int v) { return P.adv[v]; }
+// advection is added by the caller, with the dissipation
 template <typename R>
 __device__ __forceinline__ R advection(const PointLean<R>&, int) { return R(0); }
 
@@ -334,52 +298,6 @@ __device__ __forceinline__ void rhs_point(const PT<R>& P, const Gauge& gz, R iW,
       rhs[V_B1 + i] = R(0);
     }
   }
-}
-
-// Hamiltonian, momentum and Gamma constraints at a point (needs P.dAt).
-template <typename R>
-__device__ __forceinline__ void constraints_point(const PointIn<R>& P, const R dAt[3][6], R iW, R out[7]) {
-  Geo<R> G;
-  geometry<R, PointIn>(P, iW, G);
-  const R* u = P.u;
-  const R W = u[V_W], K = u[V_TRK];
-  const R* A = u + V_AT11;
-  R Am[3][3];  // At^i_j
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j)
-      Am[i][j] = G.gu[sym(i, 0)] * A[sym(0, j)] + G.gu[sym(i, 1)] * A[sym(1, j)] + G.gu[sym(i, 2)] * A[sym(2, j)];
-  R AA = R(0);
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) AA += Am[i][j] * Am[j][i];
-  R Rs = G.gu2[0] * G.Ric[0];
-#pragma unroll
-  for (int s = 1; s < 6; ++s) Rs += G.gu2[s] * G.Ric[s];
-  out[0] = W * W * Rs + R(2.0 / 3.0) * K * K - AA;
-  // M_i = gt^jk (d_k At_ij - Gt^l_ki At_lj - Gt^l_kj At_il) - 3/W At^j_i d_j W - 2/3 d_i K
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    R div = R(0);
-#pragma unroll
-    for (int s = 0; s < 6; ++s) {  // s = (j,k) symmetric pair, weight gu2
-      const int j = sym_i(s), k = sym_j(s);
-      // symmetrise the summand over (j,k): D_k At_ij + D_j At_ik
-      R t = dAt[k][sym(i, j)] + dAt[j][sym(i, k)];
-#pragma unroll
-      for (int l = 0; l < 3; ++l) {
-        t -= G.GU[l][sym(k, i)] * A[sym(l, j)] + G.GU[l][sym(k, j)] * A[sym(i, l)];
-        t -= G.GU[l][sym(j, i)] * A[sym(l, k)] + G.GU[l][sym(j, k)] * A[sym(i, l)];
-      }
-      div += G.gu2[s] * t;
-    }
-    const R aw = Am[0][i] * P.dW[0] + Am[1][i] * P.dW[1] + Am[2][i] * P.dW[2];
-    out[1 + i] = R(0.5) * div - R(3) * iW * aw - R(2.0 / 3.0) * P.dK[i];
-  }
-#pragma unroll
-  for (int i = 0; i < 3; ++i) out[4 + i] = u[V_GAM1 + i] - G.Gd[i];
 }
 
 }  // namespace bssn

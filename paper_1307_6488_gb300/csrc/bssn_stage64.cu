@@ -7,7 +7,7 @@
 #include "bssn_bounds.cuh"
 #include "bssn_fixed.cuh"
 #include "bssn_launch.h"
-#include "bssn_point.cuh"
+#include "bssn_point64.cuh"
 #include "bssn_weyl.cuh"
 
 namespace bssn {
@@ -29,7 +29,7 @@ __device__ __forceinline__ bool tile_point(const FxGrid& G, int ti, int tj, int 
 }
 
 // Threads of a block and resident blocks per SM. The kernel is bound by the
-// FP64 pipe (~1100 instructions per point at 1.68 per clock and SM), which a
+// FP64 pipe (~800 instructions per point at 1.68 per clock and SM), which a
 // few warps keep busy; small blocks spread a small grid over all SMs.
 #ifndef ALG_THREADS
 #define ALG_THREADS 64
@@ -39,7 +39,7 @@ __device__ __forceinline__ bool tile_point(const FxGrid& G, int ti, int tj, int 
 #endif
 
 // One thread per point of a slot: the pointwise right-hand side from the
-// record of k_derivs, plus its advection + dissipation sums, and the stage
+// record of k_derivs (with its advection + dissipation sums) and the stage
 // update.
 __global__ void __launch_bounds__(ALG_THREADS, ALG_MIN_BLOCKS) k_algebra(const __grid_constant__ AlgebraArgs A,
                                                                        int blocks_per_slot) {
@@ -53,12 +53,9 @@ __global__ void __launch_bounds__(ALG_THREADS, ALG_MIN_BLOCKS) k_algebra(const _
   const int vol = G.T.vol;
   const double* __restrict__ rec = A.W.rec + (long long)slot * A.W.slot + idx;
   const double* __restrict__ ys = G.buf[A.S.in] + p;
-  PointIn<double> Q;
+  Point64 Q;
 #pragma unroll
-  for (int v = 0; v < NV; ++v) {
-    Q.u[v] = __ldg(ys + v * vs);
-    Q.adv[v] = 0.0;  // added below, with the dissipation
-  }
+  for (int v = 0; v < NV; ++v) Q.u[v] = __ldg(ys + v * vs);
   auto r = [&](int o) { return __ldg(rec + o * vol); };
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
@@ -66,11 +63,11 @@ __global__ void __launch_bounds__(ALG_THREADS, ALG_MIN_BLOCKS) k_algebra(const _
     Q.da[d] = r(9 * 7 + d);
     Q.dK[d] = r(REC_K + d);
 #pragma unroll
-    for (int s = 0; s < 6; ++s) Q.dg[d][s] = r(9 * (1 + s) + d);
+    for (int s = 0; s < 6; ++s) Q.hg[d][s] = r(9 * (1 + s) + d);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       Q.db[d][c] = r(9 * (8 + c) + d);
-      Q.dGam[d][c] = r(REC_GAM + 3 * c + d);
+      Q.hG[d][c] = r(REC_GAM + 3 * c + d);
     }
   }
 #pragma unroll
@@ -80,12 +77,12 @@ __global__ void __launch_bounds__(ALG_THREADS, ALG_MIN_BLOCKS) k_algebra(const _
 #pragma unroll
     for (int c = 0; c < 3; ++c) Q.ddb[c][s] = r(9 * (8 + c) + 3 + s);
 #pragma unroll
-    for (int c = 0; c < 6; ++c) Q.ddg[c][s] = r(9 * (1 + c) + 3 + s);
+    for (int c = 0; c < 6; ++c) Q.mg[c][s] = r(9 * (1 + c) + 3 + s);
   }
   double rhs[NV];
-  rhs_point<double>(Q, A.S.gz, 1.0 / Q.u[V_W], rhs);
 #pragma unroll
-  for (int v = 0; v < NV; ++v) rhs[v] += r(REC_EXT + v);
+  for (int v = 0; v < NV; ++v) rhs[v] = r(REC_EXT + v);
+  rhs_point64(Q, A.S.gz, rhs);
   if (A.S.mode == 1) {
 #pragma unroll
     for (int v = 0; v < NV; ++v) A.S.rhs[v * vs + p] = rhs[v];
@@ -123,7 +120,7 @@ __global__ void __launch_bounds__(ALG_THREADS, ALG_MIN_BLOCKS) k_algebra(const _
 // The set of the constraints and Weyl scalars at one point.
 template <bool HONLY>
 __device__ __forceinline__ void load_con(const double* __restrict__ rec, int vol, const double* __restrict__ u,
-                                         long long vs, PointIn<double>& Q, double dAt[3][6]) {
+                                         long long vs, Point64& Q, double dAt[3][6]) {
   auto r = [&](int o) { return __ldg(rec + o * vol); };
 #pragma unroll
   for (int v = 0; v < NV; ++v) Q.u[v] = __ldg(u + v * vs);
@@ -133,17 +130,17 @@ __device__ __forceinline__ void load_con(const double* __restrict__ rec, int vol
     Q.dK[d] = HONLY ? 0.0 : r(REC_C_K + d);
 #pragma unroll
     for (int s = 0; s < 6; ++s) {
-      Q.dg[d][s] = r(9 * (1 + s) + d);
+      Q.hg[d][s] = r(9 * (1 + s) + d);
       dAt[d][s] = HONLY ? 0.0 : r(REC_C_AT + 3 * s + d);
     }
 #pragma unroll
-    for (int c = 0; c < 3; ++c) Q.dGam[d][c] = r(REC_C_GAM + 3 * c + d);
+    for (int c = 0; c < 3; ++c) Q.hG[d][c] = r(REC_C_GAM + 3 * c + d);
   }
 #pragma unroll
   for (int s = 0; s < 6; ++s) {
     Q.ddW[s] = r(3 + s);
 #pragma unroll
-    for (int c = 0; c < 6; ++c) Q.ddg[c][s] = r(9 * (1 + c) + 3 + s);
+    for (int c = 0; c < 6; ++c) Q.mg[c][s] = r(9 * (1 + c) + 3 + s);
   }
 }
 
@@ -175,13 +172,10 @@ __global__ void __launch_bounds__(CON_THREADS, 4) k_constraints(const __grid_con
     TilePoint pt;
     if (!tile_point(G, ti, tj, tk, idx, pt)) continue;
     const long long p = pt.p, vs = G.L.vs;
-    PointIn<double> Q;
+    Point64 Q;
     double dAt[3][6], c[7];
     load_con<HONLY>(A.W.rec + (long long)slot * A.W.slot + idx, G.T.vol, G.buf[1] + p, vs, Q, dAt);
-    constraints_point<double>(Q, dAt, 1.0 / Q.u[V_W], c);
-    if (HONLY)
-#pragma unroll
-      for (int q = 1; q < 7; ++q) c[q] = 0.0;
+    constraints64<HONLY>(Q, dAt, c);
     if (A.ham) A.ham[p] = c[0];
     if (A.mom && !HONLY)
 #pragma unroll
@@ -240,7 +234,7 @@ __global__ void __launch_bounds__(CON_THREADS, 4) k_psi4(const __grid_constant__
   TilePoint pt;
   if (!tile_point(G, ti, tj, tk, idx, pt)) return;
   const long long p = pt.p, vs = G.L.vs;
-  PointIn<double> Q;
+  Point64 Q;
   double dAt[3][6];
   load_con<false>(A.W.rec + (long long)slot * A.W.slot + idx, G.T.vol, G.buf[1] + p, vs, Q, dAt);
   const double xyz[3] = {A.o[0] + pt.i * A.h[0], A.o[1] + pt.j * A.h[1], A.o[2] + pt.k * A.h[2]};
