@@ -19,9 +19,10 @@
 //  * mixed derivatives apply the first-derivative weights along y or z to
 //    the exact first-derivative sums along x or y (three limbs, in shared
 //    memory).
-//  * the sum is rounded to the nearest double and scaled by 1/(denominator h).
+//  * the sum is rounded to the nearest double; the algebra (or, where h differs
+//    by axis, this kernel) scales it by 1/(denominator h).
 //
-// No rounding happens before the last two operations, so a constant field has
+// Apart from that of the paired sums (fx_pair) no rounding happens before, so a constant field has
 // exactly zero derivatives and the result does not depend on the order of the
 // terms. A tile whose values are not all finite, or so large or small that
 // the scaling could leave the range of doubles, takes double-precision
@@ -36,15 +37,17 @@
 // quadruple-precision evaluation the right-hand side's error is no larger than
 // before in any variable, and 1e-16 instead of 1e-14 for W, gt_ii and alpha.
 #pragma once
+#include <type_traits>
+
 #include "bssn_bounds.cuh"
 #include "bssn_common.cuh"
 
 namespace bssn {
 
 constexpr int FX_T = 8;          // tile edge
-constexpr int FX_THREADS = 256;  // threads of k_derivs
+constexpr int FX_THREADS = 512;  // threads of k_derivs: one tile point each
 
-// Integer weights: first derivative W1/D1, second derivative W2/D2, paired
+// Integer weights: first derivative W1/D1, second derivative W2/D1^2, paired
 // form of the upwinded first derivative
 //   sum_i UP[i] u(s o_i) = [ sum_a WT[a] (u_sa - u_-sa) + SK Delta ] / DU,
 // Delta = sum_a WK[a] (u_a + u_-a - 2 u_0) the 2r-th difference that is also
@@ -52,16 +55,18 @@ constexpr int FX_THREADS = 256;  // threads of k_derivs
 // vanish on all even powers below 2r, which leaves only this one), s = +-1.
 template <int P> struct FX;
 template <> struct FX<4> {
-  static constexpr int D1 = 12, D2 = 12, DU = 24, SK = 1;
+  static constexpr int D1 = 12, DU = 24, SK = 1;
   static __host__ __device__ constexpr int W1(int a) { return a == 1 ? 8 : -1; }
-  static __host__ __device__ constexpr int W2(int a) { return a == 1 ? 16 : -1; }
+  static __host__ __device__ constexpr int W2(int a) { return a == 1 ? 192 : -12; }
   static __host__ __device__ constexpr int WT(int a) { return a == 1 ? 21 : (a == 2 ? -6 : 1); }
   static __host__ __device__ constexpr int WK(int a) { return a == 1 ? 15 : (a == 2 ? -6 : 1); }
 };
 template <> struct FX<8> {
-  static constexpr int D1 = 840, D2 = 5040, DU = 1680, SK = 3;
+  static constexpr int D1 = 840, DU = 1680, SK = 3;
   static __host__ __device__ constexpr int W1(int a) { return a == 1 ? 672 : (a == 2 ? -168 : (a == 3 ? 32 : -3)); }
-  static __host__ __device__ constexpr int W2(int a) { return a == 1 ? 8064 : (a == 2 ? -1008 : (a == 3 ? 128 : -9)); }
+  static __host__ __device__ constexpr int W2(int a) {
+    return 140 * (a == 1 ? 8064 : (a == 2 ? -1008 : (a == 3 ? 128 : -9)));
+  }
   static __host__ __device__ constexpr int WT(int a) {
     return a == 1 ? 1470 : (a == 2 ? -480 : (a == 3 ? 145 : (a == 4 ? -30 : 3)));
   }
@@ -77,7 +82,7 @@ struct DerivList {
   short d1[NV];   // first of 3 outputs (x, y, z), or -1
   short d2[NV];   // first of 6 outputs (xx, xy, xz, yy, yz, zz), or -1
   short ext[NV];  // advection + dissipation, or -1
-  float f1[NV], f2[NV];  // factors (powers of two) of the first and second derivatives
+  signed char s1[NV], s2[NV];  // binary exponents added to the first and second derivatives
 
   void add(int v, int o1, int o2, int oe) {
     const bool gt = v >= V_GT11 && v <= V_GT33, gam = v >= V_GAM1 && v <= V_GAM3;
@@ -85,8 +90,8 @@ struct DerivList {
     d1[n] = (short)o1;
     d2[n] = (short)o2;
     ext[n] = (short)oe;
-    f1[n] = gt || gam ? 0.5f : 1.0f;  // the algebra takes half of these (Point64)
-    f2[n] = gt ? -0.5f : 1.0f;
+    s1[n] = gt || gam ? -1 : 0;  // the algebra takes half of these (Point64)
+    s2[n] = gt ? -1 : 0;
     ++n;
   }
 };
@@ -123,13 +128,21 @@ inline DerivList rhs_list() {
   return D;
 }
 
-// Scales of one grid's stencils.
+// Scales of one grid's stencils. Where h is the same along all axes (cubic)
+// the record holds the derivatives' integer sums unscaled, 1/c1 times a first
+// and 1/c1^2 times a second derivative (second-derivative weights are brought
+// to the denominator D1^2), and the algebra, homogeneous in them, applies c1
+// and c1^2 once (a and a2); the dissipation of the three axes is one exact
+// sum. Otherwise k_derivs scales every derivative and the algebra's factors
+// are 1.
 struct FxCoef {
   double c1[3];  // 1 / (D1 h_d)
-  double c2[6];  // 1 / (D2 h_d^2), mixed 1 / (D1^2 h h'), packed as sym()
+  double c2[6];  // 1 / (D1^2 h h'), packed as sym()
   double cu[3];  // 1 / (DU h_d)
   double ck[3];  // eps KOSCALE / h_d
-  int cubic;     // h equal along all axes: the dissipation is one exact sum
+  double a, a2;  // what the algebra multiplies first and second derivatives by
+  double ia;     // 1 / a
+  int cubic;
 };
 
 template <int P>
@@ -144,9 +157,12 @@ FxCoef make_fx(const bssn_grid_t& G, double eps) {
   }
   for (int s = 0; s < 6; ++s) {
     const int i = sym_i(s), j = sym_j(s);
-    C.c2[s] = i == j ? 1.0 / (X::D2 * h[i] * h[i]) : 1.0 / ((double)X::D1 * X::D1 * h[i] * h[j]);
+    C.c2[s] = 1.0 / ((double)X::D1 * X::D1 * h[i] * h[j]);
   }
   C.cubic = G.dx == G.dy && G.dy == G.dz;
+  C.a = C.cubic ? C.c1[0] : 1.0;
+  C.a2 = C.cubic ? C.c2[0] : 1.0;
+  C.ia = C.cubic ? X::D1 * h[0] : 1.0;
   return C;
 }
 
@@ -187,9 +203,10 @@ __device__ __forceinline__ int2 fx_from_double(double u, int emax) {
   const int h = __double2hiint(u);
   const unsigned int l = (unsigned int)__double2loint(u);
   const int ex = (h >> 20) & 0x7ff;
-  const unsigned int mh = ex ? ((unsigned int)h & 0xfffffu) | 0x100000u : 0u;
-  const unsigned int ml = ex ? l : 0u;  // subnormals are far below the last place
-  const unsigned long long m = ((unsigned long long)__funnelshift_l(ml, mh, 6) << 32) | (ml << 6);
+  // (the leading one is wrong for subnormals and zero, which end up 0 all the
+  // same: emax is 160 at least)
+  const unsigned int mh = ((unsigned int)h & 0xfffffu) | 0x100000u;
+  const unsigned long long m = ((unsigned long long)__funnelshift_l(l, mh, 6) << 32) | (l << 6);
   const unsigned long long s = (unsigned long long)(long long)(h >> 31);
   const long long n = (long long)((fx_shr(m, emax - ex) ^ s) - s);
   return make_int2((int)((unsigned int)n & FX_MASK), (int)(n >> FX_LIMB));
@@ -213,26 +230,25 @@ __device__ __forceinline__ int2 fx_pair(int2 p, int2 m) {
 
 // (hi 2^30 + lo) 2^(emax - 1081), rounded to nearest (ties away from zero)
 __device__ __forceinline__ double fx_to_double(long long hi, long long lo, int emax) {
-  hi += lo >> FX_LIMB;
-  unsigned int l = (unsigned int)lo & FX_MASK;
-  // magnitude
-  const unsigned int sg = (unsigned int)(hi >> 63);
-  unsigned long long H = (unsigned long long)hi;
-  if (sg) {
-    l = (0u - l) & FX_MASK;
-    H = ~H + (l == 0u ? 1u : 0u);
-  }
-  // 94 bits H:l with the top bit moved to bit 63 of y
-  const bool z = H == 0;
-  const unsigned long long A = z ? (unsigned long long)l << 34 : H;
-  const unsigned int B = z ? 0u : l << 2;
-  const int lz = __clzll((long long)A);
-  const unsigned long long y = fx_shl(A, lz) | fx_shr((unsigned long long)B << 32, 64 - lz);
-  const unsigned long long r = (y >> 11) + ((y >> 10) & 1u);
-  const int e = emax + 34 - lz - (z ? 64 : 0);
-  unsigned long long bits = ((unsigned long long)(unsigned int)e << 52) + r;
-  if (A == 0) bits = 0;
-  return __longlong_as_double((long long)(bits | ((unsigned long long)(sg & 0x80000000u) << 32)));
+  const long long t = hi + (lo >> FX_LIMB);
+  // 96 bits w2:w1:w0, the value times four; magnitude by conditional negation
+  unsigned int w0 = (unsigned int)lo << (32 - FX_LIMB), w1 = (unsigned int)t, w2 = (unsigned int)(t >> 32);
+  const unsigned int x = (unsigned int)((int)w2 >> 31);
+  w0 ^= x;
+  w1 ^= x;
+  w2 ^= x;
+  asm("sub.cc.u32 %0, %0, %3;\n\tsubc.cc.u32 %1, %1, %3;\n\tsubc.u32 %2, %2, %3;"
+      : "+r"(w0), "+r"(w1), "+r"(w2)
+      : "r"(x));
+  // the top 64 bits, leading one at bit 63
+  const bool p2 = w2 != 0u, p1 = w1 != 0u;
+  const unsigned int wa = p2 ? w2 : (p1 ? w1 : w0), wb = p2 ? w1 : (p1 ? w0 : 0u), wc = p2 ? w0 : 0u;
+  const int s = __clz((int)wa);
+  const unsigned int y1 = __funnelshift_l(wb, wa, s), y0 = __funnelshift_l(wc, wb, s);
+  const int e = emax + 34 - s - (p2 ? 0 : (p1 ? 32 : 64));
+  unsigned int ml = __funnelshift_r(y0, y1, 11), mh = (y1 >> 11) + ((unsigned int)e << 20) + (x << 31);
+  asm("add.cc.u32 %0, %0, %2;\n\taddc.u32 %1, %1, 0;" : "+r"(ml), "+r"(mh) : "r"((y0 >> 10) & 1u));
+  return __hiloint2double(y1 ? (int)mh : 0, (int)ml);
 }
 
 // ------------------------------------------------------------------ double-precision stencils
@@ -240,8 +256,8 @@ __device__ __forceinline__ double fx_to_double(long long hi, long long lo, int e
 // the point; writes the same outputs.
 template <int P>
 __device__ __noinline__ void fx_fallback(const double* __restrict__ v, long long p, long long sy, long long sz,
-                                         const FxCoef& C, const double* beta, double wa, bool want1, bool want2,
-                                         bool wante, double* o1, double* o2, double* oe) {
+                                         const FxCoef& C, const double* beta, bool adv, bool want1,
+                                         bool want2, bool wante, double* o1, double* o2, double* oe) {
   using F = FD<P>;
   using X = FX<P>;
   constexpr int H = F::H, R = F::R;
@@ -259,8 +275,8 @@ __device__ __noinline__ void fx_fallback(const double* __restrict__ v, long long
       }
       k += X::WK(a) * s;
     }
-    if (want1) o1[d] = C.c1[d] * r1;
-    if (want2) o2[sym(d, d)] = C.c2[sym(d, d)] * r2;
+    if (want1) o1[d] = C.cubic ? r1 : C.c1[d] * r1;
+    if (want2) o2[sym(d, d)] = C.cubic ? r2 : C.c2[sym(d, d)] * r2;
     if (wante) {
       // the one-sided stencil the sign of beta selects, and no other point
       const long long ss = beta[d] < 0.0 ? -st[d] : st[d];
@@ -274,7 +290,7 @@ __device__ __noinline__ void fx_fallback(const double* __restrict__ v, long long
           w = X::SK * X::WK(abs(o)) + (o > 0 ? X::WT(o) : -X::WT(-o));
         t += w * v[p + o * ss];
       }
-      ext += C.ck[d] * k + C.cu[d] * (wa * fabs(beta[d])) * t;
+      ext += C.ck[d] * k + (adv ? C.cu[d] * fabs(beta[d]) * t : 0.0);
     }
   }
   if (wante) *oe = ext;
@@ -287,7 +303,7 @@ __device__ __noinline__ void fx_fallback(const double* __restrict__ v, long long
           const long long A = a * st[i], B = b * st[j];
           r += (double)(X::W1(a) * X::W1(b)) * ((v[p + A + B] - v[p - A + B]) - (v[p + A - B] - v[p - A - B]));
         }
-      o2[sym(i, j)] = C.c2[sym(i, j)] * r;
+      o2[sym(i, j)] = C.cubic ? r : C.c2[sym(i, j)] * r;
     }
 }
 
@@ -334,9 +350,9 @@ __device__ __forceinline__ double fx_mixed(const int4* __restrict__ g, int st, i
 }
 
 // Stencils along the three axes at one point of the box, and the outputs.
-template <int P, bool D1, bool D2, bool EXT>
+template <int P, bool CUBIC, bool D1, bool D2, bool EXT>
 __device__ __forceinline__ void fx_point(const int2* __restrict__ c, const int4* const g[3], const FxCoef& C,
-                                         const double* beta, double wa, double f1, double f2, int emax,
+                                         const double* beta, bool adv, int emax, int emax1, int emax2,
                                          double* __restrict__ o1, double* __restrict__ o2, double* __restrict__ oe,
                                          int vol) {
   using F = FD<P>;
@@ -345,7 +361,7 @@ __device__ __forceinline__ void fx_point(const int2* __restrict__ c, const int4*
   const int2 u0 = c[0];
   const int m2x = -2 * u0.x, m2y = -2 * u0.y;
   long long kslo = 0, kshi = 0;
-  double ext = 0.0;
+  double ext = 0.0, ko = 0.0;
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     const int st = d == 0 ? 1 : (d == 1 ? BX : BX * BX);
@@ -354,13 +370,13 @@ __device__ __forceinline__ void fx_point(const int2* __restrict__ c, const int4*
     for (int a = 1; a <= (EXT ? F::R : F::H); ++a) {
       const int2 p = c[a * st], m = c[-a * st];
       const int dx = p.x - m.x, dy = p.y - m.y;
-      if (D1 && a <= F::H) {
-        r1l += (long long)X::W1(a) * dx;
-        r1h += (long long)X::W1(a) * dy;
+      if (D1 && !(D2 && d < 2) && a <= F::H) {
+        r1l += (long long)X::W1(a) * (dx);
+        r1h += (long long)X::W1(a) * (dy);
       }
       if (EXT) {
-        tl += (long long)X::WT(a) * dx;
-        th += (long long)X::WT(a) * dy;
+        tl += (long long)X::WT(a) * (dx);
+        th += (long long)X::WT(a) * (dy);
       }
       if (D2 && a <= F::H) {
         const int2 s = fx_pair(p, m);
@@ -372,32 +388,73 @@ __device__ __forceinline__ void fx_point(const int2* __restrict__ c, const int4*
         kh += (long long)X::WK(a) * (p.y + m.y + m2y);
       }
     }
-    if (D1) o1[d * vol] = (f1 * C.c1[d]) * fx_to_double(r1h, r1l, emax);
-    if (D2) o2[sym(d, d) * vol] = (f2 * C.c2[sym(d, d)]) * fx_to_double(r2h, r2l, emax);
+    if (D1) {
+      if (D2 && d < 2) {  // the sums the mixed derivatives are made of
+        const int4 f = *g[1 + d];
+        r1h = ((long long)f.z << FX_LIMB) | (unsigned int)f.y;
+        r1l = f.x;
+      }
+      const double r = fx_to_double(r1h, r1l, emax1);
+      o1[d * vol] = CUBIC ? r : C.c1[d] * r;
+    }
+    if (D2) {
+      const double r = fx_to_double(r2h, r2l, emax2);
+      o2[sym(d, d) * vol] = CUBIC ? r : C.c2[sym(d, d)] * r;
+    }
     if (EXT) {
-      // |b| times the stencil mirrored by the sign of b
-      const double b = wa * beta[d];
-      const long long kkl = X::SK * kl, kkh = X::SK * kh;
-      const bool neg = b < 0.0;
-      ext = fma(C.cu[d] * b, fx_to_double(neg ? th - kkh : th + kkh, neg ? tl - kkl : tl + kkl, emax), ext);
-      if (C.cubic) {
+      if (adv) {
+        // |beta| times the stencil mirrored by the sign of beta
+        const int sk = __double2hiint(beta[d]) < 0 ? -X::SK : X::SK;
+        const double U = fx_to_double(th + sk * kh, tl + sk * kl, emax);
+        ext = fma(CUBIC ? beta[d] : C.cu[d] * beta[d], U, ext);
+      }
+      if (CUBIC) {
         kslo += kl;
         kshi += kh;
       } else {
-        ext = fma(C.ck[d], fx_to_double(kh, kl, emax), ext);
+        ko = fma(C.ck[d], fx_to_double(kh, kl, emax), ko);
       }
     }
   }
-  if (EXT) {
-    if (C.cubic) ext = fma(C.ck[0], fx_to_double(kshi, kslo, emax), ext);
-    *oe = ext;
-  }
+  if (EXT) *oe = CUBIC ? fma(C.cu[0], ext, C.ck[0] * fx_to_double(kshi, kslo, emax)) : ext + ko;
   if (D2) {
-    o2[1 * vol] = (f2 * C.c2[1]) * fx_mixed<P>(g[0], FX_T, emax);
-    o2[2 * vol] = (f2 * C.c2[2]) * fx_mixed<P>(g[1], FX_T * FX_T, emax);
-    o2[4 * vol] = (f2 * C.c2[4]) * fx_mixed<P>(g[2], FX_T * FX_T, emax);
+    const double xy = fx_mixed<P>(g[0], FX_T, emax2), xz = fx_mixed<P>(g[1], FX_T * FX_T, emax2),
+                 yz = fx_mixed<P>(g[2], FX_T * FX_T, emax2);
+    o2[1 * vol] = CUBIC ? xy : C.c2[1] * xy;
+    o2[2 * vol] = CUBIC ? xz : C.c2[2] * xz;
+    o2[4 * vol] = CUBIC ? yz : C.c2[4] * yz;
   }
 }
+
+// The points of a tile's box that its stencils read, in the order they are
+// loaded: first the lines through the tile (R points beyond it along one
+// axis), then what mixed derivatives add (H beyond it along two). An entry is
+// bx | by << 5 | bz << 10 | box index << 16.
+template <int P>
+struct FxBox {
+  static constexpr int H = FD<P>::H, R = FD<P>::R, BX = FX_T + 2 * R;
+  static constexpr int LINES = FX_T * FX_T * FX_T + 3 * 2 * R * FX_T * FX_T;
+  static constexpr int ALL = LINES + 3 * (2 * H) * (2 * H) * FX_T;
+  unsigned int at[ALL];
+  constexpr FxBox() : at() {
+    int nl = 0, nm = LINES;
+    for (int z = 0; z < BX; ++z)
+      for (int y = 0; y < BX; ++y)
+        for (int x = 0; x < BX; ++x) {
+          const int ox = x < R ? R - x : (x >= R + FX_T ? x - (R + FX_T) + 1 : 0);
+          const int oy = y < R ? R - y : (y >= R + FX_T ? y - (R + FX_T) + 1 : 0);
+          const int oz = z < R ? R - z : (z >= R + FX_T ? z - (R + FX_T) + 1 : 0);
+          const int outs = (ox > 0) + (oy > 0) + (oz > 0);
+          const unsigned int e = (unsigned int)(x | y << 5 | z << 10 | ((z * BX + y) * BX + x) << 16);
+          if (outs <= 1)
+            at[nl++] = e;
+          else if (outs == 2 && ox <= H && oy <= H && oz <= H)
+            at[nm++] = e;
+        }
+  }
+};
+template <int P>
+__device__ const FxBox<P> g_fx_box{};
 
 // Point of a thread: x and the eight rows of a plane, arranged so that the
 // half-warps of an 8-byte shared-memory read take rows y and y + 4, whose
@@ -429,39 +486,42 @@ __device__ __forceinline__ void fx_tile(const Layout& L, const FxCoef& C, const 
   const long long org = L.off0 + i0 + j0 * L.sy + k0 * L.sz;
   const double* __restrict__ v = u + var * L.vs;
 
-  // ---- the box in registers: columns of the (x, y) box, cut along z. Only
-  // what the stencils read: the lines through the tile (R beyond it) and, for
-  // mixed derivatives, the planes through it (H beyond it).
-  constexpr int SEG = P == 8 ? 6 : 7, NSEG = BX / SEG, COLS = BX * BX, TASKS = COLS * NSEG;
-  constexpr int PER = (TASKS + FX_THREADS - 1) / FX_THREADS;
-  static_assert(SEG * NSEG == BX, "segments cover the box");
-  double raw[PER][SEG];
+  // ---- the box in registers. A ragged tile drops the points its stencils
+  // cannot reach (they may lie outside the array).
+  constexpr int PER = (FxBox<P>::ALL + FX_THREADS - 1) / FX_THREADS;
+  constexpr int PERL = (FxBox<P>::LINES + FX_THREADS - 1) / FX_THREADS;
+  const int count = mixed ? FxBox<P>::ALL : FxBox<P>::LINES;
+  const double* __restrict__ v0 = v + (org - R * (1 + L.sy + L.sz));
+  const bool full = ex == FX_T && ey == FX_T && ez == FX_T, wide = L.sz >= (1 << 26);
+  const int sy = (int)L.sy, sz = (int)L.sz;
+  double raw[PER];
+  unsigned int at[PER];
   unsigned int mx = 0, any = 0;
 #pragma unroll
   for (int q = 0; q < PER; ++q) {
+    raw[q] = 0.0;
+    at[q] = 0xffffffffu;
+    if (q >= PERL && !mixed) continue;
     const int c = threadIdx.x + q * FX_THREADS;
-    const int seg = c / COLS, col = c - seg * COLS;
-    const int by = col / BX, bx = col - by * BX;
-    const int ox = bx < R ? R - bx : max(0, bx - (R + ex) + 1);
-    const int oy = by < R ? R - by : max(0, by - (R + ey) + 1);
-    int reach;  // how far beyond the tile this column is read along z
-    if (c >= TASKS || ox > R || oy > R) reach = -1;
-    else if (ox == 0 && oy == 0) reach = R;
-    else if (ox == 0 || oy == 0) reach = (mixed && ox <= H && oy <= H) ? H : 0;
-    else reach = (mixed && ox <= H && oy <= H) ? 0 : -1;
-    const long long p0 = org + (bx - R) + (by - R) * L.sy + (seg * SEG - R) * L.sz;
+    if (c < count) at[q] = __ldg(&g_fx_box<P>.at[c]);
+  }
 #pragma unroll
-    for (int s = 0; s < SEG; ++s) {
-      const int bz = seg * SEG + s;
-      const int oz = bz < R ? R - bz : max(0, bz - (R + ez) + 1);
-      const long long p = p0 + s * L.sz;
-      double x = 0.0;
-      if (oz <= reach && in_range(p, p, padded_points(L))) x = __ldg(v + p);
-      raw[q][s] = x;
-      const unsigned int hw = (unsigned int)__double2hiint(x) & 0x7fffffffu;
-      mx = max(mx, hw);
-      any |= hw | (unsigned int)__double2loint(x);
+  for (int q = 0; q < PER; ++q) {
+    if (q >= PERL && !mixed) continue;
+    const int bx = at[q] & 31, by = (at[q] >> 5) & 31, bz = (at[q] >> 10) & 31;
+    // (a box spans less than 2^31 elements of a variable unless a plane of
+    // the array alone has 2^26 points)
+    const long long o = wide ? bx + by * L.sy + bz * L.sz : (long long)(bx + by * sy + bz * sz);
+    if ((full && at[q] != 0xffffffffu) || (bx < ex + 2 * R && by < ey + 2 * R && bz < ez + 2 * R)) {
+      if (in_range(org - R * (1 + L.sy + L.sz) + o, org - R * (1 + L.sy + L.sz) + o, padded_points(L)))
+        raw[q] = __ldg(v0 + o);
     }
+  }
+#pragma unroll
+  for (int q = 0; q < PER; ++q) {
+    const unsigned int hw = (unsigned int)__double2hiint(raw[q]) & 0x7fffffffu;
+    mx = max(mx, hw);
+    any |= hw | (unsigned int)__double2loint(raw[q]);
   }
   mx = __reduce_max_sync(0xffffffffu, mx);
   any = __reduce_or_sync(0xffffffffu, any);
@@ -475,30 +535,23 @@ __device__ __forceinline__ void fx_tile(const Layout& L, const FxCoef& C, const 
     mx = max(mx, red[0][w]);
     any |= red[1][w];
   }
-  const int emax = (int)(mx >> 20);
-  const bool fallback = emax >= 1900 || (emax < 160 && any != 0u);
+  const bool fallback = mx >= (1900u << 20) || (mx < (160u << 20) && any != 0u);
+  const int emax = max((int)(mx >> 20), 160);
 
   const bool d1 = list.d1[e] >= 0, ext = list.ext[e] >= 0;
   const int vol = T.vol;
-  const double f1 = list.f1[e], f2 = list.f2[e];
+  const int emax1 = emax + list.s1[e], emax2 = emax + list.s2[e];
   double* const o1 = rec + (long long)(d1 ? list.d1[e] : 0) * vol;
   double* const o2 = rec + (long long)(mixed ? list.d2[e] : 0) * vol;
   double* const oe = rec + (long long)(ext ? list.ext[e] : 0) * vol;
-  // advection weight of this variable's right-hand side
-  double wa = 1.0;
-  if (var >= V_ALPHA) {
-    const bool frozen = var == V_ALPHA ? lapse_frozen : shift_frozen;
-    wa = advect_gauge && !frozen ? 1.0 : 0.0;
-  }
+  // does this variable's right-hand side have advection?
+  const bool adv = var < V_ALPHA || (advect_gauge && !(var == V_ALPHA ? lapse_frozen : shift_frozen));
 
   if (!fallback) {
 #pragma unroll
     for (int q = 0; q < PER; ++q) {
-      const int c = threadIdx.x + q * FX_THREADS;
-      if (c >= TASKS) break;
-      const int seg = c / COLS, col = c - seg * COLS;
-#pragma unroll
-      for (int s = 0; s < SEG; ++s) box[(seg * SEG + s) * COLS + col] = fx_from_double(raw[q][s], emax);
+      if (q >= PERL && !mixed) continue;
+      if (at[q] != 0xffffffffu) box[at[q] >> 16] = fx_from_double(raw[q], emax);
     }
     __syncthreads();
     if (mixed) {
@@ -522,41 +575,47 @@ __device__ __forceinline__ void fx_tile(const Layout& L, const FxCoef& C, const 
       __syncthreads();
     }
   }
-  for (int t = threadIdx.x; t < FX_T * FX_T * FX_T; t += FX_THREADS) {
-    int x, y, z;
-    fx_lane(t, x, y, z);
-    if (x >= ex || y >= ey || z >= ez) continue;
-    const int idx = (z * T.ty + y) * T.tx + x;
-    const long long p = org + x + y * L.sy + z * L.sz;
-    if (!in_range(p - R * L.sz, p + R * L.sz, padded_points(L))) continue;
-    double beta[3] = {0.0, 0.0, 0.0};
-    if (ext)
+  // ---- one point per thread
+  int x, y, z;
+  fx_lane(threadIdx.x, x, y, z);
+  if (x >= ex || y >= ey || z >= ez) return;
+  const int idx = (z * T.ty + y) * T.tx + x;
+  const long long p = org + x + y * L.sy + z * L.sz;
+  if (!in_range(p - R * L.sz, p + R * L.sz, padded_points(L))) return;
+  double beta[3] = {0.0, 0.0, 0.0};
+  if (ext && adv)
 #pragma unroll
-      for (int d = 0; d < 3; ++d) beta[d] = __ldg(u + (V_BETA1 + d) * L.vs + p);
-    if (fallback) {
-      double r1[3], r2[6], re;
-      fx_fallback<P>(v, p, L.sy, L.sz, C, beta, wa, d1, mixed, ext, r1, r2, &re);
-      if (d1)
-        for (int d = 0; d < 3; ++d) o1[d * vol + idx] = f1 * r1[d];
-      if (mixed)
-        for (int s = 0; s < 6; ++s) o2[s * vol + idx] = f2 * r2[s];
-      if (ext) oe[idx] = re;
-      continue;
-    }
-    const int2* c = box + ((z + R) * BX + (y + R)) * BX + x + R;
-    const int4* const gt[3] = {g + (z * S::EH + (y + H)) * FX_T + x, g + S::GN + ((z + H) * FX_T + y) * FX_T + x,
-                               g + 2 * S::GN + ((z + H) * FX_T + y) * FX_T + x};
-    if (mixed && ext)
-      fx_point<P, true, true, true>(c, gt, C, beta, wa, f1, f2, emax, o1 + idx, o2 + idx, oe + idx, vol);
-    else if (mixed)
-      fx_point<P, true, true, false>(c, gt, C, beta, wa, f1, f2, emax, o1 + idx, o2 + idx, oe + idx, vol);
-    else if (d1 && ext)
-      fx_point<P, true, false, true>(c, gt, C, beta, wa, f1, f2, emax, o1 + idx, o2 + idx, oe + idx, vol);
-    else if (d1)
-      fx_point<P, true, false, false>(c, gt, C, beta, wa, f1, f2, emax, o1 + idx, o2 + idx, oe + idx, vol);
-    else
-      fx_point<P, false, false, true>(c, gt, C, beta, wa, f1, f2, emax, o1 + idx, o2 + idx, oe + idx, vol);
+    for (int d = 0; d < 3; ++d) beta[d] = __ldg(u + (V_BETA1 + d) * L.vs + p);
+  if (fallback) {
+    double r1[3], r2[6], re;
+    fx_fallback<P>(v, p, L.sy, L.sz, C, beta, adv, d1, mixed, ext, r1, r2, &re);
+    if (d1)
+      for (int d = 0; d < 3; ++d) o1[d * vol + idx] = scalbn(r1[d], list.s1[e]);
+    if (mixed)
+      for (int s = 0; s < 6; ++s) o2[s * vol + idx] = scalbn(r2[s], list.s2[e]);
+    if (ext) oe[idx] = re;
+    return;
   }
+  const int2* c = box + ((z + R) * BX + (y + R)) * BX + x + R;
+  const int4* const gt[3] = {g + (z * S::EH + (y + H)) * FX_T + x, g + S::GN + ((z + H) * FX_T + y) * FX_T + x,
+                             g + 2 * S::GN + ((z + H) * FX_T + y) * FX_T + x};
+  auto point = [&](auto cubic) {
+    constexpr bool CB = decltype(cubic)::value;
+    if (mixed && ext)
+      fx_point<P, CB, true, true, true>(c, gt, C, beta, adv, emax, emax1, emax2, o1 + idx, o2 + idx, oe + idx, vol);
+    else if (mixed)
+      fx_point<P, CB, true, true, false>(c, gt, C, beta, adv, emax, emax1, emax2, o1 + idx, o2 + idx, oe + idx, vol);
+    else if (d1 && ext)
+      fx_point<P, CB, true, false, true>(c, gt, C, beta, adv, emax, emax1, emax2, o1 + idx, o2 + idx, oe + idx, vol);
+    else if (d1)
+      fx_point<P, CB, true, false, false>(c, gt, C, beta, adv, emax, emax1, emax2, o1 + idx, o2 + idx, oe + idx, vol);
+    else
+      fx_point<P, CB, false, false, true>(c, gt, C, beta, adv, emax, emax1, emax2, o1 + idx, o2 + idx, oe + idx, vol);
+  };
+  if (C.cubic)
+    point(std::true_type{});
+  else
+    point(std::false_type{});
 }
 
 // One grid as the FP64 kernels see it: its layout, scales, tiles and buffers.

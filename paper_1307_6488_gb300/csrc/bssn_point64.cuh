@@ -23,7 +23,9 @@
 
 namespace bssn {
 
-// One point's derivatives, as the record scales them.
+// One point's derivatives, as the record scales them: first derivatives 1/a
+// times and second derivatives 1/a2 = 1/a^2 times their value, where a and a2
+// are what the functions below take (FxCoef).
 struct Point64 {
   double u[NV];
   double dW[3], dK[3], da[3];
@@ -32,9 +34,10 @@ struct Point64 {
   double db[3][3];    // db[d][i] = d_d beta^i
   double ddW[6], dda[6];
   double ddb[3][6];   // d_s beta^i
-  double mg[6][6];    // mg[s][t] = -1/2 d_t gt_s
+  double hgg[6][6];   // hgg[s][t] = 1/2 d_t gt_s
 };
 
+// Christoffel symbols in the first derivatives' units, Ricci in the second's.
 struct Conformal64 {
   double gu[6], gu2[6];  // gt^ij; with off-diagonal entries doubled
   double GU[3][6];       // Gt^k_ij
@@ -42,7 +45,8 @@ struct Conformal64 {
   double R[6];           // conformal Ricci tensor
 };
 
-__device__ __forceinline__ void conformal64(const Point64& P, Conformal64& C) {
+// ia = 1 / a brings d Gt^k to the second derivatives' units
+__device__ __forceinline__ void conformal64(const Point64& P, double ia, Conformal64& C) {
   const double* g = P.u + V_GT11;
   {
     const double c0 = g[3] * g[5] - g[4] * g[4];
@@ -87,18 +91,18 @@ __device__ __forceinline__ void conformal64(const Point64& P, Conformal64& C) {
 #pragma unroll
   for (int s = 0; s < 6; ++s) {
     const int i = sym_i(s), j = sym_j(s);
-    double r = C.gu2[0] * P.mg[s][0];
+    double r = C.Gd[0] * P.hg[0][s];
 #pragma unroll
-    for (int t = 1; t < 6; ++t) r = fma(C.gu2[t], P.mg[s][t], r);
+    for (int k = 1; k < 3; ++k) r = fma(C.Gd[k], P.hg[k][s], r);
 #pragma unroll
-    for (int k = 0; k < 3; ++k) r = fma(C.Gd[k], P.hg[k][s], r);
+    for (int t = 0; t < 6; ++t) r = fma(-C.gu2[t], P.hgg[s][t], r);
     double l = g[sym(i, 0)] * P.hG[j][0] + g[sym(i, 1)] * P.hG[j][1] + g[sym(i, 2)] * P.hG[j][2];
     if (i == j) {
-      r = fma(2.0, l, r);
+      r = fma(ia + ia, l, r);
     } else {
 #pragma unroll
       for (int k = 0; k < 3; ++k) l = fma(g[sym(j, k)], P.hG[i][k], l);
-      r += l;
+      r = fma(ia, l, r);
     }
     C.R[s] = r;
   }
@@ -137,16 +141,22 @@ __device__ __forceinline__ void conformal64(const Point64& P, Conformal64& C) {
 
 // Right-hand side of the 24 variables added to rhs (which holds advection and
 // dissipation on entry). gz.lapse / gz.shift as in bssn_point.cuh.
-__device__ __forceinline__ void rhs_point64(const Point64& P, const Gauge& gz, double rhs[NV]) {
+__device__ __forceinline__ void rhs_point64(const Point64& P, const Gauge& gz, double a, double a2, double ia,
+                                            double rhs[NV]) {
   Conformal64 C;
-  conformal64(P, C);
+  conformal64(P, ia, C);
   const double* u = P.u;
   const double* g = u + V_GT11;
   const double* A = u + V_AT11;
   const double W = u[V_W], K = u[V_TRK], al = u[V_ALPHA], al2 = al + al;
-  const double iW = 1.0 / W, W2 = W * W;
+  const double iW = 1.0 / W, W2 = a2 * (W * W);  // W2 only ever multiplies second derivatives
   const double third = 1.0 / 3.0, twothirds = 2.0 / 3.0;
-  const double div = P.db[0][0] + P.db[1][1] + P.db[2][2], d23 = twothirds * div;
+  double db[3][3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d)
+#pragma unroll
+    for (int i = 0; i < 3; ++i) db[d][i] = a * P.db[d][i];
+  const double div = db[0][0] + db[1][1] + db[2][2], d23 = twothirds * div;
 
   double dWs[3];  // d_i W / W
 #pragma unroll
@@ -213,16 +223,16 @@ __device__ __forceinline__ void rhs_point64(const Point64& P, const Gauge& gz, d
     double ra = fma(W2, X[s], fma(-cX, g[s], fma(cA, A[s], rhs[V_AT11 + s])));
     const double aa = A[sym(i, 0)] * Am[0][j] + A[sym(i, 1)] * Am[1][j] + A[sym(i, 2)] * Am[2][j];
     ra = fma(-al2, aa, ra);
-    double lg = g[sym(i, 0)] * P.db[j][0] + g[sym(i, 1)] * P.db[j][1] + g[sym(i, 2)] * P.db[j][2];
-    double la = A[sym(i, 0)] * P.db[j][0] + A[sym(i, 1)] * P.db[j][1] + A[sym(i, 2)] * P.db[j][2];
+    double lg = g[sym(i, 0)] * db[j][0] + g[sym(i, 1)] * db[j][1] + g[sym(i, 2)] * db[j][2];
+    double la = A[sym(i, 0)] * db[j][0] + A[sym(i, 1)] * db[j][1] + A[sym(i, 2)] * db[j][2];
     if (i == j) {
       rg = fma(2.0, lg, rg);
       ra = fma(2.0, la, ra);
     } else {
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
-        lg = fma(g[sym(j, k)], P.db[i][k], lg);
-        la = fma(A[sym(j, k)], P.db[i][k], la);
+        lg = fma(g[sym(j, k)], db[i][k], lg);
+        la = fma(A[sym(j, k)], db[i][k], la);
       }
       rg += lg;
       ra += la;
@@ -232,11 +242,11 @@ __device__ __forceinline__ void rhs_point64(const Point64& P, const Gauge& gz, d
   }
 
   double q[3], w[3];  // what At^ij and gt^ij are contracted with
-  const double a6 = -6.0 * al, a43 = (-4.0 / 3.0) * al;
+  const double a6 = -6.0 * al, a43 = (-4.0 / 3.0) * al, a3 = third * a;
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
     q[j] = fma(a6, dWs[j], -2.0 * P.da[j]);
-    w[j] = fma(a43, P.dK[j], third * (P.ddb[0][sym(j, 0)] + P.ddb[1][sym(j, 1)] + P.ddb[2][sym(j, 2)]));
+    w[j] = fma(a43, P.dK[j], a3 * (P.ddb[0][sym(j, 0)] + P.ddb[1][sym(j, 1)] + P.ddb[2][sym(j, 2)]));
   }
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
@@ -247,14 +257,15 @@ __device__ __forceinline__ void rhs_point64(const Point64& P, const Gauge& gz, d
       t6 = fma(Au2[s], C.GU[i][s], t6);
       r = fma(C.gu2[s], P.ddb[i][s], r);
     }
-    r = fma(al2, t6, r);
+    r = fma(a, r, al2 * t6);  // everything in units of one first derivative
     r = fma(d23, C.Gd[i], r);
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
       r = fma(Au[sym(i, j)], q[j], r);
       r = fma(C.gu[sym(i, j)], w[j], r);
-      r = fma(-C.Gd[j], P.db[j][i], r);
+      r = fma(-C.Gd[j], db[j][i], r);
     }
+    r *= a;
     rhs[V_GAM1 + i] += r;
     if (gz.shift == 0) {
       rhs[V_BETA1 + i] = fma(gz.shift_coeff, u[V_B1 + i], rhs[V_BETA1 + i]);
@@ -270,9 +281,10 @@ __device__ __forceinline__ void rhs_point64(const Point64& P, const Gauge& gz, d
 // Hamiltonian (out[0]) and, unless HONLY, momentum (1..3) and Gamma (4..6)
 // constraints at a point; dAt[d][s] = d_d At_s.
 template <bool HONLY>
-__device__ __forceinline__ void constraints64(const Point64& P, const double dAt[3][6], double out[7]) {
+__device__ __forceinline__ void constraints64(const Point64& P, const double dAt[3][6], double a, double a2, double ia,
+                                              double out[7]) {
   Conformal64 C;
-  conformal64(P, C);
+  conformal64(P, ia, C);
   const double* A = P.u + V_AT11;
   const double W = P.u[V_W], K = P.u[V_TRK], iW = 1.0 / W;
   // gt^ij R_ij: the conformal part, and 4 gt^ij DtDt_ij W / W - 6 gt^ij d_i W d_j W / W^2
@@ -298,7 +310,7 @@ __device__ __forceinline__ void constraints64(const Point64& P, const double dAt
 #pragma unroll
     for (int j = 0; j < 3; ++j) AA = fma(Am[i][j], Am[j][i], AA);
   // W^2 R = W^2 tr + 4 W tw - 6 ww
-  out[0] = fma(W, fma(W, tr, 4.0 * tw), fma(-6.0, ww, fma((2.0 / 3.0) * K, K, -AA)));
+  out[0] = fma(a2, fma(W, fma(W, tr, 4.0 * tw), -6.0 * ww), fma((2.0 / 3.0) * K, K, -AA));
 #pragma unroll
   for (int q = 1; q < 7; ++q) out[q] = 0.0;
   if constexpr (!HONLY) {
@@ -319,8 +331,8 @@ __device__ __forceinline__ void constraints64(const Point64& P, const double dAt
 #pragma unroll
         for (int k = 0; k < 3; ++k) m = fma(-C.GU[l][sym(k, i)], Am[k][l], m);
       }
-      out[1 + i] = fma(-2.0 / 3.0, P.dK[i], m);
-      out[4 + i] = P.u[V_GAM1 + i] - C.Gd[i];
+      out[1 + i] = a * fma(-2.0 / 3.0, P.dK[i], m);
+      out[4 + i] = fma(-a, C.Gd[i], P.u[V_GAM1 + i]);
     }
   }
 }

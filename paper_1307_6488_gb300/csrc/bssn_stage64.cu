@@ -77,12 +77,12 @@ __global__ void __launch_bounds__(ALG_THREADS, ALG_MIN_BLOCKS) k_algebra(const _
 #pragma unroll
     for (int c = 0; c < 3; ++c) Q.ddb[c][s] = r(9 * (8 + c) + 3 + s);
 #pragma unroll
-    for (int c = 0; c < 6; ++c) Q.mg[c][s] = r(9 * (1 + c) + 3 + s);
+    for (int c = 0; c < 6; ++c) Q.hgg[c][s] = r(9 * (1 + c) + 3 + s);
   }
   double rhs[NV];
 #pragma unroll
   for (int v = 0; v < NV; ++v) rhs[v] = r(REC_EXT + v);
-  rhs_point64(Q, A.S.gz, rhs);
+  rhs_point64(Q, A.S.gz, G.C.a, G.C.a2, G.C.ia, rhs);
   if (A.S.mode == 1) {
 #pragma unroll
     for (int v = 0; v < NV; ++v) A.S.rhs[v * vs + p] = rhs[v];
@@ -140,7 +140,7 @@ __device__ __forceinline__ void load_con(const double* __restrict__ rec, int vol
   for (int s = 0; s < 6; ++s) {
     Q.ddW[s] = r(3 + s);
 #pragma unroll
-    for (int c = 0; c < 6; ++c) Q.mg[c][s] = r(9 * (1 + c) + 3 + s);
+    for (int c = 0; c < 6; ++c) Q.hgg[c][s] = r(9 * (1 + c) + 3 + s);
   }
 }
 
@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(CON_THREADS, 4) k_constraints(const __grid_con
     Point64 Q;
     double dAt[3][6], c[7];
     load_con<HONLY>(A.W.rec + (long long)slot * A.W.slot + idx, G.T.vol, G.buf[1] + p, vs, Q, dAt);
-    constraints64<HONLY>(Q, dAt, c);
+    constraints64<HONLY>(Q, dAt, G.C.a, G.C.a2, G.C.ia, c);
     if (A.ham) A.ham[p] = c[0];
     if (A.mom && !HONLY)
 #pragma unroll
@@ -237,6 +237,25 @@ __global__ void __launch_bounds__(CON_THREADS, 4) k_psi4(const __grid_constant__
   Point64 Q;
   double dAt[3][6];
   load_con<false>(A.W.rec + (long long)slot * A.W.slot + idx, G.T.vol, G.buf[1] + p, vs, Q, dAt);
+  // Weyl scalars take the derivatives' values
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    Q.dW[d] *= G.C.a;
+    Q.dK[d] *= G.C.a;
+#pragma unroll
+    for (int s = 0; s < 6; ++s) {
+      Q.hg[d][s] *= G.C.a;
+      dAt[d][s] *= G.C.a;
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) Q.hG[d][c] *= G.C.a;
+  }
+#pragma unroll
+  for (int s = 0; s < 6; ++s) {
+    Q.ddW[s] *= G.C.a2;
+#pragma unroll
+    for (int c = 0; c < 6; ++c) Q.hgg[c][s] *= G.C.a2;
+  }
   const double xyz[3] = {A.o[0] + pt.i * A.h[0], A.o[1] + pt.j * A.h[1], A.o[2] + pt.k * A.h[2]};
   WeylOut O;
   weyl_point(Q, dAt, xyz, O);

@@ -32,7 +32,7 @@ __device__ __forceinline__ void weyl_point(const Point64& P, const double dAt[3]
   const double W = P.u[V_W], K = P.u[V_TRK];
   const double iW = 1.0 / W, iW2 = iW * iW;
   Conformal64 G;
-  conformal64(P, G);
+  conformal64(P, 1.0, G);
   const double* gt = P.u + V_GT11;
   // R_ij = Rt_ij + (DtDt_ij W + gt_ij gt^kl DtDt_kl W) / W - 2 gt_ij gt^kl d_k W d_l W / W^2
   double dWu[3], DDW[6], tr = 0.0, dWdW = 0.0;
