@@ -465,19 +465,20 @@ __device__ __forceinline__ void fx_lane(int t, int& x, int& y, int& z) {
   z = t >> 6;
 }
 
+// Barrier of the threads that work on a tile, the first FX_THREADS of a block.
+__device__ __forceinline__ void fx_sync() { asm volatile("bar.sync 1, %0;" ::"n"(FX_THREADS) : "memory"); }
+
 // All outputs of list entry e on the tile (ti, tj, tk) of the grid L, written
-// to the record slot `rec` (nout x vol doubles).
+// to the record slot `rec` (nout x vol doubles), by the
+// first FX_THREADS threads of the block. box and g: shared memory for the tile
+// and its first-derivative tables.
 template <int P>
 __device__ __forceinline__ void fx_tile(const Layout& L, const FxCoef& C, const FxTiles& T, const DerivList& list,
                                         int e, bool advect_gauge, bool lapse_frozen, bool shift_frozen,
-                                        const double* __restrict__ u, int ti, int tj, int tk,
-                                        double* __restrict__ rec) {
+                                        const double* __restrict__ u, int ti, int tj, int tk, int2* box, int4* g,
+                                        unsigned int (*red)[FX_THREADS / 32], double* __restrict__ rec) {
   using S = FxSmem<P>;
   constexpr int H = S::H, R = S::R, BX = S::BX;
-  extern __shared__ __align__(16) unsigned char fx_smem[];
-  int4* g = (int4*)fx_smem;
-  int2* box = (int2*)(g + 3 * S::GN);
-  __shared__ unsigned int red[2][FX_THREADS / 32];
 
   const int var = list.var[e];
   const bool mixed = list.d2[e] >= 0;
@@ -529,7 +530,7 @@ __device__ __forceinline__ void fx_tile(const Layout& L, const FxCoef& C, const 
     red[0][threadIdx.x >> 5] = mx;
     red[1][threadIdx.x >> 5] = any;
   }
-  __syncthreads();
+  fx_sync();
 #pragma unroll
   for (int w = 0; w < FX_THREADS / 32; ++w) {
     mx = max(mx, red[0][w]);
@@ -553,7 +554,7 @@ __device__ __forceinline__ void fx_tile(const Layout& L, const FxCoef& C, const 
       if (q >= PERL && !mixed) continue;
       if (at[q] != 0xffffffffu) box[at[q] >> 16] = fx_from_double(raw[q], emax);
     }
-    __syncthreads();
+    fx_sync();
     if (mixed) {
       // D_x sums on rows y beyond the tile (for xy) and planes z beyond it
       // (for xz), D_y sums on planes beyond it (for yz); the in-tile D_x
@@ -572,7 +573,7 @@ __device__ __forceinline__ void fx_tile(const Layout& L, const FxCoef& C, const 
         if (z >= H && z < H + FX_T) g[((z - H) * S::EH + (y + H)) * FX_T + x] = fx;
         g[2 * S::GN + (z * FX_T + y) * FX_T + x] = fx_first<P>(b, BX);
       }
-      __syncthreads();
+      fx_sync();
     }
   }
   // ---- one point per thread
@@ -684,10 +685,16 @@ struct AlgebraArgs {
 // One block per slot (blockIdx.x) and list entry (blockIdx.y).
 template <int P>
 __global__ void __launch_bounds__(FX_THREADS, 2) k_derivs(const __grid_constant__ DerivArgs A) {
+  extern __shared__ __align__(16) unsigned char fx_smem[];
+  int4* g = (int4*)fx_smem;
   int ti, tj, tk;
+  const int e = blockIdx.y;
   const FxGrid& G = fx_locate(A.W, A.W.tile0 + blockIdx.x, ti, tj, tk);
-  fx_tile<P>(G.L, G.C, G.T, A.list, blockIdx.y, A.advect_gauge, A.lapse_frozen, A.shift_frozen, G.buf[A.in], ti, tj,
-             tk, A.W.rec + (long long)blockIdx.x * A.W.slot);
+  const double* u = G.buf[A.in];
+  __shared__ unsigned int red[2][FX_THREADS / 32];
+  fx_tile<P>(G.L, G.C, G.T, A.list, e, A.advect_gauge, A.lapse_frozen, A.shift_frozen, u, ti,
+             tj, tk, (int2*)(g + 3 * FxSmem<P>::GN), g, red,
+             A.W.rec + (long long)blockIdx.x * A.W.slot);
 }
 
 }  // namespace bssn

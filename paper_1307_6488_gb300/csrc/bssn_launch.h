@@ -14,6 +14,11 @@ template <int P>
 cudaError_t derivs_init();  // raises the kernel's shared-memory limit (not during a capture)
 template <int P>
 cudaError_t launch_derivs(const DerivArgs& A, long long nslots, cudaStream_t s);
+// Derivatives of one chunk beside the algebra of another (bssn_stage64.cuh),
+// one block on each of `sms` SMs.
+struct OverlapArgs;
+template <int P>
+cudaError_t launch_overlap(const OverlapArgs& A, int sms, cudaStream_t s);
 // The FP64 stage (or right-hand side) of `ntiles` tiles from work.tile0 on,
 // through a record of `slots` slots (bssn_stage64.cu); vol: the largest tile
 // volume among the grids.

@@ -2,6 +2,7 @@
 // selected at compile time with -DBSSN_ORDER=4 or -DBSSN_ORDER=8.
 #include "bssn_fixed.cuh"
 #include "bssn_ko.cuh"
+#include "bssn_stage64.cuh"
 #include "bssn_launch.h"
 #include "bssn_bounds.cuh"
 
@@ -13,11 +14,20 @@ namespace bssn {
 
 static inline unsigned int blocks_for(long long n, int threads) { return (unsigned int)((n + threads - 1) / threads); }
 
-static std::atomic<unsigned long long> g_derivs_smem{0};  // devices whose limit is raised
+static std::atomic<unsigned long long> g_derivs_smem{0}, g_overlap_smem{0};  // devices whose limit is raised
 
 template <>
 cudaError_t derivs_init<BSSN_ORDER>() {
-  return allow_smem(k_derivs<BSSN_ORDER>, FxSmem<BSSN_ORDER>::bytes, g_derivs_smem);
+  const cudaError_t e = allow_smem(k_derivs<BSSN_ORDER>, FxSmem<BSSN_ORDER>::bytes, g_derivs_smem);
+  return e == cudaSuccess ? allow_smem(k_overlap<BSSN_ORDER>, FxSmem<BSSN_ORDER>::bytes, g_overlap_smem) : e;
+}
+
+template <>
+cudaError_t launch_overlap<BSSN_ORDER>(const OverlapArgs& A, int sms, cudaStream_t s) {
+  const cudaError_t e = derivs_init<BSSN_ORDER>();
+  if (e != cudaSuccess) return e;
+  k_overlap<BSSN_ORDER><<<sms, OVERLAP_THREADS<BSSN_ORDER>, FxSmem<BSSN_ORDER>::bytes, s>>>(A);
+  return cudaGetLastError();
 }
 
 template <>

@@ -7,26 +7,10 @@
 #include "bssn_bounds.cuh"
 #include "bssn_fixed.cuh"
 #include "bssn_launch.h"
-#include "bssn_point64.cuh"
+#include "bssn_stage64.cuh"
 #include "bssn_weyl.cuh"
 
 namespace bssn {
-
-// Point idx of a tile; false outside the grid.
-struct TilePoint {
-  int i, j, k;
-  long long p;
-};
-__device__ __forceinline__ bool tile_point(const FxGrid& G, int ti, int tj, int tk, int idx, TilePoint& q) {
-  if (idx >= G.T.vol) return false;
-  const int yz = idx / G.T.tx;
-  q.i = ti * FX_T + idx - yz * G.T.tx;
-  q.j = tj * FX_T + yz % G.T.ty;
-  q.k = tk * FX_T + yz / G.T.ty;
-  if (q.i >= G.L.nx || q.j >= G.L.ny || q.k >= G.L.nz) return false;
-  q.p = G.L.off0 + q.i + q.j * G.L.sy + q.k * G.L.sz;
-  return in_range(q.p, q.p, padded_points(G.L));
-}
 
 // Threads of a block and resident blocks per SM. The kernel is bound by the
 // FP64 pipe (~800 instructions per point at 1.68 per clock and SM), which a
@@ -38,83 +22,10 @@ __device__ __forceinline__ bool tile_point(const FxGrid& G, int ti, int tj, int 
 #define ALG_MIN_BLOCKS 4
 #endif
 
-// One thread per point of a slot: the pointwise right-hand side from the
-// record of k_derivs (with its advection + dissipation sums) and the stage
-// update.
 __global__ void __launch_bounds__(ALG_THREADS, ALG_MIN_BLOCKS) k_algebra(const __grid_constant__ AlgebraArgs A,
                                                                        int blocks_per_slot) {
   const unsigned int slot = blockIdx.x / (unsigned int)blocks_per_slot;
-  const int idx = (int)(blockIdx.x - slot * blocks_per_slot) * ALG_THREADS + threadIdx.x;
-  int ti, tj, tk;
-  const FxGrid& G = fx_locate(A.W, A.W.tile0 + slot, ti, tj, tk);
-  TilePoint pt;
-  if (!tile_point(G, ti, tj, tk, idx, pt)) return;
-  const long long p = pt.p, vs = G.L.vs;
-  const int vol = G.T.vol;
-  const double* __restrict__ rec = A.W.rec + (long long)slot * A.W.slot + idx;
-  const double* __restrict__ ys = G.buf[A.S.in] + p;
-  Point64 Q;
-#pragma unroll
-  for (int v = 0; v < NV; ++v) Q.u[v] = __ldg(ys + v * vs);
-  auto r = [&](int o) { return __ldg(rec + o * vol); };
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    Q.dW[d] = r(d);
-    Q.da[d] = r(9 * 7 + d);
-    Q.dK[d] = r(REC_K + d);
-#pragma unroll
-    for (int s = 0; s < 6; ++s) Q.hg[d][s] = r(9 * (1 + s) + d);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      Q.db[d][c] = r(9 * (8 + c) + d);
-      Q.hG[d][c] = r(REC_GAM + 3 * c + d);
-    }
-  }
-#pragma unroll
-  for (int s = 0; s < 6; ++s) {
-    Q.ddW[s] = r(3 + s);
-    Q.dda[s] = r(9 * 7 + 3 + s);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) Q.ddb[c][s] = r(9 * (8 + c) + 3 + s);
-#pragma unroll
-    for (int c = 0; c < 6; ++c) Q.hgg[c][s] = r(9 * (1 + c) + 3 + s);
-  }
-  double rhs[NV];
-#pragma unroll
-  for (int v = 0; v < NV; ++v) rhs[v] = r(REC_EXT + v);
-  rhs_point64(Q, A.S.gz, G.C.a, G.C.a2, G.C.ia, rhs);
-  if (A.S.mode == 1) {
-#pragma unroll
-    for (int v = 0; v < NV; ++v) A.S.rhs[v * vs + p] = rhs[v];
-    return;
-  }
-  const RK& rk = A.S.rk;
-  const double* y0 = G.buf[0] + p;  // may be the output: read before it is written
-  double* acc = G.buf[3] + p;
-  double* out = G.buf[A.S.out] + p;
-  if (rk.method == 3) {
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      const long long o = v * vs;
-      out[o] = fma(rk.cdt, rhs[v], fma(rk.a1, Q.u[v], rk.a0 * y0[o]));
-    }
-    return;
-  }
-#pragma unroll
-  for (int v = 0; v < NV; ++v) {
-    const long long o = v * vs;
-    double yn;
-    if (rk.stage == 0) {
-      acc[o] = rk.bdt * rhs[v];
-      yn = fma(rk.cdt, rhs[v], y0[o]);
-    } else if (rk.stage < 3) {
-      acc[o] = fma(rk.bdt, rhs[v], acc[o]);
-      yn = fma(rk.cdt, rhs[v], y0[o]);
-    } else {
-      yn = y0[o] + fma(rk.bdt, rhs[v], acc[o]);
-    }
-    out[o] = yn;
-  }
+  algebra_point(A.W, A.S, slot, (int)(blockIdx.x - slot * blocks_per_slot) * ALG_THREADS + threadIdx.x);
 }
 
 // The set of the constraints and Weyl scalars at one point.
@@ -326,23 +237,64 @@ cudaError_t launch_psi4(int order, FxWork work, size_t rec_doubles, const double
   });
 }
 
+// Chunks of an overlapped stage, about; and the fewest tiles worth it.
+constexpr int OVERLAP_CHUNKS = 8;
+constexpr long long OVERLAP_MIN_TILES = 608;
+
 cudaError_t launch_stage64(int order, const FxWork& work, int vol, long long ntiles, long long slots,
                            const Gauge& gz, const StageOut& out, cudaStream_t s) {
   if (slots < 1) return cudaErrorInvalidValue;
-  const long long chunks = (ntiles + slots - 1) / slots, per = (ntiles + chunks - 1) / chunks;
   DerivArgs D{work, rhs_list(), out.in, gz.advect_gauge != 0, gz.lapse == 2, gz.shift == 1};
   AlgebraArgs A{work, out};
   const int bps = (vol + ALG_THREADS - 1) / ALG_THREADS;
-  for (long long t = 0; t < ntiles; t += per) {
-    const long long n = std::min(per, ntiles - t);
-    D.W.tile0 = A.W.tile0 = work.tile0 + t;
-    const cudaError_t e = order == 4 ? launch_derivs<4>(D, n, s) : launch_derivs<8>(D, n, s);
-    if (e != cudaSuccess) return e;
-    k_algebra<<<(unsigned int)(n * bps), ALG_THREADS, 0, s>>>(A, bps);
-    const cudaError_t e2 = cudaGetLastError();
-    if (e2 != cudaSuccess) return e2;
+  cudaError_t e = cudaSuccess;
+  if (ntiles < OVERLAP_MIN_TILES || slots < 2 * 76) {
+    const long long chunks = (ntiles + slots - 1) / slots, per = (ntiles + chunks - 1) / chunks;
+    for (long long t = 0; t < ntiles && e == cudaSuccess; t += per) {
+      const long long n = std::min(per, ntiles - t);
+      D.W.tile0 = A.W.tile0 = work.tile0 + t;
+      e = order == 4 ? launch_derivs<4>(D, n, s) : launch_derivs<8>(D, n, s);
+      if (e != cudaSuccess) break;
+      k_algebra<<<(unsigned int)(n * bps), ALG_THREADS, 0, s>>>(A, bps);
+      e = cudaGetLastError();
+    }
+    return e;
   }
-  return cudaSuccess;
+  // the record as two halves: the derivatives of one chunk go into one while
+  // the algebra reads the chunk before from the other. Chunks are multiples
+  // of 76 tiles, so that the algebra warps of 152 SMs take equally many
+  // 32-point groups each.
+  int dev = 0, sms = 0;
+  e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  const long long half = slots / 2;
+  long long per = std::min((ntiles + OVERLAP_CHUNKS - 1) / OVERLAP_CHUNKS + 75, half) / 76 * 76;
+  OverlapArgs O;
+  O.groups = (vol + 31) / 32;
+  double* const recs[2] = {work.rec, work.rec + half * work.slot};
+  long long prev = 0;
+  int side = 0;
+  for (long long t = 0; t < ntiles && e == cudaSuccess; t += per, side ^= 1) {
+    const long long n = std::min(per, ntiles - t);
+    D.W.tile0 = work.tile0 + t;
+    D.W.rec = recs[side];
+    if (t == 0) {
+      e = order == 4 ? launch_derivs<4>(D, n, s) : launch_derivs<8>(D, n, s);
+    } else {
+      O.D = D;
+      O.A = A;
+      O.nd = (unsigned int)n;
+      O.na = (unsigned int)prev;
+      e = order == 4 ? launch_overlap<4>(O, sms, s) : launch_overlap<8>(O, sms, s);
+    }
+    A.W.tile0 = D.W.tile0;
+    A.W.rec = D.W.rec;
+    prev = n;
+  }
+  if (e != cudaSuccess) return e;
+  k_algebra<<<(unsigned int)(prev * bps), ALG_THREADS, 0, s>>>(A, bps);
+  return cudaGetLastError();
 }
 
 cudaError_t bounds_take_stage64(unsigned long long* out) { return bounds_take_local(out); }

@@ -49,6 +49,18 @@ def test_tile_edges(order, n, cubic):
     assert np.max(err) < RHS_TOL, dict(zip(inputs.VARS, err))
 
 
+# enough tiles that derivatives and algebra of different chunks run side by
+# side, with a last chunk that is smaller than the others
+@pytest.mark.parametrize("order,h", [(4, 0.1), (8, H)])
+def test_overlapped_chunks(order, h):
+    g = order // 2 + 1
+    u = perturbed_bl(70, 66, 72, g, 0.1, seed=order)
+    p = B.make_params(fd_order=order)
+    want = oracle.rhs(u, g, h, oracle_params(p), ko=True)
+    err = rel_err(gpu_stage(u, g, h, p), want, g)
+    assert np.max(err) < RHS_TOL, dict(zip(inputs.VARS, err))
+
+
 @pytest.mark.parametrize("order", [4, 8])
 @pytest.mark.parametrize("value", [np.nan, np.inf, 1e290, 1e-300])
 def test_values_outside_the_fixed_point_range(order, value):
