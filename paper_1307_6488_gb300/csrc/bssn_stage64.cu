@@ -25,7 +25,33 @@ namespace bssn {
 __global__ void __launch_bounds__(ALG_THREADS, ALG_MIN_BLOCKS) k_algebra(const __grid_constant__ AlgebraArgs A,
                                                                        int blocks_per_slot) {
   const unsigned int slot = blockIdx.x / (unsigned int)blocks_per_slot;
-  algebra_point(A.W, A.S, slot, (int)(blockIdx.x - slot * blocks_per_slot) * ALG_THREADS + threadIdx.x);
+  algebra_point<PART_ALL>(A.W, A.S, slot, (int)(blockIdx.x - slot * blocks_per_slot) * ALG_THREADS + threadIdx.x);
+}
+
+// The same for few points: At_ij and the other variables by different warps.
+// A warp's FP64 instruction holds its scheduler's FP64 unit for 64 clocks
+// whatever the other schedulers do, so where not every scheduler has a warp
+// the time is that of one warp's instructions, and two halves (with their
+// shared part done twice) take about half of it.
+__global__ void __launch_bounds__(32) k_algebra_split(const __grid_constant__ AlgebraArgs A, int groups) {
+  const unsigned int q = blockIdx.x >> 1, slot = q / (unsigned int)groups;
+  const int idx = (int)(q - slot * groups) * 32 + threadIdx.x;
+  if (blockIdx.x & 1)
+    algebra_point<PART_REST>(A.W, A.S, slot, idx);
+  else
+    algebra_point<PART_AT>(A.W, A.S, slot, idx);
+}
+
+// Algebra of n slots; few enough of them take two warps per 32 points.
+static cudaError_t launch_algebra(const AlgebraArgs& A, long long n, int vol, int schedulers, cudaStream_t s) {
+  const int groups = (vol + 31) / 32;
+  if (2 * n * groups <= schedulers) {
+    k_algebra_split<<<(unsigned int)(2 * n * groups), 32, 0, s>>>(A, groups);
+  } else {
+    const int bps = (vol + ALG_THREADS - 1) / ALG_THREADS;
+    k_algebra<<<(unsigned int)(n * bps), ALG_THREADS, 0, s>>>(A, bps);
+  }
+  return cudaGetLastError();
 }
 
 // The set of the constraints and Weyl scalars at one point.
@@ -246,8 +272,10 @@ cudaError_t launch_stage64(int order, const FxWork& work, int vol, long long nti
   if (slots < 1) return cudaErrorInvalidValue;
   DerivArgs D{work, rhs_list(), out.in, gz.advect_gauge != 0, gz.lapse == 2, gz.shift == 1};
   AlgebraArgs A{work, out};
-  const int bps = (vol + ALG_THREADS - 1) / ALG_THREADS;
-  cudaError_t e = cudaSuccess;
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
   if (ntiles < OVERLAP_MIN_TILES || slots < 2 * 76) {
     const long long chunks = (ntiles + slots - 1) / slots, per = (ntiles + chunks - 1) / chunks;
     for (long long t = 0; t < ntiles && e == cudaSuccess; t += per) {
@@ -255,8 +283,7 @@ cudaError_t launch_stage64(int order, const FxWork& work, int vol, long long nti
       D.W.tile0 = A.W.tile0 = work.tile0 + t;
       e = order == 4 ? launch_derivs<4>(D, n, s) : launch_derivs<8>(D, n, s);
       if (e != cudaSuccess) break;
-      k_algebra<<<(unsigned int)(n * bps), ALG_THREADS, 0, s>>>(A, bps);
-      e = cudaGetLastError();
+      e = launch_algebra(A, n, vol, 4 * sms, s);
     }
     return e;
   }
@@ -264,10 +291,6 @@ cudaError_t launch_stage64(int order, const FxWork& work, int vol, long long nti
   // the algebra reads the chunk before from the other. Chunks are multiples
   // of 76 tiles, so that the algebra warps of 152 SMs take equally many
   // 32-point groups each.
-  int dev = 0, sms = 0;
-  e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e != cudaSuccess) return e;
   const long long half = slots / 2;
   long long per = std::min((ntiles + OVERLAP_CHUNKS - 1) / OVERLAP_CHUNKS + 75, half) / 76 * 76;
   OverlapArgs O;
@@ -293,8 +316,7 @@ cudaError_t launch_stage64(int order, const FxWork& work, int vol, long long nti
     prev = n;
   }
   if (e != cudaSuccess) return e;
-  k_algebra<<<(unsigned int)(prev * bps), ALG_THREADS, 0, s>>>(A, bps);
-  return cudaGetLastError();
+  return launch_algebra(A, prev, vol, 4 * sms, s);
 }
 
 cudaError_t bounds_take_stage64(unsigned long long* out) { return bounds_take_local(out); }

@@ -23,8 +23,18 @@ __device__ __forceinline__ bool tile_point(const FxGrid& G, int ti, int tj, int 
   return in_range(q.p, q.p, padded_points(G.L));
 }
 
+// Which variables a call of algebra_point is for: all of them, At_ij, or the
+// others (the compiler drops the arithmetic that no stored value needs; At_ij
+// takes the Ricci tensor and about half of the instructions).
+enum AlgebraPart { PART_ALL = 0, PART_AT = 1, PART_REST = 2 };
+template <int PART>
+__host__ __device__ constexpr bool in_part(int v) {
+  return PART == PART_ALL || (v >= V_AT11 && v <= V_AT33) == (PART == PART_AT);
+}
+
 // Point idx of a slot: the pointwise right-hand side from the record of
 // k_derivs (with its advection + dissipation sums) and the stage update.
+template <int PART>
 __device__ __forceinline__ void algebra_point(const FxWork& Wk, const StageOut& S, unsigned int slot, int idx) {
   int ti, tj, tk;
   const FxGrid& G = fx_locate(Wk, Wk.tile0 + slot, ti, tj, tk);
@@ -66,7 +76,8 @@ __device__ __forceinline__ void algebra_point(const FxWork& Wk, const StageOut& 
   rhs_point64(Q, S.gz, G.C.a, G.C.a2, G.C.ia, rhs);
   if (S.mode == 1) {
 #pragma unroll
-    for (int v = 0; v < NV; ++v) S.rhs[v * vs + p] = rhs[v];
+    for (int v = 0; v < NV; ++v)
+      if (in_part<PART>(v)) S.rhs[v * vs + p] = rhs[v];
     return;
   }
   const RK& rk = S.rk;
@@ -76,6 +87,7 @@ __device__ __forceinline__ void algebra_point(const FxWork& Wk, const StageOut& 
   if (rk.method == 3) {
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
+      if (!in_part<PART>(v)) continue;
       const long long o = v * vs;
       out[o] = fma(rk.cdt, rhs[v], fma(rk.a1, Q.u[v], rk.a0 * y0[o]));
     }
@@ -83,6 +95,7 @@ __device__ __forceinline__ void algebra_point(const FxWork& Wk, const StageOut& 
   }
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
+    if (!in_part<PART>(v)) continue;
     const long long o = v * vs;
     double yn;
     if (rk.stage == 0) {
@@ -140,7 +153,7 @@ __global__ void __launch_bounds__(OVERLAP_THREADS<P>, 1) k_overlap(const __grid_
     const unsigned int warp = (threadIdx.x - FX_THREADS) >> 5, n = A.na * (unsigned int)A.groups;
     for (unsigned int q = blockIdx.x * WARPS + warp; q < n; q += gridDim.x * WARPS) {
       const unsigned int slot = q / (unsigned int)A.groups;
-      algebra_point(A.A.W, A.A.S, slot, (int)(q - slot * A.groups) * 32 + (int)(threadIdx.x & 31));
+      algebra_point<PART_ALL>(A.A.W, A.A.S, slot, (int)(q - slot * A.groups) * 32 + (int)(threadIdx.x & 31));
     }
   }
 }
