@@ -35,8 +35,8 @@ struct bssn_plan {
   Gauge gz{};
   std::vector<PatchDev> host;
   PatchDev* dev = nullptr;
-  long long* d_pad0 = nullptr;
-  long long ntiles = 0, npad = 0, points = 0;
+  long long* d_gh0 = nullptr;
+  long long ntiles = 0, nghost = 0, points = 0;
   std::vector<void*> allocations;
   int shape = 0;  // tile shape index bssn_plan_info reports
   int grid_other = 0;
@@ -82,7 +82,7 @@ void plan_free(bssn_plan* pl) {
 
 // Static ghosts of buffer `which` of every patch.
 cudaError_t fill_all(bssn_plan* pl, int which, cudaStream_t s) {
-  kb_fill<<<(unsigned int)pl->grid_other, 256, 0, s>>>(pl->dev, pl->d_pad0, pl->np, pl->npad, which);
+  kb_fill<<<dim3((unsigned int)pl->grid_other, NV / 4), 256, 0, s>>>(pl->dev, pl->d_gh0, pl->np, pl->nghost, which);
   return cudaGetLastError();
 }
 
@@ -152,7 +152,7 @@ bssn_status_t bssn_plan_create(bssn_plan_t** out, const bssn_block_t* blocks, in
   pl->host.resize(nblocks);
   cudaError_t e = cudaSuccess;
   const int H = pl->order / 2;
-  std::vector<long long> pad0(nblocks);
+  std::vector<long long> gh0(nblocks);
   for (int b = 0; b < nblocks && e == cudaSuccess; ++b) {
     const bssn_block_t& B = blocks[b];
     PatchDev& D = pl->host[b];
@@ -172,8 +172,8 @@ bssn_status_t bssn_plan_create(bssn_plan_t** out, const bssn_block_t* blocks, in
     if (e == cudaSuccess) e = cudaMemcpy(D.buf[2], B.state, n * sizeof(double), cudaMemcpyDeviceToDevice);
     if (e == cudaSuccess) e = cudaMemset(D.buf[3], 0, n * sizeof(double));
     if (e != cudaSuccess) break;
-    D.pad0 = pad0[b] = pl->npad;
-    pl->npad += (D.L.nx + 2LL * D.L.g) * (D.L.ny + 2LL * D.L.g) * (D.L.nz + 2LL * D.L.g);
+    D.gh0 = gh0[b] = pl->nghost;
+    pl->nghost += ghost_points(D.L);
     pl->points += D.L.npts;
   }
   void* p = nullptr;
@@ -253,8 +253,8 @@ bssn_status_t bssn_plan_create(bssn_plan_t** out, const bssn_block_t* blocks, in
   }
   if (e == cudaSuccess) e = plan_alloc(pl, sizeof(long long) * nblocks, &p);
   if (e == cudaSuccess) {
-    pl->d_pad0 = (long long*)p;
-    e = cudaMemcpy(pl->d_pad0, pad0.data(), sizeof(long long) * nblocks, cudaMemcpyHostToDevice);
+    pl->d_gh0 = (long long*)p;
+    e = cudaMemcpy(pl->d_gh0, gh0.data(), sizeof(long long) * nblocks, cudaMemcpyHostToDevice);
   }
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&pl->cap, cudaStreamNonBlocking);
   int dev = 0, sms = 0;

@@ -81,6 +81,44 @@ inline Layout32 make_layout32(const bssn_grid_t& G) {
   return L;
 }
 
+// Ghost points of a grid, numbered: the planes below and above the interior,
+// then the rows before and behind it, then the ends of its rows.
+inline long long ghost_points(const Layout& L) {
+  return (L.nx + 2LL * L.g) * (L.ny + 2LL * L.g) * (L.nz + 2LL * L.g) - L.npts;
+}
+__device__ __forceinline__ void ghost_point(const Layout& L, long long lin, int& i, int& j, int& k) {
+  const int g2 = 2 * L.g;
+  const long long ex = L.nx + g2, planes = ex * (L.ny + g2) * g2, rows = ex * g2 * L.nz;
+  // (a count of 2^31 would be 17 GB a variable of ghosts alone; 64-bit there)
+  auto divmod = [](long long a, int b, int& r) {
+    if (a < (1LL << 31)) {
+      const unsigned int q = (unsigned int)a / (unsigned int)b;
+      r = (int)((unsigned int)a - q * b);
+      return (long long)q;
+    }
+    r = (int)(a % b);
+    return a / b;
+  };
+  auto outside = [](int r, int g, int n) { return r < g ? r - g : n + r - g; };  // 0 .. 2g-1 -> ghost index
+  int r;
+  if (lin < planes) {
+    lin = divmod(lin, (int)ex, r);
+    i = r - L.g;
+    k = outside((int)divmod(lin, L.ny + g2, r), L.g, L.nz);
+    j = r - L.g;
+  } else if (lin < planes + rows) {
+    lin = divmod(lin - planes, (int)ex, r);
+    i = r - L.g;
+    k = (int)divmod(lin, g2, r);
+    j = outside(r, L.g, L.ny);
+  } else {
+    lin = divmod(lin - planes - rows, g2, r);
+    i = outside(r, L.g, L.nx);
+    k = (int)divmod(lin, L.ny, r);
+    j = r;
+  }
+}
+
 // padded points of one variable (the extent every index into it must respect)
 __host__ __device__ __forceinline__ long long padded_points(const Layout& L) {
   return (L.nx + 2LL * L.g) * (L.ny + 2LL * L.g) * (L.nz + 2LL * L.g);

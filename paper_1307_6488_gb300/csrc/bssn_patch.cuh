@@ -19,7 +19,7 @@ using namespace bssn;
 // Device description of one patch.
 struct PatchDev {
   Layout L;
-  long long pad0;           // first point of this patch in the flat padded-point list
+  long long gh0;            // first point of this patch in the flat ghost-point list
   double* buf[6];           // 0: state (y0, result), 1: ya, 2: yb, 3: acc; parents in a
                             // refined hierarchy also 4: third stage input, 5: y0 kept
   const double* ghost;      // t = 0 state: source of the static ghosts
@@ -36,26 +36,27 @@ __device__ __forceinline__ int find_patch(const long long* __restrict__ start, i
 
 // --- persistent kernels over all patches -------------------------------------------------
 
-// Static ghosts: copy every ghost point of `which` buffer from the t = 0 state.
-__global__ void __launch_bounds__(256) kb_fill(const PatchDev* __restrict__ P, const long long* __restrict__ pad0,
+// Static ghosts: copy every ghost point of `which` buffer from the t = 0 state,
+// the variables 4 blockIdx.y ... of it (as k_fill_ghosts).
+__global__ void __launch_bounds__(256) kb_fill(const PatchDev* __restrict__ P, const long long* __restrict__ gh0,
                                               int np, long long total, int which) {
+  constexpr int FILL_VARS = 4;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
        t += (long long)gridDim.x * blockDim.x) {
-    const int b = find_patch(pad0, np, t);
+    const int b = find_patch(gh0, np, t);
     const PatchDev& D = P[b];
     const Layout& L = D.L;
-    const long long q = t - D.pad0;
-    const long long ex = L.nx + 2LL * L.g, ey = L.ny + 2LL * L.g;
-    const int i = (int)(q % ex) - L.g;
-    const long long r = q / ex;
-    const int j = (int)(r % ey) - L.g;
-    const int k = (int)(r / ey) - L.g;
-    if (i >= 0 && i < L.nx && j >= 0 && j < L.ny && k >= 0 && k < L.nz) continue;
+    int i, j, k;
+    ghost_point(L, t - D.gh0, i, j, k);
     const long long p = L.off0 + i + j * L.sy + k * L.sz;
     if (!in_range(p, p, padded_points(L))) continue;
-    double* u = D.buf[which];
-#pragma unroll 4
-    for (int v = 0; v < NV; ++v) u[v * L.vs + p] = __ldg(D.ghost + v * L.vs + p);
+    double* u = D.buf[which] + p + blockIdx.y * FILL_VARS * L.vs;
+    const double* src = D.ghost + p + blockIdx.y * FILL_VARS * L.vs;
+    double x[FILL_VARS];
+#pragma unroll
+    for (int v = 0; v < FILL_VARS; ++v) x[v] = __ldg(src + v * L.vs);
+#pragma unroll
+    for (int v = 0; v < FILL_VARS; ++v) u[v * L.vs] = x[v];
   }
 }
 
