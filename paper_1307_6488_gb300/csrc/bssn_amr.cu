@@ -774,8 +774,8 @@ cudaError_t compute_stage(bssn_amr* A, Level& L, const RK& rk, int in, int out, 
       e = A->order == 4 ? launch_d1tab32_batch<4>(L.dev32, L.d_ext0, n, L.next, g2, s)
                         : launch_d1tab32_batch<8>(L.dev32, L.d_ext0, n, L.next, g2, s);
     if (e == cudaSuccess)
-      e = A->order == 4 ? launch_stage32_batch<4>(L.dev32, L.d_tile32, 0, n, 0, L.ntiles32, L.C32, A->gz, rk, in, out, s)
-                        : launch_stage32_batch<8>(L.dev32, L.d_tile32, 0, n, 0, L.ntiles32, L.C32, A->gz, rk, in, out, s);
+      e = A->order == 4 ? launch_stage32_batch<4>(L.dev32, nullptr, L.d_tile32, 0, n, 0, L.ntiles32, L.C32, A->gz, rk, in, out, s)
+                        : launch_stage32_batch<8>(L.dev32, nullptr, L.d_tile32, 0, n, 0, L.ntiles32, L.C32, A->gz, rk, in, out, s);
     A->nodes += 3;
     return e;
   }

@@ -49,16 +49,17 @@ cudaError_t launch_d1tab32(const Layout32& L32, const bssn_grid_t& G, const floa
 cudaError_t launch_to_f32t(const Layout& L, const Layout32& L32, const double* u, float* f, cudaStream_t s);
 // The same kernels over many patches (bssn_batch.cu): the table entry of a
 // patch (maps, layouts, weights with its spacing, buffers), the stage of the
-// patches p0 .. p0+np-1 of one spacing whose tiles start at tbase, and the
-// conversion and tables over all patches (grid-stride, `grid` blocks).
+// patches p0 .. p0+np-1 of one spacing whose tiles start at tbase (next:
+// nullable table of the same patches whose single-precision copies receive the
+// output), and the conversion and tables over all patches (grid-stride, `grid` blocks).
 template <int P>
 bool make_patch32(Patch32* D, const bssn_grid_t& G, double eps, double* const buf[6], float* f32, float* tab);
 template <int P>
 cudaError_t stage32_batch_init();  // raises the kernel's shared-memory limit (not during a capture)
 template <int P>
-cudaError_t launch_stage32_batch(const Patch32* dev, const long long* tile0, int p0, int np, long long tbase,
-                                 long long ntiles, const Coef32& C, const Gauge& gz, const RK& rk, int in, int out,
-                                 cudaStream_t s);
+cudaError_t launch_stage32_batch(const Patch32* dev, const Patch32* next, const long long* tile0, int p0, int np,
+                                 long long tbase, long long ntiles, const Coef32& C, const Gauge& gz, const RK& rk,
+                                 int in, int out, cudaStream_t s);
 template <int P>
 cudaError_t launch_d1tab32_batch(const Patch32* dev, const long long* ext0, int np, long long total, int grid,
                                  cudaStream_t s);

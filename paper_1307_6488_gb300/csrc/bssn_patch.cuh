@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "bssn_bounds.cuh"
+#include "bssn_cvt.cuh"
 #include "bssn_launch.h"
 
 namespace {
@@ -20,6 +21,7 @@ using namespace bssn;
 struct PatchDev {
   Layout L;
   long long gh0;            // first point of this patch in the flat ghost-point list
+  int slot32;               // FP32-RHS plans: the patch's place in the Patch32 tables
   double* buf[6];           // 0: state (y0, result), 1: ya, 2: yb, 3: acc; parents in a
                             // refined hierarchy also 4: third stage input, 5: y0 kept
   const double* ghost;      // t = 0 state: source of the static ghosts
@@ -37,9 +39,10 @@ __device__ __forceinline__ int find_patch(const long long* __restrict__ start, i
 // --- persistent kernels over all patches -------------------------------------------------
 
 // Static ghosts: copy every ghost point of `which` buffer from the t = 0 state,
-// the variables 4 blockIdx.y ... of it (as k_fill_ghosts).
-__global__ void __launch_bounds__(256) kb_fill(const PatchDev* __restrict__ P, const long long* __restrict__ gh0,
-                                              int np, long long total, int which) {
+// the variables 4 blockIdx.y ... of it (as k_fill_ghosts), and, where P32 is
+// given, into that table's single-precision copies.
+__global__ void __launch_bounds__(256) kb_fill(const PatchDev* __restrict__ P, const Patch32* __restrict__ P32,
+                                              const long long* __restrict__ gh0, int np, long long total, int which) {
   constexpr int FILL_VARS = 4;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
        t += (long long)gridDim.x * blockDim.x) {
@@ -57,6 +60,14 @@ __global__ void __launch_bounds__(256) kb_fill(const PatchDev* __restrict__ P, c
     for (int v = 0; v < FILL_VARS; ++v) x[v] = __ldg(src + v * L.vs);
 #pragma unroll
     for (int v = 0; v < FILL_VARS; ++v) u[v * L.vs] = x[v];
+    if (P32) {
+      const Patch32& Q = P32[D.slot32];
+      const long long q = idx32(Q.L32, i, j, k);
+      if (!in_range(q, q, padded_points32(Q.L32))) continue;
+      float* f = Q.f32 + q + blockIdx.y * FILL_VARS * Q.L32.vs;
+#pragma unroll
+      for (int v = 0; v < FILL_VARS; ++v) f[v * Q.L32.vs] = f64_to_f32_rn(x[v]);
+    }
   }
 }
 

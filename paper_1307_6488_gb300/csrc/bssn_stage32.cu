@@ -110,13 +110,13 @@ cudaError_t stage32_batch_init<BSSN_ORDER>() {
 }
 
 template <>
-cudaError_t launch_stage32_batch<BSSN_ORDER>(const Patch32* dev, const long long* tile0, int p0, int np,
-                                             long long tbase, long long ntiles, const Coef32& C, const Gauge& gz,
-                                             const RK& rk, int in, int out, cudaStream_t s) {
+cudaError_t launch_stage32_batch<BSSN_ORDER>(const Patch32* dev, const Patch32* next, const long long* tile0, int p0,
+                                             int np, long long tbase, long long ntiles, const Coef32& C,
+                                             const Gauge& gz, const RK& rk, int in, int out, cudaStream_t s) {
   using T = Tile32<BSSN_ORDER>;
   if (ntiles <= 0) return cudaSuccess;
-  k_stage32t_batch<BSSN_ORDER><<<(unsigned int)ntiles, T32N, T::SMEM, s>>>(dev, tile0, p0, np, tbase, C, gz, rk, in,
-                                                                           out);
+  k_stage32t_batch<BSSN_ORDER><<<(unsigned int)ntiles, T32N, T::SMEM, s>>>(dev, next, tile0, p0, np, tbase, C, gz,
+                                                                           rk, in, out);
   return cudaGetLastError();
 }
 

@@ -578,8 +578,9 @@ __device__ __forceinline__ int patch_of(const long long* __restrict__ start, int
 // constant operands.
 template <int P>
 __global__ void __launch_bounds__(T32N, T32_MIN_BLOCKS)
-    k_stage32t_batch(const Patch32* __restrict__ PP, const long long* __restrict__ tile0, int p0, int np,
-                     long long tbase, Coef32 C, Gauge gz, RK rk, int in, int out) {
+    k_stage32t_batch(const Patch32* __restrict__ PP, const Patch32* __restrict__ PO,
+                     const long long* __restrict__ tile0, int p0, int np, long long tbase, Coef32 C, Gauge gz, RK rk,
+                     int in, int out) {
   const long long tb = tbase + blockIdx.x;
   const int pb = p0 + patch_of(tile0 + p0, np, tb);
   const Patch32& D = PP[pb];
@@ -589,7 +590,7 @@ __global__ void __launch_bounds__(T32N, T32_MIN_BLOCKS)
   S.y0 = D.buf[0];
   S.acc = D.buf[3];
   S.out = D.buf[out];
-  S.out32 = nullptr;
+  S.out32 = PO ? PO[pb].f32 : nullptr;
   stage32_tile<P, 0>(D.L, D.L32, C, gz, rk, S, D.M, (int)(tb - D.tile0), D.ntx, D.nty);
 }
 
