@@ -15,11 +15,11 @@
 //     three output planes it neighbours (k_conv_tc below);
 //   weight gradient ("wgrad") - M = 3 dx taps x 32 input channels (+ 32
 //     discarded rows), N = 32 output channels, K = points (one x-row per
-//     step), from channels-first copies of the activation (three copies
-//     pre-shifted by dx = -1, 0, +1 so that every TMA box starts 16-byte
-//     aligned) and of the output gradient; each CTA streams a range of rows,
-//     keeps all 27 taps' sums in TMEM, and writes a partial, summed
-//     afterwards in a fixed order (k_wgrad_rows below).
+//     step). Both operands are the padded activations as they are stored:
+//     rows of points with 8 channels contiguous are an operand whose
+//     contiguous direction is M or N, which the tensor core takes. Each CTA
+//     streams a range of rows, keeps all 27 taps' sums in TMEM, and writes a
+//     partial, summed afterwards in a fixed order (k_wgrad_rows below).
 // Activations are zero outside the box (zero padding); the backward pass is
 // its exact adjoint.
 #include <cuda.h>
@@ -46,7 +46,6 @@ constexpr int CH = 32;
 constexpr int NL = 5;
 constexpr int NTAP = 27;
 constexpr int W_TAP_BYTES = CH * CH * 2;  // 2 KB per tap
-constexpr int XOFF = 8;  // interior column of the channels-first copies
 constexpr int LAYER_PARAMS = NTAP * CH * CH + CH;
 
 struct Geom {
@@ -465,13 +464,22 @@ __global__ void __launch_bounds__(CONV_THREADS, CONV_CTAS)
 // ---------------------------------------------------------------- wgrad
 // dW[t][co][ci] = sum over points p of act(p + off_t, ci) g(p, co): per CTA a
 // range of output x-rows (s, z, y), all 27 taps at once.
-//   For output row (s, z, y) the activation rows (s, z + dz, y + dy) of the
-//   three dx-shifted channels-first copies are needed, 27 boxes of
-//   32 channels x XW points. Consecutive rows of one plane share 18 of them,
-//   so the rows stream through a ring of 4 "row triples" (entry e: padded
-//   activation row y', its 3 dz planes x 3 dx copies), one new triple per
-//   output row and three at the start of a plane. Output row r uses the
-//   entries e(r) - 2, e(r) - 1, e(r) (dy = -1, 0, +1).
+//   For output row (s, z, y) the activation rows (s, z + dz, y + dy) are
+//   needed at the three shifts dx, 27 boxes of 32 channels x XW points, each
+//   one TMA copy that starts at point dx of the padded row. Consecutive rows
+//   of one plane share 18 of them, so the rows stream through a ring of 4
+//   "row triples" (entry e: padded activation row y', its 3 dz planes x 3
+//   shifts), one new triple per output row and three at the start of a
+//   plane. Output row r uses the entries e(r) - 2, e(r) - 1, e(r) (dy = -1,
+//   0, +1).
+//   In shared memory a box is [chunk of 8 channels][point][8 channels], no
+//   swizzle: 8 points x 8 channels are one 128-byte core matrix with the
+//   channels contiguous (M- and N-major operands), the next 8 points follow
+//   (leading offset 128 bytes), the next 8 channels are a chunk further
+//   (stride offset 16 XW bytes). With K-major operands the activations and
+//   the gradient had to be rewritten channels-first before every layer, once
+//   per shift: 20 passes of 25 us in a training step at 64^3, batch 4 (step
+//   2.98 -> 2.29 ms, the same bits).
 //   MMA: per (dz, dy) group one M = 128 operand: the three dx boxes of that
 //   entry and plane are adjacent in shared memory (rows: dx-major, then ci),
 //   the fourth 32-row block is whatever follows and its results are
@@ -490,15 +498,14 @@ struct WR {
   static constexpr int A_BYTES = WR_Y * 9 * BOX + BOX;   // ring + one box of pad (the 4th block of the last group)
   static constexpr int ONES = 4 * BOX;                   // 128 rows of 1.0: the bias gradient's A operand
   static constexpr int SMEM = 1024 + A_BYTES + WR_B * BOX + ONES + 256;
-  static constexpr uint32_t SBO = 8 * XW * 2;            // one 8-row swizzle atom
-  static constexpr int KSTEPS = XW / 16;
-  static constexpr tc::Swizzle SWZ = XW == 64 ? tc::SWZ_128B : tc::SWZ_64B;
+  static constexpr uint32_t SBO = 16 * XW;               // one chunk of 8 channels
+  static constexpr uint32_t LBO = 8 * 16;                // 8 points
+  static constexpr int KSTEPS = XW / 16, KSTEP = 16 * 16 / 16;  // descriptor units (16 bytes) of 16 points
 };
 
 template <int XW>
 __global__ void __launch_bounds__(WG_THREADS, 1)
-    k_wgrad_rows(const __grid_constant__ CUtensorMap tmXm, const __grid_constant__ CUtensorMap tmX0,
-                 const __grid_constant__ CUtensorMap tmXp, const __grid_constant__ CUtensorMap tmG, Geom G,
+    k_wgrad_rows(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmG, Geom G,
                  int rows_per_cta, float* __restrict__ partial, unsigned int* err) {
   using W = WR<XW>;
   extern __shared__ uint8_t smem_raw[];
@@ -539,12 +546,12 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t taddr = *tslot;
-  constexpr uint32_t IDESC = tc::idesc_bf16_f32(128, 32);
+  constexpr uint32_t MN_A = 1u << 15, MN_B = 1u << 16;  // operands stored along K, channels contiguous
+  constexpr uint32_t IDESC = tc::idesc_bf16_f32(128, 32) | MN_B;
 
   if (warp == 4) {
     // ---- TMA producer
     if (lane == 0 && nrows > 0) {
-      const CUtensorMap* tmx[3] = {&tmXm, &tmX0, &tmXp};
       int e = -1;  // last triple issued
       int issued = 0;
       bool ok = true;
@@ -576,10 +583,10 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
           for (int dz = 0; dz < 3; ++dz)
 #pragma unroll
             for (int dx = 0; dx < 3; ++dx)
-              tc::tma_load_4d(slot + (dz * 3 + dx) * W::BOX, tmx[dx], XOFF, y + t, s * (G.Z + 2) + z + dz, 0,
+              tc::tma_load_4d(slot + (dz * 3 + dx) * W::BOX, &tmX, 2 * dx, y + t, s * (G.Z + 2) + z + dz, 0,
                               &rfull[bs]);
         }
-        tc::tma_load_4d(Bst + bs * W::BOX, &tmG, XOFF, y + 1, s * (G.Z + 2) + z + 1, 0, &rfull[bs]);
+        tc::tma_load_4d(Bst + bs * W::BOX, &tmG, 2, y + 1, s * (G.Z + 2) + z + 1, 0, &rfull[bs]);
         issued = k + 1;
       }
       if (!ok) {
@@ -603,25 +610,25 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
           break;
         }
         tc::fence_after_sync();
-        const uint64_t bd = tc::smem_desc(tc::smem_u32(Bst + bs * W::BOX), 16, W::SBO, W::SWZ);
+        const uint64_t bd = tc::smem_desc(tc::smem_u32(Bst + bs * W::BOX), W::LBO, W::SBO, tc::SWZ_NONE);
 #pragma unroll
         for (int dy = 0; dy < 3; ++dy) {
           const int ent = e - 2 + dy;
 #pragma unroll
           for (int dz = 0; dz < 3; ++dz) {
             const uint64_t ad =
-                tc::smem_desc(tc::smem_u32(Ast + ((ent % WR_Y) * 9 + dz * 3) * W::BOX), 16, W::SBO, W::SWZ);
+                tc::smem_desc(tc::smem_u32(Ast + ((ent % WR_Y) * 9 + dz * 3) * W::BOX), W::LBO, W::SBO, tc::SWZ_NONE);
             const uint32_t d = taddr + (uint32_t)((dz * 3 + dy) * 32);
 #pragma unroll
             for (int j = 0; j < W::KSTEPS; ++j)
-              tc::mma_bf16_elect(d, ad + 2 * j, bd + 2 * j, IDESC, (k > 0 || j > 0) ? 1u : 0u);
+              tc::mma_bf16_elect(d, ad + W::KSTEP * j, bd + W::KSTEP * j, IDESC | MN_A, (k > 0 || j > 0) ? 1u : 0u);
           }
         }
         // bias gradient: ones x gradient row, every TMEM lane gets the row's sums
-        const uint64_t od = tc::smem_desc(tc::smem_u32(Ones), 16, W::SBO, W::SWZ);
+        const uint64_t od = tc::smem_desc(tc::smem_u32(Ones), 16, W::SBO, tc::SWZ_NONE);
 #pragma unroll
         for (int j = 0; j < W::KSTEPS; ++j)
-          tc::mma_bf16_elect(taddr + 9 * 32, od + 2 * j, bd + 2 * j, IDESC, (k > 0 || j > 0) ? 1u : 0u);
+          tc::mma_bf16_elect(taddr + 9 * 32, od + 2 * j, bd + W::KSTEP * j, IDESC, (k > 0 || j > 0) ? 1u : 0u);
         tc::mma_commit_elect(&bempty[bs]);
         // triples no later row reads: the oldest one, or all three before a new plane
         const int keep_from = (k + 1 < nrows && !fresh(k + 1)) ? e - 1 : e + 1;
@@ -703,36 +710,6 @@ __global__ void __launch_bounds__(256) k_wgrad_reduce(const float* __restrict__ 
 #pragma unroll
     for (int q = 0; q < 8; ++q) t += part[q][lane];
     dW[idx] = (float)t;
-  }
-}
-
-// Channels-last padded BF16 -> channels-first copy, interior at column XOFF,
-// shifted by dx: out[c][zz][yy][XOFF + x] = in[zz][yy][x + 1 + dx][c] for the
-// padded rows zz, yy and x in [0, X); zero elsewhere.
-__global__ void k_to_channels_first(Geom G, const __nv_bfloat16* __restrict__ in, __nv_bfloat16* __restrict__ out,
-                                    int dx, int xp) {
-  const long long rows = (long long)G.S * (G.Z + 2) * (G.Y + 2);
-  const long long n = rows * xp;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const long long row = i / xp;
-    const int xs = (int)(i % xp);
-    const int x = xs - XOFF;
-    const bool inside = x >= 0 && x < G.X;
-    __align__(16) __nv_bfloat16 v[CH];
-    if (inside) {
-      // row = (s (Z+2) + zz) (Y+2) + yy over padded planes and rows
-      const long long plane = row / (G.Y + 2);
-      const int yy = (int)(row % (G.Y + 2));
-      const uint4* src = (const uint4*)in + (plane * 4 * (G.Y + 2) + yy) * (G.X + 2) + x + 1 + dx;
-      const long long cs = chunk_stride(G);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) ((uint4*)v)[q] = __ldg(src + q * cs);
-    } else {
-#pragma unroll
-      for (int q = 0; q < 4; ++q) ((uint4*)v)[q] = make_uint4(0u, 0u, 0u, 0u);
-    }
-#pragma unroll
-    for (int c = 0; c < CH; ++c) out[(long long)c * rows * xp + i] = v[c];
   }
 }
 
@@ -1017,11 +994,12 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
 }
 
 bool encode(CUtensorMap* tm, void* ptr, int rank, const cuuint64_t* dims, const cuuint64_t* strides_bytes,
-            const cuuint32_t* box, CUtensorMapSwizzle swz) {
+            const cuuint32_t* box, CUtensorMapSwizzle swz,
+            CUtensorMapDataType type = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16) {
   auto fn = encode_fn();
   if (!fn) return false;
   cuuint32_t es[5] = {1, 1, 1, 1, 1};
-  return fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank, ptr, dims, strides_bytes, box, es,
+  return fn(tm, type, rank, ptr, dims, strides_bytes, box, es,
             CU_TENSOR_MAP_INTERLEAVE_NONE, swz, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -1046,13 +1024,16 @@ bool map_w(CUtensorMap* tm, void* ptr) {
   return encode(tm, ptr, 2, dims, str, box, CU_TENSOR_MAP_SWIZZLE_64B);
 }
 
-// channels-first copy [32][S(Z+2)][Y+2][xp]: dims {xp, Y+2, S(Z+2), 32}, box {64, 1, 1, 32}, 128B swizzle
-bool map_cf(CUtensorMap* tm, void* ptr, const Geom& G, int xp) {
-  const cuuint64_t rows = (cuuint64_t)G.S * (G.Z + 2);
-  const cuuint64_t dims[4] = {(cuuint64_t)xp, (cuuint64_t)G.Y + 2, rows, CH};
-  const cuuint64_t str[3] = {(cuuint64_t)xp * 2, (cuuint64_t)xp * 2 * (G.Y + 2), (cuuint64_t)xp * 2 * (G.Y + 2) * rows};
-  const cuuint32_t box[4] = {(cuuint32_t)G.X, 1, 1, CH};
-  return encode(tm, ptr, 4, dims, str, box, G.X == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B);
+// Rows of the same activations for the weight gradient: {X+2 points of 16
+// bytes as pairs of 8, Y+2, S (Z+2) planes, 4 chunks}, box {X points, 1, 1, 4}:
+// in shared memory [chunk][x][8 channels]. The points of a row are one
+// dimension, so that a copy moves runs of 16 X bytes.
+bool map_row(CUtensorMap* tm, void* ptr, const Geom& G) {
+  const cuuint64_t dims[4] = {2ull * (G.X + 2), (cuuint64_t)G.Y + 2, (cuuint64_t)G.S * (G.Z + 2), 4};
+  const cuuint64_t row = 16ull * (G.X + 2), chunk = row * (G.Y + 2);
+  const cuuint64_t str[3] = {row, 4 * chunk, chunk};
+  const cuuint32_t box[4] = {2 * (cuuint32_t)G.X, 1, 1, 4};
+  return encode(tm, ptr, 4, dims, str, box, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_DATA_TYPE_FLOAT64);
 }
 
 }  // namespace
@@ -1060,15 +1041,13 @@ bool map_cf(CUtensorMap* tm, void* ptr, const Geom& G, int xp) {
 // =========================================================================== corrector object
 struct bssn_corrector {
   Geom G{};          // geometry at max batch
-  int n = 0, max_batch = 0, xp = 0;
+  int n = 0, max_batch = 0;
   long long pts = 0;        // max_batch * n^3
   long long pad_pts = 0;    // max_batch * (n+2)^3
   std::vector<void*> allocs;
   __nv_bfloat16* act[NL] = {};   // padded inputs of layers 1..5 (act[0] = network input)
   float* z[NL] = {};             // pre-activations (layer outputs), unpadded FP32
   __nv_bfloat16* g[2] = {};      // padded gradients (ping-pong)
-  __nv_bfloat16* cf[3] = {};     // channels-first shifted activation copies (dx = -1, 0, +1)
-  __nv_bfloat16* cfg = nullptr;  // channels-first gradient copy
   float* target = nullptr;       // unpadded FP32 targets
   float* partial = nullptr;      // wgrad partials
   double* lpart = nullptr;       // loss partials
@@ -1238,24 +1217,13 @@ cudaError_t network_backward(bssn_corrector* c, const Geom& G, cudaStream_t s) {
   const int rpc = (int)((rows + nb - 1) / nb);
   for (int l = NL - 1; l >= 0 && e == cudaSuccess; --l) {
     float* gW = c->grads + (size_t)l * LAYER_PARAMS;
-    // channels-first copies of the layer input and of the gradient
-    for (int d = 0; d < 3 && e == cudaSuccess; ++d) {
-      k_to_channels_first<<<1024, 256, 0, s>>>(G, c->act[l], c->cf[d], d - 1, c->xp);
-      e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) {
-      k_to_channels_first<<<1024, 256, 0, s>>>(G, c->g[cur], c->cfg, 0, c->xp);
-      e = cudaGetLastError();
-    }
-    CUtensorMap tm[3], tg;
-    for (int d = 0; d < 3; ++d)
-      if (!map_cf(&tm[d], c->cf[d], G, c->xp)) return cudaErrorInvalidValue;
-    if (!map_cf(&tg, c->cfg, G, c->xp)) return cudaErrorInvalidValue;
+    CUtensorMap tx, tg;
+    if (!map_row(&tx, c->act[l], G) || !map_row(&tg, c->g[cur], G)) return cudaErrorInvalidValue;
     if (e == cudaSuccess) {
       if (G.X == 64)
-        k_wgrad_rows<64><<<nb, WG_THREADS, WR<64>::SMEM, s>>>(tm[0], tm[1], tm[2], tg, G, rpc, c->partial, c->err);
+        k_wgrad_rows<64><<<nb, WG_THREADS, WR<64>::SMEM, s>>>(tx, tg, G, rpc, c->partial, c->err);
       else
-        k_wgrad_rows<32><<<nb, WG_THREADS, WR<32>::SMEM, s>>>(tm[0], tm[1], tm[2], tg, G, rpc, c->partial, c->err);
+        k_wgrad_rows<32><<<nb, WG_THREADS, WR<32>::SMEM, s>>>(tx, tg, G, rpc, c->partial, c->err);
       e = cudaGetLastError();
     }
     if (e == cudaSuccess) {
@@ -1325,7 +1293,6 @@ bssn_status_t bssn_corrector_create(bssn_corrector_t** out, int n, int max_batch
   c->n = n;
   c->max_batch = max_batch;
   c->G = Geom{max_batch, n, n, n};
-  c->xp = n + 16;
   c->pts = (long long)max_batch * n * n * n;
   c->pad_pts = (long long)max_batch * (n + 2) * (n + 2) * (n + 2);
   // one weight-gradient CTA per SM (each streams a range of rows)
@@ -1349,13 +1316,6 @@ bssn_status_t bssn_corrector_create(bssn_corrector_t** out, int n, int max_batch
     e = calloc_dev(c, c->pad_pts * CH * 2, &p);
     c->g[i] = (__nv_bfloat16*)p;
   }
-  const size_t cf_bytes = (size_t)CH * max_batch * (n + 2) * (n + 2) * c->xp * 2;
-  for (int d = 0; d < 3 && e == cudaSuccess; ++d) {
-    e = calloc_dev(c, cf_bytes, &p);
-    c->cf[d] = (__nv_bfloat16*)p;
-  }
-  if (e == cudaSuccess) e = calloc_dev(c, cf_bytes, &p);
-  c->cfg = (__nv_bfloat16*)p;
   if (e == cudaSuccess) e = calloc_dev(c, c->pts * CH * 4, &p);
   c->target = (float*)p;
   if (e == cudaSuccess) e = calloc_dev(c, (size_t)c->wg_blocks * (NTAP * CH * CH + CH) * 4, &p);

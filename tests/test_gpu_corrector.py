@@ -205,3 +205,43 @@ def test_adam_steps_lower_the_loss(net32):
     losses = [B.corrector_train_step(net32, grid, coarse, target, 2e-3) for _ in range(10)]
     assert np.all(np.isfinite(losses))
     assert losses[-1] < 0.7 * losses[0], losses
+
+
+@pytest.mark.parametrize("n,S", [(32, 1), (32, 3), (64, 1), (64, 2)])
+def test_last_layer_weight_gradient(n, S):
+    """Every tap's weight gradient and the bias gradient of the last layer
+    against the sums over points, for both row widths of the kernel and rows
+    of several samples. The layer's input is re-formed from its
+    pre-activation, whose GELU on the GPU is good to 2^-11 and is rounded to
+    BF16 (2^-9), so a term may differ by 2^-8 of itself: 8e-3 of the norm."""
+    torch = need_gpu()
+    c = B.corrector_create(n, S, seed=9)
+    try:
+        B.corrector_params(c, seeded_params(51))
+        rng = np.random.default_rng(52 + n + S)
+        x = np.zeros((S, n, n, n, CH))
+        x[..., :24] = bf16_round(rng.standard_normal((S, n, n, n, 24)))
+        t = np.zeros((S, n ** 3, CH), dtype=np.float32)
+        t[..., :24] = 0.3 * rng.standard_normal((S, n ** 3, 24))
+        xb = to_bf16_tensor(x)
+        out = torch.empty((S * n ** 3, CH), dtype=torch.float32, device="cuda")
+        B.corrector_forward_raw(c, S, xb, out)
+        z3 = torch.empty_like(out)
+        B.corrector_layer_output(c, 3, S, z3)
+        B.corrector_loss_grad_raw(c, S, xb, torch.from_numpy(t).cuda())
+        got = B.corrector_grads(c)[4 * LAYER:5 * LAYER].astype(np.float64)
+        diff = out.cpu().numpy().reshape(t.shape) - t
+        g = bf16_round(np.float32(2.0 / (S * n ** 3 * 24.0)) * diff)
+        g[..., 24:] = 0.0
+        g = g.reshape(S, n, n, n, CH)
+        a = np.zeros((S, n + 2, n + 2, n + 2, CH))
+        a[:, 1:-1, 1:-1, 1:-1] = bf16_round(oracle.gelu(z3.cpu().numpy().astype(np.float64))).reshape(S, n, n, n, CH)
+        for tap in range(NTAP):
+            dz, dy, dx = tap // 9, tap // 3 % 3, tap % 3
+            part = a[:, dz:dz + n, dy:dy + n, dx:dx + n].reshape(-1, CH)
+            want = g.reshape(-1, CH).T @ part
+            w = got[tap * CH * CH:(tap + 1) * CH * CH].reshape(CH, CH)
+            assert rel(w, want) < 8e-3, tap
+        assert rel(got[NTAP * CH * CH:][:24], g.reshape(-1, CH).sum(0)[:24]) < 8e-3
+    finally:
+        B.corrector_destroy(c)
