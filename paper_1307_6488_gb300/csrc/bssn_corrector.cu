@@ -13,8 +13,9 @@
 //     operand of each of the 9 in-plane taps is that slab seen through a
 //     descriptor shifted by the tap's entry offset, and each slab serves the
 //     three output planes it neighbours (k_conv_tc below);
-//   weight gradient ("wgrad") - M = 3 dx taps x 32 input channels (+ 32
-//     discarded rows), N = 32 output channels, K = points (one x-row per
+//   weight gradient ("wgrad") - M = 3 dz taps x 32 input channels (+ 32
+//     rows of ones: the bias), N = up to 3 dy x 32 output channels, K = points
+//     (one x-row per
 //     step). Both operands are the padded activations as they are stored:
 //     rows of points with 8 channels contiguous are an operand whose
 //     contiguous direction is M or N, which the tensor core takes. Each CTA
@@ -471,43 +472,43 @@ __global__ void __launch_bounds__(CONV_THREADS, CONV_CTAS)
 // ---------------------------------------------------------------- wgrad
 // dW[t][co][ci] = sum over points p of act(p + off_t, ci) g(p, co): per CTA a
 // range of output x-rows (s, z, y), all 27 taps at once.
-//   For output row (s, z, y) the activation rows (s, z + dz, y + dy) are
-//   needed at the three shifts dx, 27 boxes of 32 channels x XW points, each
-//   one TMA copy that starts at point dx of the padded row. Consecutive rows
-//   of one plane share 18 of them, so the rows stream through a ring of 4
-//   "row triples" (entry e: padded activation row y', its 3 dz planes x 3
-//   shifts), one new triple per output row and three at the start of a
-//   plane. Output row r uses the entries e(r) - 2, e(r) - 1, e(r) (dy = -1,
-//   0, +1).
+//   The CTA steps through the activation rows y' that its output rows of a
+//   plane reach (one more on each side). A step loads the row's three dz
+//   planes, X + 2 points each, and the gradient row y = y' where there is
+//   one; row y' meets the gradient rows y' - dy, three of them (fewer at the
+//   ends).
 //   In shared memory a box is [chunk of 8 channels][point][8 channels], no
 //   swizzle: 8 points x 8 channels are one 128-byte core matrix with the
 //   channels contiguous (M- and N-major operands), the next 8 points follow
 //   (leading offset 128 bytes), the next 8 channels are a chunk further
-//   (stride offset 16 XW bytes). With K-major operands the activations and
-//   the gradient had to be rewritten channels-first before every layer, once
-//   per shift: 20 passes of 25 us in a training step at 64^3, batch 4 (step
-//   2.98 -> 2.29 ms, the same bits).
-//   MMA: per (dz, dy) group one M = 128 operand: the three dx boxes of that
-//   entry and plane are adjacent in shared memory (rows: dx-major, then ci),
-//   the fourth 32-row block is whatever follows and its results are
-//   discarded; N = 32 output channels from the output-gradient row; K = the
-//   row's XW points. Nine accumulators of 32 TMEM columns sum over the rows.
-//   warp 4 (one lane) streams triples and gradient rows; warp 5 (whole warp,
-//   one elected lane) issues 9 x XW/16 MMAs per row, frees each gradient
-//   slot after its row and each triple after the last row that reads it;
-//   warps 0-2 write the 27 taps' partial sums at the end (warp 3's lanes
-//   hold the discarded rows).
-constexpr int WR_Y = 4;    // row triples in the ring
-constexpr int WR_B = 4;    // gradient rows in flight
+//   (stride offset). The three dz boxes and a box of ones lie together: M = 128 rows
+//   (dz, ci) and 32 rows whose sums are the bias gradient; a shift dx is 16
+//   bytes of the start address. Gradient rows lie together too, so N is up to 3 x
+//   32 (y, co); K = the row's XW points. Per shift 96 TMEM columns sum over
+//   the rows, in row order for every tap.
+//   A copy of the operands channels-first, once per shift, had cost 20 passes
+//   of 25 us in a training step at 64^3, batch 4 (2.98 -> 2.29 ms without).
+//   Loading each shift of each row and N = 32 per MMA, a step moved 40 KB and
+//   read the M operand from shared memory nine times (168 us per layer);
+//   now 17 KB and three times (57 us; the training step 2.24 -> 1.68 ms).
+//   warp 4 (one lane) streams the rows; warp 5 (whole warp, one elected lane)
+//   issues 3 x XW/16 MMAs per step; warps 0-2 write the 27 taps' partial sums
+//   at the end, warp 3 the bias gradient's.
+constexpr int WR_Y = 6;         // activation rows in the ring
+constexpr int WR_B = WR_Y + 2;  // gradient rows in the ring: a row is last read two steps after its own, so
+                                // the free slot of an activation row implies the free slot of a gradient row
 template <int XW>
 struct WR {
-  static constexpr int BOX = CH * XW * 2;                // one box: 32 channels x XW points
-  static constexpr int A_BYTES = WR_Y * 9 * BOX + BOX;   // ring + one box of pad (the 4th block of the last group)
-  static constexpr int ONES = 4 * BOX;                   // 128 rows of 1.0: the bias gradient's A operand
-  static constexpr int SMEM = 1024 + A_BYTES + WR_B * BOX + ONES + 256;
-  static constexpr uint32_t SBO = 16 * XW;               // one chunk of 8 channels
+  static constexpr int CS = 16 * (XW + 2);               // one chunk of 8 channels of an activation row
+  static constexpr int ABOX = 4 * CS;                    // one plane of an activation row
+  static constexpr int ROW = 4 * ABOX;                   // three planes and the ones
+  static constexpr int GCS = 16 * XW, GBOX = 4 * GCS;    // gradient row
+  // the first two gradient slots are held a second time behind the last, so
+  // that three rows always lie together
+  static constexpr int SMEM = 1024 + WR_Y * ROW + (WR_B + 2) * GBOX + 256;
   static constexpr uint32_t LBO = 8 * 16;                // 8 points
   static constexpr int KSTEPS = XW / 16, KSTEP = 16 * 16 / 16;  // descriptor units (16 bytes) of 16 points
+  static_assert(ABOX % 128 == 0 && GBOX % 128 == 0, "TMA destinations stay 128-byte aligned");
 };
 
 template <int XW>
@@ -517,14 +518,12 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
   using W = WR<XW>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  uint8_t* Ast = base;                     // [entry slot][dz][dx] boxes
-  uint8_t* Bst = base + W::A_BYTES;        // [WR_B] gradient rows
-  uint8_t* Ones = Bst + WR_B * W::BOX;     // 128 x XW ones (any swizzle leaves them as they are)
-  uint64_t* bars = (uint64_t*)(Ones + W::ONES);
-  uint64_t* rfull = bars;                  // [WR_B] row r's new triples and gradient row landed
-  uint64_t* bempty = rfull + WR_B;         // [WR_B] gradient slot free
-  uint64_t* yempty = bempty + WR_B;        // [WR_Y] triple slot free
-  uint64_t* done = yempty + WR_Y;
+  uint8_t* Ast = base;                     // [WR_Y][dz, ones] boxes
+  uint8_t* Bst = base + WR_Y * W::ROW;     // [WR_B + 2] gradient rows
+  uint64_t* bars = (uint64_t*)(Bst + (WR_B + 2) * W::GBOX);
+  uint64_t* full = bars;                   // [WR_Y] a step's copies landed
+  uint64_t* empty = full + WR_Y;           // [WR_Y] a step's MMAs done
+  uint64_t* done = empty + WR_Y;
   uint32_t* tslot = (uint32_t*)(done + 1);
   __shared__ volatile int abort_flag;
 
@@ -532,19 +531,18 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
   const long long total_rows = (long long)G.S * G.Z * G.Y;
   const long long r0 = (long long)blockIdx.x * rows_per_cta;
   const int nrows = (int)(r0 >= total_rows ? 0 : (total_rows - r0 < rows_per_cta ? total_rows - r0 : rows_per_cta));
-  // plane (s, z) of a row, and whether row r starts a new window
-  auto plane_of = [&](long long R) { return R / G.Y; };
-  auto fresh = [&](int k) { return k == 0 || plane_of(r0 + k) != plane_of(r0 + k - 1); };
 
-  for (int i = tid; i < W::ONES / 4; i += blockDim.x) ((uint32_t*)Ones)[i] = 0x3F803F80u;  // BF16 1.0 pairs
+  for (int i = tid; i < WR_Y * (W::ABOX / 4); i += blockDim.x) {
+    const int slot = i / (W::ABOX / 4), q = i % (W::ABOX / 4);
+    ((uint32_t*)(Ast + slot * W::ROW + 3 * W::ABOX))[q] = 0x3F803F80u;  // BF16 1.0 pairs
+  }
   tc::fence_proxy_async();
   if (tid == 0) {
     abort_flag = 0;
-    for (int i = 0; i < WR_B; ++i) {
-      tc::mbar_init(&rfull[i], 1);
-      tc::mbar_init(&bempty[i], 1);
+    for (int i = 0; i < WR_Y; ++i) {
+      tc::mbar_init(&full[i], 1);
+      tc::mbar_init(&empty[i], 1);
     }
-    for (int i = 0; i < WR_Y; ++i) tc::mbar_init(&yempty[i], 1);
     tc::mbar_init(done, 1);
     tc::mbar_fence_init();
   }
@@ -553,93 +551,85 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t taddr = *tslot;
-  constexpr uint32_t MN_A = 1u << 15, MN_B = 1u << 16;  // operands stored along K, channels contiguous
-  constexpr uint32_t IDESC = tc::idesc_bf16_f32(128, 32) | MN_B;
+  if (warp < 4) {  // the sums start at zero: a step adds to one, two or three rows' columns at once
+#pragma unroll 1
+    for (int c = 0; c < 288; c += 8) tc::tmem_st8_zero(taddr + ((uint32_t)(warp * 32) << 16) + (uint32_t)c);
+    tc::tmem_wait_st();
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
+  constexpr uint32_t MN_MAJOR = (1u << 15) | (1u << 16);  // both operands stored along K, channels contiguous
 
   if (warp == 4) {
     // ---- TMA producer
     if (lane == 0 && nrows > 0) {
-      int e = -1;  // last triple issued
-      int issued = 0;
+      int e = 0;  // steps issued
       bool ok = true;
-      for (int k = 0; ok && k < nrows; ++k) {
+      for (int k = 0; ok && k < nrows;) {  // plane by plane: rows ya .. yb-1 of (s, z), the CTA's rows k ..
         const long long R = r0 + k;
-        const int y = (int)(R % G.Y);
+        const int ya = (int)(R % G.Y);
+        const int yb = G.Y - ya < nrows - k ? G.Y : ya + nrows - k;
         const long long rz = R / G.Y;
-        const int z = (int)(rz % G.Z);
-        const int s = (int)(rz / G.Z);
-        const int bs = k % WR_B;
-        if (k >= WR_B && !tc::mbar_wait_or_abort(&bempty[bs], ((k / WR_B) - 1) & 1, &abort_flag)) {
-          ok = false;
-          break;
-        }
-        // the triples this row adds: padded rows y, y+1, y+2 at a plane start, else y+2
-        const int first = fresh(k) ? 0 : 2;
-        const int nnew = 3 - first;
-        for (int t = first; ok && t < 3; ++t) {
-          const int ee = e + 1 + (t - first);
-          if (ee >= WR_Y && !tc::mbar_wait_or_abort(&yempty[ee % WR_Y], ((ee / WR_Y) - 1) & 1, &abort_flag)) ok = false;
-        }
-        if (!ok) break;
-        tc::mbar_expect_tx(&rfull[bs], (uint32_t)((nnew * 9 + 1) * W::BOX));
-        for (int t = first; t < 3; ++t) {
-          ++e;
-          uint8_t* slot = Ast + (e % WR_Y) * 9 * W::BOX;
-          // padded row y + t holds activation row y - 1 + t (dy = t - 1)
+        const int zp = (int)(rz / G.Z) * (G.Z + 2) + (int)(rz % G.Z);  // padded plane of dz = -1
+        for (int yp = ya; yp < yb + 2; ++yp, ++e) {
+          const int sl = e % WR_Y;
+          if (e >= WR_Y && !tc::mbar_wait_or_abort(&empty[sl], ((e / WR_Y) - 1) & 1, &abort_flag)) {
+            ok = false;
+            break;
+          }
+          const int gs = (k + yp - ya) % WR_B;
+          const int copies = yp < yb ? (gs < 2 ? 2 : 1) : 0;
+          tc::mbar_expect_tx(&full[sl], (uint32_t)(3 * W::ABOX + copies * W::GBOX));
+          // padded row yp holds activation row yp - 1
 #pragma unroll
           for (int dz = 0; dz < 3; ++dz)
-#pragma unroll
-            for (int dx = 0; dx < 3; ++dx)
-              tc::tma_load_4d(slot + (dz * 3 + dx) * W::BOX, &tmX, 2 * dx, y + t, s * (G.Z + 2) + z + dz, 0,
-                              &rfull[bs]);
+            tc::tma_load_4d(Ast + sl * W::ROW + dz * W::ABOX, &tmX, 0, yp, zp + dz, 0, &full[sl]);
+          for (int c = 0; c < copies; ++c)
+            tc::tma_load_4d(Bst + (gs + c * WR_B) * W::GBOX, &tmG, 2, yp + 1, zp + 1, 0, &full[sl]);
         }
-        tc::tma_load_4d(Bst + bs * W::BOX, &tmG, 2, y + 1, s * (G.Z + 2) + z + 1, 0, &rfull[bs]);
-        issued = k + 1;
+        k += yb - ya;
       }
       if (!ok) {
         if (!abort_flag) atomicOr(err, 4u);
         abort_flag = 1;
       }
       // every copy has landed before the CTA leaves
-      for (int k = issued > WR_B ? issued - WR_B : 0; k < issued; ++k)
-        (void)tc::mbar_wait(&rfull[k % WR_B], (k / WR_B) & 1, 100000000ull);
+      for (int q = e > WR_Y ? e - WR_Y : 0; q < e; ++q) (void)tc::mbar_wait(&full[q % WR_Y], (q / WR_Y) & 1, 100000000ull);
     }
   } else if (warp == 5) {
     // ---- MMA issuer (warp-uniform, one elected lane issues)
     if (nrows > 0) {
       bool ok = true;
-      int e = -1;
-      for (int k = 0; k < nrows; ++k) {
-        const int bs = k % WR_B;
-        e += fresh(k) ? 3 : 1;
-        if (!tc::warp_wait_or_abort(&rfull[bs], (k / WR_B) & 1, &abort_flag)) {
-          ok = false;
-          break;
-        }
-        tc::fence_after_sync();
-        const uint64_t bd = tc::smem_desc(tc::smem_u32(Bst + bs * W::BOX), W::LBO, W::SBO, tc::SWZ_NONE);
+      int e = 0;
+      for (int k = 0; ok && k < nrows;) {
+        const int ya = (int)((r0 + k) % G.Y);
+        const int yb = G.Y - ya < nrows - k ? G.Y : ya + nrows - k;
+        for (int yp = ya; yp < yb + 2; ++yp, ++e) {
+          const int sl = e % WR_Y;
+          if (!tc::warp_wait_or_abort(&full[sl], (e / WR_Y) & 1, &abort_flag)) {
+            ok = false;
+            break;
+          }
+          tc::fence_after_sync();
+          // gradient rows ylo .. yhi meet this row; row yp - 2 + c has columns 32 c ..
+          const int ylo = yp - 2 > ya ? yp - 2 : ya, yhi = yp < yb ? yp : yb - 1;
+          const int n = yhi - ylo + 1;
+          const uint32_t idesc = tc::idesc_bf16_f32(128, 32 * n) | MN_MAJOR;
+          const uint64_t bd = tc::smem_desc(tc::smem_u32(Bst + (k + ylo - ya) % WR_B * W::GBOX), W::LBO, W::GCS,
+                                            tc::SWZ_NONE);
 #pragma unroll
-        for (int dy = 0; dy < 3; ++dy) {
-          const int ent = e - 2 + dy;
-#pragma unroll
-          for (int dz = 0; dz < 3; ++dz) {
+          for (int dx = 0; dx < 3; ++dx) {
             const uint64_t ad =
-                tc::smem_desc(tc::smem_u32(Ast + ((ent % WR_Y) * 9 + dz * 3) * W::BOX), W::LBO, W::SBO, tc::SWZ_NONE);
-            const uint32_t d = taddr + (uint32_t)((dz * 3 + dy) * 32);
+                tc::smem_desc(tc::smem_u32(Ast + sl * W::ROW + dx * 16), W::LBO, W::CS, tc::SWZ_NONE);
+            const uint32_t d = taddr + (uint32_t)(dx * 96 + (ylo - yp + 2) * 32);
 #pragma unroll
             for (int j = 0; j < W::KSTEPS; ++j)
-              tc::mma_bf16_elect(d, ad + W::KSTEP * j, bd + W::KSTEP * j, IDESC | MN_A, (k > 0 || j > 0) ? 1u : 0u);
+              tc::mma_bf16_elect(d, ad + W::KSTEP * j, bd + W::KSTEP * j, idesc, 1u);
           }
+          tc::mma_commit_elect(&empty[sl]);
         }
-        // bias gradient: ones x gradient row, every TMEM lane gets the row's sums
-        const uint64_t od = tc::smem_desc(tc::smem_u32(Ones), 16, W::SBO, tc::SWZ_NONE);
-#pragma unroll
-        for (int j = 0; j < W::KSTEPS; ++j)
-          tc::mma_bf16_elect(taddr + 9 * 32, od + 2 * j, bd + W::KSTEP * j, IDESC, (k > 0 || j > 0) ? 1u : 0u);
-        tc::mma_commit_elect(&bempty[bs]);
-        // triples no later row reads: the oldest one, or all three before a new plane
-        const int keep_from = (k + 1 < nrows && !fresh(k + 1)) ? e - 1 : e + 1;
-        for (int q = e - 2; q < keep_from; ++q) tc::mma_commit_elect(&yempty[q % WR_Y]);
+        k += yb - ya;
       }
       if (!ok && lane == 0) {
         if (!abort_flag) atomicOr(err, 4u);
@@ -649,8 +639,8 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
       tc::mma_commit_elect(done);
     }
   }
-  // ---- epilogue (warps 0-2: TMEM lanes 32 w .. = input channels of dx = w - 1;
-  // warp 3: the bias gradient, columns 288 .. 319 of any lane)
+  // ---- epilogue (warps 0-2: TMEM lanes 32 w .. = input channels of dz = w - 1;
+  // warp 3: the bias gradient, the lanes of the ones, any shift and row)
   bool ok = false;
   if (warp < 4 && nrows > 0) {
     ok = tc::mbar_wait(done, 0);
@@ -661,7 +651,7 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
   tc::fence_after_sync();
   if (warp < 3) {
     for (int g = 0; g < 9; ++g) {
-      const int dz = g / 3, dy = g % 3, t = dz * 9 + dy * 3 + warp;
+      const int dx = g / 3, dy = 2 - g % 3, t = warp * 9 + dy * 3 + dx;
       // partial[b][t][co][ci]: lane = ci, so each co is one coalesced 128-byte row
       float* out = partial + ((long long)blockIdx.x * NTAP + t) * CH * CH + lane;
       float acc[32];
@@ -677,7 +667,7 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
   } else if (warp == 3) {
     float acc[32];
     if (ok) {
-      tc::tmem_ld32(taddr + ((uint32_t)(3 * 32) << 16) + (uint32_t)(9 * 32), acc);
+      tc::tmem_ld32(taddr + ((uint32_t)(3 * 32) << 16), acc);
     } else {
 #pragma unroll
       for (int co = 0; co < 32; ++co) acc[co] = 0.f;
@@ -1039,14 +1029,14 @@ bool map_w(CUtensorMap* tm, void* ptr) {
 }
 
 // Rows of the same activations for the weight gradient: {X+2 points of 16
-// bytes as pairs of 8, Y+2, S (Z+2) planes, 4 chunks}, box {X points, 1, 1, 4}:
+// bytes as pairs of 8, Y+2, S (Z+2) planes, 4 chunks}, box {points, 1, 1, 4}:
 // in shared memory [chunk][x][8 channels]. The points of a row are one
-// dimension, so that a copy moves runs of 16 X bytes.
-bool map_row(CUtensorMap* tm, void* ptr, const Geom& G) {
+// dimension, so that a copy moves runs of 16 bytes times the points.
+bool map_row(CUtensorMap* tm, void* ptr, const Geom& G, int points) {
   const cuuint64_t dims[4] = {2ull * (G.X + 2), (cuuint64_t)G.Y + 2, (cuuint64_t)G.S * (G.Z + 2), 4};
   const cuuint64_t row = 16ull * (G.X + 2), chunk = row * (G.Y + 2);
   const cuuint64_t str[3] = {row, 4 * chunk, chunk};
-  const cuuint32_t box[4] = {2 * (cuuint32_t)G.X, 1, 1, 4};
+  const cuuint32_t box[4] = {2 * (cuuint32_t)points, 1, 1, 4};
   return encode(tm, ptr, 4, dims, str, box, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_DATA_TYPE_FLOAT64);
 }
 
@@ -1232,7 +1222,7 @@ cudaError_t network_backward(bssn_corrector* c, const Geom& G, cudaStream_t s) {
   for (int l = NL - 1; l >= 0 && e == cudaSuccess; --l) {
     float* gW = c->grads + (size_t)l * LAYER_PARAMS;
     CUtensorMap tx, tg;
-    if (!map_row(&tx, c->act[l], G) || !map_row(&tg, c->g[cur], G)) return cudaErrorInvalidValue;
+    if (!map_row(&tx, c->act[l], G, G.X + 2) || !map_row(&tg, c->g[cur], G, G.X)) return cudaErrorInvalidValue;
     if (e == cudaSuccess) {
       if (G.X == 64)
         k_wgrad_rows<64><<<nb, WG_THREADS, WR<64>::SMEM, s>>>(tx, tg, G, rpc, c->partial, c->err);
