@@ -694,7 +694,9 @@ __global__ void __launch_bounds__(256) k_wgrad_reduce(const float* __restrict__ 
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int idx = blockIdx.x * 32 + lane;  // over 27*32*32 + 32
   double s = 0.0;
+  // the loads of several partials ahead of their sums
   if (idx < NTAP * CH * CH) {
+#pragma unroll 10
     for (int b = w; b < nb; b += 8) s += partial[(long long)b * NTAP * CH * CH + idx];
   } else if (idx < NTAP * CH * CH + CH) {
     const float* bp = partial + (long long)nb * NTAP * CH * CH + (idx - NTAP * CH * CH);
@@ -726,8 +728,39 @@ __global__ void k_pad_copy(Geom G, const __nv_bfloat16* __restrict__ in, __nv_bf
 // Loss: mean over points and the first nout channels of (out - target)^2;
 // the gradient 2 (out - target) / (pts nout) goes to g (padded BF16, zero in
 // the other channels). Per-block partial sums of squares in part.
-__global__ void k_mse(Geom G, int nout, const float* __restrict__ out, const float* __restrict__ target,
-                      __nv_bfloat16* __restrict__ g, double* __restrict__ part) {
+// Targets as FP32 points of all samples, or (TargetsBf16) as the samples'
+// BF16 pointers, 16-byte aligned: a training step's targets are read where
+// they are. Two blocks of 512 threads on each SM: a thread's loads lie 128
+// bytes from its neighbour's, so it takes many lines in flight.
+struct TargetsF32 {
+  const float* p;
+  __device__ __forceinline__ void get(long long i, int, long long, float (&t)[CH]) const {
+#pragma unroll
+    for (int q = 0; q < CH / 4; ++q) ((float4*)t)[q] = __ldg((const float4*)(p + i * CH) + q);
+  }
+};
+struct TargetsBf16 {
+  const __nv_bfloat16* p[64];
+  __device__ __forceinline__ void get(long long i, int s, long long per_sample, float (&t)[CH]) const {
+    const uint4* src = (const uint4*)(p[s] + (i - s * per_sample) * CH);
+#pragma unroll
+    for (int q = 0; q < CH / 8; ++q) {
+      const uint4 v = __ldg(src + q);
+      const unsigned w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        t[8 * q + 2 * c] = __uint_as_float(w[c] << 16);
+        t[8 * q + 2 * c + 1] = __uint_as_float(w[c] & 0xFFFF0000u);
+      }
+    }
+  }
+};
+constexpr int MSE_BLOCKS = 304, MSE_THREADS = 512;  // two blocks on each of 152 SMs
+
+template <typename Targets>
+__global__ void __launch_bounds__(MSE_THREADS)
+    k_mse(Geom G, int nout, const float* __restrict__ out, const __grid_constant__ Targets target,
+          __nv_bfloat16* __restrict__ g, double* __restrict__ part) {
   const long long pts = (long long)G.S * G.Z * G.Y * G.X;
   const float gscale = (float)(2.0 / ((double)pts * nout));  // d loss / d out = 2 (out - target) / (pts nout)
   double acc = 0.0;
@@ -741,8 +774,8 @@ __global__ void k_mse(Geom G, int nout, const float* __restrict__ out, const flo
 #pragma unroll
     for (int q = 0; q < CH / 4; ++q) {
       ((float4*)o)[q] = __ldg((const float4*)(out + i * CH) + q);
-      ((float4*)t)[q] = __ldg((const float4*)(target + i * CH) + q);
     }
+    target.get(i, s, (long long)G.Z * G.Y * G.X, t);
     __align__(16) __nv_bfloat16 h[32];
     float sq = 0.f;  // this point's sum of squares (at most 32 terms)
 #pragma unroll
@@ -758,7 +791,7 @@ __global__ void k_mse(Geom G, int nout, const float* __restrict__ out, const flo
     acc += (double)sq;
     store_point(G, g, s, z, y, x, h);
   }
-  __shared__ double sh[256];
+  __shared__ double sh[MSE_THREADS];
   sh[threadIdx.x] = acc;
   __syncthreads();
   for (int o = blockDim.x / 2; o > 0; o >>= 1) {
@@ -774,6 +807,9 @@ __global__ void k_weights_bf16(const float* __restrict__ W, __nv_bfloat16* __res
                                __nv_bfloat16* __restrict__ wb) {
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= NTAP * CH * CH) return;
+  W += (size_t)blockIdx.y * LAYER_PARAMS;  // layer
+  wf += (size_t)blockIdx.y * NTAP * CH * CH;
+  wb += (size_t)blockIdx.y * NTAP * CH * CH;
   const int t = idx / (CH * CH), co = (idx / CH) % CH, ci = idx % CH;
   const __nv_bfloat16 v = __float2bfloat16_rn(W[idx]);
   wf[idx] = v;
@@ -1251,25 +1287,26 @@ cudaError_t network_backward(bssn_corrector* c, const Geom& G, cudaStream_t s) {
 }
 
 cudaError_t refresh_weights(bssn_corrector* c, cudaStream_t s) {
-  for (int l = 0; l < NL; ++l) {
-    k_weights_bf16<<<(NTAP * CH * CH + 255) / 256, 256, 0, s>>>(c->params + (size_t)l * LAYER_PARAMS,
-                                                                 c->wf + (size_t)l * NTAP * CH * CH,
-                                                                 c->wb + (size_t)l * NTAP * CH * CH);
-  }
+  k_weights_bf16<<<dim3((NTAP * CH * CH + 255) / 256, NL), 256, 0, s>>>(c->params, c->wf, c->wb);
   return cudaGetLastError();
 }
 
-// loss and output gradient for targets already in c->target; returns the loss (synchronizes)
-cudaError_t loss_and_grad(bssn_corrector* c, const Geom& G, double* loss, cudaStream_t s) {
-  k_mse<<<256, 256, 0, s>>>(G, NV, c->z[NL - 1], c->target, c->g[0], c->lpart);
+// loss and output gradient for targets in c->target, or for the samples' BF16
+// ones if given; returns the loss (synchronizes)
+cudaError_t loss_and_grad(bssn_corrector* c, const Geom& G, double* loss, cudaStream_t s,
+                          const TargetsBf16* bf16 = nullptr) {
+  if (bf16)
+    k_mse<<<MSE_BLOCKS, MSE_THREADS, 0, s>>>(G, NV, c->z[NL - 1], *bf16, c->g[0], c->lpart);
+  else
+    k_mse<<<MSE_BLOCKS, MSE_THREADS, 0, s>>>(G, NV, c->z[NL - 1], TargetsF32{c->target}, c->g[0], c->lpart);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = network_backward(c, G, s);
-  double h[256];
+  double h[MSE_BLOCKS];
   if (e == cudaSuccess) e = cudaMemcpyAsync(h, c->lpart, sizeof(h), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e == cudaSuccess) {
     double sum = 0.0;
-    for (int i = 0; i < 256; ++i) sum += h[i];
+    for (int i = 0; i < MSE_BLOCKS; ++i) sum += h[i];
     *loss = sum / ((double)G.S * G.Z * G.Y * G.X * NV);
   }
   return e;
@@ -1324,7 +1361,7 @@ bssn_status_t bssn_corrector_create(bssn_corrector_t** out, int n, int max_batch
   c->target = (float*)p;
   if (e == cudaSuccess) e = calloc_dev(c, (size_t)c->wg_blocks * (NTAP * CH * CH + CH) * 4, &p);
   c->partial = (float*)p;
-  if (e == cudaSuccess) e = calloc_dev(c, 256 * sizeof(double), &p);
+  if (e == cudaSuccess) e = calloc_dev(c, MSE_BLOCKS * sizeof(double), &p);
   c->lpart = (double*)p;
   const size_t np = (size_t)NL * LAYER_PARAMS;
   if (e == cudaSuccess) e = calloc_dev(c, np * 4, &p);
@@ -1569,15 +1606,21 @@ bssn_status_t bssn_corrector_train_step_raw(bssn_corrector_t* c, int S, const vo
   const Geom G1 = geom_for(c, 1);
   const long long pts1 = (long long)c->n * c->n * c->n;
   const long long pad1 = (long long)(c->n + 2) * (c->n + 2) * (c->n + 2);
+  // targets on 16-byte boundaries are read by the loss itself; others are
+  // widened to FP32 first (14 us more per sample of 64^3)
+  TargetsBf16 bf16{};
+  bool wide = true;
+  for (int i = 0; i < S; ++i) wide = wide && ((uintptr_t)t_bf16[i] & 15) == 0;
   cudaError_t e = cudaMemsetAsync(c->err, 0, 4, s);
   for (int i = 0; i < S && e == cudaSuccess; ++i) {
     if (!x_bf16[i] || !t_bf16[i]) return BSSN_ERR_INVALID_ARG;
     k_pad_copy<<<512, 256, 0, s>>>(G1, (const __nv_bfloat16*)x_bf16[i], c->act[0] + i * pad1 * CH);
-    k_bf16_to_f32<<<512, 256, 0, s>>>(pts1 * CH, (const __nv_bfloat16*)t_bf16[i], c->target + i * pts1 * CH);
+    bf16.p[i] = (const __nv_bfloat16*)t_bf16[i];
+    if (!wide) k_bf16_to_f32<<<512, 256, 0, s>>>(pts1 * CH, bf16.p[i], c->target + i * pts1 * CH);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = network_forward(c, G, s);
-  if (e == cudaSuccess) e = loss_and_grad(c, G, loss, s);
+  if (e == cudaSuccess) e = loss_and_grad(c, G, loss, s, wide ? &bf16 : nullptr);
   if (e == cudaSuccess && lr > 0) {
     c->adam_t += 1;
     const float b1 = 0.9f, b2 = 0.999f;

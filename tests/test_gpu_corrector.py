@@ -245,3 +245,29 @@ def test_last_layer_weight_gradient(n, S):
         assert rel(got[NTAP * CH * CH:][:24], g.reshape(-1, CH).sum(0)[:24]) < 8e-3
     finally:
         B.corrector_destroy(c)
+
+
+@pytest.mark.parametrize("shift", [1, 8])
+def test_training_step_takes_targets_at_any_address(shift):
+    """Targets on 16-byte boundaries are read by the loss itself, others are
+    widened first: the same loss and gradients, bit for bit."""
+    torch = need_gpu()
+    n, S = 32, 2
+    rng = np.random.default_rng(61)
+    x = np.zeros((S, n, n, n, CH))
+    x[..., :24] = bf16_round(rng.standard_normal((S, n, n, n, 24)))
+    xs = [to_bf16_tensor(v) for v in x]
+    ts = [to_bf16_tensor(0.3 * rng.standard_normal((n ** 3, CH))) for _ in range(S)]
+    room = torch.zeros(n ** 3 * CH + shift, dtype=torch.bfloat16, device="cuda")
+    moved = room[shift:].view(n ** 3, CH)
+    moved.copy_(ts[1])
+    got = []
+    for t in (ts, [ts[0], moved]):
+        c = B.corrector_create(n, S, seed=13)
+        try:
+            loss = B.corrector_train_step_raw(c, xs, t, 1e-3)
+            got.append((loss, B.corrector_grads(c).copy()))
+        finally:
+            B.corrector_destroy(c)
+    assert got[0][0] == got[1][0]
+    assert np.array_equal(got[0][1], got[1][1])
