@@ -5,7 +5,7 @@
 // A block of 128 threads owns a tile of 8 x 4 x 4 interior points, one
 // point per thread. For each of the 24 variables in turn, one thread issues
 // the TMA copies of that variable's stencil region around the tile into one
-// slot of a 3-deep ring in shared memory:
+// slot of a 2-deep ring in shared memory:
 //   SX  the tile's rows widened by 8 points on each side in x (the copy
 //       starts 8 points left of the tile so that it stays 16-byte aligned;
 //       the stencil uses 5),
@@ -13,7 +13,7 @@
 // and, for the 11 variables with mixed second derivatives, the D_x u table
 // widened by p/2 in y and in z and the D_y u table widened by p/2 in z. An
 // mbarrier per slot signals the copy's completion; the last of the four warps
-// to finish with a slot (a per-slot counter) refills it with the variable 3
+// to finish with a slot (a per-slot counter) refills it with the variable 2
 // places later, so no thread waits for the others.
 // Every value a thread reads comes from shared memory at a fixed offset from
 // its own point, and feeds the first derivative, the diagonal second
@@ -74,10 +74,23 @@ constexpr int T32X = 8, T32Y = 4, T32Z = 4, T32N = T32X * T32Y * T32Z;
 #ifndef T32_PF_AT
 #define T32_PF_AT 16
 #endif
+// Two slots: a third bought nothing (the other blocks of the SM cover a
+// copy's latency) and took 7 to 10 KB per block from the L1 cache that the
+// centre values and the update go through (42.3 -> 40.5 ms per RK4 step of
+// 256^3 in 4th order).
 #ifndef T32_NBUF_DEF
-#define T32_NBUF_DEF 3
+#define T32_NBUF_DEF 2
 #endif
 constexpr int T32_NBUF = T32_NBUF_DEF;
+// Variables whose update is in registers at a time. All 24 at once spilled
+// 256 bytes a thread, 98 KB per SM through an L1 of 49 KB (44.9 -> 42.3 ms
+// per step of 256^3); with 4 or 6 the loads in flight are too few (43.7,
+// 42.2 against 40.5 ms), 12 are 1 % slower.
+#ifndef U32_VARS_DEF
+#define U32_VARS_DEF 8
+#endif
+constexpr int U32_VARS = U32_VARS_DEF;
+static_assert(NV % U32_VARS == 0, "whole groups");
 constexpr int T32_NTAB = 2 * NM;  // D_x tables of the 11 mixed variables, then their D_y tables
 
 template <int P>
@@ -491,57 +504,65 @@ __device__ __forceinline__ void stage32_tile(const Layout& L, const Layout32& L3
   rhs_point<float>(Q, gz, iW, rhs);
   if (valid && in_range(p, p, padded_points(L)) && in_range(q, q, padded_points32(L32))) {
   const long long vs = L.vs;
-  double kd[NV];
-  {
-    float kf[NV];
+  // the right-hand side goes back to the record, so that the update below
+  // holds U32_VARS variables in registers at a time
 #pragma unroll
-    for (int v = 0; v < NV; ++v) kf[v] = rhs[v] + my[(rec::EXT + v) * T32N];
-    f32_to_f64_vec<NV>(kf, kd);
-  }
-  if constexpr (MODE == 1) {
+  for (int v = 0; v < NV; ++v) my[(rec::EXT + v) * T32N] = rhs[v] + my[(rec::EXT + v) * T32N];
+#pragma unroll 1
+  for (int v0 = 0; v0 < NV; v0 += U32_VARS) {
+    const long long o0 = v0 * vs + p;
+    double kd[U32_VARS];
+    {
+      float kf[U32_VARS];
 #pragma unroll
-    for (int v = 0; v < NV; ++v) S.out[v * vs + p] = kd[v];
-  } else {
-    // every input of the update is read before any output is written:
-    // ynext may be y0, and the loads can then all be in flight at once
-    double y0r[NV], br[NV];
-#pragma unroll
-    for (int v = 0; v < NV; ++v) y0r[v] = __ldg(S.y0 + v * vs + p);
-    if (rk.method == 3) {
-#pragma unroll
-      for (int v = 0; v < NV; ++v) br[v] = __ldg(S.ys64 + v * vs + p);
-    } else if (rk.stage > 0) {
-#pragma unroll
-      for (int v = 0; v < NV; ++v) br[v] = S.acc[v * vs + p];
+      for (int v = 0; v < U32_VARS; ++v) kf[v] = my[(rec::EXT + v0 + v) * T32N];
+      f32_to_f64_vec<U32_VARS>(kf, kd);
     }
-    double yn[NV];
-    if (rk.method == 3) {
+    if constexpr (MODE == 1) {
 #pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        yn[v] = fma(rk.cdt, kd[v], fma(rk.a1, br[v], rk.a0 * y0r[v]));
-        S.out[v * vs + p] = yn[v];
-      }
+      for (int v = 0; v < U32_VARS; ++v) S.out[o0 + v * vs] = kd[v];
     } else {
+      // the inputs of these variables are read before their outputs are
+      // written: ynext may be y0, and the loads are in flight together
+      double y0r[U32_VARS], br[U32_VARS];
 #pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        const long long o = v * vs + p;
-        if (rk.stage == 0) {
-          S.acc[o] = rk.bdt * kd[v];
-          yn[v] = fma(rk.cdt, kd[v], y0r[v]);
-        } else if (rk.stage < 3) {
-          S.acc[o] = fma(rk.bdt, kd[v], br[v]);
-          yn[v] = fma(rk.cdt, kd[v], y0r[v]);
-        } else {
-          yn[v] = y0r[v] + fma(rk.bdt, kd[v], br[v]);
-        }
-        S.out[o] = yn[v];
+      for (int v = 0; v < U32_VARS; ++v) y0r[v] = __ldg(S.y0 + o0 + v * vs);
+      if (rk.method == 3) {
+#pragma unroll
+        for (int v = 0; v < U32_VARS; ++v) br[v] = __ldg(S.ys64 + o0 + v * vs);
+      } else if (rk.stage > 0) {
+#pragma unroll
+        for (int v = 0; v < U32_VARS; ++v) br[v] = S.acc[o0 + v * vs];
       }
-    }
-    if (S.out32) {
-      float y32[NV];
-      f64_to_f32_vec<NV>(yn, y32);
+      double yn[U32_VARS];
+      if (rk.method == 3) {
 #pragma unroll
-      for (int v = 0; v < NV; ++v) S.out32[v * L32.vs + q] = y32[v];
+        for (int v = 0; v < U32_VARS; ++v) {
+          yn[v] = fma(rk.cdt, kd[v], fma(rk.a1, br[v], rk.a0 * y0r[v]));
+          S.out[o0 + v * vs] = yn[v];
+        }
+      } else {
+#pragma unroll
+        for (int v = 0; v < U32_VARS; ++v) {
+          const long long o = o0 + v * vs;
+          if (rk.stage == 0) {
+            S.acc[o] = rk.bdt * kd[v];
+            yn[v] = fma(rk.cdt, kd[v], y0r[v]);
+          } else if (rk.stage < 3) {
+            S.acc[o] = fma(rk.bdt, kd[v], br[v]);
+            yn[v] = fma(rk.cdt, kd[v], y0r[v]);
+          } else {
+            yn[v] = y0r[v] + fma(rk.bdt, kd[v], br[v]);
+          }
+          S.out[o] = yn[v];
+        }
+      }
+      if (S.out32) {
+        float y32[U32_VARS];
+        f64_to_f32_vec<U32_VARS>(yn, y32);
+#pragma unroll
+        for (int v = 0; v < U32_VARS; ++v) S.out32[(v0 + v) * L32.vs + q] = y32[v];
+      }
     }
   }
   }
