@@ -23,8 +23,9 @@
 // instruction cache (the unrolled loop spent most of its stalls fetching
 // instructions). Each thread writes its results (the lean per-point set:
 // second derivatives of gt_ij and beta^i contracted with gt^ij as they are
-// produced) into its own column of a record in shared memory, and the
-// pointwise algebra reads the record back.
+// produced), the second derivatives in registers and the rest in its own
+// column of a record in shared memory, and the pointwise algebra reads the
+// record back.
 //
 // The y and z stencils of a variable run as the two lanes of packed
 // single-precision operations (sm_100's two-wide FMA, add and multiply, one
@@ -63,21 +64,26 @@ namespace bssn {
 
 // ---------------------------------------------------------------- tile
 constexpr int T32X = 8, T32Y = 4, T32Z = 4, T32N = T32X * T32Y * T32Z;
+// Four blocks on each SM: 128 registers a thread without spills, and 56 KB
+// of shared memory. For the latter the contracted second derivatives and
+// those of W and alpha stay in registers, 21 of a thread's 90 values (256^3
+// in 8th order 40.5 -> 39.0 ms per RK4 step against three blocks, 67 x 61 x 53
+// in 4th 726 -> 691 us).
 #ifndef T32_MIN_BLOCKS
-#define T32_MIN_BLOCKS 3
+#define T32_MIN_BLOCKS 4
 #endif
 // variable before whose stencils the update's operands are prefetched into
-// L2 (-1: before the variable loop). Two thirds of the way through the loop
+// L2 (-1: before the variable loop). Late in the loop
 // the lines arrive in time and are still there when the update reads them;
 // prefetched at the start, a 128^3 stage streams more than the L2 holds
 // before they are used (1.35 -> 1.28 ms per stage).
 #ifndef T32_PF_AT
-#define T32_PF_AT 16
+#define T32_PF_AT 20
 #endif
 // Two slots: a third bought nothing (the other blocks of the SM cover a
 // copy's latency) and took 7 to 10 KB per block from the L1 cache that the
 // centre values and the update go through (42.3 -> 40.5 ms per RK4 step of
-// 256^3 in 4th order).
+// 256^3 in 8th order).
 #ifndef T32_NBUF_DEF
 #define T32_NBUF_DEF 2
 #endif
@@ -91,6 +97,7 @@ constexpr int T32_NBUF = T32_NBUF_DEF;
 #endif
 constexpr int U32_VARS = U32_VARS_DEF;
 static_assert(NV % U32_VARS == 0, "whole groups");
+constexpr int T32_REC = 69;      // floats of a thread's record (namespace rec)
 constexpr int T32_NTAB = 2 * NM;  // D_x tables of the 11 mixed variables, then their D_y tables
 
 template <int P>
@@ -111,7 +118,7 @@ struct Tile32 {
   // empty barriers, the abort flag; 128 bytes of slack to align the ring
   static constexpr size_t RING = (size_t)T32_NBUF * SLOT * 4;
   // ring, record, full barriers, per-slot counters, abort flag, issued count
-  static constexpr size_t SMEM = 128 + RING + (size_t)90 * T32N * 4 + T32_NBUF * sizeof(uint64_t) +
+  static constexpr size_t SMEM = 128 + RING + (size_t)T32_REC * T32N * 4 + T32_NBUF * sizeof(uint64_t) +
                                  (T32_NBUF + 2) * sizeof(int) + 16;
   static_assert(N_X % 32 == 0 && N_Y % 32 == 0 && N_Z % 32 == 0 && N_TY % 32 == 0 && N_TZ % 32 == 0,
                 "TMA destinations must stay 128-byte aligned");
@@ -179,7 +186,7 @@ static __device__ unsigned int g_stage32_err;
 // derivatives are stored per variable as a triple (d = x, y, z) in the order
 // W, gt11..gt33, K, Gt1..Gt3, alpha, beta1..beta3.
 namespace rec {
-constexpr int EXT = 0, D1 = 24, DDW = 69, DDA = 75, LAPG = 81, LAPB = 87, N = 90;
+constexpr int EXT = 0, D1 = 24, N = T32_REC;
 }
 // first-derivative triple of variable v in the record, or -1
 __host__ __device__ constexpr int d1_slot(int v) {
@@ -311,6 +318,8 @@ __device__ __forceinline__ void stage32_tile(const Layout& L, const Layout32& L3
   constexpr int DY = T32X, DZ = T32X * T32Y;
   float* my = recb + t;
 
+  float ddW[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, dda[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  float lapg[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, lapb[3] = {0.f, 0.f, 0.f};
   float dddb[3] = {0.f, 0.f, 0.f};  // d_j d_k beta^k, summed as the shift components arrive
   bool ok = true;
   int consumed = 0;
@@ -435,20 +444,24 @@ __device__ __forceinline__ void stage32_tile(const Layout& L, const Layout32& L3
       for (int a = 2; a <= H; ++a) yz = fmaf(C.c1[2][a], TZY[tzi + a * DZ] - TZY[tzi - a * DZ], yz);
       const float d2s[6] = {d2v[0], xy, xz, d2v[1], yz, d2v[2]};
       if (m == 0 || m == 7) {
-        const int base = m == 0 ? rec::DDW : rec::DDA;
 #pragma unroll
-        for (int w = 0; w < 6; ++w) my[(base + w) * T32N] = d2s[w];
+        for (int w = 0; w < 6; ++w) {
+          ddW[w] = m == 0 ? d2s[w] : ddW[w];
+          dda[w] = d2s[w];  // alpha comes after W
+        }
       } else if (m <= 6) {
         float r = hgu[0] * d2s[0];
 #pragma unroll
         for (int w = 1; w < 6; ++w) r = fmaf(hgu[w], d2s[w], r);
-        my[(rec::LAPG + m - 1) * T32N] = r;
+#pragma unroll
+        for (int w = 0; w < 6; ++w) lapg[w] = m == w + 1 ? r : lapg[w];
       } else {
         const int ib = m - 8;  // beta^ib
         float r = gu2[0] * d2s[0];
 #pragma unroll
         for (int w = 1; w < 6; ++w) r = fmaf(gu2[w], d2s[w], r);
-        my[(rec::LAPB + ib) * T32N] = r;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) lapb[c] = ib == c ? r : lapb[c];
         // d_j d_ib beta^ib for j = x, y, z: packed pairs (j, ib)
         dddb[0] += ib == 0 ? d2s[0] : (ib == 1 ? d2s[1] : d2s[2]);
         dddb[1] += ib == 0 ? d2s[1] : (ib == 1 ? d2s[3] : d2s[4]);
@@ -491,13 +504,13 @@ __device__ __forceinline__ void stage32_tile(const Layout& L, const Layout32& L3
   }
 #pragma unroll
   for (int w = 0; w < 6; ++w) {
-    Q.ddW[w] = my[(rec::DDW + w) * T32N];
-    Q.dda[w] = my[(rec::DDA + w) * T32N];
-    Q.lapg[w] = my[(rec::LAPG + w) * T32N];
+    Q.ddW[w] = ddW[w];
+    Q.dda[w] = dda[w];
+    Q.lapg[w] = lapg[w];
   }
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    Q.lapb[c] = my[(rec::LAPB + c) * T32N];
+    Q.lapb[c] = lapb[c];
     Q.dddb[c] = dddb[c];
   }
   float rhs[NV];
