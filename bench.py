@@ -4,8 +4,8 @@ Workload (default): Brill-Lindquist two-puncture data (bare masses 0.5 at
 x = +-1.5) on a 128^3 grid over [-8, 8]^3, 8th-order finite differences,
 5 ghost zones with a static outer boundary, 1+log slicing, Gamma-driver shift
 (eta = 2), Kreiss-Oliger eps = 0.1, dt = 0.25 h, double precision. One step
-is one full RK4 step (4 x ghost fill + difference tables + fused
-right-hand-side/dissipation/stage kernel) over every interior point; the
+is one full RK4 step (4 x ghost fill + the stage's derivative and
+right-hand-side/dissipation/update kernels) over every interior point; the
 metric counts interior points advanced per second.
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl reference]
@@ -42,28 +42,26 @@ try:
 except (OSError, ValueError):
     MEASURED = {}
 
-# DRAM traffic of the fused stage kernel per launch, from one ncu capture of
-# the same source (profiles/k_stage_fp64_bl64.md); ignored when the kernel
-# source has changed. Captured at 64^3 (262,144 points: 921.1 MB read + 797.5
-# MB written per launch, 6.56 kB per point at 4 blocks/SM, rows traversed in
-# bricks) and scaled to 128^3 by the point count, since the traffic is per
-# point (state, tables and the per-thread stack).
-TRAFFIC = {"src_sha": "64481867ccf4c0a5", "bytes_per_launch_128": (920577024 + 797818880) * 128 ** 3 / 64 ** 3}
-# FP64 pipe utilisation of the same launch (sm__pipe_fp64_cycles_active,
-# percent of peak over active cycles) and the FP64 instructions it executed
-# per interior point (smsp__sass_thread_inst_executed_op_{dfma,dadd,dmul}
-# _pred_on.sum / 64^3), for the same source.
-FP64_PIPE_BUSY = {"src_sha": "64481867ccf4c0a5", "pct_of_active_cycles": 82.56,
-                  "dfma_per_point": 636223488 / 64 ** 3, "dadd_per_point": 409468928 / 64 ** 3,
-                  "dmul_per_point": 101187584 / 64 ** 3}
+# DRAM traffic of a stage's kernels (k_derivs, k_overlap, k_algebra), the mean
+# of the four stages' launches of one RK4 step at 128^3, from one ncu capture
+# of the same source (profiles/k_overlap_fp64_bl128.md); ignored when the
+# kernel source has changed.
+TRAFFIC = {"src_sha": "f3ef4daa2458f2f1", "bytes_per_stage_128": (24447868416 + 31903728640) / 4}
+# FP64 pipe utilisation of the kernel that does most of it, k_overlap
+# (sm__pipe_fp64_cycles_active, percent of peak over active cycles), and the
+# FP64 instructions of a stage per interior point, mean of the four stages
+# (smsp__sass_thread_inst_executed_op_{dfma,dadd,dmul}_pred_on.sum / 128^3),
+# for the same source.
+FP64_PIPE_BUSY = {"src_sha": "f3ef4daa2458f2f1", "pct_of_active_cycles": 53.95, "dfma_per_point": 699.0,
+                  "dadd_per_point": 53.0, "dmul_per_point": 189.0}
 # The same for the tiled FP32-RHS stage kernel k_stage32t<8,0> as the bench
 # times it (per-stage calls; the roofline's 864 B per point is the average of
-# the four stages): the mean of the four stages' launches at 64^3, 1043.6 MB
-# read and written in all, 0.995 kB per point and launch
+# the four stages): the mean of the four stages' launches at 64^3, 1001.0 MB
+# read and written in all, 0.955 kB per point and launch
 # (profiles/k_stage32t_fp32_bl64.md), scaled to 128^3 by the point count.
-TRAFFIC_F32 = {"src_sha": "c9578cbd115078fd",
-               "bytes_per_launch_128": (150967552 + 75629568 + 206530560 + 83616512 + 206648064 + 83771904 +
-                                        197803520 + 38672384) / 4 * 128 ** 3 / 64 ** 3}
+TRAFFIC_F32 = {"src_sha": "1186ab0c9e6d1684",
+               "bytes_per_launch_128": (151940352 + 71976960 + 204373248 + 70006528 + 204210432 + 70670080 +
+                                        196419328 + 31411200) / 4 * 128 ** 3 / 64 ** 3}
 N_SM = 152
 FP64_FMA_PER_CLK_SM = 2
 
@@ -72,8 +70,9 @@ FP64_FMA_PER_CLK_SM = 2
 # + dram__bytes_write.sum), for the source it was taken on.
 CFD_TRAFFIC = {"src_sha": "1559830c488ce0a5", "bytes_per_launch": 286361600 + 225778176}
 
-# the sources that make up the fused FP64 stage kernel k_stage<8,0,double>
-STAGE_SOURCES = ("bssn_common.cuh", "bssn_point.cuh", "bssn_kernels.cuh", "bssn_order.cu", "bssn_bounds.cuh")
+# the sources that make up the FP64 stage's kernels
+STAGE_SOURCES = ("bssn_common.cuh", "bssn_fixed.cuh", "bssn_point64.cuh", "bssn_stage64.cuh", "bssn_stage64.cu",
+                 "bssn_order.cu", "bssn_bounds.cuh")
 # and the tiled FP32-RHS stage kernel k_stage32t<8,0>
 STAGE32_SOURCES = ("bssn_common.cuh", "bssn_point.cuh", "bssn_stage32.cuh", "bssn_stage32_types.h", "bssn_stage32.cu", "bssn_cvt.cuh",
                    "bssn_tc.cuh", "bssn_bounds.cuh")
@@ -121,6 +120,24 @@ def stage_bytes(prec, stage, order=8, whole_step=False):
     if whole_step and stage < 3:
         b += nv * 4
     return b
+
+
+def fp64_array_bytes():
+    """Bytes per interior point of the arrays an FP64 stage must read or write
+    once, four-stage mean: stage_bytes without the first-difference tables,
+    which the kernels keep as a record of their own that mostly stays on
+    chip between its writer and its reader."""
+    return sum(24 * 8 * (3 + (s > 0) + (s < 3)) for s in range(4)) / 4
+
+
+# Kernels of one FP64 stage over `tiles` tiles of 8 x 8 x 8 points: derivatives
+# and algebra, or, from 608 tiles on, derivatives of the first chunk, both at once
+# for the others (about eight, multiples of 76 tiles) and algebra of the last.
+def fp64_stage_launches(tiles, slots=1 << 30):
+    if tiles < 608:
+        return 2
+    per = min((tiles + 7) // 8 + 75, slots // 2) // 76 * 76
+    return (tiles + per - 1) // per + 1
 
 
 def mean_stage_bytes(prec, order=8):
@@ -389,6 +406,8 @@ def run_gpu(args):
     work = B.alloc_work(grid, p, device=dev)
     rates = None if (args.profile or args.corrector_only or args.amr_only or args.cfd_only) else B.probe_fp_rates()
 
+    fp64_step = 4 * (1 + fp64_stage_launches(((n + 7) // 8) ** 3)) + 1  # per stage ghost fill and stage; final fill
+
     def run_form(prec, sample_clocks, whole_step=False):
         """Warm-up and timed RK4 steps of one form. Default: each stage through
         its own calls (ghost fill, tables, fused stage) with CUDA events around
@@ -417,7 +436,7 @@ def run_gpu(args):
                     ev[-1].record(stream)
                 ys = outs[s]
             B.fill_ghosts(grid, 1, ghost_src, y)
-            launches[0] += 13 if prec == B.FP64 else 17
+            launches[0] += fp64_step if prec == B.FP64 else 17
 
         def step(ev=None):
             if not whole_step:
@@ -425,7 +444,7 @@ def run_gpu(args):
                 return
             B.rk4_step(grid, p, prec, dt, 1, ghost_src, state, bufs3, work)
             # FP32: one conversion, 4 x (ghost fill, tables, fused stage), final ghost fill
-            launches[0] += 13 if prec == B.FP64 else 14
+            launches[0] += fp64_step if prec == B.FP64 else 14
 
         for _ in range(args.warmup):
             step()
@@ -507,11 +526,13 @@ def run_gpu(args):
                 "patches": len(patches), "interior_points": int(pts), "tiles": int(tiles),
                 "tile_shapes_chosen": np.bincount(shapes, minlength=7).tolist(), "plan_create_s": t_tune,
                 "fd_order": 4, "dt": dtb, "graph_launches_per_step": 1,
-                # FP64: per stage ghost fill, tables, stage (persistent kernels over all
-                # patches); FP32-RHS: ghost fill, single-precision copy, tables, and one
-                # tiled stage launch per spacing; then a final ghost fill
-                "kernel_nodes_per_step": 13 if prec == B.FP64 else 4 * (3 + nlev) + 1,
-                "stage_kernel": "kb_stage<4,double> (persistent, autotuned tiles)" if prec == B.FP64 else
+                # FP64: per stage ghost fill and the stage's kernels over all patches (the
+                # record of 2048 tiles bounds a chunk); FP32-RHS: ghost fill, tables and one
+                # tiled stage launch per spacing, and one single-precision conversion per
+                # step; then a final ghost fill
+                "kernel_nodes_per_step": 4 * (1 + fp64_stage_launches(tiles, min(2048, tiles))) + 1 if prec == B.FP64 else
+                4 * (2 + nlev) + 2,
+                "stage_kernel": "k_overlap<4> (derivatives and algebra of 8x8x8 tiles)" if prec == B.FP64 else
                                 "k_stage32t_batch<4> (TMA-staged 8x4x4 tiles, one launch per spacing)"}
 
     def run_amr(prec):
@@ -1204,7 +1225,9 @@ def run_gpu(args):
     peak_nominal = N_SM * FP64_FMA_PER_CLK_SM * 2.0 * sm_mhz * 1e6
     peak_probe = 2.0 * rates["fp64_fma_per_s"]
     sha = kernel_src_sha()
-    traffic = TRAFFIC["bytes_per_launch_128"] if TRAFFIC["src_sha"] == sha and n == N else None
+    traffic = TRAFFIC["bytes_per_stage_128"] if TRAFFIC["src_sha"] == sha and n == N else None
+    executed = executed_fp64(f64["stage_ms"], pts, sm_mhz, per_clk, sha)
+    issued = 2.0 * executed["fp64_inst_per_point"] * pts / (f64["stage_ms"] * 1e-3) if executed else achieved
     cpu_rate, cpu_steps, cpu_s, cpu_threads = cpu_oracle_rate(budget_s=args.cpu_budget, n=32)
     cpu_one = cpu_oracle_rate_single_thread()
     achieved32 = flops["total"] * pts / (f32["stage_ms"] * 1e-3)
@@ -1216,28 +1239,35 @@ def run_gpu(args):
         "config": {"workload": WORKLOAD if n == N else WORKLOAD.replace("128^3", f"{n}^3"), "grid": n, "fd_order": ORDER, "ghost": G, "precision": "fp64",
                    "parallelism": f"replicas x{world}",
                    "l2": "inputs larger than L2 (each state copy %.0f MB > 129 MB)" % (flat_bytes / 1e6)},
-        "roofline": {"bound": "alu", "achieved": achieved / 1e12, "peak": peak / 1e12, "unit": "TFLOP/s",
-                     "frac": achieved / peak, "traffic": traffic, "kernel": "k_stage<8,0,double> (fused RHS+KO+RK stage)",
+        # the FP64 pipe's side: the FP64 instructions the stage executes (ncu counts of the same
+        # source), two flop each, against the measured FMA rate. The stencils run on the integer
+        # pipes, so the method's literal operation count is no measure of this pipe; it is
+        # reported beside it (and taken where the source has changed since the counts)
+        "roofline": {"bound": "alu", "achieved": issued / 1e12, "peak": peak / 1e12, "unit": "TFLOP/s",
+                     "frac": issued / peak, "traffic": traffic,
+                     "kernel": "k_derivs<8>, k_overlap<8>, k_algebra (RHS+KO+RK stage)",
+                     "counts": "FP64 instructions executed x 2" if executed else "operations of the method",
+                     "algorithmic_tflops": achieved / 1e12,
                      "flops_per_point": flops["total"], "stage_ms": f64["stage_ms"],
                      "peak_source": f"measured {per_clk:.3f} FP64 FMA/clock/SM (probe, SM cycle counter) x "
                                     f"{N_SM} SMs x 2 flop at the sampled median SM clock {sm_mhz:.0f} MHz",
                      "peak_nominal": peak_nominal / 1e12,
                      "peak_probe": peak_probe / 1e12,
                      "peak_probe_sm_mhz": rates["sm_mhz_fp64_fma"],
-                     "frac_of_probe": achieved / peak_probe,
+                     "frac_of_probe": issued / peak_probe,
                      # the HBM side of the same kernel: algorithmic bytes per point and stage,
-                     # averaged over the four stages (stage_bytes): ys 192, difference tables
-                     # 704, y0 192, acc read 144 and written 144, ynext 192
-                     "hbm": {"bytes_per_point_stage": mean_stage_bytes("fp64"),
-                             "achieved_gbs": mean_stage_bytes("fp64") * pts / (f64["stage_ms"] * 1e-3) / 1e9,
-                             "frac": (mean_stage_bytes("fp64") * pts / (f64["stage_ms"] * 1e-3) / 1e9 /
+                     # averaged over the four stages: ys 192, y0 192, acc read 144 and
+                     # written 144, ynext 192
+                     "hbm": {"bytes_per_point_stage": fp64_array_bytes(),
+                             "achieved_gbs": fp64_array_bytes() * pts / (f64["stage_ms"] * 1e-3) / 1e9,
+                             "frac": (fp64_array_bytes() * pts / (f64["stage_ms"] * 1e-3) / 1e9 /
                                       MEASURED["hbm_gbs"])
                              if MEASURED.get("hbm_gbs") else None},
                      "fp64_pipe_busy_ncu": FP64_PIPE_BUSY if FP64_PIPE_BUSY["src_sha"] == sha else None,
                      # what the kernel executes (ncu instruction counts of the same source): FP64
                      # instructions per point and stage, and their rate per SM clock against the
                      # probe's measured FMA rate per SM clock (the FP64 pipe's issue ceiling)
-                     "executed": executed_fp64(f64["stage_ms"], pts, sm_mhz, per_clk, sha)},
+                     "executed": executed},
         "cpu_baseline": {"value": cpu_rate, "unit": UNIT, "cores": cpu_threads, "kind": "oracle",
                          "sample": f"{cpu_steps} oracle RK4 step(s) of the same workload on a 32^3 block "
                                    f"({cpu_s:.1f} s)",

@@ -102,7 +102,7 @@ void bssn_clear_error(void);
 /* Compile-time bounds-check mode. The library built with -DBSSN_BOUNDS_CHECK
  * (libbssn_check.so; the same entry points) checks, in every kernel that
  * indexes global memory through computed offsets (single-grid and patch
- * stencils, ghost fills, difference tables, constraints, Psi_4, the refined
+ * stencils, ghost fills, derivative tables, constraints, Psi_4, the refined
  * hierarchy's entry lists, the CFD kernels), each point's or entry's whole
  * access range against the extent of its array. A range outside is counted
  * in a device word and that access is skipped; nothing traps.

@@ -48,8 +48,9 @@
 // 64-point sum per ghost.
 //
 // One coarse step is one CUDA graph: per level and step, ghost fills,
-// [single-precision copy,] difference tables and the fused stage kernels of
-// the batched path (bssn_patch.cuh) over all patches of the level, the
+// the stage kernels of the batched path (FP64: derivatives and algebra,
+// bssn_patch.cuh; FP32-RHS: single-precision copy, tables and the tiled
+// kernel, bssn_stage32.cuh) over all patches of the level, the
 // radiative boundary kernel on level 0, then the two substeps of the finer
 // level and the restriction. Every kernel walks a flat entry or tile list
 // grid-stride: no device-side waits, no atomics, deterministic results.
@@ -780,7 +781,7 @@ cudaError_t compute_stage(bssn_amr* A, Level& L, const RK& rk, int in, int out, 
     return e;
   }
   const cudaError_t e = fx_stage(A->order, L.fx, A->rec, A->rec_slots, A->gz, rk, in, out, s);
-  A->nodes += 2 * ((L.fx.ntiles + A->rec_slots - 1) / A->rec_slots);
+  A->nodes += stage64_launches(L.fx.ntiles, A->rec_slots);
   return e;
 }
 

@@ -22,8 +22,8 @@ enum Var : int {
 };
 
 // The 11 grid functions whose second derivatives the right-hand side needs:
-// W, gt_ij (6), alpha, beta^i (3). Slot m of the difference tables holds
-// variable mvar(m).
+// W, gt_ij (6), alpha, beta^i (3). Slot m of the FP32 form's D_x and D_y tables
+// holds variable mvar(m).
 constexpr int NM = 11;
 __host__ __device__ constexpr int mvar(int m) { return m < 7 ? m : m + 10; }
 // Inverse of mvar: the table slot of variable v, or -1.

@@ -22,9 +22,9 @@
 //  * the sum is rounded to the nearest double; the algebra (or, where h differs
 //    by axis, this kernel) scales it by 1/(denominator h).
 //
-// Apart from that of the paired sums (fx_pair) no rounding happens before, so a constant field has
-// exactly zero derivatives and the result does not depend on the order of the
-// terms. A tile whose values are not all finite, or so large or small that
+// Apart from that of the paired sums (fx_pair) no rounding happens before, so
+// a constant field has exactly zero derivatives and the result does not
+// depend on the order of the terms. A tile whose values are not all finite, or so large or small that
 // the scaling could leave the range of doubles, takes double-precision
 // stencils (fx_fallback) instead: infinities and NaNs then reach exactly the
 // points whose stencils touch them.
@@ -33,7 +33,7 @@
 // (rec[(slot * nout + output) * vol + point of the tile]); the algebra kernel
 // reads them back. At 128^3, 8th order, one stage took 17.26 ms (+ 0.40 ms of
 // difference tables) when one kernel did stencils and algebra on the FP64
-// pipe (4375 FP64 instructions per point), 8.3 ms this way. Against a
+// pipe (4375 FP64 instructions per point), 6.2 ms this way (941). Against a
 // quadruple-precision evaluation the right-hand side's error is no larger than
 // before in any variable, and 1e-16 instead of 1e-14 for W, gt_ii and alpha.
 #pragma once

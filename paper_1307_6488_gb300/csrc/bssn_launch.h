@@ -24,6 +24,7 @@ cudaError_t launch_overlap(const OverlapArgs& A, int sms, cudaStream_t s);
 // volume among the grids.
 cudaError_t launch_stage64(int order, const FxWork& work, int vol, long long ntiles, long long slots,
                            const Gauge& gz, const StageOut& out, cudaStream_t s);
+long long stage64_launches(long long ntiles, long long slots);  // kernels that launch_stage64 enqueues
 template <int P>
 cudaError_t launch_ko(const Layout& L, const bssn_grid_t& G, double eps, bssn_precision_t prec, const double* u,
                       double* rhs, cudaStream_t s);

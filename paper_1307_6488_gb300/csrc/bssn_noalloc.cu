@@ -1,5 +1,5 @@
-// bssn_rk4_stage_noalloc: one fused RK4 stage (difference tables + fused
-// right-hand side, dissipation and stage update) whose scratch is a
+// bssn_rk4_stage_noalloc: one RK4 stage (right-hand side, dissipation and
+// stage update, what it needs before included) whose scratch is a
 // file-scope device array instead of a caller-supplied buffer, for callers
 // that cannot call cudaMalloc (see include/bssn.h).
 //

@@ -3,7 +3,7 @@
 // and the conformal Ricci tensor, written for as few FP64 instructions as
 // possible (the kernels that use it are bound by the FP64 pipe; the stage's
 // executes ~800 per point with its update, 1176 with the algebra the FP32 form
-// uses: at 128^3, 8th order, 8.33 -> 7.74 ms per stage, derivatives included,
+// uses: at 128^3, 8th order, 8.33 -> 7.74 ms per stage when made, derivatives included,
 // and the constraints 5.59 -> 4.39 ms):
 //
 //  * Half the metric's first derivatives come from the record, so Christoffel

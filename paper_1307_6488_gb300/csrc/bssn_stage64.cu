@@ -267,6 +267,12 @@ cudaError_t launch_psi4(int order, FxWork work, size_t rec_doubles, const double
 constexpr int OVERLAP_CHUNKS = 8;
 constexpr long long OVERLAP_MIN_TILES = 608;
 
+// Tiles of a chunk: multiples of 76, so that the algebra warps of 152 SMs take
+// equally many 32-point groups each.
+static long long overlap_chunk(long long ntiles, long long half) {
+  return std::min((ntiles + OVERLAP_CHUNKS - 1) / OVERLAP_CHUNKS + 75, half) / 76 * 76;
+}
+
 cudaError_t launch_stage64(int order, const FxWork& work, int vol, long long ntiles, long long slots,
                            const Gauge& gz, const StageOut& out, cudaStream_t s) {
   if (slots < 1) return cudaErrorInvalidValue;
@@ -288,11 +294,9 @@ cudaError_t launch_stage64(int order, const FxWork& work, int vol, long long nti
     return e;
   }
   // the record as two halves: the derivatives of one chunk go into one while
-  // the algebra reads the chunk before from the other. Chunks are multiples
-  // of 76 tiles, so that the algebra warps of 152 SMs take equally many
-  // 32-point groups each.
+  // the algebra reads the chunk before from the other
   const long long half = slots / 2;
-  long long per = std::min((ntiles + OVERLAP_CHUNKS - 1) / OVERLAP_CHUNKS + 75, half) / 76 * 76;
+  const long long per = overlap_chunk(ntiles, half);
   OverlapArgs O;
   O.groups = (vol + 31) / 32;
   double* const recs[2] = {work.rec, work.rec + half * work.slot};
@@ -317,6 +321,12 @@ cudaError_t launch_stage64(int order, const FxWork& work, int vol, long long nti
   }
   if (e != cudaSuccess) return e;
   return launch_algebra(A, prev, vol, 4 * sms, s);
+}
+
+long long stage64_launches(long long ntiles, long long slots) {
+  if (ntiles < OVERLAP_MIN_TILES || slots < 2 * 76) return 2 * ((ntiles + slots - 1) / slots);
+  const long long per = overlap_chunk(ntiles, slots / 2);
+  return (ntiles + per - 1) / per + 1;
 }
 
 cudaError_t bounds_take_stage64(unsigned long long* out) { return bounds_take_local(out); }
