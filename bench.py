@@ -68,7 +68,7 @@ FP64_FMA_PER_CLK_SM = 2
 
 # DRAM traffic of one k_cfd_mass_rb iteration at 256^3 (ncu dram__bytes_read.sum
 # + dram__bytes_write.sum), for the source it was taken on.
-CFD_TRAFFIC = {"src_sha": "29316462371b0522", "bytes_per_launch": 284790000 + 227070000}
+CFD_TRAFFIC = {"src_sha": "3ebb37ba50622be7", "bytes_per_launch": 284790000 + 227070000}
 
 # the sources that make up the FP64 stage's kernels
 STAGE_SOURCES = ("bssn_common.cuh", "bssn_fixed.cuh", "bssn_point64.cuh", "bssn_stage64.cuh", "bssn_stage64.cu",

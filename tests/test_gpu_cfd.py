@@ -219,3 +219,34 @@ def test_mass_iteration_equals_two_half_sweeps(case):
             lo = [slice(1, -1)] * 3
             lo[2 - ax] = 0
             assert torch.equal(got[tuple(lo)], want[tuple(lo)]), "uvw"[ax]
+
+
+@pytest.mark.parametrize("case", range(len(STEP_CASES)))
+def test_boundary_equals_axis_by_axis_fill(case):
+    """The one-launch boundary against the fill axis by axis (x, y, z, each over
+    the full padded extent of the others): every padded entry's bits, edges and
+    corners and the signs of zeros included."""
+    torch = need_gpu()
+    n, h, per, kw = STEP_CASES[case]
+    d = _desc(_flow(n, h, per, np.float32, **kw))
+    rng = np.random.default_rng(500 + case)
+    F = [rng.standard_normal((n[2] + 2, n[1] + 2, n[0] + 2)).astype(np.float32) for _ in range(4)]
+    dev = [torch.from_numpy(x).cuda().flatten() for x in F]
+    B.cfd_boundary(d, *dev)
+    torch.cuda.synchronize()
+    lid = np.float32(kw.get("lid", 0.0))
+    for a in range(3):
+        for f, x in enumerate(F):
+            x = np.moveaxis(x, 2 - a, 0)  # a view: padded index along a first
+            m = n[a]
+            if per[a]:
+                x[0], x[m + 1] = x[m].copy(), x[1].copy()
+            elif f == a:
+                x[0] = x[m] = x[m + 1] = 0.0
+            elif f == 3:
+                x[0], x[m + 1] = x[1], x[m]
+            else:
+                uw = lid if (a == 2 and f == 0) else np.float32(0)
+                x[0], x[m + 1] = -x[1], np.float32(2) * uw - x[m]
+    for got, want in zip(dev, F):
+        assert np.array_equal(got.cpu().numpy().view(np.uint32), want.ravel().view(np.uint32))
