@@ -138,9 +138,11 @@ bssn_status_t bssn_check_device(void* stream);
 bssn_status_t bssn_test_conversions(long long n, const double* din, const float* fin, float* f_bits, float* f_hw,
                                     double* d_bits, double* d_hw, void* stream);
 
-/* Bytes of scratch ("work") that bssn_rhs, bssn_rk4_stage and
- * bssn_constraints need for this grid, order and precision. Returns 0 and
- * sets *bytes to 0 for invalid arguments. */
+/* Bytes of scratch ("work") for bssn_rhs, bssn_rk4_stage, bssn_constraints
+ * and the other entry points that take it, for this grid, order and precision.
+ * On small FP64 grids this is more than they insist on: they accept the size
+ * of two single-precision copies and the derivative tables, and are faster
+ * with the rest. Returns 0 for invalid arguments. */
 unsigned long long bssn_work_bytes(const bssn_grid_t* grid, const bssn_params_t* params,
                                    bssn_precision_t prec);
 
@@ -208,8 +210,8 @@ bssn_status_t bssn_rk4_stage_fused(const bssn_grid_t* grid, const bssn_params_t*
  * and ynext.
  * Scratch: a file-scope device array of BSSN_NOALLOC_SCRATCH_BYTES, created on
  * each GPU where this entry point runs and held until the process exits. A
- * grid whose scratch need (bssn_work_bytes() for the same grid, params and
- * precision) exceeds it is rejected with BSSN_ERR_INVALID_ARG before anything
+ * grid whose least scratch (for the same grid, params and precision) exceeds
+ * it is rejected with BSSN_ERR_INVALID_ARG before anything
  * is launched. For example, at 8th order in FP64 n <= 35 interior points per
  * axis fit; at 4th order, n <= 51.
  * Set-up: the first call on a device looks up the array's device address

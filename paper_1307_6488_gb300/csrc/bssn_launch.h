@@ -24,6 +24,7 @@ cudaError_t launch_overlap(const OverlapArgs& A, int sms, cudaStream_t s);
 // volume among the grids.
 cudaError_t launch_stage64(int order, const FxWork& work, int vol, long long ntiles, long long slots,
                            const Gauge& gz, const StageOut& out, cudaStream_t s);
+long long stage64_slots(long long ntiles);  // record slots beyond which more would not be used
 long long stage64_launches(long long ntiles, long long slots);  // kernels that launch_stage64 enqueues
 template <int P>
 cudaError_t launch_ko(const Layout& L, const bssn_grid_t& G, double eps, bssn_precision_t prec, const double* u,
@@ -71,11 +72,12 @@ cudaError_t launch_to_f32t_batch(const Patch32* dev, const long long* pad0, int 
 template <int P>
 cudaError_t stage32_take_error(unsigned int* out);
 
-// bssn_api.cu: one fused RK4 stage (tables + fused kernel) on a scratch
-// buffer laid out like `work` (shared with the allocation-free entry point),
-// and the error latch of the C ABI.
-cudaError_t rk4_stage_on_work(void* work, const bssn_grid_t& G, const bssn_params_t& P, bssn_precision_t prec,
-                              int stage, double dt, const double* y0, const double* ys, double* acc, double* ynext,
+// bssn_api.cu: the least scratch the entry points accept, one RK4 stage on a
+// scratch buffer laid out like `work` (shared with the allocation-free entry
+// point), and the error latch of the C ABI.
+unsigned long long work_min_bytes(const bssn_grid_t& G, const bssn_params_t& P);
+cudaError_t rk4_stage_on_work(void* work, unsigned long long work_bytes, const bssn_grid_t& G,
+                              const bssn_params_t& P, bssn_precision_t prec, int stage, double dt, const double* y0, const double* ys, double* acc, double* ynext,
                               cudaStream_t s);
 bssn_status_t latch_cuda(cudaError_t e);
 // The argument rules every stepping entry point applies to a grid and its

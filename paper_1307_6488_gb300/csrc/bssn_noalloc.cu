@@ -55,9 +55,8 @@ extern "C" bssn_status_t bssn_rk4_stage_noalloc(const bssn_grid_t* grid, const b
                                                 const double* ys, double* acc, double* ynext, void* stream) {
   // Same argument rules as bssn_rk4_stage; bssn_work_bytes validates grid,
   // params and precision and returns 0 when any is invalid.
-  const unsigned long long need = bssn_work_bytes(grid, params, prec);
-  if (need == 0) return BSSN_ERR_INVALID_ARG;
-  if (need > BSSN_NOALLOC_SCRATCH_BYTES) return BSSN_ERR_INVALID_ARG;
+  if (bssn_work_bytes(grid, params, prec) == 0) return BSSN_ERR_INVALID_ARG;
+  if (work_min_bytes(*grid, *params) > BSSN_NOALLOC_SCRATCH_BYTES) return BSSN_ERR_INVALID_ARG;
   if (stage < 0 || stage > 3 || !std::isfinite(dt)) return BSSN_ERR_INVALID_ARG;
   if (!aligned16(y0) || !aligned16(ys) || !aligned16(acc) || !aligned16(ynext)) return BSSN_ERR_INVALID_ARG;
   if (ynext == ys || ynext == acc || acc == ys || acc == y0) return BSSN_ERR_INVALID_ARG;
@@ -67,6 +66,6 @@ extern "C" bssn_status_t bssn_rk4_stage_noalloc(const bssn_grid_t* grid, const b
   if (st != BSSN_OK) return st;
   // the scratch is laid out exactly like a caller's work buffer, so this is
   // bssn_rk4_stage's own code path
-  return latch_cuda(rk4_stage_on_work(scratch, *grid, *params, prec, stage, dt, y0, ys, acc, ynext,
+  return latch_cuda(rk4_stage_on_work(scratch, BSSN_NOALLOC_SCRATCH_BYTES, *grid, *params, prec, stage, dt, y0, ys, acc, ynext,
                                       (cudaStream_t)stream));
 }

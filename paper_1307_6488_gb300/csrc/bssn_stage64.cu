@@ -323,6 +323,10 @@ cudaError_t launch_stage64(int order, const FxWork& work, int vol, long long nti
   return launch_algebra(A, prev, vol, 4 * sms, s);
 }
 
+long long stage64_slots(long long ntiles) {
+  return ntiles < OVERLAP_MIN_TILES ? ntiles : 2 * overlap_chunk(ntiles, ntiles);
+}
+
 long long stage64_launches(long long ntiles, long long slots) {
   if (ntiles < OVERLAP_MIN_TILES || slots < 2 * 76) return 2 * ((ntiles + slots - 1) / slots);
   const long long per = overlap_chunk(ntiles, slots / 2);

@@ -98,3 +98,28 @@ def test_wide_range_within_a_tile(order):
     bound = 4 * 2.0 ** -58 * big * (16 / h ** 2 + 4 / h)
     scale = np.max(np.abs(want[:, far]), axis=1, keepdims=True)
     assert np.all(np.abs((got - want)[:, far]) <= bound + RHS_TOL * scale)
+
+
+# a scratch that holds some of the tiles at a time, and one that holds them
+# all: 27, 36 and 80 tiles also lie on both sides of the rule that divides the
+# algebra of 32 points between two warps
+@pytest.mark.parametrize("n", [(24, 24, 24), (32, 24, 23), (40, 32, 31)])
+@pytest.mark.parametrize("least", [False, True])
+def test_scratch_sizes(n, least):
+    torch = need_gpu()
+    g, p = 3, B.make_params(fd_order=4)
+    u = perturbed_bl(*n, g, 0.1, seed=7)
+    grid = grid_for(u, g, 0.1)
+    nb = B.work_bytes(grid, p, B.FP32_RHS if least else B.FP64)  # the FP32 form's is the least either accepts
+    assert nb <= B.work_bytes(grid, p, B.FP64)
+    y0 = B.upload(u, grid)
+    acc, out = B.alloc_state(grid), B.alloc_state(grid)
+    work = torch.empty(nb // 8, dtype=torch.float64, device="cuda")
+    B.rk4_stage(grid, p, B.FP64, 0, 6.0, y0, y0, acc, out, work)
+    torch.cuda.synchronize()
+    want = oracle.rhs(u, g, 0.1, oracle_params(p), ko=True)
+    err = rel_err(B.download(acc, grid), want, g)
+    assert np.max(err) < RHS_TOL, dict(zip(inputs.VARS, err))
+    if least:
+        with pytest.raises(Exception):
+            B.rk4_stage(grid, p, B.FP64, 0, 6.0, y0, y0, acc, out, work[:-1])
