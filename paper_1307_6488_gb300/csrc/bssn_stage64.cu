@@ -42,10 +42,18 @@ __global__ void __launch_bounds__(32) k_algebra_split(const __grid_constant__ Al
     algebra_point<PART_AT>(A.W, A.S, slot, idx);
 }
 
-// Algebra of n slots; few enough of them take two warps per 32 points.
+// Algebra of n slots, split where that is shorter: where whole warps would
+// leave schedulers without one (one RK4 step of 24^3 points, 27 tiles, 298 ->
+// 271 us; of 32 x 24 x 24, 36 tiles, 328 -> 332, so not there), and where the
+// schedulers' last whole warp is the only one of most of them (40 x 32 x 32, 80
+// tiles, 738 -> 658 us; 36^3 901 -> 831; with fewer than two warps each it does
+// not pay, 32 x 32 x 24 425 -> 433). A half takes about 0.55 of a warp's time.
 static cudaError_t launch_algebra(const AlgebraArgs& A, long long n, int vol, int schedulers, cudaStream_t s) {
   const int groups = (vol + 31) / 32;
-  if (2 * n * groups <= schedulers) {
+  const long long warps = n * groups;
+  auto rounds = [&](long long w) { return (w + schedulers - 1) / schedulers; };
+  if (2 * warps <= schedulers + schedulers / 2 ||
+      (warps > 2 * schedulers && 0.55 * rounds(2 * warps) < (double)rounds(warps))) {
     k_algebra_split<<<(unsigned int)(2 * n * groups), 32, 0, s>>>(A, groups);
   } else {
     const int bps = (vol + ALG_THREADS - 1) / ALG_THREADS;
