@@ -66,7 +66,8 @@ bool params_ok(const bssn_grid_t* G, const bssn_params_t* P) {
 //   [tables region][constraint partials][finals + flag]
 // The tables region is as large as 2 x 11 x p/2 arrays of var_stride doubles:
 // for BSSN_FP64 stages and the constraints it holds the derivative record (as
-// many tiles at a time as fit); for BSSN_FP32_RHS, two single
+// many tiles at a time as fit; a larger scratch widens it, work_ptrs); for
+// BSSN_FP32_RHS, two single
 // precision copies of the state (24 x var_stride floats each: a whole step
 // alternates between them) followed by the single precision tables.
 constexpr int RMS_BLOCKS = 304, RMS_THREADS = 256;

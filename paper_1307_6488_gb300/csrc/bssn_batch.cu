@@ -3,13 +3,13 @@
 // and Sec. 1.1; tile selection prior art, Sec. 2.6).
 //
 // A plan holds, for every patch, three stage buffers (and in the FP32-RHS
-// form a single-precision copy and derivative tables), device tables that
+// form two single-precision copies and derivative tables), device tables that
 // describe the patches, in FP64 the derivative record, and one CUDA graph per
 // step size. One RK4 step of all patches is one graph launch: four times
 // (static ghost fill, stage), then a final ghost fill. A stage is the single
 // grids' kernels over the tiles of all patches: k_derivs and k_algebra in
-// FP64 (bssn_stage64.cu), conversion, tables and k_stage32t_batch in the
-// FP32-RHS form. No device-side waiting between blocks, no atomics, and a
+// FP64 (bssn_stage64.cu), tables and k_stage32t_batch in the FP32-RHS form (the
+// first stage also converts the state). No device-side waiting between blocks, no atomics, and a
 // deterministic result; the per-point arithmetic is the single grids'.
 #include <cuda_runtime.h>
 

@@ -15,8 +15,7 @@
 //     three output planes it neighbours (k_conv_tc below);
 //   weight gradient ("wgrad") - M = 3 dz taps x 32 input channels (+ 32
 //     rows of ones: the bias), N = up to 3 dy x 32 output channels, K = points
-//     (one x-row per
-//     step). Both operands are the padded activations as they are stored:
+//     (one x-row per step). Both operands are padded arrays as they are stored:
 //     rows of points with 8 channels contiguous are an operand whose
 //     contiguous direction is M or N, which the tensor core takes. Each CTA
 //     streams a range of rows, keeps all 27 taps' sums in TMEM, and writes a
