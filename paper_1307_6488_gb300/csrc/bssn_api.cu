@@ -769,8 +769,9 @@ bssn_status_t constraints_impl(const bssn_grid_t* grid, const bssn_params_t* par
   const WorkPtrs w = work_ptrs(work, work_bytes, *grid, *params, BSSN_FP64);
   cudaError_t e = cudaMemsetAsync(w.flag, 0, sizeof(unsigned int), s);
   int nparts = 0;
+  const double h[3] = {grid->dx, grid->dy, grid->dz};
   if (e == cudaSuccess)
-    e = launch_constraints(params->fd_order, fx_work(params->fd_order, *grid, 0.0, state, w), w.rec_doubles, ham, mom,
+    e = launch_constraints(params->fd_order, fx_work(params->fd_order, *grid, 0.0, state, w), h, w.rec_doubles, ham, mom,
                            gcon, w.part, (long long)(w.part_doubles / 14), &nparts, w.flag, ham_only, s);
   if (e == cudaSuccess) {
     k_reduce_partials<<<1, 256, 0, s>>>(w.part, nparts, w.finals);

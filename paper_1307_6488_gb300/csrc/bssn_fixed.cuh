@@ -100,8 +100,8 @@ struct DerivList {
 // then the 24 advection + dissipation sums.
 constexpr int REC_K = 9 * NM, REC_GAM = REC_K + 3, REC_EXT = REC_GAM + 9, REC_RHS = REC_EXT + NV;
 
-// Constraints and Weyl scalars: W and gt (9 each), Gt^i (3 each) - all the
-// Hamiltonian constraint needs - then K (3) and At (3 each).
+// Hamiltonian constraint: W and gt (9 each), Gt^i (3 each). Weyl scalars: K (3)
+// and At (3 each) too.
 constexpr int REC_C_GAM = 9 * 7, REC_HAM = REC_C_GAM + 9, REC_C_K = REC_HAM, REC_C_AT = REC_C_K + 3,
               REC_CON = REC_C_AT + 18;
 

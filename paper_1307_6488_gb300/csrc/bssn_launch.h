@@ -33,9 +33,9 @@ cudaError_t launch_ko(const Layout& L, const bssn_grid_t& G, double eps, bssn_pr
 // sums and maxima per block in part (14 doubles each; *nparts of at most
 // max_parts are written), and the Weyl scalars. Single grids, through a record
 // of rec_doubles.
-cudaError_t launch_constraints(int order, FxWork work, size_t rec_doubles, double* ham, double* mom, double* gcon,
-                               double* part, long long max_parts, int* nparts, unsigned int* flag, bool ham_only,
-                               cudaStream_t s);
+cudaError_t launch_constraints(int order, FxWork work, const double h[3], size_t rec_doubles, double* ham, double* mom,
+                               double* gcon, double* part, long long max_parts, int* nparts, unsigned int* flag,
+                               bool ham_only, cudaStream_t s);
 cudaError_t launch_psi4(int order, FxWork work, size_t rec_doubles, const double origin[3], const double h[3],
                         double* psi_re, double* psi_im, double* inv_re, double* inv_im, double* E, double* B,
                         unsigned int* flag, cudaStream_t s);

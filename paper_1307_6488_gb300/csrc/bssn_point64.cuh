@@ -1,10 +1,11 @@
 // Pointwise algebra of the FP64 forms: the right-hand side of the BSSN system
-// (the equations at the head of bssn_point.cuh), the constraints' share of it
+// (the equations at the head of bssn_point.cuh), the Hamiltonian constraint
 // and the conformal Ricci tensor, written for as few FP64 instructions as
 // possible (the kernels that use it are bound by the FP64 pipe; the stage's
 // executes ~800 per point with its update, 1176 with the algebra the FP32 form
-// uses: at 128^3, 8th order, 8.33 -> 7.74 ms per stage when made, derivatives included,
-// and the constraints 5.59 -> 4.39 ms):
+// uses: at 128^3, 8th order, 8.33 -> 7.74 ms per stage when made, derivatives
+// included). The momentum and Gamma constraints have a form of their own
+// (momentum64).
 //
 //  * Half the metric's first derivatives come from the record, so Christoffel
 //    symbols of the first kind are sums of them, most of them a single one.
@@ -20,6 +21,7 @@
 //    gt^ij times one vector, Gt^k_ij times one vector).
 #pragma once
 #include "bssn_common.cuh"
+#include "bssn_point.cuh"
 
 namespace bssn {
 
@@ -278,15 +280,12 @@ __device__ __forceinline__ void rhs_point64(const Point64& P, const Gauge& gz, d
     rhs[V_ALPHA] = fma(-al * al, K, rhs[V_ALPHA]);
 }
 
-// Hamiltonian (out[0]) and, unless HONLY, momentum (1..3) and Gamma (4..6)
-// constraints at a point; dAt[d][s] = d_d At_s.
-template <bool HONLY>
-__device__ __forceinline__ void constraints64(const Point64& P, const double dAt[3][6], double a, double a2, double ia,
-                                              double out[7]) {
+// Hamiltonian constraint at a point.
+__device__ __forceinline__ double hamiltonian64(const Point64& P, double a2, double ia) {
   Conformal64 C;
   conformal64(P, ia, C);
   const double* A = P.u + V_AT11;
-  const double W = P.u[V_W], K = P.u[V_TRK], iW = 1.0 / W;
+  const double W = P.u[V_W], K = P.u[V_TRK];
   // gt^ij R_ij: the conformal part, and 4 gt^ij DtDt_ij W / W - 6 gt^ij d_i W d_j W / W^2
   double tr = C.gu2[0] * C.R[0], tw = C.gu2[0] * P.ddW[0], ww = 0.0;
 #pragma unroll
@@ -310,31 +309,95 @@ __device__ __forceinline__ void constraints64(const Point64& P, const double dAt
 #pragma unroll
     for (int j = 0; j < 3; ++j) AA = fma(Am[i][j], Am[j][i], AA);
   // W^2 R = W^2 tr + 4 W tw - 6 ww
-  out[0] = fma(a2, fma(W, fma(W, tr, 4.0 * tw), -6.0 * ww), fma((2.0 / 3.0) * K, K, -AA));
+  return fma(a2, fma(W, fma(W, tr, 4.0 * tw), -6.0 * ww), fma((2.0 / 3.0) * K, K, -AA));
+}
+
+// First derivative along a stride: sum_a c_a (u_a - u_-a).
+template <int H>
+__device__ __forceinline__ double d1_direct(const double* __restrict__ v, long long s, const double* c) {
+  double r = c[1] * (__ldg(v + s) - __ldg(v - s));
 #pragma unroll
-  for (int q = 1; q < 7; ++q) out[q] = 0.0;
-  if constexpr (!HONLY) {
-    // M_i = gt^jk (d_k At_ij - Gt^l_ki At_lj) - Gd^l At_il - 3/W At^j_i d_j W - 2/3 d_i K,
-    // gt^jk Gt^l_ki At_lj = Gt^l_ki At^k_l
+  for (int a = 2; a <= H; ++a) r = fma(c[a], __ldg(v + a * s) - __ldg(v - a * s), r);
+  return r;
+}
+
+// Momentum (out[0..2]) and Gamma (out[3..5]) constraints of the state u at a
+// point, c1 the first-derivative weights over the spacing. Where the
+// constraints hold they are what is left of terms that cancel: on a gauge wave
+// (A = 0.05, noise 1e-10) terms of order 1 leave 1e-8 to 1e-10, and
+// parts in 1e-9 to 1e-8 of the result are the rounding of whatever form is
+// evaluated. This form, stencils and expressions in double precision, is the
+// one that the constraints' values have always had, so they stay the same to
+// the last bit; from the derivative record, rounded once and gathered
+// differently, they were as close to a quadruple-precision evaluation but up
+// to 9e-9 of their norm apart from these. All constraints at 128^3, 8th order:
+// 12.0 ms with every stencil in double precision, 6.15 with these alone, 4.0
+// with none.
+template <int H>
+__device__ __forceinline__ void momentum64(const double* __restrict__ up, long long vs, const long long st[3],
+                                           const double (*c1)[5], double out[6]) {
+  double u[V_ALPHA], dW[3], dK[3], dg[3][6], dAt[3][6];
 #pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      double m = 0.0;
+  for (int v = 0; v < V_ALPHA; ++v) u[v] = __ldg(up + v * vs);
 #pragma unroll
-      for (int s = 0; s < 6; ++s) {
-        const int j = sym_i(s), k = sym_j(s);
-        m = fma(C.gu[s], j == k ? dAt[k][sym(i, j)] : dAt[k][sym(i, j)] + dAt[j][sym(i, k)], m);
-      }
+  for (int d = 0; d < 3; ++d) {
+    dW[d] = d1_direct<H>(up + V_W * vs, st[d], c1[d]);
+    dK[d] = d1_direct<H>(up + V_TRK * vs, st[d], c1[d]);
 #pragma unroll
-      for (int l = 0; l < 3; ++l) {
-        m = fma(-C.Gd[l], A[sym(i, l)], m);
-        m = fma(-3.0 * iW * Am[l][i], P.dW[l], m);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) m = fma(-C.GU[l][sym(k, i)], Am[k][l], m);
-      }
-      out[1 + i] = a * fma(-2.0 / 3.0, P.dK[i], m);
-      out[4 + i] = fma(-a, C.Gd[i], P.u[V_GAM1 + i]);
+    for (int s = 0; s < 6; ++s) {
+      dg[d][s] = d1_direct<H>(up + (V_GT11 + s) * vs, st[d], c1[d]);
+      dAt[d][s] = d1_direct<H>(up + (V_AT11 + s) * vs, st[d], c1[d]);
     }
   }
+  const double iW = 1.0 / u[V_W];
+  double gu[6], gu2[6], GL[3][6], GU[3][6], Gd[3];  // gt^ij, Gt_k,ij, Gt^k_ij, gt^ij Gt^k_ij
+  inverse_metric<double>(u + V_GT11, gu);
+#pragma unroll
+  for (int s = 0; s < 6; ++s) gu2[s] = (s == 1 || s == 2 || s == 4) ? gu[s] + gu[s] : gu[s];
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+#pragma unroll
+    for (int s = 0; s < 6; ++s) {
+      const int i = sym_i(s), j = sym_j(s);
+      GL[k][s] = 0.5 * (dg[i][sym(k, j)] + dg[j][sym(k, i)] - dg[k][s]);
+    }
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+#pragma unroll
+    for (int s = 0; s < 6; ++s)
+      GU[k][s] = gu[sym(k, 0)] * GL[0][s] + gu[sym(k, 1)] * GL[1][s] + gu[sym(k, 2)] * GL[2][s];
+    double t = gu2[0] * GU[k][0];
+#pragma unroll
+    for (int s = 1; s < 6; ++s) t += gu2[s] * GU[k][s];
+    Gd[k] = t;
+  }
+  const double* A = u + V_AT11;
+  double Am[3][3];  // At^i_j
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+      Am[i][j] = gu[sym(i, 0)] * A[sym(0, j)] + gu[sym(i, 1)] * A[sym(1, j)] + gu[sym(i, 2)] * A[sym(2, j)];
+  // M_i = gt^jk (d_k At_ij - Gt^l_ki At_lj - Gt^l_kj At_il) - 3/W At^j_i d_j W - 2/3 d_i K
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    double div = 0.0;
+#pragma unroll
+    for (int s = 0; s < 6; ++s) {  // twice the summand, symmetrised over (j, k)
+      const int j = sym_i(s), k = sym_j(s);
+      double t = dAt[k][sym(i, j)] + dAt[j][sym(i, k)];
+#pragma unroll
+      for (int l = 0; l < 3; ++l) {
+        t -= GU[l][sym(k, i)] * A[sym(l, j)] + GU[l][sym(k, j)] * A[sym(i, l)];
+        t -= GU[l][sym(j, i)] * A[sym(l, k)] + GU[l][sym(j, k)] * A[sym(i, l)];
+      }
+      div += gu2[s] * t;
+    }
+    const double aw = Am[0][i] * dW[0] + Am[1][i] * dW[1] + Am[2][i] * dW[2];
+    out[i] = 0.5 * div - 3.0 * iW * aw - (2.0 / 3.0) * dK[i];
+  }
+#pragma unroll
+  for (int i = 0; i < 3; ++i) out[3 + i] = u[V_GAM1 + i] - Gd[i];
 }
 
 }  // namespace bssn

@@ -62,22 +62,17 @@ static cudaError_t launch_algebra(const AlgebraArgs& A, long long n, int vol, in
   return cudaGetLastError();
 }
 
-// The set of the constraints and Weyl scalars at one point.
-template <bool HONLY>
-__device__ __forceinline__ void load_con(const double* __restrict__ rec, int vol, const double* __restrict__ u,
-                                         long long vs, Point64& Q, double dAt[3][6]) {
+// The set of the Hamiltonian constraint at one point.
+__device__ __forceinline__ void load_ham(const double* __restrict__ rec, int vol, const double* __restrict__ u,
+                                         long long vs, Point64& Q) {
   auto r = [&](int o) { return __ldg(rec + o * vol); };
 #pragma unroll
   for (int v = 0; v < NV; ++v) Q.u[v] = __ldg(u + v * vs);
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     Q.dW[d] = r(d);
-    Q.dK[d] = HONLY ? 0.0 : r(REC_C_K + d);
 #pragma unroll
-    for (int s = 0; s < 6; ++s) {
-      Q.hg[d][s] = r(9 * (1 + s) + d);
-      dAt[d][s] = HONLY ? 0.0 : r(REC_C_AT + 3 * s + d);
-    }
+    for (int s = 0; s < 6; ++s) Q.hg[d][s] = r(9 * (1 + s) + d);
 #pragma unroll
     for (int c = 0; c < 3; ++c) Q.hG[d][c] = r(REC_C_GAM + 3 * c + d);
   }
@@ -89,20 +84,35 @@ __device__ __forceinline__ void load_con(const double* __restrict__ rec, int vol
   }
 }
 
+// And of the Weyl scalars, which take the derivatives of K and At_ij too.
+__device__ __forceinline__ void load_weyl(const double* __restrict__ rec, int vol, const double* __restrict__ u,
+                                          long long vs, Point64& Q, double dAt[3][6]) {
+  load_ham(rec, vol, u, vs, Q);
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    Q.dK[d] = __ldg(rec + (REC_C_K + d) * vol);
+#pragma unroll
+    for (int s = 0; s < 6; ++s) dAt[d][s] = __ldg(rec + (REC_C_AT + 3 * s + d) * vol);
+  }
+}
+
 struct ConArgs {
   FxWork W;
   double *ham, *mom, *gcon, *part;
   unsigned int* flag;
+  double c1[3][5];  // first-derivative weights over the spacing
 };
 
 // Constraints of the points of `nblocks` blocks of CON_THREADS points
 // (blocks_per_slot to a slot), grid-stride. Per-block partial results, 7 sums
 // of squares and 7 maxima, are added to part[blockIdx.x * 14 + q] (written by
 // the first chunk), so that one small array serves any number of tiles in a
-// fixed order. With HONLY the Hamiltonian constraint alone (the momentum and
+// fixed order. H = 0: the Hamiltonian constraint alone (the momentum and
 // Gamma slots stay 0); its values are the same bits as in the full evaluation.
-// Bound by the FP64 pipe (128 registers and 4 blocks an SM, as the algebra).
-template <bool HONLY>
+// H = p/2: the momentum and Gamma constraints too, from the state itself
+// (momentum64). Bound by the FP64 pipe (128 registers and 4 blocks an SM, as
+// the algebra).
+template <int H>
 __global__ void __launch_bounds__(CON_THREADS, 4) k_constraints(const __grid_constant__ ConArgs A, unsigned int nblocks,
                                                                int blocks_per_slot, bool first) {
   double sum[7], top[7];
@@ -117,23 +127,32 @@ __global__ void __launch_bounds__(CON_THREADS, 4) k_constraints(const __grid_con
     TilePoint pt;
     if (!tile_point(G, ti, tj, tk, idx, pt)) continue;
     const long long p = pt.p, vs = G.L.vs;
-    Point64 Q;
-    double dAt[3][6], c[7];
-    load_con<HONLY>(A.W.rec + (long long)slot * A.W.slot + idx, G.T.vol, G.buf[1] + p, vs, Q, dAt);
-    constraints64<HONLY>(Q, dAt, G.C.a, G.C.a2, G.C.ia, c);
-    if (A.ham) A.ham[p] = c[0];
-    if (A.mom && !HONLY)
+    const double* __restrict__ u = G.buf[1] + p;
+    double c[7];
+    if constexpr (H > 0) {
+      if (!in_range(p - H * G.L.sz, p + H * G.L.sz, padded_points(G.L))) continue;
+      const long long st[3] = {1, G.L.sy, G.L.sz};
+      momentum64<H>(u, vs, st, A.c1, c + 1);
+      if (A.mom)
 #pragma unroll
-      for (int a = 0; a < 3; ++a) A.mom[a * vs + p] = c[1 + a];
-    if (A.gcon && !HONLY)
+        for (int a = 0; a < 3; ++a) A.mom[a * vs + p] = c[1 + a];
+      if (A.gcon)
 #pragma unroll
-      for (int a = 0; a < 3; ++a) A.gcon[a * vs + p] = c[4 + a];
+        for (int a = 0; a < 3; ++a) A.gcon[a * vs + p] = c[4 + a];
 #pragma unroll
-    for (int q = 0; q < 7; ++q) {
-      bad |= !isfinite(c[q]);
-      sum[q] += c[q] * c[q];
-      top[q] = fmax(top[q], fabs(c[q]));  // a NaN is left out here and reported by the flag
+      for (int q = 1; q < 7; ++q) {
+        bad |= !isfinite(c[q]);
+        sum[q] += c[q] * c[q];
+        top[q] = fmax(top[q], fabs(c[q]));  // a NaN is left out here and reported by the flag
+      }
     }
+    Point64 Q;
+    load_ham(A.W.rec + (long long)slot * A.W.slot + idx, G.T.vol, u, vs, Q);
+    c[0] = hamiltonian64(Q, G.C.a2, G.C.ia);
+    if (A.ham) A.ham[p] = c[0];
+    bad |= !isfinite(c[0]);
+    sum[0] += c[0] * c[0];
+    top[0] = fmax(top[0], fabs(c[0]));
     bad |= !(Q.u[V_W] > 0.0);  // the conformal factor must stay positive
   }
   if (bad) atomicOr(A.flag, 1u);
@@ -181,7 +200,7 @@ __global__ void __launch_bounds__(CON_THREADS, 4) k_psi4(const __grid_constant__
   const long long p = pt.p, vs = G.L.vs;
   Point64 Q;
   double dAt[3][6];
-  load_con<false>(A.W.rec + (long long)slot * A.W.slot + idx, G.T.vol, G.buf[1] + p, vs, Q, dAt);
+  load_weyl(A.W.rec + (long long)slot * A.W.slot + idx, G.T.vol, G.buf[1] + p, vs, Q, dAt);
   // Weyl scalars take the derivatives' values
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
@@ -240,13 +259,15 @@ static cudaError_t through_record(int order, const FxWork& work, const DerivList
   return cudaSuccess;
 }
 
-cudaError_t launch_constraints(int order, FxWork work, size_t rec_doubles, double* ham, double* mom, double* gcon,
-                               double* part, long long max_parts, int* nparts, unsigned int* flag, bool ham_only,
-                               cudaStream_t s) {
-  ConArgs A{work, ham, mom, gcon, part, flag};
+cudaError_t launch_constraints(int order, FxWork work, const double h[3], size_t rec_doubles, double* ham, double* mom,
+                               double* gcon, double* part, long long max_parts, int* nparts, unsigned int* flag,
+                               bool ham_only, cudaStream_t s) {
+  ConArgs A{work, ham, mom, gcon, part, flag, {}};
+  for (int d = 0; d < 3; ++d)
+    for (int a = 1; a <= order / 2; ++a) A.c1[d][a] = (order == 4 ? FD<4>::W1[a] : FD<8>::W1[a]) / h[d];
   const int bps = (work.one.T.vol + CON_THREADS - 1) / CON_THREADS;
   *nparts = 0;
-  return through_record(order, work, con_list(ham_only), rec_doubles, s, [&](const FxWork& W, long long n, bool first) {
+  return through_record(order, work, con_list(true), rec_doubles, s, [&](const FxWork& W, long long n, bool first) {
     A.W = W;
     // as many blocks as are resident (4 on each of 152 SMs): each takes the
     // points of several tiles, and the partial sums stay few
@@ -254,9 +275,11 @@ cudaError_t launch_constraints(int order, FxWork work, size_t rec_doubles, doubl
     if (first) *nparts = (int)std::min<long long>(std::min<long long>(nb, max_parts), 608);
     const unsigned int g = (unsigned int)*nparts;  // the last chunk may be smaller: idle blocks add nothing
     if (ham_only)
-      k_constraints<true><<<g, CON_THREADS, 0, s>>>(A, nb, bps, first);
+      k_constraints<0><<<g, CON_THREADS, 0, s>>>(A, nb, bps, first);
+    else if (order == 4)
+      k_constraints<2><<<g, CON_THREADS, 0, s>>>(A, nb, bps, first);
     else
-      k_constraints<false><<<g, CON_THREADS, 0, s>>>(A, nb, bps, first);
+      k_constraints<4><<<g, CON_THREADS, 0, s>>>(A, nb, bps, first);
   });
 }
 
