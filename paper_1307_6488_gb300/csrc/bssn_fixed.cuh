@@ -6,12 +6,23 @@
 // fixed point, and rounded to double once:
 //
 //  * one block takes one variable on one tile of 8 x 8 x 8 interior points
-//    with its halo. E is the largest exponent among the values the tile's
-//    stencils read, and every value becomes the integer
+//    with its halo. 2^E is the power of two above the largest value of the
+//    tile and its halo, and every value becomes the integer
 //    n = trunc(u 2^(59-E)), |n| < 2^59: six bits more than a double's
-//    significand has. Values of at least 2^-6 of the tile's largest are held
-//    exactly, smaller ones to 2^-59 of the largest (the rounding error a
-//    double-precision stencil makes on the largest itself is 2^-53).
+//    significand has. Values within 2^-6 of 2^E are held exactly, smaller ones
+//    to 2^(E-59).
+//  * a derivative is taken from these integers only where they are no coarser
+//    than the rounding of a double-precision stencil: where some value that its
+//    own stencil reads is at least 2^(E-7), so that 2^(E-59) is no more than that
+//    value's last bit (which a difference of two such values is rounded to). The
+//    others (of points beside a spike or a steep front of the tile, or along a
+//    line or in a plane on which the variable is nearly zero: some 0.05 % of
+//    the points of puncture data) are made from the doubles (fx_fallback), and
+//    so are all of a tile whose values are not all finite, or so large or small
+//    that the scaling could leave the range of doubles: infinities and NaNs
+//    then reach exactly the points whose stencils touch them. What a derivative
+//    is good to depends on what its stencil reads, and not on what else its
+//    tile holds.
 //  * n is kept as two limbs, n = hi 2^30 + lo with 0 <= lo < 2^30, so that
 //    differences a - b and paired sums a + b - 2c of limbs fit 32 bits and a
 //    weighted sum is one 32 x 32 + 64 bit multiply-add per limb. The weights
@@ -24,10 +35,7 @@
 //
 // Apart from that of the paired sums (fx_pair) no rounding happens before, so
 // a constant field has exactly zero derivatives and the result does not
-// depend on the order of the terms. A tile whose values are not all finite, or so large or small that
-// the scaling could leave the range of doubles, takes double-precision
-// stencils (fx_fallback) instead: infinities and NaNs then reach exactly the
-// points whose stencils touch them.
+// depend on the order of the terms.
 //
 // k_derivs writes the derivatives to a record, one slot per tile
 // (rec[(slot * nout + output) * vol + point of the tile]); the algebra kernel
@@ -36,6 +44,8 @@
 // pipe (4375 FP64 instructions per point), 6.2 ms this way (941). Against a
 // quadruple-precision evaluation the right-hand side's error is no larger than
 // before in any variable, and 1e-16 instead of 1e-14 for W, gt_ii and alpha.
+// Looking after coarse derivatives costs 2 % of a step at 128^3, 6 % of a small
+// hierarchy's, whose launches end with the slowest tile.
 #pragma once
 #include <type_traits>
 
@@ -82,7 +92,7 @@ struct DerivList {
   short d1[NV];   // first of 3 outputs (x, y, z), or -1
   short d2[NV];   // first of 6 outputs (xx, xy, xz, yy, yz, zz), or -1
   short ext[NV];  // advection + dissipation, or -1
-  signed char s1[NV], s2[NV];  // binary exponents added to the first and second derivatives
+  signed char s1[NV], s2[NV];  // binary exponents added to the first and second derivatives (0 or -1)
 
   void add(int v, int o1, int o2, int oe) {
     const bool gt = v >= V_GT11 && v <= V_GT33, gam = v >= V_GAM1 && v <= V_GAM3;
@@ -143,6 +153,7 @@ struct FxCoef {
   double a, a2;  // what the algebra multiplies first and second derivatives by
   double ia;     // 1 / a
   int cubic;
+  int weak;      // little or no dissipation
 };
 
 template <int P>
@@ -160,6 +171,7 @@ FxCoef make_fx(const bssn_grid_t& G, double eps) {
     C.c2[s] = 1.0 / ((double)X::D1 * X::D1 * h[i] * h[j]);
   }
   C.cubic = G.dx == G.dy && G.dy == G.dz;
+  C.weak = eps < 0.05;
   C.a = C.cubic ? C.c1[0] : 1.0;
   C.a2 = C.cubic ? C.c2[0] : 1.0;
   C.ia = C.cubic ? X::D1 * h[0] : 1.0;
@@ -197,6 +209,7 @@ __device__ __forceinline__ unsigned long long fx_shl(unsigned long long x, int n
 
 constexpr int FX_LIMB = 30;
 constexpr unsigned int FX_MASK = (1u << FX_LIMB) - 1;
+constexpr int FX_HELD = 1 << 22;  // high limb of a value of 2^(E-7)
 
 // limbs (lo, hi) of trunc(u 2^(1081 - emax)), emax the largest biased exponent
 __device__ __forceinline__ int2 fx_from_double(double u, int emax) {
@@ -252,59 +265,98 @@ __device__ __forceinline__ double fx_to_double(long long hi, long long lo, int e
 }
 
 // ------------------------------------------------------------------ double-precision stencils
-// One point of a tile that fixed point does not hold. v: the variable, p:
-// the point; writes the same outputs.
+// Which derivatives of a point: the first and second along axis d (FX_AXIS << d),
+// the mixed ones (FX_MIXED for xy, then xz, yz), the axis' share of advection
+// and dissipation (FX_EXT << d).
+constexpr int FX_AXIS = 1, FX_MIXED = 8, FX_EXT = 64, FX_ALL = 511;
+
+// The derivatives `which` of a point that fixed point does not hold. v: the
+// variable, p: the point; has1, has2, hase: which of them the variable's record
+// has, half1 and half2: whether it has half the first and second ones. oe holds
+// the sum of the other axes unless `which` is FX_ALL. beta: the shift's first
+// component at the point, the others vs apart. Each axis' values are
+// loaded before any is used: what these points cost is mostly that latency.
 template <int P>
 __device__ __noinline__ void fx_fallback(const double* __restrict__ v, long long p, long long sy, long long sz,
-                                         const FxCoef& C, const double* beta, bool adv, bool want1,
-                                         bool want2, bool wante, double* o1, double* o2, double* oe) {
+                                         const FxCoef& C, const double* __restrict__ beta, long long vs, bool adv,
+                                         int which, bool has1, bool has2, bool hase, bool half1, bool half2,
+                                         double* __restrict__ o1, double* __restrict__ o2, double* __restrict__ oe,
+                                         int vol) {
   using F = FD<P>;
   using X = FX<P>;
   constexpr int H = F::H, R = F::R;
-  const long long st[3] = {1, sy, sz};
-  const double m2 = -2.0 * v[p];
-  double ext = 0.0;
+  const double f1 = half1 ? 0.5 : 1.0, f2 = half2 ? 0.5 : 1.0;
+  v += p;
+  const double u0 = v[0], m2 = -2.0 * u0;
+  const bool wante = hase && which >= FX_EXT;
+  double ext = wante && which != FX_ALL ? *oe : 0.0;
+#pragma unroll 1
   for (int d = 0; d < 3; ++d) {
-    double r1 = 0.0, r2 = 0.0, k = 0.0;
+    const bool axis = which & (FX_AXIS << d), share = hase && (which & (FX_EXT << d));
+    if (!axis && !share) continue;
+    const long long st = d == 0 ? 1 : (d == 1 ? sy : sz);
+    double up[R + 1], um[R + 1];
+#pragma unroll
     for (int a = 1; a <= R; ++a) {
-      const double up = v[p + a * st[d]], um = v[p - a * st[d]];
-      const double df = up - um, s = (up + um) + m2;
-      if (a <= H) {
-        r1 += X::W1(a) * df;
-        r2 += X::W2(a) * s;
+      up[a] = um[a] = 0.0;
+      if (a <= H || share) {
+        up[a] = v[a * st];
+        um[a] = v[-a * st];
       }
-      k += X::WK(a) * s;
     }
-    if (want1) o1[d] = C.cubic ? r1 : C.c1[d] * r1;
-    if (want2) o2[sym(d, d)] = C.cubic ? r2 : C.c2[sym(d, d)] * r2;
-    if (wante) {
-      // the one-sided stencil the sign of beta selects, and no other point
-      const long long ss = beta[d] < 0.0 ? -st[d] : st[d];
-      double t = 0.0;
-      for (int i = 0; i < F::UPN; ++i) {
-        const int o = F::UPLO + i;
-        int w = 0;
-        if (o == 0)
-          for (int a = 1; a <= R; ++a) w -= 2 * X::SK * X::WK(a);
-        else
-          w = X::SK * X::WK(abs(o)) + (o > 0 ? X::WT(o) : -X::WT(-o));
-        t += w * v[p + o * ss];
+    if (axis) {
+      double r1 = 0.0, r2 = 0.0;
+#pragma unroll
+      for (int a = 1; a <= H; ++a) {
+        r1 += X::W1(a) * (up[a] - um[a]);
+        if (has2) r2 += X::W2(a) * ((up[a] + um[a]) + m2);
       }
-      ext += C.ck[d] * k + (adv ? C.cu[d] * fabs(beta[d]) * t : 0.0);
+      if (has1) o1[d * vol] = f1 * (C.cubic ? r1 : C.c1[d] * r1);
+      if (has2) o2[sym(d, d) * vol] = f2 * (C.cubic ? r2 : C.c2[sym(d, d)] * r2);
+    }
+    if (share) {
+      double k = 0.0;
+#pragma unroll
+      for (int a = 1; a <= R; ++a) k += X::WK(a) * ((up[a] + um[a]) + m2);
+      ext += C.ck[d] * k;
+      if (adv) {
+        // the one-sided stencil the sign of beta selects, and no other point
+        const double bd = beta[d * vs];
+        const bool neg = bd < 0.0;
+        double t = 0.0;
+#pragma unroll
+        for (int i = 0; i < F::UPN; ++i) {
+          const int o = F::UPLO + i, b = o < 0 ? -o : o;
+          int w = 0;
+          if (o == 0)
+            for (int a = 1; a <= R; ++a) w -= 2 * X::SK * X::WK(a);
+          else
+            w = X::SK * X::WK(b) + (o > 0 ? X::WT(o) : -X::WT(-o));
+          t += w * (o == 0 ? u0 : ((o < 0) != neg ? um[b] : up[b]));
+        }
+        ext += C.cu[d] * fabs(bd) * t;
+      }
     }
   }
   if (wante) *oe = ext;
-  if (!want2) return;
-  for (int i = 0; i < 3; ++i)
-    for (int j = i + 1; j < 3; ++j) {
-      double r = 0.0;
-      for (int a = 1; a <= H; ++a)
-        for (int b = 1; b <= H; ++b) {
-          const long long A = a * st[i], B = b * st[j];
-          r += (double)(X::W1(a) * X::W1(b)) * ((v[p + A + B] - v[p - A + B]) - (v[p + A - B] - v[p - A - B]));
-        }
-      o2[sym(i, j)] = C.cubic ? r : C.c2[sym(i, j)] * r;
+  if (!has2) return;
+  int pair = FX_MIXED;
+#pragma unroll 1
+  for (int q = 0; q < 3; ++q, pair <<= 1) {
+    if (!(which & pair)) continue;
+    const long long si = q < 2 ? 1 : sy, sj = q == 0 ? sy : sz;
+    double r = 0.0;
+#pragma unroll 1
+    for (int a = 1; a <= H; ++a) {
+      const double *vp = v + a * si, *vm = v - a * si;
+      double t = 0.0;
+#pragma unroll
+      for (int b = 1; b <= H; ++b) t += X::W1(b) * ((vp[b * sj] - vm[b * sj]) - (vp[-b * sj] - vm[-b * sj]));
+      r += X::W1(a) * t;
     }
+    const int c = q == 2 ? 4 : q + 1;  // packed xy, xz, yz
+    o2[c * vol] = f2 * (C.cubic ? r : C.c2[c] * r);
+  }
 }
 
 // ------------------------------------------------------------------ one tile of one variable
@@ -318,43 +370,71 @@ struct FxSmem {
   static constexpr size_t bytes = sizeof(int2) * BOX + 3 * sizeof(int4) * GN;
 };
 
-// three limbs of sum_a W1[a] (n_a - n_-a) along stride st
+// three limbs of sum_a W1[a] (n_a - n_-a) along stride st, and the largest
+// magnitude (high limb) among the n
 template <int P>
 __device__ __forceinline__ int4 fx_first(const int2* __restrict__ b, int st) {
   long long lo = 0, hi = 0;
+  int top = 0, low = 0;
 #pragma unroll
   for (int a = 1; a <= FD<P>::H; ++a) {
     const int2 p = b[a * st], m = b[-a * st];
     lo += (long long)FX<P>::W1(a) * (p.x - m.x);
     hi += (long long)FX<P>::W1(a) * (p.y - m.y);
+    top = __vimax3_s32(top, p.y, m.y);
+    low = __vimin3_s32(low, p.y, m.y);
   }
   hi += lo >> FX_LIMB;
-  return make_int4((int)((unsigned int)lo & FX_MASK), (int)((unsigned int)hi & FX_MASK), (int)(hi >> FX_LIMB), 0);
+  return make_int4((int)((unsigned int)lo & FX_MASK), (int)((unsigned int)hi & FX_MASK), (int)(hi >> FX_LIMB),
+                   max(top, ~low));
 }
 
-// the first-derivative weights along stride st of a table of such sums
+// the first-derivative weights along stride st of a table of such sums, and
+// the largest magnitude among the values they are made of
 template <int P>
-__device__ __forceinline__ double fx_mixed(const int4* __restrict__ g, int st, int emax) {
+__device__ __forceinline__ double fx_mixed(const int4* __restrict__ g, int st, int emax, int& mag) {
   long long l0 = 0, l1 = 0;
   int l2 = 0;
+  mag = 0;
 #pragma unroll
   for (int b = 1; b <= FD<P>::H; ++b) {
     const int4 p = g[b * st], m = g[-b * st];
     l0 += (long long)FX<P>::W1(b) * (p.x - m.x);
     l1 += (long long)FX<P>::W1(b) * (p.y - m.y);
     l2 += FX<P>::W1(b) * (p.z - m.z);
+    mag = __vimax3_s32(mag, p.w, m.w);
   }
   l1 += l0 >> FX_LIMB;
   const long long hi = ((long long)(l2 + (int)(l1 >> FX_LIMB)) << FX_LIMB) | (l1 & (long long)FX_MASK);
   return fx_to_double(hi, l0 & (long long)FX_MASK, emax);
 }
 
+// Whether some value that the upwinded stencil along st reads is as large as FX_HELD.
+template <int P>
+__device__ __noinline__ bool fx_upwind_held(const int2* __restrict__ c, int st) {
+  int top = 0, low = 0;
+#pragma unroll
+  for (int i = 0; i < FD<P>::UPN; ++i) {
+    const int v = c[(FD<P>::UPLO + i) * st].y;
+    top = max(top, v);
+    low = min(low, v);
+  }
+  return max(top, ~low) >= FX_HELD;
+}
+
 // Stencils along the three axes at one point of the box, and the outputs.
+// Returns those that fixed point holds too coarsely, where no value that the
+// stencil reads is as large as FX_HELD. Advection and dissipation leave such
+// axes out, for fx_fallback to add. Along an axis the values looked at are those
+// of the centred stencils, H on each side. The upwinded stencil does not read
+// the last of them on one side: a large value there enters through the
+// dissipation, and advection is good to parts in 1e14 of that; where there
+// is little or none (weak) its own values are looked at.
 template <int P, bool CUBIC, bool D1, bool D2, bool EXT>
-__device__ __forceinline__ void fx_point(const int2* __restrict__ c, const int4* const g[3], const FxCoef& C,
-                                         const double* beta, bool adv, int emax, int emax1, int emax2,
-                                         double* __restrict__ o1, double* __restrict__ o2, double* __restrict__ oe,
-                                         int vol) {
+__device__ __forceinline__ int fx_point(const int2* __restrict__ c, const int4* const g[3], const FxCoef& C,
+                                        const double* beta, bool adv, bool inexact, int emax, int emax1, int emax2,
+                                        double* __restrict__ o1, double* __restrict__ o2, double* __restrict__ oe,
+                                        int vol) {
   using F = FD<P>;
   using X = FX<P>;
   constexpr int BX = FxSmem<P>::BX;
@@ -362,14 +442,22 @@ __device__ __forceinline__ void fx_point(const int2* __restrict__ c, const int4*
   const int m2x = -2 * u0.x, m2y = -2 * u0.y;
   long long kslo = 0, kshi = 0;
   double ext = 0.0, ko = 0.0;
+  int coarse = 0;
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     const int st = d == 0 ? 1 : (d == 1 ? BX : BX * BX);
+    int top = 0, low = 0;  // (the point itself is not read by first derivatives)
+    int4 f = make_int4(0, 0, 0, 0);  // the sums that mixed derivatives are made of, and their values' magnitude
+    if (D2 && d < 2) f = *g[1 + d];
     long long r1l = 0, r1h = 0, r2l = 0, r2h = 0, tl = 0, th = 0, kl = 0, kh = 0;
 #pragma unroll
     for (int a = 1; a <= (EXT ? F::R : F::H); ++a) {
       const int2 p = c[a * st], m = c[-a * st];
       const int dx = p.x - m.x, dy = p.y - m.y;
+      if (!(D2 && d < 2) && a <= F::H) {
+        top = __vimax3_s32(top, p.y, m.y);
+        low = __vimin3_s32(low, p.y, m.y);
+      }
       if (D1 && !(D2 && d < 2) && a <= F::H) {
         r1l += (long long)X::W1(a) * (dx);
         r1h += (long long)X::W1(a) * (dy);
@@ -388,9 +476,15 @@ __device__ __forceinline__ void fx_point(const int2* __restrict__ c, const int4*
         kh += (long long)X::WK(a) * (p.y + m.y + m2y);
       }
     }
+    const bool held = (D2 && d < 2 ? f.w : max(top, ~low)) >= FX_HELD || !inexact;
+    bool share = held;
+    if ((D1 || D2) && !held) coarse |= FX_AXIS << d;
+    if (EXT) {
+      if (C.weak && inexact && adv) share = fx_upwind_held<P>(c, beta[d] < 0.0 ? -st : st);
+      if (!share) coarse |= FX_EXT << d;
+    }
     if (D1) {
-      if (D2 && d < 2) {  // the sums the mixed derivatives are made of
-        const int4 f = *g[1 + d];
+      if (D2 && d < 2) {
         r1h = ((long long)f.z << FX_LIMB) | (unsigned int)f.y;
         r1l = f.x;
       }
@@ -401,7 +495,7 @@ __device__ __forceinline__ void fx_point(const int2* __restrict__ c, const int4*
       const double r = fx_to_double(r2h, r2l, emax2);
       o2[sym(d, d) * vol] = CUBIC ? r : C.c2[sym(d, d)] * r;
     }
-    if (EXT) {
+    if (EXT && share) {
       if (adv) {
         // |beta| times the stencil mirrored by the sign of beta
         const int sk = __double2hiint(beta[d]) < 0 ? -X::SK : X::SK;
@@ -418,12 +512,17 @@ __device__ __forceinline__ void fx_point(const int2* __restrict__ c, const int4*
   }
   if (EXT) *oe = CUBIC ? fma(C.cu[0], ext, C.ck[0] * fx_to_double(kshi, kslo, emax)) : ext + ko;
   if (D2) {
-    const double xy = fx_mixed<P>(g[0], FX_T, emax2), xz = fx_mixed<P>(g[1], FX_T * FX_T, emax2),
-                 yz = fx_mixed<P>(g[2], FX_T * FX_T, emax2);
+    int mag[3];
+    const double xy = fx_mixed<P>(g[0], FX_T, emax2, mag[0]), xz = fx_mixed<P>(g[1], FX_T * FX_T, emax2, mag[1]),
+                 yz = fx_mixed<P>(g[2], FX_T * FX_T, emax2, mag[2]);
+#pragma unroll
+    for (int q = 0; q < 3; ++q)
+      if (mag[q] < FX_HELD && inexact) coarse |= FX_MIXED << q;
     o2[1 * vol] = CUBIC ? xy : C.c2[1] * xy;
     o2[2 * vol] = CUBIC ? xz : C.c2[2] * xz;
     o2[4 * vol] = CUBIC ? yz : C.c2[4] * yz;
   }
+  return coarse;
 }
 
 // The points of a tile's box that its stencils read, in the order they are
@@ -497,7 +596,7 @@ __device__ __forceinline__ void fx_tile(const Layout& L, const FxCoef& C, const 
   const int sy = (int)L.sy, sz = (int)L.sz;
   double raw[PER];
   unsigned int at[PER];
-  unsigned int mx = 0, any = 0;
+  unsigned int mx = 0, any = 0, mn = 0xffffffffu;
 #pragma unroll
   for (int q = 0; q < PER; ++q) {
     raw[q] = 0.0;
@@ -521,23 +620,29 @@ __device__ __forceinline__ void fx_tile(const Layout& L, const FxCoef& C, const 
 #pragma unroll
   for (int q = 0; q < PER; ++q) {
     const unsigned int hw = (unsigned int)__double2hiint(raw[q]) & 0x7fffffffu;
+    const unsigned int bits = hw | (unsigned int)__double2loint(raw[q]);
     mx = max(mx, hw);
-    any |= hw | (unsigned int)__double2loint(raw[q]);
+    mn = min(mn, bits ? hw : 0xffffffffu);
+    any |= bits;
   }
   mx = __reduce_max_sync(0xffffffffu, mx);
+  mn = __reduce_min_sync(0xffffffffu, mn);
   any = __reduce_or_sync(0xffffffffu, any);
   if ((threadIdx.x & 31) == 0) {
     red[0][threadIdx.x >> 5] = mx;
     red[1][threadIdx.x >> 5] = any;
+    red[2][threadIdx.x >> 5] = mn;
   }
   fx_sync();
 #pragma unroll
   for (int w = 0; w < FX_THREADS / 32; ++w) {
     mx = max(mx, red[0][w]);
     any |= red[1][w];
+    mn = min(mn, red[2][w]);
   }
   const bool fallback = mx >= (1900u << 20) || (mx < (160u << 20) && any != 0u);
   const int emax = max((int)(mx >> 20), 160);
+  const bool inexact = (int)(mn >> 20) < emax - 6;  // some value loses bits
 
   const bool d1 = list.d1[e] >= 0, ext = list.ext[e] >= 0;
   const int vol = T.vol;
@@ -587,36 +692,29 @@ __device__ __forceinline__ void fx_tile(const Layout& L, const FxCoef& C, const 
   if (ext && adv)
 #pragma unroll
     for (int d = 0; d < 3; ++d) beta[d] = __ldg(u + (V_BETA1 + d) * L.vs + p);
-  if (fallback) {
-    double r1[3], r2[6], re;
-    fx_fallback<P>(v, p, L.sy, L.sz, C, beta, adv, d1, mixed, ext, r1, r2, &re);
-    if (d1)
-      for (int d = 0; d < 3; ++d) o1[d * vol + idx] = scalbn(r1[d], list.s1[e]);
-    if (mixed)
-      for (int s = 0; s < 6; ++s) o2[s * vol + idx] = scalbn(r2[s], list.s2[e]);
-    if (ext) oe[idx] = re;
-    return;
+  int coarse = FX_ALL;
+  if (!fallback) {
+    const int2* c = box + ((z + R) * BX + (y + R)) * BX + x + R;
+    const int4* const gt[3] = {g + (z * S::EH + (y + H)) * FX_T + x, g + S::GN + ((z + H) * FX_T + y) * FX_T + x,
+                               g + 2 * S::GN + ((z + H) * FX_T + y) * FX_T + x};
+    auto point = [&](auto cubic) {
+      constexpr bool CB = decltype(cubic)::value;
+      double *const p1 = o1 + idx, *const p2 = o2 + idx, *const pe = oe + idx;
+      if (mixed && ext)
+        return fx_point<P, CB, true, true, true>(c, gt, C, beta, adv, inexact, emax, emax1, emax2, p1, p2, pe, vol);
+      if (mixed)
+        return fx_point<P, CB, true, true, false>(c, gt, C, beta, adv, inexact, emax, emax1, emax2, p1, p2, pe, vol);
+      if (d1 && ext)
+        return fx_point<P, CB, true, false, true>(c, gt, C, beta, adv, inexact, emax, emax1, emax2, p1, p2, pe, vol);
+      if (d1)
+        return fx_point<P, CB, true, false, false>(c, gt, C, beta, adv, inexact, emax, emax1, emax2, p1, p2, pe, vol);
+      return fx_point<P, CB, false, false, true>(c, gt, C, beta, adv, inexact, emax, emax1, emax2, p1, p2, pe, vol);
+    };
+    coarse = C.cubic ? point(std::true_type{}) : point(std::false_type{});
   }
-  const int2* c = box + ((z + R) * BX + (y + R)) * BX + x + R;
-  const int4* const gt[3] = {g + (z * S::EH + (y + H)) * FX_T + x, g + S::GN + ((z + H) * FX_T + y) * FX_T + x,
-                             g + 2 * S::GN + ((z + H) * FX_T + y) * FX_T + x};
-  auto point = [&](auto cubic) {
-    constexpr bool CB = decltype(cubic)::value;
-    if (mixed && ext)
-      fx_point<P, CB, true, true, true>(c, gt, C, beta, adv, emax, emax1, emax2, o1 + idx, o2 + idx, oe + idx, vol);
-    else if (mixed)
-      fx_point<P, CB, true, true, false>(c, gt, C, beta, adv, emax, emax1, emax2, o1 + idx, o2 + idx, oe + idx, vol);
-    else if (d1 && ext)
-      fx_point<P, CB, true, false, true>(c, gt, C, beta, adv, emax, emax1, emax2, o1 + idx, o2 + idx, oe + idx, vol);
-    else if (d1)
-      fx_point<P, CB, true, false, false>(c, gt, C, beta, adv, emax, emax1, emax2, o1 + idx, o2 + idx, oe + idx, vol);
-    else
-      fx_point<P, CB, false, false, true>(c, gt, C, beta, adv, emax, emax1, emax2, o1 + idx, o2 + idx, oe + idx, vol);
-  };
-  if (C.cubic)
-    point(std::true_type{});
-  else
-    point(std::false_type{});
+  if (coarse)
+    fx_fallback<P>(v, p, L.sy, L.sz, C, u + V_BETA1 * L.vs + p, L.vs, adv, coarse, d1, mixed, ext, list.s1[e] < 0, list.s2[e] < 0, o1 + idx,
+                   o2 + idx, oe + idx, vol);
 }
 
 // One grid as the FP64 kernels see it: its layout, scales, tiles and buffers.
@@ -691,7 +789,7 @@ __global__ void __launch_bounds__(FX_THREADS, 2) k_derivs(const __grid_constant_
   const int e = blockIdx.y;
   const FxGrid& G = fx_locate(A.W, A.W.tile0 + blockIdx.x, ti, tj, tk);
   const double* u = G.buf[A.in];
-  __shared__ unsigned int red[2][FX_THREADS / 32];
+  __shared__ unsigned int red[3][FX_THREADS / 32];
   fx_tile<P>(G.L, G.C, G.T, A.list, e, A.advect_gauge, A.lapse_frozen, A.shift_frozen, u, ti,
              tj, tk, (int2*)(g + 3 * FxSmem<P>::GN), g, red,
              A.W.rec + (long long)blockIdx.x * A.W.slot);

@@ -134,7 +134,7 @@ template <int P>
 __global__ void __launch_bounds__(OVERLAP_THREADS<P>, 1) k_overlap(const __grid_constant__ OverlapArgs A) {
   if (threadIdx.x < FX_THREADS) {
     extern __shared__ __align__(16) unsigned char fx_smem[];
-    __shared__ unsigned int red[2][FX_THREADS / 32];
+    __shared__ unsigned int red[3][FX_THREADS / 32];
     int4* g = (int4*)fx_smem;
     int2* box = (int2*)(g + 3 * FxSmem<P>::GN);
     const DerivArgs& D = A.D;

@@ -1,0 +1,82 @@
+"""A point's FP64 derivatives are as good as what its own stencils read allows,
+whatever else lies in its tile of 8 x 8 x 8 points (bssn_fixed.cuh): one value
+far larger than the rest must leave every result that does not read it where
+the other right-hand side tests have it (1e-12 of the variable's largest value
+among them).
+
+Which results read the value is what a NaN in its place reaches in the oracle."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1307_6488_gb300 import binding as B
+from paper_1307_6488_gb300.inputs import IDX
+
+from gpu_common import RHS_TOL, grid_for, interior, need_gpu, oracle_params, perturbed_bl
+
+pytestmark = pytest.mark.gpu
+
+SPIKE = (6, 7, 10)  # z, y, x among 16 x 16 x 24 points, inside a tile
+
+
+def check(got, want, nan):
+    """Every variable where the NaN does not reach."""
+    for v in range(len(want)):
+        far = np.isfinite(nan[v])
+        assert np.count_nonzero(far) > 0.5 * far.size
+        err = np.max(np.abs((got[v] - want[v])[far]))
+        assert err <= RHS_TOL * np.max(np.abs(want[v][far])), (v, err)
+
+
+def spiked(g, names, value, seed=9):
+    u = perturbed_bl(24, 16, 16, g, 0.1, seed=seed)
+    for name in names:
+        u[IDX[name]][tuple(g + i for i in SPIKE)] = value
+    return u
+
+
+@pytest.mark.parametrize("order", [4, 8])
+@pytest.mark.parametrize("h", [0.1, (0.11, 0.1, 0.13)])
+@pytest.mark.parametrize("big", [2.0 ** 20, 2.0 ** 60, 1e100])
+def test_spike_in_a_stage(order, h, big):
+    torch = need_gpu()
+    g, names = order // 2 + 1, ("Gt1", "trK", "At12", "beta2", "B3")
+    u = spiked(g, names, big)
+    p = B.make_params(fd_order=order, advect_gauge=0)
+    grid = grid_for(u, g, h)
+    y0, acc, out = B.upload(u, grid), B.alloc_state(grid), B.alloc_state(grid)
+    B.rk4_stage(grid, p, B.FP64, 0, 6.0, y0, y0, acc, out, B.alloc_work(grid, p))  # acc: RHS + dissipation
+    torch.cuda.synchronize()
+    f = lambda w: interior(oracle.rhs(w, g, h, oracle_params(p), ko=True), g)
+    check(interior(B.download(acc, grid), g), f(u), f(spiked(g, names, np.nan)))
+
+
+@pytest.mark.parametrize("order", [4, 8])
+@pytest.mark.parametrize("big", [2.0 ** 20, 1e100])
+def test_spike_in_a_right_hand_side(order, big):
+    """Without dissipation a variable's stencils reach further on one side."""
+    torch = need_gpu()
+    g, names = order // 2 + 1, ("At12", "B3")
+    u = spiked(g, names, big)
+    p = B.make_params(fd_order=order)
+    grid = grid_for(u, g, 0.1)
+    d, out = B.upload(u, grid), B.alloc_state(grid)
+    B.rhs(grid, p, B.FP64, d, out, B.alloc_work(grid, p))
+    torch.cuda.synchronize()
+    f = lambda w: interior(oracle.rhs(w, g, 0.1, oracle_params(p), ko=False), g)
+    check(interior(B.download(out, grid), g), f(u), f(spiked(g, names, np.nan)))
+
+
+@pytest.mark.parametrize("order", [4, 8])
+@pytest.mark.parametrize("big", [2.0 ** 20, 1e100])
+def test_spike_in_the_hamiltonian_constraint(order, big):
+    torch = need_gpu()
+    g = order // 2 + 1
+    u = spiked(g, ("Gt2",), big)
+    p = B.make_params(fd_order=order)
+    grid = grid_for(u, g, 0.1)
+    ham = torch.zeros(grid.var_stride, dtype=torch.float64, device="cuda")
+    B.hamiltonian(grid, p, B.upload(u, grid), B.alloc_work(grid, p), ham=ham)
+    torch.cuda.synchronize()
+    f = lambda w: interior(oracle.constraints(w, g, 0.1, order, fields=True)[3][0], g)[None]
+    check(interior(B.view4(ham, grid, 1).cpu().numpy(), g), f(u), f(spiked(g, ("Gt2",), np.nan)))
