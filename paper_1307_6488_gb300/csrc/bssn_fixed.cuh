@@ -586,13 +586,22 @@ __device__ __forceinline__ void fx_tile(const Layout& L, const FxCoef& C, const 
   const long long org = L.off0 + i0 + j0 * L.sy + k0 * L.sz;
   const double* __restrict__ v = u + var * L.vs;
 
-  // ---- the box in registers. A ragged tile drops the points its stencils
-  // cannot reach (they may lie outside the array).
+  // ---- the box in registers. A ragged tile drops the points that its own
+  // stencils do not read (they may lie outside the array, or be ghosts that
+  // nothing fills), and so does a variable without dissipation, whose lines
+  // are shorter.
   constexpr int PER = (FxBox<P>::ALL + FX_THREADS - 1) / FX_THREADS;
   constexpr int PERL = (FxBox<P>::LINES + FX_THREADS - 1) / FX_THREADS;
   const int count = mixed ? FxBox<P>::ALL : FxBox<P>::LINES;
   const double* __restrict__ v0 = v + (org - R * (1 + L.sy + L.sz));
-  const bool full = ex == FX_T && ey == FX_T && ez == FX_T, wide = L.sz >= (1 << 26);
+  const bool d1 = list.d1[e] >= 0, ext = list.ext[e] >= 0;
+  const bool full = ex == FX_T && ey == FX_T && ez == FX_T && ext, wide = L.sz >= (1 << 26);
+  auto reads = [&](int bx, int by, int bz) {  // does some point of the tile read this one?
+    const int ox = max(max(R - bx, bx - (R + ex - 1)), 0), oy = max(max(R - by, by - (R + ey - 1)), 0),
+              oz = max(max(R - bz, bz - (R + ez - 1)), 0), far = max(ox, max(oy, oz));
+    const int axes = (ox > 0) + (oy > 0) + (oz > 0);
+    return axes < 2 ? far <= (ext ? R : H) : axes == 2 && mixed && far <= H;
+  };
   const int sy = (int)L.sy, sz = (int)L.sz;
   double raw[PER];
   unsigned int at[PER];
@@ -612,7 +621,7 @@ __device__ __forceinline__ void fx_tile(const Layout& L, const FxCoef& C, const 
     // (a box spans less than 2^31 elements of a variable unless a plane of
     // the array alone has 2^26 points)
     const long long o = wide ? bx + by * L.sy + bz * L.sz : (long long)(bx + by * sy + bz * sz);
-    if ((full && at[q] != 0xffffffffu) || (bx < ex + 2 * R && by < ey + 2 * R && bz < ez + 2 * R)) {
+    if (full ? at[q] != 0xffffffffu : reads(bx, by, bz)) {
       if (in_range(org - R * (1 + L.sy + L.sz) + o, org - R * (1 + L.sy + L.sz) + o, padded_points(L)))
         raw[q] = __ldg(v0 + o);
     }
@@ -644,7 +653,6 @@ __device__ __forceinline__ void fx_tile(const Layout& L, const FxCoef& C, const 
   const int emax = max((int)(mx >> 20), 160);
   const bool inexact = (int)(mn >> 20) < emax - 6;  // some value loses bits
 
-  const bool d1 = list.d1[e] >= 0, ext = list.ext[e] >= 0;
   const int vol = T.vol;
   const int emax1 = emax + list.s1[e], emax2 = emax + list.s2[e];
   double* const o1 = rec + (long long)(d1 ? list.d1[e] : 0) * vol;
@@ -713,8 +721,8 @@ __device__ __forceinline__ void fx_tile(const Layout& L, const FxCoef& C, const 
     coarse = C.cubic ? point(std::true_type{}) : point(std::false_type{});
   }
   if (coarse)
-    fx_fallback<P>(v, p, L.sy, L.sz, C, u + V_BETA1 * L.vs + p, L.vs, adv, coarse, d1, mixed, ext, list.s1[e] < 0, list.s2[e] < 0, o1 + idx,
-                   o2 + idx, oe + idx, vol);
+    fx_fallback<P>(v, p, L.sy, L.sz, C, u + V_BETA1 * L.vs + p, L.vs, adv, coarse, d1, mixed, ext, list.s1[e] < 0,
+                   list.s2[e] < 0, o1 + idx, o2 + idx, oe + idx, vol);
 }
 
 // One grid as the FP64 kernels see it: its layout, scales, tiles and buffers.

@@ -80,3 +80,42 @@ def test_spike_in_the_hamiltonian_constraint(order, big):
     torch.cuda.synchronize()
     f = lambda w: interior(oracle.constraints(w, g, 0.1, order, fields=True)[3][0], g)[None]
     check(interior(B.view4(ham, grid, 1).cpu().numpy(), g), f(u), f(spiked(g, ("Gt2",), np.nan)))
+
+
+def unread(u, g, line, square):
+    """The padded points that no stencil of an interior point reads: further out
+    than `line` along one axis, than `square` along two, or along all three."""
+    out = []
+    for m in u.shape[1:]:
+        i = np.arange(m)
+        out.append(np.maximum(np.maximum(g - i, i - (m - g - 1)), 0))
+    d = np.sort(np.stack(np.meshgrid(*out, indexing="ij")), axis=0)  # distances outside, the smallest first
+    return (d[0] > 0) | (d[1] > square) | ((d[1] == 0) & (d[2] > line)) | ((d[1] > 0) & (d[2] > square))
+
+
+@pytest.mark.parametrize("order", [4, 8])
+@pytest.mark.parametrize("n", [(13, 21, 5), (16, 8, 8)])
+@pytest.mark.parametrize("value", [1e200, np.nan])
+def test_unread_ghosts_do_not_matter(order, n, value):
+    """Bit for bit, in a stage (lines of r = p/2 + 1 points) and in the constraints (p/2)."""
+    torch = need_gpu()
+    g, H = order // 2 + 2, order // 2
+    u = perturbed_bl(*n, g, 0.1, seed=3)
+    p = B.make_params(fd_order=order)
+    grid = grid_for(u, g, 0.1)
+
+    def stage(w):
+        y0, acc, out = B.upload(w, grid), B.alloc_state(grid), B.alloc_state(grid)
+        B.rk4_stage(grid, p, B.FP64, 0, 0.1, y0, y0, acc, out, B.alloc_work(grid, p))
+        return interior(B.download(out, grid), g)
+
+    def constraints(w):
+        vs = grid.var_stride
+        f = [torch.zeros(k * vs, dtype=torch.float64, device="cuda") for k in (1, 3, 3)]
+        l2, mx, _ = B.constraints(grid, p, B.upload(w, grid), B.alloc_work(grid, p), *f)
+        return np.concatenate([interior(B.view4(x, grid, k).cpu().numpy(), g) for x, k in zip(f, (1, 3, 3))])
+
+    for run, line in ((stage, H + 1), (constraints, H)):
+        w = u.copy()
+        w[:, unread(u, g, line, H)] = value
+        assert np.array_equal(run(w), run(u)), run.__name__
