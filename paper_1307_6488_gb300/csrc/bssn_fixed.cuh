@@ -274,12 +274,13 @@ constexpr int FX_AXIS = 1, FX_MIXED = 8, FX_EXT = 64, FX_ALL = 511;
 // variable, p: the point; has1, has2, hase: which of them the variable's record
 // has, half1 and half2: whether it has half the first and second ones. oe holds
 // the sum of the other axes unless `which` is FX_ALL. beta: the shift's first
-// component at the point, the others vs apart. Each axis' values are
+// component at the point, the others vs apart; ko: whether there is a
+// dissipation, whose stencil reads further than the upwinded one. Each axis' values are
 // loaded before any is used: what these points cost is mostly that latency.
 template <int P>
 __device__ __noinline__ void fx_fallback(const double* __restrict__ v, long long p, long long sy, long long sz,
                                          const FxCoef& C, const double* __restrict__ beta, long long vs, bool adv,
-                                         int which, bool has1, bool has2, bool hase, bool half1, bool half2,
+                                         bool ko, int which, bool has1, bool has2, bool hase, bool half1, bool half2,
                                          double* __restrict__ o1, double* __restrict__ o2, double* __restrict__ oe,
                                          int vol) {
   using F = FD<P>;
@@ -315,10 +316,12 @@ __device__ __noinline__ void fx_fallback(const double* __restrict__ v, long long
       if (has2) o2[sym(d, d) * vol] = f2 * (C.cubic ? r2 : C.c2[sym(d, d)] * r2);
     }
     if (share) {
-      double k = 0.0;
+      if (ko) {
+        double k = 0.0;
 #pragma unroll
-      for (int a = 1; a <= R; ++a) k += X::WK(a) * ((up[a] + um[a]) + m2);
-      ext += C.ck[d] * k;
+        for (int a = 1; a <= R; ++a) k += X::WK(a) * ((up[a] + um[a]) + m2);
+        ext += C.ck[d] * k;
+      }
       if (adv) {
         // the one-sided stencil the sign of beta selects, and no other point
         const double bd = beta[d * vs];
@@ -573,7 +576,7 @@ __device__ __forceinline__ void fx_sync() { asm volatile("bar.sync 1, %0;" ::"n"
 // and its first-derivative tables.
 template <int P>
 __device__ __forceinline__ void fx_tile(const Layout& L, const FxCoef& C, const FxTiles& T, const DerivList& list,
-                                        int e, bool advect_gauge, bool lapse_frozen, bool shift_frozen,
+                                        int e, bool advect_gauge, bool lapse_frozen, bool shift_frozen, bool ko,
                                         const double* __restrict__ u, int ti, int tj, int tk, int2* box, int4* g,
                                         unsigned int (*red)[FX_THREADS / 32], double* __restrict__ rec) {
   using S = FxSmem<P>;
@@ -721,7 +724,7 @@ __device__ __forceinline__ void fx_tile(const Layout& L, const FxCoef& C, const 
     coarse = C.cubic ? point(std::true_type{}) : point(std::false_type{});
   }
   if (coarse)
-    fx_fallback<P>(v, p, L.sy, L.sz, C, u + V_BETA1 * L.vs + p, L.vs, adv, coarse, d1, mixed, ext, list.s1[e] < 0,
+    fx_fallback<P>(v, p, L.sy, L.sz, C, u + V_BETA1 * L.vs + p, L.vs, adv, ko, coarse, d1, mixed, ext, list.s1[e] < 0,
                    list.s2[e] < 0, o1 + idx, o2 + idx, oe + idx, vol);
 }
 
@@ -772,6 +775,7 @@ struct DerivArgs {
   DerivList list;
   int in;  // buffer the stencils read
   bool advect_gauge, lapse_frozen, shift_frozen;
+  bool ko;  // a stage (its dissipation may be 0); a right-hand side alone has none
 };
 
 // What a thread does with the right-hand side of its point.
@@ -798,8 +802,8 @@ __global__ void __launch_bounds__(FX_THREADS, 2) k_derivs(const __grid_constant_
   const FxGrid& G = fx_locate(A.W, A.W.tile0 + blockIdx.x, ti, tj, tk);
   const double* u = G.buf[A.in];
   __shared__ unsigned int red[3][FX_THREADS / 32];
-  fx_tile<P>(G.L, G.C, G.T, A.list, e, A.advect_gauge, A.lapse_frozen, A.shift_frozen, u, ti,
-             tj, tk, (int2*)(g + 3 * FxSmem<P>::GN), g, red,
+  fx_tile<P>(G.L, G.C, G.T, A.list, e, A.advect_gauge, A.lapse_frozen, A.shift_frozen, A.ko, u,
+             ti, tj, tk, (int2*)(g + 3 * FxSmem<P>::GN), g, red,
              A.W.rec + (long long)blockIdx.x * A.W.slot);
 }
 

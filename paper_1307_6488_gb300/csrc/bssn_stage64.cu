@@ -242,7 +242,7 @@ template <typename F>
 static cudaError_t through_record(int order, const FxWork& work, const DerivList& list, size_t rec_doubles,
                                   cudaStream_t s, F use) {
   const FxTiles& T = work.one.T;
-  DerivArgs D{work, list, 1, false, false, false};
+  DerivArgs D{work, list, 1, false, false, false, false};
   D.W.slot = (long long)list.nout * T.vol;
   const long long ntiles = (long long)T.ntx * T.nty * T.ntz, slots = (long long)(rec_doubles / (size_t)D.W.slot);
   if (slots < 1) return cudaErrorInvalidValue;
@@ -307,7 +307,7 @@ static long long overlap_chunk(long long ntiles, long long half) {
 cudaError_t launch_stage64(int order, const FxWork& work, int vol, long long ntiles, long long slots,
                            const Gauge& gz, const StageOut& out, cudaStream_t s) {
   if (slots < 1) return cudaErrorInvalidValue;
-  DerivArgs D{work, rhs_list(), out.in, gz.advect_gauge != 0, gz.lapse == 2, gz.shift == 1};
+  DerivArgs D{work, rhs_list(), out.in, gz.advect_gauge != 0, gz.lapse == 2, gz.shift == 1, out.mode == 0};
   AlgebraArgs A{work, out};
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);

@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(OVERLAP_THREADS<P>, 1) k_overlap(const __grid_
       int ti, tj, tk;
       const FxGrid& G = fx_locate(D.W, D.W.tile0 + slot, ti, tj, tk);
       const double* u = G.buf[D.in];
-      fx_tile<P>(G.L, G.C, G.T, D.list, (int)e, D.advect_gauge, D.lapse_frozen, D.shift_frozen, u,
+      fx_tile<P>(G.L, G.C, G.T, D.list, (int)e, D.advect_gauge, D.lapse_frozen, D.shift_frozen, D.ko, u,
                  ti, tj, tk, box, g, red, D.W.rec + (long long)slot * D.W.slot);
       fx_sync();  // the next tile reuses the shared memory
     }

@@ -119,3 +119,38 @@ def test_unread_ghosts_do_not_matter(order, n, value):
         w = u.copy()
         w[:, unread(u, g, line, H)] = value
         assert np.array_equal(run(w), run(u)), run.__name__
+
+
+@pytest.mark.parametrize("order", [4, 8])
+@pytest.mark.parametrize("gauge", [dict(lapse=0, shift=0), dict(lapse=2, shift=1)])
+def test_reach_of_a_right_hand_side(order, gauge):
+    """A right-hand side without dissipation reads the outermost ghosts on the
+    side that the shift points to, and no others (with a frozen gauge, none at
+    all for the gauge variables): NaNs there reach those points alone."""
+    torch = need_gpu()
+    g = order // 2 + 1
+    u = perturbed_bl(13, 18, 11, g, 0.1, seed=order)
+    p = B.make_params(fd_order=order, **gauge)
+    want = interior(oracle.rhs(u, g, 0.1, oracle_params(p), ko=False), g)
+    beta = interior(u, g)[IDX["beta1"]:IDX["beta1"] + 3]
+    reached = np.zeros(want.shape[1:], dtype=bool)
+    w = u.copy()
+    for a in range(3):
+        ends = [tuple(e if b == 2 - a else slice(None) for b in range(3)) for e in (0, -1)]
+        for e in ends:
+            w[(slice(None),) + e] = np.nan
+        reached[ends[0]] |= beta[a][ends[0]] < 0
+        reached[ends[1]] |= beta[a][ends[1]] >= 0
+    assert 0 < np.count_nonzero(reached) < reached.size / 2
+    grid = grid_for(u, g, 0.1)
+    d, out = B.upload(w, grid), B.alloc_state(grid)
+    B.rhs(grid, p, B.FP64, d, out, B.alloc_work(grid, p))
+    torch.cuda.synchronize()
+    got = interior(B.download(out, grid), g)
+    for v in range(len(want)):
+        if gauge["lapse"] == 2 and v >= IDX["alpha"]:
+            assert np.all(got[v] == 0.0), v
+            continue
+        assert np.array_equal(np.isnan(got[v]), reached), v
+        err = np.max(np.abs((got[v] - want[v])[~reached]))
+        assert err <= RHS_TOL * np.max(np.abs(want[v][~reached])), v
