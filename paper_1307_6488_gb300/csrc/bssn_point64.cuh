@@ -26,8 +26,8 @@
 namespace bssn {
 
 // One point's derivatives, as the record scales them: first derivatives 1/a
-// times and second derivatives 1/a2 = 1/a^2 times their value, where a and a2
-// are what the functions below take (FxCoef).
+// times and second derivatives 1/a2 = 1/a^2 times their value, where a, a2 and
+// b = a2 / a are what the functions below take (FxCoef).
 struct Point64 {
   double u[NV];
   double dW[3], dK[3], da[3];
@@ -144,7 +144,7 @@ __device__ __forceinline__ void conformal64(const Point64& P, double ia, Conform
 // Right-hand side of the 24 variables added to rhs (which holds advection and
 // dissipation on entry). gz.lapse / gz.shift as in bssn_point.cuh.
 __device__ __forceinline__ void rhs_point64(const Point64& P, const Gauge& gz, double a, double a2, double ia,
-                                            double rhs[NV]) {
+                                            double b, double rhs[NV]) {
   Conformal64 C;
   conformal64(P, ia, C);
   const double* u = P.u;
@@ -244,34 +244,36 @@ __device__ __forceinline__ void rhs_point64(const Point64& P, const Gauge& gz, d
   }
 
   double q[3], w[3];  // what At^ij and gt^ij are contracted with
-  const double a6 = -6.0 * al, a43 = (-4.0 / 3.0) * al, a3 = third * a;
+  const double a6 = -6.0 * al, a43 = (-4.0 / 3.0) * al, b3 = third * b;
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
     q[j] = fma(a6, dWs[j], -2.0 * P.da[j]);
-    w[j] = fma(a43, P.dK[j], a3 * (P.ddb[0][sym(j, 0)] + P.ddb[1][sym(j, 1)] + P.ddb[2][sym(j, 2)]));
+    w[j] = fma(a43, P.dK[j], b3 * (P.ddb[0][sym(j, 0)] + P.ddb[1][sym(j, 1)] + P.ddb[2][sym(j, 2)]));
   }
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
+    // everything in units of one first derivative; the second derivatives of
+    // beta, the largest terms where beta is rough, are added last
     double t6 = Au2[0] * C.GU[i][0];
-    double r = C.gu2[0] * P.ddb[i][0];
+    double lap = C.gu2[0] * P.ddb[i][0];
 #pragma unroll
     for (int s = 1; s < 6; ++s) {
       t6 = fma(Au2[s], C.GU[i][s], t6);
-      r = fma(C.gu2[s], P.ddb[i][s], r);
+      lap = fma(C.gu2[s], P.ddb[i][s], lap);
     }
-    r = fma(a, r, al2 * t6);  // everything in units of one first derivative
-    r = fma(d23, C.Gd[i], r);
+    double r = fma(d23, C.Gd[i], al2 * t6);
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
       r = fma(Au[sym(i, j)], q[j], r);
-      r = fma(C.gu[sym(i, j)], w[j], r);
       r = fma(-C.Gd[j], db[j][i], r);
     }
-    r *= a;
-    rhs[V_GAM1 + i] += r;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) r = fma(C.gu[sym(i, j)], w[j], r);
+    r = fma(b, lap, r);
+    rhs[V_GAM1 + i] = fma(a, r, rhs[V_GAM1 + i]);
     if (gz.shift == 0) {
       rhs[V_BETA1 + i] = fma(gz.shift_coeff, u[V_B1 + i], rhs[V_BETA1 + i]);
-      rhs[V_B1 + i] += fma(-gz.eta, u[V_B1 + i], r);
+      rhs[V_B1 + i] = fma(a, r, fma(-gz.eta, u[V_B1 + i], rhs[V_B1 + i]));
     }
   }
   if (gz.lapse == 0)

@@ -73,7 +73,7 @@ __device__ __forceinline__ void algebra_point(const FxWork& Wk, const StageOut& 
   double rhs[NV];
 #pragma unroll
   for (int v = 0; v < NV; ++v) rhs[v] = r(REC_EXT + v);
-  rhs_point64(Q, S.gz, G.C.a, G.C.a2, G.C.ia, rhs);
+  rhs_point64(Q, S.gz, G.C.a, G.C.a2, G.C.ia, G.C.b, rhs);
   if (S.mode == 1) {
 #pragma unroll
     for (int v = 0; v < NV; ++v)
