@@ -281,7 +281,7 @@ typedef struct {
  * The plan allocates and owns, per patch, three stage buffers (and in the
  * FP32-RHS form a single-precision copy and derivative tables), plus the
  * patch table, one CUDA graph per step size and, in FP64, the derivative
- * record of up to 2048 tiles (1.1 GB). The stage kernels' tiles are fixed in
+ * record of the tiles that are worked on at a time, up to 2048 (1.1 GB). The stage kernels' tiles are fixed in
  * both precisions (8 x 8 x 8 points in FP64, 8 x 4 x 4 in FP32-RHS), so
  * autotune (0 or 1) has nothing to choose. Synchronizes the device. Returns
  * BSSN_ERR_NOMEM if an allocation fails (nothing is leaked). */

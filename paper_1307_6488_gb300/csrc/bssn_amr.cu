@@ -585,7 +585,7 @@ struct bssn_amr {
   std::vector<void*> allocations;
   int grid_other = 0;
   double* rec = nullptr;        // FP64 form: the derivative record all levels share
-  long long rec_slots = 0;
+  size_t rec_doubles = 0;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   cudaStream_t cap = nullptr;
@@ -811,8 +811,8 @@ cudaError_t compute_stage(bssn_amr* A, Level& L, const RK& rk, int in, int out, 
     A->nodes += 3;
     return e;
   }
-  const cudaError_t e = fx_stage(A->order, L.fx, A->rec, A->rec_slots, A->gz, rk, in, out, s);
-  A->nodes += stage64_launches(L.fx.ntiles, A->rec_slots);
+  const cudaError_t e = fx_stage(A->order, L.fx, A->rec, A->gz, rk, in, out, s);
+  A->nodes += stage64_launches(L.fx.ntiles, L.fx.slots);
   return e;
 }
 
@@ -1069,7 +1069,7 @@ bssn_status_t bssn_amr_create(bssn_amr_t** out, const bssn_amr_patch_t* patches,
     L.npad = npd;
     if (prec == BSSN_FP64) {
       e = fx_upload(tab, &L.fx, [&](size_t n, void** q) { return amr_alloc(A, n, q); });
-      A->rec_slots = std::max(A->rec_slots, std::min(FX_MAX_SLOTS, L.fx.ntiles));
+      A->rec_doubles = std::max(A->rec_doubles, L.fx.record_doubles());
     }
     if (e == cudaSuccess) e = amr_alloc(A, sizeof(long long) * nl, &p);
     if (e == cudaSuccess) {
@@ -1112,7 +1112,7 @@ bssn_status_t bssn_amr_create(bssn_amr_t** out, const bssn_amr_patch_t* patches,
     e = A->order == 4 ? stage32_batch_init<4>() : stage32_batch_init<8>();
   if (e == cudaSuccess && nested) e = cudaStreamCreateWithFlags(&A->cap, cudaStreamNonBlocking);
   if (e == cudaSuccess && nested && prec == BSSN_FP64) {
-    e = amr_alloc(A, (size_t)A->rec_slots * FX_SLOT_DOUBLES * sizeof(double), &p);
+    e = amr_alloc(A, A->rec_doubles * sizeof(double), &p);
     A->rec = (double*)p;
     if (e == cudaSuccess) e = A->order == 4 ? derivs_init<4>() : derivs_init<8>();
   }

@@ -43,7 +43,6 @@ struct bssn_plan {
   // FP64 form: the patches as the stage kernels see them, and their record
   FxTable fx;
   double* rec = nullptr;
-  long long rec_slots = 0;
   // FP32-RHS form: the tiled kernels of bssn_stage32.cuh over a second table,
   // ordered by spacing so that each spacing's patches are one range,
   // and numbered by that order; two tables that differ in the single-precision
@@ -159,7 +158,7 @@ cudaError_t enqueue_step(bssn_plan* pl, double dt, cudaStream_t s) {
     const RK rk = make_rk(st, dt);
     e = pl->prec == BSSN_FP32_RHS
             ? stage32_all(pl, rk, ins[st], outs[st], cur, two && st < 3 ? pl->dev32[1 - (st & 1)] : nullptr, convert, s)
-            : fx_stage(pl->order, pl->fx, pl->rec, pl->rec_slots, pl->gz, rk, ins[st], outs[st], s);
+            : fx_stage(pl->order, pl->fx, pl->rec, pl->gz, rk, ins[st], outs[st], s);
   }
   if (e == cudaSuccess) e = fill_all(pl, 0, nullptr, s);
   return e;
@@ -287,8 +286,7 @@ bssn_status_t bssn_plan_create(bssn_plan_t** out, const bssn_block_t* blocks, in
     for (int b = 0; b < nblocks; ++b) grids.push_back(fx_grid(blocks[b].grid, pl->order, params->ko_eps, pl->host[b].buf));
     e = fx_upload(grids, &pl->fx, [&](size_t n, void** q) { return plan_alloc(pl, n, q); });
     pl->ntiles = pl->fx.ntiles;
-    pl->rec_slots = std::min(FX_MAX_SLOTS, pl->fx.ntiles);
-    if (e == cudaSuccess) e = plan_alloc(pl, (size_t)pl->rec_slots * FX_SLOT_DOUBLES * sizeof(double), &p);
+    if (e == cudaSuccess) e = plan_alloc(pl, pl->fx.record_doubles() * sizeof(double), &p);
     if (e == cudaSuccess) pl->rec = (double*)p;
     if (e == cudaSuccess) e = pl->order == 4 ? derivs_init<4>() : derivs_init<8>();
   }

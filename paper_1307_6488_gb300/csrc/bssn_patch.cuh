@@ -8,6 +8,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "bssn_bounds.cuh"
@@ -77,13 +78,15 @@ struct FxTable {
   FxGrid* dev = nullptr;
   long long* tile0s = nullptr;
   int n = 0;
+  int vol = 1;              // points of the largest tile
   long long ntiles = 0;
+  long long slots = 0;      // tiles of its record, and the record's size
+  size_t record_doubles() const { return (size_t)slots * REC_RHS * vol; }
 };
 
-// Slots of the shared record: at most this many tiles (of 512 points, 135
-// doubles each) are between the two kernels of a stage at a time.
+// Slots of the shared record: at most this many tiles are between the two
+// kernels of a stage at a time (1.1 GB where tiles have 512 points).
 constexpr long long FX_MAX_SLOTS = 2048;
-constexpr long long FX_SLOT_DOUBLES = (long long)REC_RHS * FX_T * FX_T * FX_T;
 
 FxGrid fx_grid(const bssn_grid_t& G, int order, double eps, double* const buf[6]) {
   FxGrid F{};
@@ -104,7 +107,9 @@ cudaError_t fx_upload(std::vector<FxGrid>& grids, FxTable* T, Alloc alloc) {
   for (size_t b = 0; b < grids.size(); ++b) {
     grids[b].tile0 = t0[b] = T->ntiles;
     T->ntiles += (long long)grids[b].T.ntx * grids[b].T.nty * grids[b].T.ntz;
+    T->vol = std::max(T->vol, grids[b].T.vol);
   }
+  T->slots = std::min(FX_MAX_SLOTS, stage64_slots(T->ntiles));
   void* p = nullptr;
   cudaError_t e = alloc(sizeof(FxGrid) * grids.size(), &p);
   T->dev = (FxGrid*)p;
@@ -115,17 +120,17 @@ cudaError_t fx_upload(std::vector<FxGrid>& grids, FxTable* T, Alloc alloc) {
   return e;
 }
 
-// One FP64 stage of every patch of the table, buffer `in` to buffer `out`.
-cudaError_t fx_stage(int order, const FxTable& T, double* rec, long long slots, const Gauge& gz, const RK& rk, int in,
-                     int out, cudaStream_t s) {
-  constexpr int vol = FX_T * FX_T * FX_T;
+// One FP64 stage of every patch of the table, buffer `in` to buffer `out`,
+// through a record of at least T.record_doubles().
+cudaError_t fx_stage(int order, const FxTable& T, double* rec, const Gauge& gz, const RK& rk, int in, int out,
+                     cudaStream_t s) {
   FxWork W{};
   W.table = T.dev;
   W.tile0s = T.tile0s;
   W.ngrids = T.n;
   W.rec = rec;
-  W.slot = FX_SLOT_DOUBLES;
-  return launch_stage64(order, W, vol, T.ntiles, slots, gz, StageOut{0, gz, rk, in, out, nullptr}, s);
+  W.slot = (long long)REC_RHS * T.vol;
+  return launch_stage64(order, W, T.vol, T.ntiles, T.slots, gz, StageOut{0, gz, rk, in, out, nullptr}, s);
 }
 
 }  // namespace
