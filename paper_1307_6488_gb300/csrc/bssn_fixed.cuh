@@ -111,20 +111,15 @@ struct DerivList {
 // then the 24 advection + dissipation sums.
 constexpr int REC_K = 9 * NM, REC_GAM = REC_K + 3, REC_EXT = REC_GAM + 9, REC_RHS = REC_EXT + NV;
 
-// Hamiltonian constraint: W and gt (9 each), Gt^i (3 each). Weyl scalars: K (3)
-// and At (3 each) too.
-constexpr int REC_C_GAM = 9 * 7, REC_HAM = REC_C_GAM + 9, REC_C_K = REC_HAM, REC_C_AT = REC_C_K + 3,
-              REC_CON = REC_C_AT + 18;
+// Constraints and Weyl scalars: W and gt (9 each), Gt^i (3 each), all that the
+// Hamiltonian constraint and the conformal Ricci tensor need.
+constexpr int REC_C_GAM = 9 * 7, REC_HAM = REC_C_GAM + 9;
 
-inline DerivList con_list(bool ham_only) {
+inline DerivList ham_list() {
   DerivList D{};
   for (int m = 0; m < 7; ++m) D.add(m, 9 * m, 9 * m + 3, -1);
   for (int i = 0; i < 3; ++i) D.add(V_GAM1 + i, REC_C_GAM + 3 * i, -1, -1);
-  if (!ham_only) {
-    D.add(V_TRK, REC_C_K, -1, -1);
-    for (int s = 0; s < 6; ++s) D.add(V_AT11 + s, REC_C_AT + 3 * s, -1, -1);
-  }
-  D.nout = ham_only ? REC_HAM : REC_CON;
+  D.nout = REC_HAM;
   return D;
 }
 

@@ -323,63 +323,75 @@ __device__ __forceinline__ double d1_direct(const double* __restrict__ v, long l
   return r;
 }
 
-// Momentum (out[0..2]) and Gamma (out[3..5]) constraints of the state u at a
-// point, c1 the first-derivative weights over the spacing. Where the
-// constraints hold they are what is left of terms that cancel: on a gauge wave
-// (A = 0.05, noise 1e-10) terms of order 1 leave 1e-8 to 1e-10, and
-// parts in 1e-9 to 1e-8 of the result are the rounding of whatever form is
-// evaluated. This form, stencils and expressions in double precision, is the
-// one that the constraints' values have always had, so they stay the same to
-// the last bit; from the derivative record, rounded once and gathered
-// differently, they were as close to a quadruple-precision evaluation but up
-// to 9e-9 of their norm apart from these. All constraints at 128^3, 8th order:
-// 12.0 ms with every stencil in double precision, 6.15 with these alone, 4.0
-// with none.
+// What the momentum and Gamma constraints and the magnetic part of the Weyl
+// tensor are made of, from the state itself: first derivatives by stencils in
+// double precision and the Christoffel symbols.
+//
+// On data that satisfies the constraints these are what is left of terms that
+// cancel: on a gauge wave (A = 0.05, noise 1e-10) terms of order 1 leave 1e-8 to
+// 1e-10, and parts in 1e-9 to 1e-8 of the result are the rounding of whatever
+// form is evaluated. This form is the one that their values have always had, so
+// they stay the same to the last bit; from the derivative record, rounded once
+// and gathered differently, they were as close to a quadruple-precision
+// evaluation but up to 9e-9 of their norm apart from these. All constraints at
+// 128^3, 8th order: 12.0 ms with every stencil in double precision, 6.4 with
+// these alone, 4.0 with none.
+struct First64 {
+  double u[V_ALPHA];  // the variables up to Gt^i
+  double dW[3], dK[3], dg[3][6], dAt[3][6];
+  double gu[6], gu2[6];  // gt^ij; with off-diagonal entries doubled
+  double GU[3][6], Gd[3];  // Gt^k_ij, gt^ij Gt^k_ij
+};
+
+// c1: the first-derivative weights over the spacing
 template <int H>
-__device__ __forceinline__ void momentum64(const double* __restrict__ up, long long vs, const long long st[3],
-                                           const double (*c1)[5], double out[6]) {
-  double u[V_ALPHA], dW[3], dK[3], dg[3][6], dAt[3][6];
+__device__ __forceinline__ void first64(const double* __restrict__ up, long long vs, const long long st[3],
+                                        const double (*c1)[5], First64& F) {
 #pragma unroll
-  for (int v = 0; v < V_ALPHA; ++v) u[v] = __ldg(up + v * vs);
+  for (int v = 0; v < V_ALPHA; ++v) F.u[v] = __ldg(up + v * vs);
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    dW[d] = d1_direct<H>(up + V_W * vs, st[d], c1[d]);
-    dK[d] = d1_direct<H>(up + V_TRK * vs, st[d], c1[d]);
+    F.dW[d] = d1_direct<H>(up + V_W * vs, st[d], c1[d]);
+    F.dK[d] = d1_direct<H>(up + V_TRK * vs, st[d], c1[d]);
 #pragma unroll
     for (int s = 0; s < 6; ++s) {
-      dg[d][s] = d1_direct<H>(up + (V_GT11 + s) * vs, st[d], c1[d]);
-      dAt[d][s] = d1_direct<H>(up + (V_AT11 + s) * vs, st[d], c1[d]);
+      F.dg[d][s] = d1_direct<H>(up + (V_GT11 + s) * vs, st[d], c1[d]);
+      F.dAt[d][s] = d1_direct<H>(up + (V_AT11 + s) * vs, st[d], c1[d]);
     }
   }
-  const double iW = 1.0 / u[V_W];
-  double gu[6], gu2[6], GL[3][6], GU[3][6], Gd[3];  // gt^ij, Gt_k,ij, Gt^k_ij, gt^ij Gt^k_ij
-  inverse_metric<double>(u + V_GT11, gu);
+  double GL[3][6];  // Gt_k,ij
+  inverse_metric<double>(F.u + V_GT11, F.gu);
 #pragma unroll
-  for (int s = 0; s < 6; ++s) gu2[s] = (s == 1 || s == 2 || s == 4) ? gu[s] + gu[s] : gu[s];
+  for (int s = 0; s < 6; ++s) F.gu2[s] = (s == 1 || s == 2 || s == 4) ? F.gu[s] + F.gu[s] : F.gu[s];
 #pragma unroll
   for (int k = 0; k < 3; ++k)
 #pragma unroll
     for (int s = 0; s < 6; ++s) {
       const int i = sym_i(s), j = sym_j(s);
-      GL[k][s] = 0.5 * (dg[i][sym(k, j)] + dg[j][sym(k, i)] - dg[k][s]);
+      GL[k][s] = 0.5 * (F.dg[i][sym(k, j)] + F.dg[j][sym(k, i)] - F.dg[k][s]);
     }
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
 #pragma unroll
     for (int s = 0; s < 6; ++s)
-      GU[k][s] = gu[sym(k, 0)] * GL[0][s] + gu[sym(k, 1)] * GL[1][s] + gu[sym(k, 2)] * GL[2][s];
-    double t = gu2[0] * GU[k][0];
+      F.GU[k][s] = F.gu[sym(k, 0)] * GL[0][s] + F.gu[sym(k, 1)] * GL[1][s] + F.gu[sym(k, 2)] * GL[2][s];
+    double t = F.gu2[0] * F.GU[k][0];
 #pragma unroll
-    for (int s = 1; s < 6; ++s) t += gu2[s] * GU[k][s];
-    Gd[k] = t;
+    for (int s = 1; s < 6; ++s) t += F.gu2[s] * F.GU[k][s];
+    F.Gd[k] = t;
   }
-  const double* A = u + V_AT11;
+}
+
+// Momentum (out[0..2]) and Gamma (out[3..5]) constraints.
+__device__ __forceinline__ void momentum64(const First64& F, double out[6]) {
+  const double iW = 1.0 / F.u[V_W];
+  const double* A = F.u + V_AT11;
   double Am[3][3];  // At^i_j
 #pragma unroll
   for (int i = 0; i < 3; ++i)
 #pragma unroll
     for (int j = 0; j < 3; ++j)
-      Am[i][j] = gu[sym(i, 0)] * A[sym(0, j)] + gu[sym(i, 1)] * A[sym(1, j)] + gu[sym(i, 2)] * A[sym(2, j)];
+      Am[i][j] = F.gu[sym(i, 0)] * A[sym(0, j)] + F.gu[sym(i, 1)] * A[sym(1, j)] + F.gu[sym(i, 2)] * A[sym(2, j)];
   // M_i = gt^jk (d_k At_ij - Gt^l_ki At_lj - Gt^l_kj At_il) - 3/W At^j_i d_j W - 2/3 d_i K
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
@@ -387,19 +399,19 @@ __device__ __forceinline__ void momentum64(const double* __restrict__ up, long l
 #pragma unroll
     for (int s = 0; s < 6; ++s) {  // twice the summand, symmetrised over (j, k)
       const int j = sym_i(s), k = sym_j(s);
-      double t = dAt[k][sym(i, j)] + dAt[j][sym(i, k)];
+      double t = F.dAt[k][sym(i, j)] + F.dAt[j][sym(i, k)];
 #pragma unroll
       for (int l = 0; l < 3; ++l) {
-        t -= GU[l][sym(k, i)] * A[sym(l, j)] + GU[l][sym(k, j)] * A[sym(i, l)];
-        t -= GU[l][sym(j, i)] * A[sym(l, k)] + GU[l][sym(j, k)] * A[sym(i, l)];
+        t -= F.GU[l][sym(k, i)] * A[sym(l, j)] + F.GU[l][sym(k, j)] * A[sym(i, l)];
+        t -= F.GU[l][sym(j, i)] * A[sym(l, k)] + F.GU[l][sym(j, k)] * A[sym(i, l)];
       }
-      div += gu2[s] * t;
+      div += F.gu2[s] * t;
     }
-    const double aw = Am[0][i] * dW[0] + Am[1][i] * dW[1] + Am[2][i] * dW[2];
-    out[i] = 0.5 * div - 3.0 * iW * aw - (2.0 / 3.0) * dK[i];
+    const double aw = Am[0][i] * F.dW[0] + Am[1][i] * F.dW[1] + Am[2][i] * F.dW[2];
+    out[i] = 0.5 * div - 3.0 * iW * aw - (2.0 / 3.0) * F.dK[i];
   }
 #pragma unroll
-  for (int i = 0; i < 3; ++i) out[3 + i] = u[V_GAM1 + i] - Gd[i];
+  for (int i = 0; i < 3; ++i) out[3 + i] = F.u[V_GAM1 + i] - F.Gd[i];
 }
 
 }  // namespace bssn

@@ -62,7 +62,7 @@ static cudaError_t launch_algebra(const AlgebraArgs& A, long long n, int vol, in
   return cudaGetLastError();
 }
 
-// The set of the Hamiltonian constraint at one point.
+// What the Hamiltonian constraint and the conformal Ricci tensor take, at one point.
 __device__ __forceinline__ void load_ham(const double* __restrict__ rec, int vol, const double* __restrict__ u,
                                          long long vs, Point64& Q) {
   auto r = [&](int o) { return __ldg(rec + o * vol); };
@@ -84,18 +84,6 @@ __device__ __forceinline__ void load_ham(const double* __restrict__ rec, int vol
   }
 }
 
-// And of the Weyl scalars, which take the derivatives of K and At_ij too.
-__device__ __forceinline__ void load_weyl(const double* __restrict__ rec, int vol, const double* __restrict__ u,
-                                          long long vs, Point64& Q, double dAt[3][6]) {
-  load_ham(rec, vol, u, vs, Q);
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    Q.dK[d] = __ldg(rec + (REC_C_K + d) * vol);
-#pragma unroll
-    for (int s = 0; s < 6; ++s) dAt[d][s] = __ldg(rec + (REC_C_AT + 3 * s + d) * vol);
-  }
-}
-
 struct ConArgs {
   FxWork W;
   double *ham, *mom, *gcon, *part;
@@ -110,7 +98,7 @@ struct ConArgs {
 // fixed order. H = 0: the Hamiltonian constraint alone (the momentum and
 // Gamma slots stay 0); its values are the same bits as in the full evaluation.
 // H = p/2: the momentum and Gamma constraints too, from the state itself
-// (momentum64). Bound by the FP64 pipe (128 registers and 4 blocks an SM, as
+// (first64). Bound by the FP64 pipe (128 registers and 4 blocks an SM, as
 // the algebra).
 template <int H>
 __global__ void __launch_bounds__(CON_THREADS, 4) k_constraints(const __grid_constant__ ConArgs A, unsigned int nblocks,
@@ -132,7 +120,9 @@ __global__ void __launch_bounds__(CON_THREADS, 4) k_constraints(const __grid_con
     if constexpr (H > 0) {
       if (!in_range(p - H * G.L.sz, p + H * G.L.sz, padded_points(G.L))) continue;
       const long long st[3] = {1, G.L.sy, G.L.sz};
-      momentum64<H>(u, vs, st, A.c1, c + 1);
+      First64 F;
+      first64<H>(u, vs, st, A.c1, F);
+      momentum64(F, c + 1);
       if (A.mom)
 #pragma unroll
         for (int a = 0; a < 3; ++a) A.mom[a * vs + p] = c[1 + a];
@@ -186,10 +176,14 @@ struct WeylArgs {
   double o[3], h[3];
   double *psi_re, *psi_im, *inv_re, *inv_im, *E, *B;
   unsigned int* flag;
+  double c1[3][5];  // first-derivative weights over the spacing
 };
 
 // Weyl scalars, one point per thread; outputs in the state's padded layout
-// (E and B as 6 arrays var_stride apart), each nullable. FP64-pipe bound.
+// (E and B as 6 arrays var_stride apart), each nullable. The conformal Ricci
+// tensor comes from the record, the rest from the state (first64, H = p/2).
+// FP64-pipe bound.
+template <int H>
 __global__ void __launch_bounds__(CON_THREADS, 4) k_psi4(const __grid_constant__ WeylArgs A, int blocks_per_slot) {
   const unsigned int slot = blockIdx.x / (unsigned int)blocks_per_slot;
   const int idx = (int)(blockIdx.x - slot * blocks_per_slot) * CON_THREADS + threadIdx.x;
@@ -198,31 +192,26 @@ __global__ void __launch_bounds__(CON_THREADS, 4) k_psi4(const __grid_constant__
   TilePoint pt;
   if (!tile_point(G, ti, tj, tk, idx, pt)) return;
   const long long p = pt.p, vs = G.L.vs;
-  Point64 Q;
-  double dAt[3][6];
-  load_weyl(A.W.rec + (long long)slot * A.W.slot + idx, G.T.vol, G.buf[1] + p, vs, Q, dAt);
-  // Weyl scalars take the derivatives' values
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    Q.dW[d] *= G.C.a;
-    Q.dK[d] *= G.C.a;
+  if (!in_range(p - H * G.L.sz, p + H * G.L.sz, padded_points(G.L))) return;
+  const double* __restrict__ u = G.buf[1] + p;
+  double ddW[6], R[6];
+  {
+    Point64 Q;
+    load_ham(A.W.rec + (long long)slot * A.W.slot + idx, G.T.vol, u, vs, Q);
+    Conformal64 C;
+    conformal64(Q, G.C.ia, C);
 #pragma unroll
     for (int s = 0; s < 6; ++s) {
-      Q.hg[d][s] *= G.C.a;
-      dAt[d][s] *= G.C.a;
+      ddW[s] = Q.ddW[s] * G.C.a2;
+      R[s] = C.R[s] * G.C.a2;
     }
-#pragma unroll
-    for (int c = 0; c < 3; ++c) Q.hG[d][c] *= G.C.a;
   }
-#pragma unroll
-  for (int s = 0; s < 6; ++s) {
-    Q.ddW[s] *= G.C.a2;
-#pragma unroll
-    for (int c = 0; c < 6; ++c) Q.hgg[c][s] *= G.C.a2;
-  }
+  First64 F;
+  const long long st[3] = {1, G.L.sy, G.L.sz};
+  first64<H>(u, vs, st, A.c1, F);
   const double xyz[3] = {A.o[0] + pt.i * A.h[0], A.o[1] + pt.j * A.h[1], A.o[2] + pt.k * A.h[2]};
   WeylOut O;
-  weyl_point(Q, dAt, xyz, O);
+  weyl_point(F, ddW, R, xyz, O);
   const bool bad = !isfinite(O.psi_re) || !isfinite(O.psi_im) || !isfinite(O.inv_re) || !isfinite(O.inv_im);
   if (A.psi_re) A.psi_re[p] = O.psi_re;
   if (A.psi_im) A.psi_im[p] = O.psi_im;
@@ -259,15 +248,19 @@ static cudaError_t through_record(int order, const FxWork& work, const DerivList
   return cudaSuccess;
 }
 
+static void first_weights(int order, const double h[3], double c1[3][5]) {
+  for (int d = 0; d < 3; ++d)
+    for (int a = 1; a <= order / 2; ++a) c1[d][a] = (order == 4 ? FD<4>::W1[a] : FD<8>::W1[a]) / h[d];
+}
+
 cudaError_t launch_constraints(int order, FxWork work, const double h[3], size_t rec_doubles, double* ham, double* mom,
                                double* gcon, double* part, long long max_parts, int* nparts, unsigned int* flag,
                                bool ham_only, cudaStream_t s) {
   ConArgs A{work, ham, mom, gcon, part, flag, {}};
-  for (int d = 0; d < 3; ++d)
-    for (int a = 1; a <= order / 2; ++a) A.c1[d][a] = (order == 4 ? FD<4>::W1[a] : FD<8>::W1[a]) / h[d];
+  first_weights(order, h, A.c1);
   const int bps = (work.one.T.vol + CON_THREADS - 1) / CON_THREADS;
   *nparts = 0;
-  return through_record(order, work, con_list(true), rec_doubles, s, [&](const FxWork& W, long long n, bool first) {
+  return through_record(order, work, ham_list(), rec_doubles, s, [&](const FxWork& W, long long n, bool first) {
     A.W = W;
     // as many blocks as are resident (4 on each of 152 SMs): each takes the
     // points of several tiles, and the partial sums stay few
@@ -286,11 +279,15 @@ cudaError_t launch_constraints(int order, FxWork work, const double h[3], size_t
 cudaError_t launch_psi4(int order, FxWork work, size_t rec_doubles, const double origin[3], const double h[3],
                         double* psi_re, double* psi_im, double* inv_re, double* inv_im, double* E, double* B,
                         unsigned int* flag, cudaStream_t s) {
-  WeylArgs A{work, {origin[0], origin[1], origin[2]}, {h[0], h[1], h[2]}, psi_re, psi_im, inv_re, inv_im, E, B, flag};
+  WeylArgs A{work, {origin[0], origin[1], origin[2]}, {h[0], h[1], h[2]}, psi_re, psi_im, inv_re, inv_im, E, B, flag, {}};
+  first_weights(order, h, A.c1);
   const int bps = (work.one.T.vol + CON_THREADS - 1) / CON_THREADS;
-  return through_record(order, work, con_list(false), rec_doubles, s, [&](const FxWork& W, long long n, bool) {
+  return through_record(order, work, ham_list(), rec_doubles, s, [&](const FxWork& W, long long n, bool) {
     A.W = W;
-    k_psi4<<<(unsigned int)(n * bps), CON_THREADS, 0, s>>>(A, bps);
+    if (order == 4)
+      k_psi4<2><<<(unsigned int)(n * bps), CON_THREADS, 0, s>>>(A, bps);
+    else
+      k_psi4<4><<<(unsigned int)(n * bps), CON_THREADS, 0, s>>>(A, bps);
   });
 }
 

@@ -27,34 +27,34 @@ __device__ __forceinline__ double sdot3(const double* g, const double* a, const 
          a[2] * (g[2] * b[0] + g[4] * b[1] + g[5] * b[2]);
 }
 
-__device__ __forceinline__ void weyl_point(const Point64& P, const double dAt[3][6], const double xyz[3],
+// P: the state's first derivatives and what is made of them; ddW and R: second
+// derivatives of W, conformal Ricci tensor (overwritten with R_ij).
+__device__ __forceinline__ void weyl_point(const First64& P, const double ddW[6], double R[6], const double xyz[3],
                                            WeylOut& O) {
   const double W = P.u[V_W], K = P.u[V_TRK];
   const double iW = 1.0 / W, iW2 = iW * iW;
-  Conformal64 G;
-  conformal64(P, 1.0, G);
   const double* gt = P.u + V_GT11;
   // R_ij = Rt_ij + (DtDt_ij W + gt_ij gt^kl DtDt_kl W) / W - 2 gt_ij gt^kl d_k W d_l W / W^2
   double dWu[3], DDW[6], tr = 0.0, dWdW = 0.0;
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    dWu[k] = G.gu[sym(k, 0)] * P.dW[0] + G.gu[sym(k, 1)] * P.dW[1] + G.gu[sym(k, 2)] * P.dW[2];
+    dWu[k] = P.gu[sym(k, 0)] * P.dW[0] + P.gu[sym(k, 1)] * P.dW[1] + P.gu[sym(k, 2)] * P.dW[2];
     dWdW += dWu[k] * P.dW[k];
   }
 #pragma unroll
   for (int s = 0; s < 6; ++s) {
-    DDW[s] = P.ddW[s] - (G.GU[0][s] * P.dW[0] + G.GU[1][s] * P.dW[1] + G.GU[2][s] * P.dW[2]);
-    tr += G.gu2[s] * DDW[s];
+    DDW[s] = ddW[s] - (P.GU[0][s] * P.dW[0] + P.GU[1][s] * P.dW[1] + P.GU[2][s] * P.dW[2]);
+    tr += P.gu2[s] * DDW[s];
   }
   const double fac = (tr - 2.0 * dWdW * iW) * iW;
 #pragma unroll
-  for (int s = 0; s < 6; ++s) G.R[s] += DDW[s] * iW + gt[s] * fac;
+  for (int s = 0; s < 6; ++s) R[s] += DDW[s] * iW + gt[s] * fac;
   const double* At = P.u + V_AT11;
   double gam[6], gamu[6], Kd[6];
 #pragma unroll
   for (int s = 0; s < 6; ++s) {
     gam[s] = gt[s] * iW2;
-    gamu[s] = G.gu[s] * (W * W);
+    gamu[s] = P.gu[s] * (W * W);
     Kd[s] = (At[s] + gt[s] * (K / 3.0)) * iW2;
   }
   // K^k_j (full) and E
@@ -68,7 +68,7 @@ __device__ __forceinline__ void weyl_point(const Point64& P, const double dAt[3]
   for (int s = 0; s < 6; ++s) {
     const int i = sym_i(s), j = sym_j(s);
     const double kk = Kd[sym(i, 0)] * Km[0][j] + Kd[sym(i, 1)] * Km[1][j] + Kd[sym(i, 2)] * Km[2][j];
-    O.E[s] = G.R[s] + K * Kd[s] - kk;
+    O.E[s] = R[s] + K * Kd[s] - kk;
   }
   // physical Christoffels Gamma^k_ij = Gt^k_ij - (d^k_i W_j + d^k_j W_i - gt_ij gt^kl W_l) / W
   double Gp[3][6];
@@ -80,13 +80,13 @@ __device__ __forceinline__ void weyl_point(const Point64& P, const double dAt[3]
       double t = -gt[s] * dWu[k];
       if (k == i) t += P.dW[j];
       if (k == j) t += P.dW[i];
-      Gp[k][s] = G.GU[k][s] - t * iW;
+      Gp[k][s] = P.GU[k][s] - t * iW;
     }
   // curl part: C_ij = gamma_im eps^mkl D_k K_lj, with D_k K_lj = d_k K_lj - Gp^n_kl K_nj - Gp^n_kj K_ln
   auto DK = [&](int k, int l, int j) {
     const int s = sym(l, j);
     const double num = At[s] + gt[s] * (K / 3.0);
-    double d = (dAt[k][s] + P.hg[k][s] * (K * (2.0 / 3.0)) + gt[s] * (P.dK[k] / 3.0)) * iW2 - 2.0 * num * P.dW[k] * iW2 * iW;
+    double d = (P.dAt[k][s] + P.dg[k][s] * (K / 3.0) + gt[s] * (P.dK[k] / 3.0)) * iW2 - 2.0 * num * P.dW[k] * iW2 * iW;
 #pragma unroll
     for (int n = 0; n < 3; ++n) d -= Gp[n][sym(k, l)] * Kd[sym(n, j)] + Gp[n][sym(k, j)] * Kd[sym(l, n)];
     return d;

@@ -26,9 +26,9 @@ GOLDEN = os.path.join(os.path.dirname(os.path.abspath(__file__)), "golden", "mom
 NX, NY, NZ, ORDER, G = 40, 3, 4, 8, 5
 
 
-def read_golden():
+def read_golden(path=GOLDEN):
     d = {}
-    with open(GOLDEN) as f:
+    with open(path) as f:
         for line in f:
             kind, name, *v = line.split()
             d[kind, name] = np.array([float.fromhex(x) for x in v])
@@ -67,3 +67,23 @@ def test_momentum_constraint_of_a_gauge_wave():
         # they do cancel: far below the derivatives they are made of
         assert 0 < np.max(np.abs(want)) < 1e-6
         assert np.linalg.norm(got[kind] - want) <= 1e-9 * np.linalg.norm(want), kind
+
+
+def gpu_weyl_b(u):
+    torch = need_gpu()
+    grid, p = grid_for(u, G, 1.0 / NX), B.make_params(fd_order=ORDER)
+    b = torch.zeros(6 * grid.var_stride, dtype=torch.float64, device="cuda")
+    B.psi4(grid, p, B.upload(u, grid), (0.1, 0.2, 0.3), B.alloc_work(grid, p), B=b)
+    torch.cuda.synchronize()
+    return interior(B.view4(b, grid, 6).cpu().numpy(), G)
+
+
+def test_magnetic_weyl_tensor_of_a_gauge_wave():
+    """It vanishes on a gauge wave by the same kind of cancellation (golden/
+    weyl_b_gauge_wave.txt: "B <packed component> <values>")."""
+    d = read_golden()
+    got = gpu_weyl_b(state({n: p for (k, n), p in d.items() if k == "profile"}))
+    w = read_golden(GOLDEN.replace("momentum", "weyl_b"))
+    want = np.array([w["B", str(c)].reshape(NZ, NY, NX) for c in range(6)])
+    assert 0 < np.max(np.abs(want)) < 1e-6
+    assert np.linalg.norm(got - want) <= 1e-9 * np.linalg.norm(want)
