@@ -11,18 +11,20 @@
 //    n = trunc(u 2^(59-E)), |n| < 2^59: six bits more than a double's
 //    significand has. Values within 2^-6 of 2^E are held exactly, smaller ones
 //    to 2^(E-59).
-//  * a derivative is taken from these integers only where they are no coarser
-//    than the rounding of a double-precision stencil: where some value that its
-//    own stencil reads is at least 2^(E-7), so that 2^(E-59) is no more than that
-//    value's last bit (which a difference of two such values is rounded to). The
-//    others (of points beside a spike or a steep front of the tile, or along a
-//    line or in a plane on which the variable is nearly zero: some 0.05 % of
-//    the points of puncture data) are made from the doubles (fx_fallback), and
-//    so are all of a tile whose values are not all finite, or so large or small
-//    that the scaling could leave the range of doubles: infinities and NaNs
-//    then reach exactly the points whose stencils touch them. What a derivative
-//    is good to depends on what its stencil reads, and not on what else its
-//    tile holds.
+//  * that is enough for a derivative whose own stencil reads some value of at
+//    least 2^(E-7): 2^(E-59) is then no more than that value's last bit, which a
+//    difference of two such values is rounded to in double precision. Where a
+//    point has others (beside a spike or a steep front of the tile, or along a
+//    line or in a plane on which the variable is nearly zero: 1 to 3 % of the
+//    points of evolved puncture data, in 5 to 15 % of the tiles), what the
+//    integers leave out of the tile's values is kept as single-precision
+//    fractions of their unit, and the same stencils of those are added
+//    (fx_refine). What is coarser still (values of 2^(E-28), 24 bits of the
+//    fractions), and all of a tile whose values are not all finite, or so large
+//    or small that the scaling could leave the range of doubles, is made from
+//    the doubles (fx_fallback): infinities and NaNs then reach exactly the
+//    points whose stencils touch them. What a derivative is good to depends on
+//    what its stencil reads, and not on what else its tile holds.
 //  * n is kept as two limbs, n = hi 2^30 + lo with 0 <= lo < 2^30, so that
 //    differences a - b and paired sums a + b - 2c of limbs fit 32 bits and a
 //    weighted sum is one 32 x 32 + 64 bit multiply-add per limb. The weights
@@ -44,8 +46,9 @@
 // pipe (4375 FP64 instructions per point), 6.2 ms this way (941). Against a
 // quadruple-precision evaluation the right-hand side's error is no larger than
 // before in any variable, and 1e-16 instead of 1e-14 for W, gt_ii and alpha.
-// Looking after coarse derivatives costs 2 % of a step at 128^3, 6 % of a small
-// hierarchy's, whose launches end with the slowest tile.
+// Looking after coarse derivatives costs 3 % of an RK4 step of evolved punctures
+// at 128^3 (25.5 -> 26.25 ms), 5 % of a small hierarchy's, 6 % of an RK3 step at
+// 100^3; from the doubles alone, 18 %, 8 % and 57 %.
 #pragma once
 #include <cmath>
 #include <type_traits>
@@ -218,6 +221,7 @@ __device__ __forceinline__ unsigned long long fx_shl(unsigned long long x, int n
 constexpr int FX_LIMB = 30;
 constexpr unsigned int FX_MASK = (1u << FX_LIMB) - 1;
 constexpr int FX_HELD = 1 << 22;  // high limb of a value of 2^(E-7)
+constexpr int FX_FINE = 2;        // of a value of 2^(E-28), of which fx_rest adds enough
 
 // limbs (lo, hi) of trunc(u 2^(1081 - emax)), emax the largest biased exponent
 __device__ __forceinline__ int2 fx_from_double(double u, int emax) {
@@ -231,6 +235,17 @@ __device__ __forceinline__ int2 fx_from_double(double u, int emax) {
   const unsigned long long s = (unsigned long long)(long long)(h >> 31);
   const long long n = (long long)((fx_shr(m, emax - ex) ^ s) - s);
   return make_int2((int)((unsigned int)n & FX_MASK), (int)(n >> FX_LIMB));
+}
+
+// What fx_from_double leaves out: u 2^(1081 - emax) - n, in (-1, 1), to 2^-32
+__device__ __forceinline__ float fx_rest(double u, int emax) {
+  const int h = __double2hiint(u);
+  const unsigned int l = (unsigned int)__double2loint(u);
+  const int sh = emax - ((h >> 20) & 0x7ff);
+  const unsigned int mh = ((unsigned int)h & 0xfffffu) | 0x100000u;
+  const unsigned long long m = ((unsigned long long)__funnelshift_l(l, mh, 6) << 32) | (l << 6);
+  const float r = __uint2float_rn((unsigned int)((fx_shl(m, 64 - sh) | fx_shr(m, sh - 64)) >> 32)) * 0x1p-32f;
+  return h < 0 ? -r : r;
 }
 
 // The sum of two values, rounded to 53 significant bits (ties to even) as a
@@ -277,6 +292,7 @@ __device__ __forceinline__ double fx_to_double(long long hi, long long lo, int e
 // the mixed ones (FX_MIXED for xy, then xz, yz), the axis' share of advection
 // and dissipation (FX_EXT << d).
 constexpr int FX_AXIS = 1, FX_MIXED = 8, FX_EXT = 64, FX_ALL = 511;
+constexpr int FX_BEYOND = 9;  // those shifted by this: too coarse for fx_refine as well
 
 // The derivatives `which` of a point that fixed point does not hold. v: the
 // variable, p: the point; has1, has2, hase: which of them the variable's record
@@ -381,6 +397,73 @@ struct FxSmem {
   static constexpr size_t bytes = sizeof(int2) * BOX + 3 * sizeof(int4) * GN;
 };
 
+// Adds to the derivatives `which` of a point what the integers left out of the
+// values that its stencils read (r: fx_rest of the point's, in a box like the
+// integers'). That is less than one unit a value, so single precision brings a
+// sum to 2^-24 of a unit and a derivative to what its own stencil's doubles
+// allow. Added in memory, where the point's thread has just written the rest.
+template <int P>
+__device__ __noinline__ void fx_refine(const float* __restrict__ r, const FxCoef& C, const double* __restrict__ beta,
+                                       long long vs, bool adv, int which, bool has1, bool has2, int emax, int emax1,
+                                       int emax2, double* __restrict__ o1, double* __restrict__ o2,
+                                       double* __restrict__ oe, int vol) {
+  using F = FD<P>;
+  using X = FX<P>;
+  constexpr int H = F::H, R = F::R, BX = FxSmem<P>::BX;
+  // 2^(emax - 1081), the integers' unit
+  const double unit = __hiloint2double((emax - 58) << 20, 0), unit1 = __hiloint2double((emax1 - 58) << 20, 0),
+               unit2 = __hiloint2double((emax2 - 58) << 20, 0);
+  const float r0 = r[0];
+  double ext = 0.0;
+#pragma unroll 1
+  for (int d = 0; d < 3; ++d) {
+    if (!(which & ((FX_AXIS | FX_EXT) << d))) continue;
+    const int st = d == 0 ? 1 : (d == 1 ? BX : BX * BX);
+    float c1 = 0.f, c2 = 0.f, k = 0.f, t = 0.f;
+#pragma unroll
+    for (int a = 1; a <= R; ++a) {
+      const float p = r[a * st], m = r[-a * st], df = p - m, s = p + m - 2.f * r0;
+      if (a <= H) {
+        c1 = fmaf((float)X::W1(a), df, c1);
+        c2 = fmaf((float)X::W2(a), s, c2);
+      }
+      k = fmaf((float)X::WK(a), s, k);
+      t = fmaf((float)X::WT(a), df, t);
+    }
+    if (which & (FX_AXIS << d)) {
+      if (has1) atomicAdd(o1 + d * vol, (double)c1 * (C.cubic ? unit1 : C.c1[d] * unit1));
+      if (has2) atomicAdd(o2 + sym(d, d) * vol, (double)c2 * (C.cubic ? unit2 : C.c2[sym(d, d)] * unit2));
+    }
+    if (which & (FX_EXT << d)) {
+      ext = fma(C.ck[d], (double)k, ext);
+      if (adv) {
+        const double b = beta[d * vs];
+        ext = fma(C.cu[d] * b, (double)(t + (b < 0.0 ? -(float)X::SK : (float)X::SK) * k), ext);
+      }
+    }
+  }
+  if (which & (FX_EXT | FX_EXT << 1 | FX_EXT << 2)) atomicAdd(oe, ext * unit);
+  int pair = FX_MIXED;
+#pragma unroll 1
+  for (int q = 0; q < 3; ++q, pair <<= 1) {
+    if (!(which & pair)) continue;
+    const int si = q < 2 ? 1 : BX, sj = q == 0 ? BX : BX * BX;
+    float c = 0.f;
+#pragma unroll
+    for (int a = 1; a <= H; ++a) {
+      float t = 0.f;
+#pragma unroll
+      for (int b = 1; b <= H; ++b) {
+        const float *p = r + a * si, *m = r - a * si;
+        t = fmaf((float)X::W1(b), (p[b * sj] - m[b * sj]) - (p[-b * sj] - m[-b * sj]), t);
+      }
+      c = fmaf((float)X::W1(a), t, c);
+    }
+    const int o = q == 2 ? 4 : q + 1;
+    atomicAdd(o2 + o * vol, (double)c * (C.cubic ? unit2 : C.c2[o] * unit2));
+  }
+}
+
 // three limbs of sum_a W1[a] (n_a - n_-a) along stride st, and the largest
 // magnitude (high limb) among the n
 template <int P>
@@ -420,9 +503,9 @@ __device__ __forceinline__ double fx_mixed(const int4* __restrict__ g, int st, i
   return fx_to_double(hi, l0 & (long long)FX_MASK, emax);
 }
 
-// Whether some value that the upwinded stencil along st reads is as large as FX_HELD.
+// The largest magnitude among the values that the upwinded stencil along st reads.
 template <int P>
-__device__ __noinline__ bool fx_upwind_held(const int2* __restrict__ c, int st) {
+__device__ __noinline__ int fx_upwind_mag(const int2* __restrict__ c, int st) {
   int top = 0, low = 0;
 #pragma unroll
   for (int i = 0; i < FD<P>::UPN; ++i) {
@@ -430,17 +513,18 @@ __device__ __noinline__ bool fx_upwind_held(const int2* __restrict__ c, int st) 
     top = max(top, v);
     low = min(low, v);
   }
-  return max(top, ~low) >= FX_HELD;
+  return max(top, ~low);
 }
 
 // Stencils along the three axes at one point of the box, and the outputs.
 // Returns those that fixed point holds too coarsely, where no value that the
-// stencil reads is as large as FX_HELD. Advection and dissipation leave such
-// axes out, for fx_fallback to add. Along an axis the values looked at are those
-// of the centred stencils, H on each side. The upwinded stencil does not read
-// the last of them on one side: a large value there enters through the
-// dissipation, and advection is good to parts in 1e14 of that; where there
-// is little or none (weak) its own values are looked at.
+// stencil reads is as large as FX_HELD, and << FX_BEYOND those where none is
+// even as large as FX_FINE (advection and dissipation leave such axes out, for
+// fx_fallback to add). Along an axis the values looked at are those of the
+// centred stencils, H on each side. The upwinded stencil does not read the last
+// of them on one side: a large value there enters through the dissipation, and
+// advection is good to parts in 1e14 of that; where there is little or none
+// (weak) its own values are looked at.
 template <int P, bool CUBIC, bool D1, bool D2, bool EXT>
 __device__ __forceinline__ int fx_point(const int2* __restrict__ c, const int4* const g[3], const FxCoef& C,
                                         const double* beta, bool adv, bool inexact, int emax, int emax1, int emax2,
@@ -487,12 +571,19 @@ __device__ __forceinline__ int fx_point(const int2* __restrict__ c, const int4* 
         kh += (long long)X::WK(a) * (p.y + m.y + m2y);
       }
     }
-    const bool held = (D2 && d < 2 ? f.w : max(top, ~low)) >= FX_HELD || !inexact;
-    bool share = held;
-    if ((D1 || D2) && !held) coarse |= FX_AXIS << d;
-    if (EXT) {
-      if (C.weak && inexact && adv) share = fx_upwind_held<P>(c, beta[d] < 0.0 ? -st : st);
-      if (!share) coarse |= FX_EXT << d;
+    const int mag = D2 && d < 2 ? f.w : max(top, ~low);
+    bool share = true;
+    if (mag < FX_HELD && inexact) {
+      const int far = mag < FX_FINE ? 1 | 1 << FX_BEYOND : 1;
+      if (D1 || D2) coarse |= far * (FX_AXIS << d);
+      if (EXT) coarse |= far * (FX_EXT << d);
+      share = mag >= FX_FINE;
+    }
+    if (EXT && C.weak && inexact && adv) {
+      const int um = fx_upwind_mag<P>(c, beta[d] < 0.0 ? -st : st);
+      coarse &= ~((1 | 1 << FX_BEYOND) * (FX_EXT << d));
+      if (um < FX_HELD) coarse |= (um < FX_FINE ? 1 | 1 << FX_BEYOND : 1) * (FX_EXT << d);
+      share = um >= FX_FINE;
     }
     if (D1) {
       if (D2 && d < 2) {
@@ -528,7 +619,7 @@ __device__ __forceinline__ int fx_point(const int2* __restrict__ c, const int4* 
                  yz = fx_mixed<P>(g[2], FX_T * FX_T, emax2, mag[2]);
 #pragma unroll
     for (int q = 0; q < 3; ++q)
-      if (mag[q] < FX_HELD && inexact) coarse |= FX_MIXED << q;
+      if (mag[q] < FX_HELD && inexact) coarse |= (mag[q] < FX_FINE ? 1 | 1 << FX_BEYOND : 1) * (FX_MIXED << q);
     o2[1 * vol] = CUBIC ? xy : C.c2[1] * xy;
     o2[2 * vol] = CUBIC ? xz : C.c2[2] * xz;
     o2[4 * vol] = CUBIC ? yz : C.c2[4] * yz;
@@ -617,26 +708,29 @@ __device__ __forceinline__ void fx_tile(const Layout& L, const FxCoef& C, const 
   double raw[PER];
   unsigned int at[PER];
   unsigned int mx = 0, any = 0, mn = 0xffffffffu;
+  auto load = [&]() {
 #pragma unroll
-  for (int q = 0; q < PER; ++q) {
-    raw[q] = 0.0;
-    at[q] = 0xffffffffu;
-    if (q >= PERL && !mixed) continue;
-    const int c = threadIdx.x + q * FX_THREADS;
-    if (c < count) at[q] = __ldg(&g_fx_box<P>.at[c]);
-  }
-#pragma unroll
-  for (int q = 0; q < PER; ++q) {
-    if (q >= PERL && !mixed) continue;
-    const int bx = at[q] & 31, by = (at[q] >> 5) & 31, bz = (at[q] >> 10) & 31;
-    // (a box spans less than 2^31 elements of a variable unless a plane of
-    // the array alone has 2^26 points)
-    const long long o = wide ? bx + by * L.sy + bz * L.sz : (long long)(bx + by * sy + bz * sz);
-    if (full ? at[q] != 0xffffffffu : reads(bx, by, bz)) {
-      if (in_range(org - R * (1 + L.sy + L.sz) + o, org - R * (1 + L.sy + L.sz) + o, padded_points(L)))
-        raw[q] = __ldg(v0 + o);
+    for (int q = 0; q < PER; ++q) {
+      raw[q] = 0.0;
+      at[q] = 0xffffffffu;
+      if (q >= PERL && !mixed) continue;
+      const int c = threadIdx.x + q * FX_THREADS;
+      if (c < count) at[q] = __ldg(&g_fx_box<P>.at[c]);
     }
-  }
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+      if (q >= PERL && !mixed) continue;
+      const int bx = at[q] & 31, by = (at[q] >> 5) & 31, bz = (at[q] >> 10) & 31;
+      // (a box spans less than 2^31 elements of a variable unless a plane of
+      // the array alone has 2^26 points)
+      const long long o = wide ? bx + by * L.sy + bz * L.sz : (long long)(bx + by * sy + bz * sz);
+      if (full ? at[q] != 0xffffffffu : reads(bx, by, bz)) {
+        if (in_range(org - R * (1 + L.sy + L.sz) + o, org - R * (1 + L.sy + L.sz) + o, padded_points(L)))
+          raw[q] = __ldg(v0 + o);
+      }
+    }
+  };
+  load();
 #pragma unroll
   for (int q = 0; q < PER; ++q) {
     const unsigned int hw = (unsigned int)__double2hiint(raw[q]) & 0x7fffffffu;
@@ -703,16 +797,16 @@ __device__ __forceinline__ void fx_tile(const Layout& L, const FxCoef& C, const 
   // ---- one point per thread
   int x, y, z;
   fx_lane(threadIdx.x, x, y, z);
-  if (x >= ex || y >= ey || z >= ez) return;
   const int idx = (z * T.ty + y) * T.tx + x;
   const long long p = org + x + y * L.sy + z * L.sz;
-  if (!in_range(p - R * L.sz, p + R * L.sz, padded_points(L))) return;
+  const bool inside =
+      x < ex && y < ey && z < ez && in_range(p - R * L.sz, p + R * L.sz, padded_points(L));
   double beta[3] = {0.0, 0.0, 0.0};
-  if (ext && adv)
+  if (inside && ext && adv)
 #pragma unroll
     for (int d = 0; d < 3; ++d) beta[d] = __ldg(u + (V_BETA1 + d) * L.vs + p);
-  int coarse = FX_ALL;
-  if (!fallback) {
+  int coarse = inside && fallback ? FX_ALL | FX_ALL << FX_BEYOND : 0;
+  if (inside && !fallback) {
     const int2* c = box + ((z + R) * BX + (y + R)) * BX + x + R;
     const int4* const gt[3] = {g + (z * S::EH + (y + H)) * FX_T + x, g + S::GN + ((z + H) * FX_T + y) * FX_T + x,
                                g + 2 * S::GN + ((z + H) * FX_T + y) * FX_T + x};
@@ -731,9 +825,33 @@ __device__ __forceinline__ void fx_tile(const Layout& L, const FxCoef& C, const 
     };
     coarse = C.cubic ? point(std::true_type{}) : point(std::false_type{});
   }
-  if (coarse)
-    fx_fallback<P>(v, p, L.sy, L.sz, C, u + V_BETA1 * L.vs + p, L.vs, adv, ko, coarse, d1, mixed, ext, list.s1[e] < 0,
-                   list.s2[e] < 0, o1 + idx, o2 + idx, oe + idx, vol);
+  // ---- where some value lost bits that a point needs, what the integers left
+  // out of all of them takes the box's place
+  if (!fallback && inexact) {
+    const bool some = __any_sync(0xffffffffu, coarse != 0);
+    if ((threadIdx.x & 31) == 0) red[0][threadIdx.x >> 5] = some;
+    fx_sync();
+    bool tile = false;
+#pragma unroll
+    for (int w = 0; w < FX_THREADS / 32; ++w) tile |= red[0][w] != 0;
+    if (tile) {
+      float* rest = (float*)box;
+      load();
+#pragma unroll
+      for (int q = 0; q < PER; ++q) {
+        if (q >= PERL && !mixed) continue;
+        if (at[q] != 0xffffffffu) rest[at[q] >> 16] = fx_rest(raw[q], emax);
+      }
+      fx_sync();
+      const int which = coarse & FX_ALL & ~(coarse >> FX_BEYOND);
+      if (which)
+        fx_refine<P>(rest + ((z + R) * BX + (y + R)) * BX + x + R, C, u + V_BETA1 * L.vs + p, L.vs, adv, which, d1,
+                     mixed, emax, emax1, emax2, o1 + idx, o2 + idx, oe + idx, vol);
+    }
+  }
+  if (coarse >> FX_BEYOND)
+    fx_fallback<P>(v, p, L.sy, L.sz, C, u + V_BETA1 * L.vs + p, L.vs, adv, ko, coarse >> FX_BEYOND, d1, mixed, ext,
+                   list.s1[e] < 0, list.s2[e] < 0, o1 + idx, o2 + idx, oe + idx, vol);
 }
 
 // One grid as the FP64 kernels see it: its layout, scales, tiles and buffers.

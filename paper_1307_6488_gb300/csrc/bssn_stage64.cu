@@ -279,7 +279,8 @@ cudaError_t launch_constraints(int order, FxWork work, const double h[3], size_t
 cudaError_t launch_psi4(int order, FxWork work, size_t rec_doubles, const double origin[3], const double h[3],
                         double* psi_re, double* psi_im, double* inv_re, double* inv_im, double* E, double* B,
                         unsigned int* flag, cudaStream_t s) {
-  WeylArgs A{work, {origin[0], origin[1], origin[2]}, {h[0], h[1], h[2]}, psi_re, psi_im, inv_re, inv_im, E, B, flag, {}};
+  WeylArgs A{work,   {origin[0], origin[1], origin[2]}, {h[0], h[1], h[2]}, psi_re, psi_im, inv_re, inv_im, E, B, flag,
+             {}};
   first_weights(order, h, A.c1);
   const int bps = (work.one.T.vol + CON_THREADS - 1) / CON_THREADS;
   return through_record(order, work, ham_list(), rec_doubles, s, [&](const FxWork& W, long long n, bool) {

@@ -139,8 +139,14 @@ __global__ void __launch_bounds__(OVERLAP_THREADS<P>, 1) k_overlap(const __grid_
     int2* box = (int2*)(g + 3 * FxSmem<P>::GN);
     const DerivArgs& D = A.D;
     const unsigned int items = A.nd * (unsigned int)D.list.n;
+    const unsigned int turn = A.nd / (unsigned int)D.list.n;
     for (unsigned int it = blockIdx.x; it < items; it += gridDim.x) {
-      const unsigned int e = it / A.nd, slot = it - e * A.nd;
+      // the chunk's tiles from another one on for every variable: a tile that
+      // takes long (fx_refine) does so for several, which are not to meet in one
+      // block (chunks are multiples of half a round; RK3 at 100^3 11.3 -> 10.4 ms)
+      const unsigned int e = it / A.nd;
+      unsigned int slot = it - e * A.nd + e * turn;
+      if (slot >= A.nd) slot -= A.nd;
       int ti, tj, tk;
       const FxGrid& G = fx_locate(D.W, D.W.tile0 + slot, ti, tj, tk);
       const double* u = G.buf[D.in];

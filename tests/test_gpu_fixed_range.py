@@ -37,7 +37,9 @@ def spiked(g, names, value, seed=9):
 
 @pytest.mark.parametrize("order", [4, 8])
 @pytest.mark.parametrize("h", [0.1, (0.11, 0.1, 0.13)])
-@pytest.mark.parametrize("big", [2.0 ** 20, 2.0 ** 60, 1e100])
+# on both sides of the ranges that integers alone (2^7), integers and fractions
+# (2^28) and doubles serve
+@pytest.mark.parametrize("big", [2.0 ** 4, 2.0 ** 9, 2.0 ** 20, 2.0 ** 26, 2.0 ** 30, 2.0 ** 60, 1e100])
 def test_spike_in_a_stage(order, h, big):
     torch = need_gpu()
     g, names = order // 2 + 1, ("Gt1", "trK", "At12", "beta2", "B3")
