@@ -669,6 +669,45 @@ __device__ __forceinline__ void fx_lane(int t, int& x, int& y, int& z) {
 // Barrier of the threads that work on a tile, the first FX_THREADS of a block.
 __device__ __forceinline__ void fx_sync() { asm volatile("bar.sync 1, %0;" ::"n"(FX_THREADS) : "memory"); }
 
+// Does some stencil of a tile of ex x ey x ez points read point (bx, by, bz) of
+// its box? (mixed: the variable has mixed derivatives, ext: dissipation, whose
+// lines are longer)
+template <int P>
+__device__ __forceinline__ bool fx_reads(int bx, int by, int bz, int ex, int ey, int ez, bool mixed, bool ext) {
+  constexpr int H = FxBox<P>::H, R = FxBox<P>::R;
+  const int ox = max(max(R - bx, bx - (R + ex - 1)), 0), oy = max(max(R - by, by - (R + ey - 1)), 0),
+            oz = max(max(R - bz, bz - (R + ez - 1)), 0), far = max(ox, max(oy, oz));
+  const int axes = (ox > 0) + (oy > 0) + (oz > 0);
+  return axes < 2 ? far <= (ext ? R : H) : axes == 2 && mixed && far <= H;
+}
+
+// fx_rest of the points of a tile's box (v: its first point, number `first` of
+// the `room` points of a variable). Apart from the rest of fx_tile, whose
+// registers it would share.
+template <int P>
+__device__ __noinline__ void fx_rest_box(const double* __restrict__ v, long long first, long long room, long long sy,
+                                         long long sz, int ex, int ey, int ez, bool mixed, bool ext, int emax,
+                                         float* __restrict__ rest) {
+  constexpr int PER = (FxBox<P>::ALL + FX_THREADS - 1) / FX_THREADS;
+  const int count = mixed ? FxBox<P>::ALL : FxBox<P>::LINES;
+  double raw[PER];
+#pragma unroll
+  for (int q = 0; q < PER; ++q) {
+    const int c = threadIdx.x + q * FX_THREADS;
+    raw[q] = 0.0;
+    if (c >= count) continue;
+    const unsigned int at = __ldg(&g_fx_box<P>.at[c]);
+    const int bx = at & 31, by = (at >> 5) & 31, bz = (at >> 10) & 31;
+    const long long o = bx + by * sy + bz * sz;
+    if (fx_reads<P>(bx, by, bz, ex, ey, ez, mixed, ext) && in_range(first + o, first + o, room)) raw[q] = __ldg(v + o);
+  }
+#pragma unroll
+  for (int q = 0; q < PER; ++q) {
+    const int c = threadIdx.x + q * FX_THREADS;
+    if (c < count) rest[__ldg(&g_fx_box<P>.at[c]) >> 16] = fx_rest(raw[q], emax);
+  }
+}
+
 // All outputs of list entry e on the tile (ti, tj, tk) of the grid L, written
 // to the record slot `rec` (nout x vol doubles), by the
 // first FX_THREADS threads of the block. box and g: shared memory for the tile
@@ -698,25 +737,19 @@ __device__ __forceinline__ void fx_tile(const Layout& L, const FxCoef& C, const 
   const double* __restrict__ v0 = v + (org - R * (1 + L.sy + L.sz));
   const bool d1 = list.d1[e] >= 0, ext = list.ext[e] >= 0;
   const bool full = ex == FX_T && ey == FX_T && ez == FX_T && ext, wide = L.sz >= (1 << 26);
-  auto reads = [&](int bx, int by, int bz) {  // does some point of the tile read this one?
-    const int ox = max(max(R - bx, bx - (R + ex - 1)), 0), oy = max(max(R - by, by - (R + ey - 1)), 0),
-              oz = max(max(R - bz, bz - (R + ez - 1)), 0), far = max(ox, max(oy, oz));
-    const int axes = (ox > 0) + (oy > 0) + (oz > 0);
-    return axes < 2 ? far <= (ext ? R : H) : axes == 2 && mixed && far <= H;
-  };
   const int sy = (int)L.sy, sz = (int)L.sz;
   double raw[PER];
   unsigned int at[PER];
   unsigned int mx = 0, any = 0, mn = 0xffffffffu;
-  auto load = [&]() {
 #pragma unroll
-    for (int q = 0; q < PER; ++q) {
-      raw[q] = 0.0;
-      at[q] = 0xffffffffu;
-      if (q >= PERL && !mixed) continue;
-      const int c = threadIdx.x + q * FX_THREADS;
-      if (c < count) at[q] = __ldg(&g_fx_box<P>.at[c]);
-    }
+  for (int q = 0; q < PER; ++q) {
+    raw[q] = 0.0;
+    at[q] = 0xffffffffu;
+    if (q >= PERL && !mixed) continue;
+    const int c = threadIdx.x + q * FX_THREADS;
+    if (c < count) at[q] = __ldg(&g_fx_box<P>.at[c]);
+  }
+  auto load = [&](auto all) {
 #pragma unroll
     for (int q = 0; q < PER; ++q) {
       if (q >= PERL && !mixed) continue;
@@ -724,13 +757,16 @@ __device__ __forceinline__ void fx_tile(const Layout& L, const FxCoef& C, const 
       // (a box spans less than 2^31 elements of a variable unless a plane of
       // the array alone has 2^26 points)
       const long long o = wide ? bx + by * L.sy + bz * L.sz : (long long)(bx + by * sy + bz * sz);
-      if (full ? at[q] != 0xffffffffu : reads(bx, by, bz)) {
+      if (decltype(all)::value ? at[q] != 0xffffffffu : fx_reads<P>(bx, by, bz, ex, ey, ez, mixed, ext)) {
         if (in_range(org - R * (1 + L.sy + L.sz) + o, org - R * (1 + L.sy + L.sz) + o, padded_points(L)))
           raw[q] = __ldg(v0 + o);
       }
     }
   };
-  load();
+  if (full)
+    load(std::true_type{});
+  else
+    load(std::false_type{});
 #pragma unroll
   for (int q = 0; q < PER; ++q) {
     const unsigned int hw = (unsigned int)__double2hiint(raw[q]) & 0x7fffffffu;
@@ -836,12 +872,7 @@ __device__ __forceinline__ void fx_tile(const Layout& L, const FxCoef& C, const 
     for (int w = 0; w < FX_THREADS / 32; ++w) tile |= red[0][w] != 0;
     if (tile) {
       float* rest = (float*)box;
-      load();
-#pragma unroll
-      for (int q = 0; q < PER; ++q) {
-        if (q >= PERL && !mixed) continue;
-        if (at[q] != 0xffffffffu) rest[at[q] >> 16] = fx_rest(raw[q], emax);
-      }
+      fx_rest_box<P>(v0, org - R * (1 + L.sy + L.sz), padded_points(L), L.sy, L.sz, ex, ey, ez, mixed, ext, emax, rest);
       fx_sync();
       const int which = coarse & FX_ALL & ~(coarse >> FX_BEYOND);
       if (which)
