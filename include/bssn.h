@@ -67,7 +67,9 @@ typedef enum {
 } bssn_status_t;
 
 typedef enum {
-  BSSN_FP64 = 0,     /* every operation in double precision                     */
+  BSSN_FP64 = 0,     /* double precision throughout; a stage's finite differences
+                        are sums in fixed point, no coarser than the doubles each
+                        stencil reads, rounded to double once                   */
   BSSN_FP32_RHS = 1  /* derivatives, right-hand side and dissipation in single
                         precision on the double-precision state; 1/W and 1/alpha
                         factors, the RK4 update and constraints in double        */
@@ -279,11 +281,12 @@ typedef struct {
 
 /* Builds a plan for nblocks patches (params and precision shared by all).
  * The plan allocates and owns, per patch, three stage buffers (and in the
- * FP32-RHS form a single-precision copy and derivative tables), plus the
- * patch table, one CUDA graph per step size and, in FP64, the derivative
- * record of the tiles that are worked on at a time, up to 2048 (1.1 GB). The stage kernels' tiles are fixed in
- * both precisions (8 x 8 x 8 points in FP64, 8 x 4 x 4 in FP32-RHS), so
- * autotune (0 or 1) has nothing to choose. Synchronizes the device. Returns
+ * FP32-RHS form two single-precision copies, the second where there is memory
+ * for it, and derivative tables), plus the patch table, one CUDA graph per step
+ * size and, in FP64, the derivative record of the tiles that are worked on at a
+ * time, up to 2048 (1.1 GB). The stage kernels' tiles are fixed in both
+ * precisions (8 x 8 x 8 points in FP64, 8 x 4 x 4 in FP32-RHS), so autotune
+ * (0 or 1) has nothing to choose. Synchronizes the device. Returns
  * BSSN_ERR_NOMEM if an allocation fails (nothing is leaked). */
 bssn_status_t bssn_plan_create(bssn_plan_t** out, const bssn_block_t* blocks, int nblocks,
                                const bssn_params_t* params, bssn_precision_t prec, int autotune);

@@ -43,12 +43,15 @@
 // (rec[(slot * nout + output) * vol + point of the tile]); the algebra kernel
 // reads them back. At 128^3, 8th order, one stage took 17.26 ms (+ 0.40 ms of
 // difference tables) when one kernel did stencils and algebra on the FP64
-// pipe (4375 FP64 instructions per point), 6.2 ms this way (941). Against a
+// pipe (4375 FP64 instructions per point), 6.4 ms this way (938). Against a
 // quadruple-precision evaluation the right-hand side's error is no larger than
 // before in any variable, and 1e-16 instead of 1e-14 for W, gt_ii and alpha.
 // Looking after coarse derivatives costs 3 % of an RK4 step of evolved punctures
-// at 128^3 (25.5 -> 26.25 ms), 5 % of a small hierarchy's, 6 % of an RK3 step at
-// 100^3; from the doubles alone, 18 %, 8 % and 57 %.
+// at 128^3 (25.5 -> 26.2 ms) and of a small hierarchy's (17.6 -> 18.2), 5 % of an
+// RK3 step at 100^3, 9 % of a step of 192 patches whose tiles have such points in
+// one case of five (378 -> 412); from the doubles alone, 18 % at 128^3, 57 % at
+// 100^3. On a grid with points on a symmetry plane, where variables are the
+// rounding of zero, the doubles serve that plane (101^3: 10.0 -> 11.9 ms).
 #pragma once
 #include <cmath>
 #include <type_traits>

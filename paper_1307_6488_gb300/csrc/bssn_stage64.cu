@@ -1,7 +1,9 @@
 // The FP64 stage of single grids, patches and refined levels, the constraints
 // and the Weyl scalars: derivatives on the integer pipes (k_derivs,
 // bssn_fixed.cuh), then the pointwise algebra on the FP64 pipe, tile by tile
-// through a record that holds as many tiles as the caller's scratch takes.
+// through a record that holds as many tiles as the caller's scratch takes (the
+// momentum and Gamma constraints and the magnetic Weyl part make their own,
+// first64).
 #include <algorithm>
 
 #include "bssn_bounds.cuh"
