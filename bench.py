@@ -46,13 +46,13 @@ except (OSError, ValueError):
 # of the four stages' launches of one RK4 step at 128^3, from one ncu capture
 # of the same source (profiles/k_overlap_fp64_bl128.md); ignored when the
 # kernel source has changed.
-TRAFFIC = {"src_sha": "08d1f25a78d5368d", "bytes_per_stage_128": (25530335488 + 33049517056) / 4}
+TRAFFIC = {"src_sha": "074d0257d7a073e4", "bytes_per_stage_128": (25530335488 + 33049517056) / 4}
 # FP64 pipe utilisation of the kernel that does most of it, k_overlap
 # (sm__pipe_fp64_cycles_active, percent of peak over active cycles), and the
 # FP64 instructions of a stage per interior point, mean of the four stages
 # (smsp__sass_thread_inst_executed_op_{dfma,dadd,dmul}_pred_on.sum / 128^3),
 # for the same source.
-FP64_PIPE_BUSY = {"src_sha": "08d1f25a78d5368d", "pct_of_active_cycles": 52.46, "dfma_per_point": 705.0,
+FP64_PIPE_BUSY = {"src_sha": "074d0257d7a073e4", "pct_of_active_cycles": 52.46, "dfma_per_point": 705.0,
                   "dadd_per_point": 47.0, "dmul_per_point": 186.0}
 # The same for the tiled FP32-RHS stage kernel k_stage32t<8,0> as the bench
 # times it (per-stage calls; the roofline's 864 B per point is the average of

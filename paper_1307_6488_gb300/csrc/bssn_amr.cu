@@ -53,7 +53,8 @@
 // kernel, bssn_stage32.cuh) over all patches of the level, the
 // radiative boundary kernel on level 0, then the two substeps of the finer
 // level and the restriction. Every kernel walks a flat entry or tile list
-// grid-stride: no device-side waits, no atomics, deterministic results.
+// grid-stride: no device-side waits, no sums across threads, deterministic
+// results.
 #include <cuda_runtime.h>
 
 #include <algorithm>

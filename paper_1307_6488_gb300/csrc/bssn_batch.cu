@@ -9,8 +9,9 @@
 // (static ghost fill, stage), then a final ghost fill. A stage is the single
 // grids' kernels over the tiles of all patches: k_derivs and k_algebra in
 // FP64 (bssn_stage64.cu), tables and k_stage32t_batch in the FP32-RHS form (the
-// first stage also converts the state). No device-side waiting between blocks, no atomics, and a
-// deterministic result; the per-point arithmetic is the single grids'.
+// first stage also converts the state). No device-side waiting between blocks, no
+// sums across threads, and a deterministic result; the per-point arithmetic is
+// the single grids'.
 #include <cuda_runtime.h>
 
 #include <algorithm>
